@@ -21,13 +21,10 @@ constexpr int kClosureWarps = kClosureThreads / 32;
 //  * warps 1..3 meanwhile sum the FM bands (Eq. fm, n = 0 outside the domain) from the slice
 //    densities staged in shared memory; chi = chi_SET(pi sigma^3 nbar / 6) (Eqs. chi, chi_ret),
 //    or chi at the local density;
-//  * the J1 gradients (Eq. j1) as stencils of logarithms of ratios to the own cell, exact
-//    because the stencil weights sum to zero:  sum_q w_q ln(n_q^2 chi_q T_q) = sum_q w_q
-//    [2 log1p(dn_q / n) + log1p(dchi_q / chi) + log1p(dT_q / T)], the differences taken in the
-//    wide type; velocity gradients from wide differences;
-//  * mu, Pr, tau (Eqs. viscosity, prandtl, tau), the covariant strain and the Shakhov
-//    coefficient; the recurrences of the expansion coefficients of the equilibria (Sec. III.C;
-//    warp = axis, lane = cell) and the per-axis vectors g_2, g_R, g_3 (whole block).
+//  * the J1 gradients (Eq. j1) from the differences of neighbouring reach cells (clo_pair_terms), the
+//    covariant strain;
+//  * mu, Pr, tau (Eqs. viscosity, prandtl, tau) and the Shakhov coefficient; the recurrences of the
+//    expansion coefficients of the equilibria (Sec. III.C) and the per-axis vectors g_2, g_R, g_3.
 // chi and nbar of the own cells also go to a small side buffer, from which ca_kernel forms the
 // FP64 closure record of the moments and closure queries.
 // Wall items (kind 1 + side, part): the block sums the outgoing flux of one part of the momenta
@@ -35,32 +32,36 @@ constexpr int kClosureWarps = kClosureThreads / 32;
 // Output: the per-cell collision record in the populations' precision, [20 scalars | g_2 | g_R
 // | g_3].
 __host__ __device__ inline int closure_tab_elems(int nR, int n2, int n3) {
-    return 4 * kMaxE + 2 + (nR + n2 + n3) * kMaxE + 2 * nR + n2 + n3;
+    return (2 * (nR + n2 + n3) + 3) / 4 * 4 + (nR + n2 + n3) * kMaxE + 4 * kMaxE + 2;
 }
 // dynamic shared memory: [staged band rows | tables | band-union densities]
 __host__ __device__ inline size_t closure_smem_bytes(int nR, int n2, int n3, int max_union, int wst_elems, int tsize) {
     return (size_t)wst_elems * tsize + ((size_t)closure_tab_elems(nR, n2, n3) + (size_t)max_union) * tsize + 16;
 }
 
-// Position q of the five-point derivative stencil of cell c (the stencils of stencil5).
+// The five-point derivative stencil of cell c in the mapped coordinate (gradients of Eq. j1; fourth
+// order: central in the interior, one-sided at the two cells next to each wall) as weights of the four
+// differences y[base + p + 1] - y[base + p] of its ascending cells: the weights of the values sum to
+// zero, so weight p is the sum of the value weights above position p.
 template <typename R>
-__device__ __forceinline__ void stencil5_at(int c, int N, int q, int& cell, R& w) {
+__device__ __forceinline__ void stencil5_pairs(int c, int N, int& base, R (&w)[4]) {
     const R k = R(1) / R(12);
     if (c >= 2 && c <= N - 3) {
-        cell = c - 2 + q;
-        w = q == 0 ? k : q == 1 ? R(-8) * k : q == 2 ? R(0) : q == 3 ? R(8) * k : -k;
-    } else if (c == 0) {
-        cell = q;
-        w = q == 0 ? R(-25) * k : q == 1 ? R(48) * k : q == 2 ? R(-36) * k : q == 3 ? R(16) * k : R(-3) * k;
-    } else if (c == 1) {
-        cell = q;
-        w = q == 0 ? R(-3) * k : q == 1 ? R(-10) * k : q == 2 ? R(18) * k : q == 3 ? R(-6) * k : k;
-    } else if (c == N - 2) {
-        cell = N - 1 - q;
-        w = q == 0 ? R(3) * k : q == 1 ? R(10) * k : q == 2 ? R(-18) * k : q == 3 ? R(6) * k : -k;
+        base = c - 2;
+        w[0] = w[3] = -k;
+        w[1] = w[2] = R(7) * k;
+    } else if (c < 2) {
+        base = 0;
+        w[0] = (c == 0 ? R(25) : R(3)) * k;
+        w[1] = (c == 0 ? R(-23) : R(13)) * k;
+        w[2] = (c == 0 ? R(13) : R(-5)) * k;
+        w[3] = (c == 0 ? R(-3) : R(1)) * k;
     } else {
-        cell = N - 1 - q;
-        w = q == 0 ? R(25) * k : q == 1 ? R(-48) * k : q == 2 ? R(36) * k : q == 3 ? R(-16) * k : R(3) * k;
+        base = N - 5;
+        w[0] = (c == N - 1 ? R(-3) : R(1)) * k;
+        w[1] = (c == N - 1 ? R(13) : R(-5)) * k;
+        w[2] = (c == N - 1 ? R(-23) : R(13)) * k;
+        w[3] = (c == N - 1 ? R(25) : R(3)) * k;
     }
 }
 
@@ -77,80 +78,76 @@ struct ClosureTabs {
 };
 
 // The closure's tables in shared memory (closure_tab_elems elements from `base`), filled by the
-// block's threads; the caller synchronises.
+// block's threads; the caller synchronises.  The two spans of the device table that hold them (nodes
+// and weights from o_pR; equilibrium tables and recurrence from o_GR) are contiguous, so the copy is
+// one loop whose loads are all in flight: table by table, each with its own wait on L2, the copy took
+// 5000 cycles before every closure (cylinder, 16 x 8 x 8).
 template <typename T>
 __device__ ClosureTabs<T> closure_tables(T* base, const void* tabTv, const MomSet& M, int tid, int NT) {
-    const int nR = M.nR, n2 = M.n2, n3 = M.n3;
+    const int nR = M.nR, n2 = M.n2, n3 = M.n3, ng = nR + n2 + n3;
+    const int nA = 2 * ng, oB = (nA + 3) / 4 * 4, nB = ng * kMaxE + 3 * kMaxE + 1;  // (rows of GR on 16 bytes)
     ClosureTabs<T> t;
-    t.ha = base;
-    t.hb = t.ha + kMaxE;
-    t.ihb = t.hb + kMaxE + 1;  // 1 / hb
-    t.h0t = t.ihb + kMaxE + 1;
-    t.GR = t.h0t + kMaxE;
+    t.pRt = base;
+    t.wRt = t.pRt + nR;
+    t.w2t = t.wRt + nR + n2;
+    t.w3t = t.w2t + n2 + n3;
+    t.GR = base + oB;
     t.G2 = t.GR + nR * kMaxE;
     t.G3 = t.G2 + n2 * kMaxE;
-    t.pRt = t.G3 + n3 * kMaxE;
-    t.wRt = t.pRt + nR;
-    t.w2t = t.wRt + nR;
-    t.w3t = t.w2t + n2;
+    t.ha = t.G3 + n3 * kMaxE;
+    t.hb = t.ha + kMaxE;
+    t.h0t = t.hb + kMaxE + 1;
+    t.ihb = base + oB + nB;  // 1 / hb
     const T* tabT = reinterpret_cast<const T*>(tabTv);
-    for (int e = tid; e < kMaxE; e += NT) {
-        t.ha[e] = tabT[M.o_ha + e];
-        t.h0t[e] = tabT[M.o_h0 + e];
-    }
+#pragma unroll 4
+    for (int e = tid; e < oB + nB; e += NT) base[e] = tabT[e < oB ? M.o_pR + e : M.o_GR + e - oB];
     for (int e = tid; e <= kMaxE; e += NT) {
-        t.hb[e] = tabT[M.o_hb + e];
-        t.ihb[e] = t.hb[e] != T(0) ? T(1) / t.hb[e] : T(0);
+        const T h = tabT[M.o_hb + e];
+        t.ihb[e] = h != T(0) ? T(1) / h : T(0);
     }
-    for (int e = tid; e < nR * kMaxE; e += NT) t.GR[e] = tabT[M.o_GR + e];
-    for (int e = tid; e < n2 * kMaxE; e += NT) t.G2[e] = tabT[M.o_G2 + e];
-    for (int e = tid; e < n3 * kMaxE; e += NT) t.G3[e] = tabT[M.o_G3 + e];
-    for (int e = tid; e < nR; e += NT) {
-        t.pRt[e] = tabT[M.o_pR + e];
-        t.wRt[e] = tabT[M.o_wR + e];
-    }
-    for (int e = tid; e < n2; e += NT) t.w2t[e] = tabT[M.o_w2 + e];
-    for (int e = tid; e < n3; e += NT) t.w3t[e] = tabT[M.o_w3 + e];
     return t;
 }
 
 // One thread's share of part `part` (of P) of the outgoing flux through a wall (side 0: inner,
-// 1: outer): the sum over the outgoing momenta of |p_R| w vhat, vhat the WENO5 value at the
-// wall face from the wall cell, its neighbour and the cubic extrapolation outside.  `wall` points
-// at the populations of the wall cell (cell 0 or N-1), `st` is the step to the next cell inward
-// (the rows may be in global or shared memory).  `tl` is the thread's index in a block of
-// kClosureThreads threads, whose order of the sums this follows.
+// 1: outer): the sum over the outgoing momenta (half of the radial nodes; of the reduced pair phi's
+// alone, the mass flux) of |p_R| times the WENO5 value at the wall face, from the wall cell, its
+// neighbours and the cubic extrapolation outside, in the stage kernel's form (f itself, epsilon
+// scaled by w^2).  `wall` points at the populations of the wall cell (cell 0 or N-1), `st` is the step
+// to the next cell inward (the rows may be in global or shared memory).  `tl` is the thread's index in
+// a block of kClosureThreads threads, whose order of the sums this follows.
 template <typename T>
 __device__ T wall_flux_partial(const T* wall, long long st, const MomSet& M, const ClosureTabs<T>& tb, int side, int part,
                                int P, int tl) {
-    const int Np = M.Np, nR = M.nR, n2 = M.n2, NT = kClosureThreads;
-    const int mlo = (int)((long long)Np * part / P), mhi = (int)((long long)Np * (part + 1) / P);
-    const long long base = 0;
+    const int nR = M.nR, n2 = M.n2, QR = nR / 2, NT = kClosureThreads;
+    const int Nout = QR * n2 * (M.reduced ? 1 : M.n3);
+    const int mlo = (int)((long long)Nout * part / P), mhi = (int)((long long)Nout * (part + 1) / P);
+    const T sg = side == 0 ? T(-3) : T(3), dL = side == 0 ? T(0.3) : T(0.1), dR = side == 0 ? T(0.1) : T(0.3);
     T acc = T(0);
     for (int m0 = mlo + tl; m0 < mhi; m0 += 4 * NT) {
         // four momenta per pass so that their sixteen loads are in flight together
         T fv[4][4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int m = min(m0 + u * NT, mhi - 1);
+            const int mo = m0 + u * NT;
+            if (mo < mhi) {
+                const int k = mo / (QR * n2), rem = mo % (QR * n2);
+                const int m = k * nR * n2 + (side == 0 ? QR * n2 : 0) + rem;
 #pragma unroll
-            for (int r = 0; r < 4; ++r) fv[u][r] = wall[base + m + r * st];
+                for (int r = 0; r < 4; ++r) fv[u][r] = wall[m + r * st];
+            }
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int m = m0 + u * NT;
-            if (m >= mhi) continue;
-            const int k = m / (nR * n2), rem = m % (nR * n2), i = rem / n2, j = rem % n2;
-            const T pr = tb.pRt[i];
-            if (side == 0 ? !(pr < T(0)) : !(pr > T(0))) continue;
-            if (M.reduced && k > 0) continue;  // the mass flux is phi's (chi = int p_z^2 f)
-            const T wm = tb.wRt[i] * tb.w2t[j] * tb.w3t[k];
-            const T iw = wm > (sizeof(T) == 4 ? T(1e-30) : T(0)) ? T(1) / wm : T(0);  // as the stage kernel
+            const int mo = m0 + u * NT;
+            if (mo >= mhi) continue;
+            const int k = mo / (QR * n2), rem = mo % (QR * n2), i = (side == 0 ? QR : 0) + rem / n2, j = rem % n2;
+            const T wm = mul_rn(mul_rn(tb.wRt[i], tb.w3t[k]), tb.w2t[j]), ew = mul_rn(mul_rn(T(4e-6), wm), wm);
+            const T e4 = sizeof(T) == 4 ? fmax(ew, T(1e-37)) : ew;
             const T f0 = fv[u][0], f1 = fv[u][1], f2 = fv[u][2], f3 = fv[u][3];
-            const T g1 = T(4) * f0 - T(6) * f1 + T(4) * f2 - f3;
-            const T g2 = T(10) * f0 - T(20) * f1 + T(15) * f2 - T(4) * f3;
-            const T vh = weno5(f2 * iw, f1 * iw, f0 * iw, g1 * iw, g2 * iw);
-            acc += fabs(pr) * wm * vh;
+            const T g1 = fma(T(4), f0, fma(T(-6), f1, fma(T(4), f2, -f3)));
+            const T g2 = fma(T(10), f0, fma(T(-20), f1, fma(T(15), f2, mul_rn(T(-4), f3))));
+            const T vh = side == 0 ? weno5_one(g2, g1, f0, f1, f2, sg, dL, dR, e4) : weno5_one(f2, f1, f0, g1, g2, sg, dL, dR, e4);
+            acc = fma(fabs(tb.pRt[i]), vh, acc);
         }
     }
     return acc;
@@ -162,10 +159,25 @@ __device__ __forceinline__ T wall_part_sum(const T* r) {
     return (r[0] + r[1]) + (r[2] + r[3]);
 }
 
+// A part of the wall flux by one warp, in the order of the closure kernel's block of kClosureThreads
+// threads: lane L takes the momenta of its threads L, L + 32, L + 64, L + 96 and the four warp sums are
+// combined as there.  Lane 0 returns the part.
+template <typename T>
+__device__ T wall_part_of_warp(const T* fin, const MomSet& M, const ClosureTabs<T>& tb, const InstDev& I, int side, int part,
+                               int P, int lane) {
+    const T* wall = fin + I.f_off + (side == 0 ? 0LL : (long long)(I.n_cells - 1) * M.Np);
+    T r[kClosureWarps];
+#pragma unroll
+    for (int vw = 0; vw < kClosureWarps; ++vw)
+        r[vw] = warp_sum(wall_flux_partial<T>(wall, side == 0 ? (long long)M.Np : -(long long)M.Np, M, tb, side, part, P,
+                                              32 * vw + lane));
+    return wall_part_sum(r);
+}
+
 struct NoExtra {
     __device__ void operator()(int, int) const {}
 };
-struct NoAfterLoads {
+struct NoHook {
     __device__ void operator()() const {}
 };
 
@@ -208,20 +220,32 @@ __device__ __forceinline__ void clo_fields(const Wide<T> (&sv)[kSums], Wide<T>& 
                                            T (&q)[3]) {
     using W = Wide<T>;
     n = sv[0];
-    u[0] = w_div(sv[1], n);
-    u[1] = w_div(sv[2], n);
-    u[2] = w_div(sv[3], n);
     const W tr = w_add(w_add(sv[4], sv[5]), sv[6]);
-    const W uu = w_add(w_add(w_mul(u[0], u[0]), w_mul(u[1], u[1])), w_mul(u[2], u[2]));
-    Tc = w_div(w_sub(tr, w_mul(n, uu)), w_scale(n, T(3)));
-    const T tn = w_hi(n), t0 = w_hi(u[0]), t1 = w_hi(u[1]), t2 = w_hi(u[2]), ttr = w_hi(tr), tuu = w_hi(uu);
+    if constexpr (sizeof(T) == 8) {
+        // one division for the four quotients by n (a division is nine FP64 operations)
+        const T in = T(1) / n.v;
+        u[0].v = mul_rn(sv[1].v, in);
+        u[1].v = mul_rn(sv[2].v, in);
+        u[2].v = mul_rn(sv[3].v, in);
+        const T uu = fma(u[0].v, u[0].v, fma(u[1].v, u[1].v, mul_rn(u[2].v, u[2].v)));
+        Tc.v = mul_rn(mul_rn(fma(-n.v, uu, tr.v), in), T(1.0 / 3.0));
+    } else {
+        u[0] = w_div(sv[1], n);
+        u[1] = w_div(sv[2], n);
+        u[2] = w_div(sv[3], n);
+        const W uu = w_add(w_add(w_mul(u[0], u[0]), w_mul(u[1], u[1])), w_mul(u[2], u[2]));
+        Tc = w_div(w_sub(tr, w_mul(n, uu)), w_scale(n, T(3)));
+    }
+    const T tn = w_hi(n), t0 = w_hi(u[0]), t1 = w_hi(u[1]), t2 = w_hi(u[2]), ttr = w_hi(tr);
+    const T tuu = fma(t0, t0, fma(t1, t1, mul_rn(t2, t2))), nuu = mul_rn(tn, tuu);
     const T s4 = w_hi(sv[4]), s5 = w_hi(sv[5]), s6 = w_hi(sv[6]), s7 = w_hi(sv[7]), s8 = w_hi(sv[8]), s9 = w_hi(sv[9]);
-    const T m0 = s4 * t0 + s7 * t1 + s8 * t2;
-    const T m1 = s7 * t0 + s5 * t1 + s9 * t2;
-    const T m2 = s8 * t0 + s9 * t1 + s6 * t2;
-    q[0] = T(0.5) * (w_hi(sv[10]) - T(2) * m0 - t0 * ttr + T(2) * tn * tuu * t0);
-    q[1] = T(0.5) * (w_hi(sv[11]) - T(2) * m1 - t1 * ttr + T(2) * tn * tuu * t1);
-    q[2] = T(0.5) * (w_hi(sv[12]) - T(2) * m2 - t2 * ttr + T(2) * tn * tuu * t2);
+    const T m0 = fma(s4, t0, fma(s7, t1, mul_rn(s8, t2)));
+    const T m1 = fma(s7, t0, fma(s5, t1, mul_rn(s9, t2)));
+    const T m2 = fma(s8, t0, fma(s9, t1, mul_rn(s6, t2)));
+    // (S3_a - 2 m_a - u_a tr S2 + 2 n u^2 u_a) / 2
+    q[0] = mul_rn(T(0.5), fma(mul_rn(T(2), nuu), t0, fma(-t0, ttr, fma(T(-2), m0, w_hi(sv[10])))));
+    q[1] = mul_rn(T(0.5), fma(mul_rn(T(2), nuu), t1, fma(-t1, ttr, fma(T(-2), m1, w_hi(sv[11])))));
+    q[2] = mul_rn(T(0.5), fma(mul_rn(T(2), nuu), t2, fma(-t2, ttr, fma(T(-2), m2, w_hi(sv[12])))));
 }
 
 // The FM band sum of one row (Eq. fm; a whole warp, every lane returns the sum): weights Wr[k]
@@ -305,6 +329,40 @@ __device__ __forceinline__ void clo_band_row2(const T* WrA, const DensA& dnA, in
     totB = warp_sum((b0 + b1) + (b2 + b3));
 }
 
+// R rows of at most 32 U columns (U <= 4) by one warp, each summed exactly as clo_band_row sums it, with
+// the loads of all rows in flight together; every lane passes the row pointers and extents.
+template <typename T, int R, int U>
+__device__ __forceinline__ void clo_band_rows(const T* const (&Wr)[R], const T* const (&nd)[R], const int (&kmax)[R],
+                                              int slices, int lane, T (&tot)[R]) {
+    T w[R][4], d[R][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = lane + 32 * u;
+            w[r][u] = d[r][u] = T(0);
+            if (u < U && k < kmax[r]) {
+                w[r][u] = Wr[r][k];
+                d[r][u] = nd[r][(long long)k * slices];
+                for (int sl = 1; sl < slices; ++sl) d[r][u] += nd[r][(long long)k * slices + sl];
+            }
+        }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        // four accumulators where all four columns are in the row, else one
+        T a0 = fma(w[r][0], d[r][0], T(0)), a1 = T(0), a2 = T(0), a3 = T(0);
+        if (U == 4 && lane + 96 < kmax[r]) {
+            a1 = fma(w[r][1], d[r][1], T(0));
+            a2 = fma(w[r][2], d[r][2], T(0));
+            a3 = fma(w[r][3], d[r][3], T(0));
+        } else {
+            a0 = fma(w[r][1], d[r][1], a0);
+            if (U == 4) a0 = fma(w[r][2], d[r][2], a0);
+        }
+        tot[r] = warp_sum((a0 + a1) + (a2 + a3));
+    }
+}
+
 // chi = chi_SET(eta), eta = etafac x (Eqs. chi, chi_ret), in the wide type, rounded once: J1
 // scales with b rho chi, and near finely resolved walls J1 is large enough that a few roundings of
 // chi show in the right-hand side.
@@ -323,92 +381,99 @@ struct ReachView {
     const Wide<T>* n;
     const Wide<T>* Tc;
     const Wide<T>* u[3];
-    const T* chi;
     const T* nb;
 };
 
-// Position q of the J1 gradient stencils of own cell c (reach index lt; the stencil cell has
-// reach index k, weight wq): the five gradient terms, logarithms of ratios to the own cell, exact
-// because the stencil weights sum to zero:
-//   sum_q w_q ln(n_q^2 chi_q T_q) = sum_q w_q [2 log1p(dn_q / n) + log1p(dchi_q / chi) + log1p(dT_q / T)],
-// the differences taken in the wide type; ln chi_q - ln chi_c from the packing-fraction
-// difference alone, since ln chi(eta) = ln(2 - eta) - ln 2 - 3 ln(1 - eta) (no rounding noise of
-// chi itself); velocity differences in the wide type.
+// The terms of the J1 gradients (Eq. j1) of the neighbouring reach cells lt and lt + 1: the
+// differences of ln(n^2 chi T), ln T and the three velocities.  A derivative stencil is a weighted sum
+// of four such differences (stencil5_pairs), so each is formed once per pair of cells instead of once
+// per cell and stencil position, with two logarithms instead of four: the ratio of n^2 chi T is the
+// product of 1 + x over the factors' relative differences, and its deviation from one is carried as
+// E <- E + x + E x (every factor is formed from a difference of the wide values, so nothing cancels);
+// ln chi(eta) = ln(2 - eta) - ln 2 - 3 ln(1 - eta) from the packing-fraction difference alone (no
+// rounding noise of chi itself).  The gradients of two cells' closure in FP64 took 20800 cycles with
+// twenty logarithms per cell, a third of the whole chain in FP32.
 template <typename T>
-__device__ __forceinline__ void clo_grad_terms(const ReachView<T>& R, int k, int lt, T wq, T etaf, bool chi_local,
-                                               T (&g)[5]) {
+__device__ __forceinline__ void clo_pair_terms(const ReachView<T>& R, int lt, T etaf, bool chi_local, T (&d)[5]) {
     const Wide<T> nw = R.n[lt], Tw = R.Tc[lt];
-    const T lT = log1p(ratio_fast(w_hi(w_sub(R.Tc[k], Tw)), w_hi(Tw)));
-    const T ln = log1p(ratio_fast(w_hi(w_sub(R.n[k], nw)), w_hi(nw)));
-    const T dnb = chi_local ? w_hi(w_sub(R.n[k], nw)) : R.nb[k] - R.nb[lt];
-    const T etac = etaf * (chi_local ? w_hi(nw) : R.nb[lt]), deta = etaf * dnb;
-    const T lchi = log1p(ratio_fast(-deta, T(2) - etac)) - T(3) * log1p(ratio_fast(-deta, T(1) - etac));
-    g[0] = wq * (T(2) * ln + lchi + lT);
-    g[1] = wq * lT;
-    g[2] = wq * w_hi(w_sub(R.u[0][k], R.u[0][lt]));
-    g[3] = wq * w_hi(w_sub(R.u[1][k], R.u[1][lt]));
-    g[4] = wq * w_hi(w_sub(R.u[2][k], R.u[2][lt]));
+    const T dn = w_hi(w_sub(R.n[lt + 1], nw));
+    const T a = ratio_fast(dn, w_hi(nw)), b = ratio_fast(w_hi(w_sub(R.Tc[lt + 1], Tw)), w_hi(Tw));
+    const T eta = mul_rn(etaf, chi_local ? w_hi(nw) : R.nb[lt]);
+    const T deta = mul_rn(etaf, chi_local ? dn : R.nb[lt + 1] - R.nb[lt]);
+    const T x = ratio_fast(-deta, T(2) - eta);               // (2 - eta') / (2 - eta) - 1
+    const T y = ratio_fast(deta, (T(1) - eta) - deta);        // (1 - eta) / (1 - eta') - 1
+    T E = fma(a, a, mul_rn(T(2), a));                                // (1 + a)^2 - 1
+    E = fma(E, b, E + b);
+    E = fma(E, x, E + x);
+    E = fma(E, y, E + y);
+    E = fma(E, y, E + y);
+    E = fma(E, y, E + y);
+    d[0] = log1p(E);
+    d[1] = log1p(b);
+    d[2] = w_hi(w_sub(R.u[0][lt + 1], R.u[0][lt]));
+    d[3] = w_hi(w_sub(R.u[1][lt + 1], R.u[1][lt]));
+    d[4] = w_hi(w_sub(R.u[2][lt + 1], R.u[2][lt]));
 }
 
-// The 20 scalars of an own cell's collision record: n, u, 1/T, 1/tau (Eq. tau), the Shakhov
-// coefficient (Eq. prandtl), q, -b rho chi, the J1 gradients X = d ln(n^2 chi T), Y = d ln T, the
-// velocity derivative, the covariant strain (cylinder / sphere) and its divergence (Eq. j1);
-// mu from Eq. viscosity.  Products the stage kernel would otherwise form per cell and thread are
-// stored in place of their factors that it uses nowhere else: 0.4 S_11 / T in place of S_11,
-// 2 S_01 / T in place of S_01, 1 / (2T) in the spare slot 18.  gp[v][q]: the gradient terms of the cell's five stencil positions.
+// The collision record's 20 scalars of an own cell, in two independent halves (entry 0, the density of
+// f^MB, follows with the equilibrium vectors).  The transport half: u, 1/T, 1/tau (Eq. tau, mu from Eq. viscosity), the Shakhov coefficient (Eq. prandtl), q and
+// -b rho chi.  With x = b rho chi and P(x) = 1 + 4/5 x + 4/25 (1 + 12/pi) x^2, mu is mu0 P / chi and the
+// Prandtl number 2/3 P / Q, so the two share P and 1/tau = n sqrt(T) chi (16 sigma^2 sqrt(pi) / 5) / P.
 template <typename T>
-__device__ __forceinline__ void clo_record_scalars(T* ct, const ReachView<T>& R, int lt, const T (&gp)[5][5], T geo0,
-                                                   T geo1, const T (&q)[3], const InstDev& I) {
+__device__ __forceinline__ void clo_record_transport(T* ct, Wide<T> nw, T cu0, T cu1, T cu2, T cT, T cchi, const T (&q)[3],
+                                                     const InstDev& I) {
     using C = T;
-    const C cn = w_hi(R.n[lt]), cT = w_hi(R.Tc[lt]), cchi = R.chi[lt];
-    const C in = ratio_fast(C(1), cn), iT = ratio_fast(C(1), cT), ichi = ratio_fast(C(1), cchi);
-    C gsum[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) gsum[v] = (gp[v][0] + gp[v][1]) + (gp[v][2] + gp[v][3]) + gp[v][4];
-    const C sc = geo1 * inst_param<C>(1.0 / I.ds, I.f_ids);
-    const C X = gsum[0] * sc, Y = gsum[1] * sc;
-    const C cd0 = gsum[2] * sc, cd1 = gsum[3] * sc, cd2 = gsum[4] * sc;
-    const C iR = ratio_fast(C(1), geo0);
-    const C cu0 = w_hi(R.u[0][lt]), cu1 = w_hi(R.u[1][lt]), cu2 = w_hi(R.u[2][lt]);
+    const C cn = w_hi(nw);
+    const C in = ratio_fast(C(1), cn), iT = ratio_fast(C(1), cT);
     const C sg = inst_param<C>(I.sigma, I.f_sigma);
-    const C br = inst_param<C>(I.bfac, I.f_bfac) * cn, x = br * cchi;
-    const C pi = C(3.14159265358979323846);
-    const C mu = ratio_fast(C(5), C(16) * sg * sg) * sqrt(cT * C(0.31830988618379067154)) *
-                 (ichi + C(0.8) * br + C(4.0 / 25.0) * (C(1) + C(12) / pi) * br * br * cchi);
-    const C Pr = ratio_fast(C(2.0 / 3.0) * (C(1) + C(0.8) * x + C(4.0 / 25.0) * (C(1) + C(12) / pi) * x * x),
-                            C(1) + C(1.2) * x + C(9.0 / 25.0) * (C(1) + C(32) / (C(9) * pi)) * x * x);
-    C S11, S22, S01, S02, div;
-    if (I.geometry == 0) {
-        S11 = cu0 * iR;
-        S22 = C(0);
-        S01 = C(0.5) * (cd1 - cu1 * iR);
-        S02 = C(0.5) * cd2;
-        div = cd0 + cu0 * iR;
-    } else {
-        S11 = S22 = cu0 * iR;
-        S01 = C(0.5) * (cd1 - cu1 * iR);
-        S02 = C(0.5) * (cd2 - cu2 * iR);
-        div = cd0 + C(2) * cu0 * iR;
-    }
-    ct[0] = cn;
+    const C x = mul_rn(mul_rn(inst_param<C>(I.bfac, I.f_bfac), cn), cchi);
+    constexpr double pi = 3.14159265358979323846;
+    const C P = fma(x, fma(C(4.0 / 25.0 * (1.0 + 12.0 / pi)), x, C(0.8)), C(1));
+    const C Q = fma(x, fma(C(9.0 / 25.0 * (1.0 + 32.0 / (9.0 * pi))), x, C(1.2)), C(1));
+    const C Pr1 = fma(C(-2.0 / 3.0), ratio_fast(P, Q), C(1));  // 1 - Pr
     ct[1] = cu0;
     ct[2] = cu1;
     ct[3] = cu2;
     ct[4] = iT;
-    ct[5] = ratio_fast(cn * cT, mu);
-    ct[6] = (C(1) - Pr) * iT * iT * in;
+    ct[5] = ratio_fast(mul_rn(mul_rn(mul_rn(cn, sqrt(cT)), cchi), mul_rn(mul_rn(C(5.671852322897651), sg), sg)), P);
+    ct[6] = mul_rn(mul_rn(mul_rn(Pr1, iT), iT), in);
     ct[7] = q[0];
     ct[8] = q[1];
     ct[9] = q[2];
     ct[10] = -x;
-    ct[11] = X;
-    ct[12] = Y;
-    ct[13] = cd0;
-    ct[14] = T(0.4) * iT * S11;
+}
+
+// The gradient half: X = d ln(n^2 chi T), Y = d ln T, the radial velocity's derivative, the covariant
+// strain (cylinder / sphere) and its divergence (Eq. j1).  Products the stage kernel would otherwise
+// form per cell and thread are stored in place of their factors that it uses nowhere else:
+// 0.4 S_11 / T in place of S_11, 2 S_01 / T in place of S_01, 1 / (2T) in the spare slot 18.
+// gp[v]: the pair terms of the reach (32 per term); base - h0: the stencil's first pair.
+template <typename T>
+__device__ __forceinline__ void clo_record_gradients(T* ct, int c, int N, int h0, const T (*gp)[32], T cu0, T cu1, T cu2,
+                                                     T cT, T geo0, T geo1, const InstDev& I) {
+    using C = T;
+    const C iT = ratio_fast(C(1), cT), iR = ratio_fast(C(1), geo0);
+    const C sc = mul_rn(geo1, inst_param<C>(1.0 / I.ds, I.f_ids));
+    int base;
+    C w[4];
+    stencil5_pairs<C>(c, N, base, w);
+    base -= h0;
+    C g[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v)
+        g[v] = mul_rn(sc, fma(w[3], gp[v][base + 3], fma(w[2], gp[v][base + 2], fma(w[1], gp[v][base + 1], mul_rn(w[0], gp[v][base])))));
+    const C S11 = mul_rn(cu0, iR), S22 = I.geometry == 0 ? C(0) : S11;
+    const C S01 = mul_rn(C(0.5), fma(-cu1, iR, g[3]));
+    const C S02 = mul_rn(C(0.5), I.geometry == 0 ? g[4] : fma(-cu2, iR, g[4]));
+    const C div = I.geometry == 0 ? g[2] + S11 : fma(C(2), S11, g[2]);
+    ct[11] = g[0];
+    ct[12] = g[1];
+    ct[13] = g[2];
+    ct[14] = mul_rn(mul_rn(T(0.4), iT), S11);
     ct[15] = S22;
-    ct[16] = T(2) * iT * S01;
+    ct[16] = mul_rn(mul_rn(T(2), iT), S01);
     ct[17] = S02;
-    ct[18] = T(0.5) * iT;
+    ct[18] = mul_rn(T(0.5), iT);
     ct[19] = div;
 }
 
@@ -437,27 +502,28 @@ __device__ __forceinline__ void clo_eq_coeffs(int job, T cT, T tm1, T ur, T ua, 
         //   b_{l+1} d_{l+1} = (v - a_l) d_l + (T - 1) b_l e_{l-1}
         //                     + T h_l(0) [D - sum_{k<l} h_k(0) d_k] / sqrt(2 pi).
         const C v = job == 0 ? ur : -ur;
-        const C sT = sqrt(cT), z = v * rsqrt(C(2) * cT);
-        const C D = (expm1(-z * z) - tm1 / (C(1) + sT)) / sT;
+        const C sT = sqrt(cT), z = mul_rn(ur, rsqrt(mul_rn(C(2), cT)));  // (odd in z: the two halves share erf)
+        const C D = (expm1(mul_rn(-z, z)) - tm1 / (C(1) + sT)) / sT;
+        const C ez = erf(z);
         const C is2pi = C(0.39894228040143267794);
-        const C r0 = h0t[0] * C(0.5);
+        const C r0 = mul_rn(h0t[0], C(0.5));
         C d[kMaxE + 1];
 #pragma unroll
         for (int l = 0; l <= kMaxE; ++l) d[l] = C(0);
-        d[0] = r0 * erf(z);
+        d[0] = mul_rn(r0, job == 0 ? ez : -ez);
         C run = C(0);  // sum_{k<l} h_k(0) d_k
 #pragma unroll
         for (int l = 0; l < kMaxE; ++l) {
             if (l < M.NR) {
                 C val;
                 if (l == 0) {
-                    val = v * r0 + (v - ha[0]) * d[0] + h0t[0] * (tm1 + cT * D) * is2pi;
+                    val = fma(v - ha[0], d[0], fma(v, r0, mul_rn(mul_rn(h0t[0], fma(cT, D, tm1)), is2pi)));
                 } else {
                     const C em1 = (l == 1 ? r0 : C(0)) + d[l > 0 ? l - 1 : 0];
-                    val = (v - ha[l]) * d[l] + tm1 * hb[l] * em1 + cT * h0t[l] * (D - run) * is2pi;
+                    val = fma(v - ha[l], d[l], fma(mul_rn(tm1, hb[l]), em1, mul_rn(mul_rn(cT, h0t[l]), mul_rn(D - run, is2pi))));
                 }
-                run += h0t[l] * d[l];
-                d[l + 1] = val * ihb[l + 1];
+                run = fma(h0t[l], d[l], run);
+                d[l + 1] = mul_rn(val, ihb[l + 1]);
             }
         }
 #pragma unroll
@@ -470,66 +536,69 @@ __device__ __forceinline__ void clo_eq_coeffs(int job, T cT, T tm1, T ur, T ua, 
         ev[1] = Nax >= 1 ? ua : C(0);
 #pragma unroll
         for (int l = 1; l < kMaxE; ++l)
-            if (l < Nax) ev[l + 1] = ua * ev[l] + C(l) * tm1 * ev[l - 1];
+            if (l < Nax) ev[l + 1] = fma(ua, ev[l], mul_rn(mul_rn(C(l), tm1), ev[l - 1]));
     }
 }
 
-// Entry k (of nR + n2 + n3) of an own cell's per-axis equilibrium vectors g_R, g_2, g_3 in the
-// populations' precision; ecs: the cell's coefficients [job][l]; cT its temperature (the reduced
-// pair's chi factor).  Returns the value, *dst its offset in the record.
+// The expansion coefficients of an item's own cells, [job][l][cell]: consecutive cells on consecutive
+// banks for the lane-per-cell writes.
+constexpr int kEcsCells = kClosureCells + 1;
 template <typename T>
-__device__ __forceinline__ T clo_g_entry(int k, const T (*ecs)[kMaxE], T cT, const ClosureTabs<T>& tb, const MomSet& M,
-                                         int& dst) {
+struct EqCoeffs {
+    T v[4][kMaxE][kEcsCells];
+};
+
+// The per-axis equilibrium vectors g_R, g_2, g_3 of an own cell into its record, and the density
+// stored for f^MB, by eight lanes (sub = 0..7, aligned in the warp; every lane of the warp calls, `on`
+// false where there is no cell): two lanes for each job of clo_eq_coeffs (equal shares for equal
+// orders), each holding the job's coefficients and summing its stored entries in the wide type as it
+// forms them.  The rounded vectors need not sum to exactly one per axis, and for FP32 populations that
+// bias, times dt / tau every step, would make the total mass drift: the density for f^MB = n g_R g_2 g_3
+// is the wide n divided by the wide product of the three sums; lane sub = 0 returns it.  ec: the item's
+// coefficients, t: the cell's place in them; cT its temperature (the reduced pair's chi factor).  (Entries
+// by one thread each and then a thread per cell reading them all back cost 4000 cycles of 17600 in the
+// cylinder's closure.)
+template <typename T>
+__device__ __forceinline__ T clo_equilibrium(bool on, int sub, T* ct, Wide<T> n, T cT, const EqCoeffs<T>& ec, int t,
+                                             const ClosureTabs<T>& tb, const MomSet& M) {
+    using W = Wide<T>;
     const int nR = M.nR, n2 = M.n2, QR = nR / 2;
-    T acc = T(0);
-    // (the expansion orders are at most kMaxE - 1: every loop runs unrolled, predicated)
-    if (k < nR) {
-        const T* eh = ecs[k >= QR ? 1 : 0];
+    const int job = sub >> 1;
+    const int len = job < 2 ? QR : job == 2 ? n2 : M.n3;
+    const int N = job < 2 ? M.NR : job == 2 ? M.N2 : M.N3;
+    const T* G = job < 2 ? tb.GR + job * QR * kMaxE : job == 2 ? tb.G2 : tb.G3;
+    T* dst = ct + (job < 2 ? rec_off_gR(n2) + job * QR : job == 2 ? rec_off_g2() : rec_off_g3(nR, n2));
+    const bool pair = job == 3 && M.reduced;  // the pair's factors: int g_z = 1 (phi), int p_z^2 g_z = T (chi)
+    W sum = w_from_t(T(0));
+    if (on) {
+        // (the expansion orders are at most kMaxE - 1: the coefficients beyond are zero)
+        T e[kMaxE];
 #pragma unroll
-        for (int l = 0; l < kMaxE; ++l)
-            if (l <= M.NR) acc += tb.GR[k * kMaxE + l] * eh[l];
-        dst = rec_off_gR(n2) + k;
-    } else if (k < nR + n2) {
-        const int j = k - nR;
+        for (int l = 0; l < kMaxE; ++l) e[l] = l <= N ? ec.v[job][l][t] : T(0);
+        for (int k = sub & 1; k < len; k += 2) {
+            T g[kMaxE];
+            if constexpr (sizeof(T) == 4) {
+                const float4 x = reinterpret_cast<const float4*>(G + k * kMaxE)[0], y = reinterpret_cast<const float4*>(G + k * kMaxE)[1];
+                g[0] = x.x; g[1] = x.y; g[2] = x.z; g[3] = x.w; g[4] = y.x; g[5] = y.y; g[6] = y.z; g[7] = y.w;
+            } else {
 #pragma unroll
-        for (int l = 0; l < kMaxE; ++l)
-            if (l <= M.N2) acc += tb.G2[j * kMaxE + l] * ecs[2][l];
-        dst = rec_off_g2() + j;
-    } else {
-        const int j = k - nR - n2;
-        if (M.reduced) {
-            // the pair's Gaussian factors: int g_z = 1 (phi), int p_z^2 g_z = T (chi)
-            acc = j == 0 ? T(1) : cT;
-        } else {
+                for (int l = 0; l < kMaxE; ++l) g[l] = G[k * kMaxE + l];
+            }
+            T acc = T(0);
 #pragma unroll
             for (int l = 0; l < kMaxE; ++l)
-                if (l <= M.N3) acc += tb.G3[j * kMaxE + l] * ecs[3][l];
+                if (l <= N) acc = fma(g[l], e[l], acc);
+            if (pair) acc = k == 0 ? T(1) : cT;
+            dst[k] = acc;
+            if (!pair || k == 0) sum = w_add(sum, w_from_t(acc));  // (the pair's mass is phi's)
         }
-        dst = rec_off_g3(nR, n2) + j;
     }
-    return acc;
-}
-
-// Discrete mass of the stored equilibrium (one thread per own cell): the rounded vectors need not
-// sum to exactly one per axis, and for FP32 populations that bias, times dt / tau every step, would
-// make the total mass drift.  The density stored for f^MB = n g_R g_2 g_3 is the wide n divided by
-// the wide product of the sums of the stored vectors (wide sums in the order of the entries).
-template <typename T>
-__device__ __forceinline__ void clo_mass_normalise(T* ct, Wide<T> n, const MomSet& M) {
-    using W = Wide<T>;
-    const int nR = M.nR, n2 = M.n2, n3 = M.n3;
-    W sR = w_from_t(T(0)), s2 = w_from_t(T(0)), s3 = w_from_t(T(0));
-    const T* gR = ct + rec_off_gR(n2);
-    const T* g2 = ct + rec_off_g2();
-    const T* g3 = ct + rec_off_g3(nR, n2);
-    for (int k = 0; k < nR; ++k) sR = w_add(sR, w_from_t(gR[k]));
-    for (int k = 0; k < n2; ++k) s2 = w_add(s2, w_from_t(g2[k]));
-    if (M.reduced) {
-        s3 = w_from_t(T(1));  // the mass is phi's: its p_z factor is exactly 1
-    } else {
-        for (int k = 0; k < n3; ++k) s3 = w_add(s3, w_from_t(g3[k]));
-    }
-    ct[0] = w_hi(w_div(n, w_mul(w_mul(sR, s2), s3)));
+    sum = w_add(sum, w_shfl_xor(sum, 1));
+    const W r2 = w_shfl_xor(sum, 2);
+    // lanes 0..3: g_R's two halves added; lanes 4..7: the product of the two full-range sums
+    const W s = job < 2 ? w_add(sum, r2) : w_mul(sum, r2);
+    const W p23 = w_shfl_xor(s, 4);
+    return w_hi(w_div(n, w_mul(s, p23)));
 }
 
 // Reach of an item of own cells [c0, c0 + cnt) of an instance of N cells: the own cells, two on
@@ -543,21 +612,22 @@ __device__ __forceinline__ void clo_reach(int c0, int cnt, int N, int& h0, int& 
 // records go to `recb` (the record of cell c0, stride A.rec_stride), chi and nbar to A.cw.
 // Every thread of the block calls it (it holds block barriers); the block has at least
 // kClosureWarps warps, and warps beyond them run extra(w, nw) (the w-th of nw such warps)
-// while warps 0..2 run the chains of step 3; every thread runs after_loads() once the item's
-// global loads are issued.  `wst` holds A.wst_elems staged band elements, `nbuf`
+// while the closure's own run the chains of step 3; every thread runs before_loads() once the item's
+// constants (geometry, band extents and rows) are requested and before it reads what the previous
+// kernel wrote, and after_loads() once the item's global loads are issued.  `wst` holds A.wst_elems staged band elements, `nbuf`
 // A.max_union densities.  Returns false on every thread when the band-row copy never
 // completed (A.err is set).
-template <typename T, typename Extra, typename AfterLoads>
+template <typename T, typename Extra, typename BeforeLoads, typename AfterLoads>
 __device__ bool closure_cells(const ClosureArgs& A, const MomSet& M, const ClosureTabs<T>& tb, const InstDev& I, int c0,
                               int cnt, T* recb, T* wst, T* nbuf, uint64_t* cbar, uint32_t& phase, const Extra& extra,
-                              const AfterLoads& after_loads) {
+                              const BeforeLoads& before_loads, const AfterLoads& after_loads) {
     using W = Wide<T>;
     __shared__ W sw_n[32], sw_T[32], sw_u[3][32];  // reach cells, wide
-    __shared__ T s_chi[32], snb[32];               // reach cells: chi, band density
+    __shared__ T snb[32];                          // reach cells: band density
     __shared__ int sblo[32], scnt[32];             // reach cells: first band column, stored extent
     __shared__ T sq[3][32];                        // own cells: q
-    __shared__ T ecs[kClosureCells][4][kMaxE];     // own cells: expansion coefficients
-    __shared__ T sgp[kClosureCells][5][5];         // gradient terms per own cell and stencil position
+    __shared__ EqCoeffs<T> ecs;                    // own cells: expansion coefficients
+    __shared__ T sgp[5][32];                       // gradient terms per pair of neighbouring reach cells
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x;
     const T* band = reinterpret_cast<const T*>(A.band);
     const T* dens = reinterpret_cast<const T*>(A.dens);
@@ -568,14 +638,13 @@ __device__ bool closure_cells(const ClosureArgs& A, const MomSet& M, const Closu
     clo_reach(c0, cnt, N, h0, h1);
     const int nh = h1 - h0;
     const int rs = A.rec_stride;
-    const ReachView<T> RV{sw_n, sw_T, {sw_u[0], sw_u[1], sw_u[2]}, s_chi, snb};
-    // ---- 1. every global load of the item at once: the raw sums of the reach cells and the
-    // geometry of the own cells (warp 0, lane per cell), the band rows of the reach cells
-    // (bulk copies of their stored extents, issued by warp 0) and the densities of the union
-    // of the bands (all threads)
+    const ReachView<T> RV{sw_n, sw_T, {sw_u[0], sw_u[1], sw_u[2]}, snb};
+    // ---- 1. the constants: the geometry of the own cells (lane per cell of warp 0) and, by bulk
+    // copies issued by warp 0, the band rows of the reach cells (their stored extents); then, past
+    // before_loads(), every load of the previous kernel's output at once: the raw sums of the reach
+    // cells (lane per cell of warp 0) and the densities of the union of the bands (all threads)
     W sv[kSums];
     T geo0 = T(1), geo1 = T(0);
-    if (warp == 0 && lane < nh) clo_load_sums<T>(A, (long long)I.cell_off + h0 + lane, sv);
     if (warp == 0 && lane < cnt) {
         const T* gc = geoT + (long long)(I.cell_off + c0 + lane) * kGeo;
         geo0 = gc[0];
@@ -612,6 +681,10 @@ __device__ bool closure_cells(const ClosureArgs& A, const MomSet& M, const Closu
                              (uint32_t)(mine.y * sizeof(T)), cbar);
             }
         }
+    }
+    before_loads();
+    if (warp == 0 && lane < nh) clo_load_sums<T>(A, (long long)I.cell_off + h0 + lane, sv);
+    if (!I.chi_local) {
         const T* nd = dens + ((long long)I.cell_off + jlo) * slices;
         for (int j0 = tid; j0 < nu; j0 += 4 * NT) {
             // four loads in flight per thread
@@ -672,33 +745,23 @@ __device__ bool closure_cells(const ClosureArgs& A, const MomSet& M, const Closu
         }
     }
     __syncthreads();
-    // ---- 3. two concurrent chains.  Warp 0: chi of the reach cells, the gradient terms (one
-    // lane per own cell and stencil position), then transport, strain and Shakhov coefficient
-    // (lane per own cell).  Warps 1 and 2: the expansion coefficients of the equilibria (Sec.
-    // III.C), lane per (own cell, axis half): warp 1 the half-range axis (+ and -), warp 2 the
-    // axes 2 and 3.
+    // ---- 3. concurrent chains.  Warp 0: the gradient terms (lane per pair of neighbouring reach
+    // cells), then the own cells' gradients and strain.  Warp 3: chi, transport and Shakhov coefficient
+    // (lane per own cell).  Warps 1 and 2: the expansion coefficients of the equilibria (Sec. III.C),
+    // lane per (own cell, axis half): warp 1 the half-range axis (+ and -), warp 2 the axes 2 and 3.
+    const T etaf = inst_param<T>(I.etafac, I.f_etafac);
     if (warp == 0) {
-        const T etaf = inst_param<T>(I.etafac, I.f_etafac);
-        if (lane < nh) s_chi[lane] = clo_chi<T>(etaf, I.chi_local ? w_hi(sw_n[lane]) : snb[lane]);
-        __syncwarp();
-        for (int e = lane; e < cnt * 5; e += 32) {
-            const int t = e / 5, q = e % 5, c = c0 + t;
-            int cq;
-            T wq;
-            stencil5_at<T>(c, N, q, cq, wq);
-            T g[5];
-            clo_grad_terms<T>(RV, cq - h0, c - h0, wq, etaf, I.chi_local != 0, g);
+        if (lane < nh - 1) {
+            T d[5];
+            clo_pair_terms<T>(RV, lane, etaf, I.chi_local != 0, d);
 #pragma unroll
-            for (int v = 0; v < 5; ++v) sgp[t][v][q] = g[v];
+            for (int v = 0; v < 5; ++v) sgp[v][lane] = d[v];
         }
         __syncwarp();
         if (lane < cnt) {
-            const int t = lane, lt = c0 + t - h0;
-            const T q[3] = {sq[0][t], sq[1][t], sq[2][t]};
-            clo_record_scalars<T>(recb + (long long)t * rs, RV, lt, sgp[t], geo0, geo1, q, I);
-            T* cw = reinterpret_cast<T*>(A.cw) + (long long)(I.cell_off + c0 + t) * 2;
-            cw[0] = s_chi[lt];
-            cw[1] = I.chi_local ? w_hi(sw_n[lt]) : snb[lt];
+            const int lt = c0 + lane - h0;
+            clo_record_gradients<T>(recb + (long long)lane * rs, c0 + lane, N, h0, sgp, w_hi(sw_u[0][lt]), w_hi(sw_u[1][lt]),
+                                    w_hi(sw_u[2][lt]), w_hi(sw_T[lt]), geo0, geo1, I);
         }
     } else if (warp <= 2) {
         for (int e = lane; e < 2 * cnt; e += 32) {
@@ -708,23 +771,30 @@ __device__ bool closure_cells(const ClosureArgs& A, const MomSet& M, const Closu
             T ev[kMaxE + 1];
             clo_eq_coeffs<T>(job, cT, tm1, w_hi(sw_u[0][lt]), w_hi(sw_u[job == 2 ? 1 : 2][lt]), tb, M, ev);
 #pragma unroll
-            for (int l = 0; l < kMaxE; ++l) ecs[t][job][l] = ev[l];
+            for (int l = 0; l < kMaxE; ++l) ecs.v[job][l][t] = ev[l];
         }
-    } else if (warp >= kClosureWarps) {
+    } else if (warp == 3) {
+        if (lane < cnt) {
+            const int lt = c0 + lane - h0;
+            const T q[3] = {sq[0][lane], sq[1][lane], sq[2][lane]};
+            const T nb = I.chi_local ? w_hi(sw_n[lt]) : snb[lt], chi = clo_chi<T>(etaf, nb);
+            clo_record_transport<T>(recb + (long long)lane * rs, sw_n[lt], w_hi(sw_u[0][lt]), w_hi(sw_u[1][lt]),
+                                    w_hi(sw_u[2][lt]), w_hi(sw_T[lt]), chi, q, I);
+            T* cw = reinterpret_cast<T*>(A.cw) + (long long)(I.cell_off + c0 + lane) * 2;
+            cw[0] = chi;
+            cw[1] = nb;
+        }
+    } else {
         extra(warp - kClosureWarps, NT / 32 - kClosureWarps);
     }
     __syncthreads();
-    // ---- 5. per-axis equilibrium vectors of the own cells, in the populations' precision
-    const int ng = M.nR + M.n2 + M.n3;
-    for (int e = tid; e < cnt * ng; e += NT) {
-        const int t = e / ng, k = e % ng;
-        int dst;
-        const T g = clo_g_entry<T>(k, ecs[t], w_hi(sw_T[c0 + t - h0]), tb, M, dst);
-        recb[(long long)t * rs + dst] = g;
+    // ---- 4. the equilibrium vectors and the normalised density (eight lanes per own cell)
+    for (int e = tid; e < (8 * cnt + 31) / 32 * 32; e += NT) {
+        const int t = min(e >> 3, cnt - 1), lt = c0 + t - h0;
+        const bool on = (e >> 3) < cnt;
+        const T nf = clo_equilibrium<T>(on, e & 7, recb + (long long)t * rs, sw_n[lt], w_hi(sw_T[lt]), ecs, t, tb, M);
+        if (on && (e & 7) == 0) recb[(long long)t * rs] = nf;
     }
-    __syncthreads();
-    // ---- 6. discrete mass of the stored equilibrium (a thread per own cell)
-    for (int t = tid; t < cnt; t += NT) clo_mass_normalise<T>(recb + (long long)t * rs, sw_n[c0 + t - h0], M);
     __syncthreads();  // shared arrays are reused by the next call
     return true;
 }

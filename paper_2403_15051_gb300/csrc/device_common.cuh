@@ -95,33 +95,13 @@ __device__ __forceinline__ T ldg_t(const T* p) {
     return __ldg(p);
 }
 
+// A product that is rounded by itself: never contracted into a following addition, so code that must
+// give the same bits from every kernel it is inlined into says with fma() and mul_rn() what is fused.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 __device__ __forceinline__ float ratio_fast(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double ratio_fast(double a, double b) { return a / b; }
-
-// Fifth-order WENO reconstruction (Jiang & Shu 1996; epsilon 1e-6, power 2) at the right face
-// of the cell holding c, upwind from the left; reversing the five arguments gives the value at
-// the left face of the cell holding c, upwind from the right.  The nonlinear weights
-// d_k / (eps + beta_k)^2 are scaled by the square of the smallest (eps + beta_k), which leaves
-// the normalised weights unchanged and keeps every intermediate in [0, 1] (no FP32 overflow for
-// large populations).
-template <typename T>
-__device__ __forceinline__ T weno5(T a, T b, T c, T d, T e) {
-    const T eps = T(1e-6);
-    const T k13 = T(13.0 / 12.0), q = T(0.25);
-    const T t0 = a - T(2) * b + c, t1 = a - T(4) * b + T(3) * c;
-    const T t2 = b - T(2) * c + d, t3 = b - d;
-    const T t4 = c - T(2) * d + e, t5 = T(3) * c - T(4) * d + e;
-    const T e0 = eps + k13 * t0 * t0 + q * t1 * t1;
-    const T e1 = eps + k13 * t2 * t2 + q * t3 * t3;
-    const T e2 = eps + k13 * t4 * t4 + q * t5 * t5;
-    const T m = fmin(e0, fmin(e1, e2));
-    const T s0 = ratio_fast(m, e0), s1 = ratio_fast(m, e1), s2 = ratio_fast(m, e2);
-    const T a0 = T(0.1) * s0 * s0, a1 = T(0.6) * s1 * s1, a2 = T(0.3) * s2 * s2;
-    const T r0 = T(2) * a - T(7) * b + T(11) * c;
-    const T r1 = -b + T(5) * c + T(2) * d;
-    const T r2 = T(2) * c + T(5) * d - e;
-    return ratio_fast(a0 * r0 + a1 * r1 + a2 * r2, T(6) * (a0 + a1 + a2));
-}
 
 // ---- pairs of lanes: two momenta of a vector per instruction.  FP32 pairs use the packed FP32x2
 // operations of the sm_100 family (__ffma2_rn, __fadd2_rn, __fmul2_rn: one issue slot for two
@@ -157,7 +137,6 @@ __device__ __forceinline__ double2 p_mul(double2 a, double2 b) { return make_dou
 __device__ __forceinline__ float2 p_sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 __device__ __forceinline__ double2 p_sub(double2 a, double2 b) { return make_double2(__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y)); }
 __device__ __forceinline__ float2 p_min(float2 a, float2 b) { return make_float2(fminf(a.x, b.x), fminf(a.y, b.y)); }
-__device__ __forceinline__ double2 p_min(double2 a, double2 b) { return make_double2(fmin(a.x, b.x), fmin(a.y, b.y)); }
 // Approximate FP32 reciprocal (the PTX rcp.approx instruction: at most one unit in the last place
 // off, subnormals flushed to zero).
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -165,49 +144,107 @@ __device__ __forceinline__ float rcp_approx(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-// a / b lane by lane: for FP32 the product with the approximate reciprocal (the operands here are
-// normal numbers well inside the range); for FP64 the correctly rounded quotient.
+// a / b lane by lane, as the product with the approximate reciprocal (the operands here are normal
+// numbers well inside the range).
 __device__ __forceinline__ float2 p_ratio(float2 a, float2 b) {
     return __fmul2_rn(a, make_float2(rcp_approx(b.x), rcp_approx(b.y)));
 }
-__device__ __forceinline__ double2 p_ratio(double2 a, double2 b) { return make_double2(a.x / b.x, a.y / b.y); }
 
-// The same reconstruction written on the window in ascending cell order, w0..w4, for either
-// upwind direction: sigma = +1 gives weno5(w0, .., w4) (value at the right face of w2's cell,
-// from the left), sigma = -1 gives weno5(w4, .., w0) (left face, from the right).  The three
-// smoothness indicators belong to the left, centre and right stencils whatever the direction,
+// Fifth-order WENO reconstruction (Jiang & Shu 1996; epsilon 1e-6, power 2) of the face value on
+// the window w0..w4 in ascending cell order, for either upwind direction: sigma = +1 gives the value at
+// the right face of w2's cell, from the left; sigma = -1 the value at its left face, from the right.
+// The three smoothness indicators belong to the left, centre and right stencils whatever the direction,
 // and every candidate value is (D_k + 12 w2 -+ 3 sigma t_k) / 2 with D_k the stencil's second
 // difference and t_k the first-difference part of its indicator, so the value is
 // w2 + sum_k a_k X_k / (12 sum_k a_k), X_k = D_k +- 3 sigma t_k.  The linear weights follow the
 // direction: (dL, dC, dR) = (0.1, 0.6, 0.3) or (0.3, 0.6, 0.1); s3 = 3 sigma.  Indicators are
 // taken four times over (e4 + 13/3 D^2 + t^2, e4 = 4 eps): the normalised weights are unchanged.
 // The reconstruction is homogeneous of degree one in the window once eps scales with its square:
-// the value for c w0..c w4 with c^2 e4 is c times the value for w0..w4 with e4.
-// Written for a pair of momenta (one packed operation per step for FP32 pairs).  The window's
+// the value for c w0..c w4 with c^2 e4 is c times the value for w0..w4 with e4.  The window's
 // first difference enters negated (w0 - w1), and so does the centre stencil's first-difference
 // part (-tC = d1 + d2), which the indicators square and the candidate values take with the
-// opposite sign: no negation is ever formed.  s3, ns3 = 3 sigma and its negative; dL, dR the
-// linear weights of the outer stencils; e4 = 4 eps (w^2 for the reconstruction of f, below).
-template <typename T>
-__device__ __forceinline__ Pair<T> weno5_pair(Pair<T> w0, Pair<T> w1, Pair<T> w2, Pair<T> w3, Pair<T> w4, Pair<T> s3,
-                                              Pair<T> ns3, Pair<T> dL, Pair<T> dR, Pair<T> e4) {
-    using P = Pair<T>;
+// opposite sign: no negation is ever formed.
+//
+// FP32: a pair of momenta, one packed operation per step.  The nonlinear weights d_k / E_k^2 are
+// scaled by the square of the smallest indicator, which leaves the normalised weights unchanged and
+// keeps every intermediate in [0, 1] (no overflow for large populations).  ns3 = -3 sigma.
+__device__ __forceinline__ float2 weno5_pair(float2 w0, float2 w1, float2 w2, float2 w3, float2 w4, float2 s3, float2 ns3,
+                                             float2 dL, float2 dR, float2 e4) {
+    using P = float2;
     const P nd0 = p_sub(w0, w1), d1 = p_sub(w2, w1), d2 = p_sub(w3, w2), d3 = p_sub(w4, w3);
     const P D1 = p_add(d1, nd0), D2 = p_sub(d2, d1), D3 = p_sub(d3, d2);
-    const P tL = p_fma(p_splat(T(3)), d1, nd0);    // 3 d1 - d0
+    const P tL = p_fma(p_splat(3.f), d1, nd0);    // 3 d1 - d0
     const P ntC = p_add(d1, d2);                    // -tC
-    const P tR = p_fma(p_splat(T(-3)), d2, d3);     // d3 - 3 d2
-    const P c = p_splat(T(13.0 / 3.0));
+    const P tR = p_fma(p_splat(-3.f), d2, d3);     // d3 - 3 d2
+    const P c = p_splat((float)(13.0 / 3.0));
     const P EL = p_fma(tL, tL, p_fma(p_mul(c, D1), D1, e4));
     const P EC = p_fma(ntC, ntC, p_fma(p_mul(c, D2), D2, e4));
     const P ER = p_fma(tR, tR, p_fma(p_mul(c, D3), D3, e4));
     const P m = p_min(EL, p_min(EC, ER));
     const P sL = p_ratio(m, EL), sC = p_ratio(m, EC), sR = p_ratio(m, ER);
-    const P aL = p_mul(dL, p_mul(sL, sL)), aC = p_mul(p_splat(T(0.6)), p_mul(sC, sC)), aR = p_mul(dR, p_mul(sR, sR));
+    const P aL = p_mul(dL, p_mul(sL, sL)), aC = p_mul(p_splat(0.6f), p_mul(sC, sC)), aR = p_mul(dR, p_mul(sR, sR));
     const P XL = p_fma(s3, tL, D1), XC = p_fma(s3, ntC, D2), XR = p_fma(ns3, tR, D3);
     const P num = p_fma(aR, XR, p_fma(aC, XC, p_mul(aL, XL)));
-    const P den = p_mul(p_splat(T(12)), p_add(p_add(aL, aC), aR));
+    const P den = p_mul(p_splat(12.f), p_add(p_add(aL, aC), aR));
     return p_add(w2, p_ratio(num, den));
+}
+
+// FP64: the FP64 unit takes a warp instruction every 16 cycles, so its operations are what a stage
+// costs, and each of the four quotients above is nine of them.  The weights are taken without a
+// quotient, d_k times the square of the product of the other two indicators, with the indicators'
+// exponents lowered by the smallest one's (an integer operation on the high words, exact) and held
+// below 2^200 (a stencil that much rougher than the smoothest has no weight left either way), so the
+// products stay within the range.  The remaining quotient: the instruction's approximate reciprocal
+// (relative error 2^-20), one cubic step x (1 + e + e^2), e = 1 - d x (2^-60), and the quotient
+// corrected by its residual (correct to an ulp).
+__device__ __forceinline__ double f64_quot(double num, double den) {
+    double x;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(den));
+    const double e = __fma_rn(-den, x, 1.0);
+    x = __fma_rn(x, __fma_rn(e, e, e), x);
+    const double q = __dmul_rn(num, x);
+    return __fma_rn(__fma_rn(-den, q, num), x, q);
+}
+__device__ __forceinline__ double f64_lowered(double E, int sh) {
+    return __hiloint2double(min(__double2hiint(E) - sh, (1023 + 200) << 20), __double2loint(E));
+}
+__device__ __forceinline__ double weno5_f64(double w0, double w1, double w2, double w3, double w4, double s3, double dL,
+                                            double dR, double e4) {
+    const double nd0 = __dsub_rn(w0, w1), d1 = __dsub_rn(w2, w1), d2 = __dsub_rn(w3, w2), d3 = __dsub_rn(w4, w3);
+    const double D1 = __dadd_rn(d1, nd0), D2 = __dsub_rn(d2, d1), D3 = __dsub_rn(d3, d2);
+    const double tL = __fma_rn(3.0, d1, nd0), ntC = __dadd_rn(d1, d2), tR = __fma_rn(-3.0, d2, d3);
+    const double c = 13.0 / 3.0;
+    double EL = __fma_rn(tL, tL, __fma_rn(__dmul_rn(c, D1), D1, e4));
+    double EC = __fma_rn(ntC, ntC, __fma_rn(__dmul_rn(c, D2), D2, e4));
+    double ER = __fma_rn(tR, tR, __fma_rn(__dmul_rn(c, D3), D3, e4));
+    // (positive doubles order like their high words; a window that is not finite keeps the value not
+    // finite through the candidates)
+    const int hm = min(__double2hiint(EL), min(__double2hiint(EC), __double2hiint(ER)));
+    const int sh = (hm & 0x7ff00000) - (1023 << 20);
+    EL = f64_lowered(EL, sh);
+    EC = f64_lowered(EC, sh);
+    ER = f64_lowered(ER, sh);
+    const double pL = __dmul_rn(EC, ER), pC = __dmul_rn(EL, ER), pR = __dmul_rn(EL, EC);
+    const double aL = __dmul_rn(dL, __dmul_rn(pL, pL)), aC = __dmul_rn(0.6, __dmul_rn(pC, pC)),
+                 aR = __dmul_rn(dR, __dmul_rn(pR, pR));
+    const double XL = __fma_rn(s3, tL, D1), XC = __fma_rn(s3, ntC, D2), XR = __fma_rn(-s3, tR, D3);
+    const double num = __fma_rn(aR, XR, __fma_rn(aC, XC, __dmul_rn(aL, XL)));
+    return __fma_rn(f64_quot(num, __dadd_rn(__dadd_rn(aL, aC), aR)), 1.0 / 12.0, w2);
+}
+__device__ __forceinline__ double2 weno5_pair(double2 w0, double2 w1, double2 w2, double2 w3, double2 w4, double2 s3,
+                                              double2, double2 dL, double2 dR, double2 e4) {
+    return make_double2(weno5_f64(w0.x, w1.x, w2.x, w3.x, w4.x, s3.x, dL.x, dR.x, e4.x),
+                        weno5_f64(w0.y, w1.y, w2.y, w3.y, w4.y, s3.y, dL.y, dR.y, e4.y));
+}
+// One momentum (the wall fluxes).
+__device__ __forceinline__ double weno5_one(double w0, double w1, double w2, double w3, double w4, double s3, double dL,
+                                            double dR, double e4) {
+    return weno5_f64(w0, w1, w2, w3, w4, s3, dL, dR, e4);
+}
+__device__ __forceinline__ float weno5_one(float w0, float w1, float w2, float w3, float w4, float s3, float dL, float dR,
+                                           float e4) {
+    return weno5_pair(p_splat(w0), p_splat(w1), p_splat(w2), p_splat(w3), p_splat(w4), p_splat(s3), p_splat(-s3), p_splat(dL),
+                      p_splat(dR), p_splat(e4)).x;
 }
 
 // ---- wide accumulators: plain FP64 for FP64 populations; for FP32 populations a double-float
@@ -237,9 +274,9 @@ __device__ __forceinline__ double w_hi(Wide<double> a) { return a.v; }
 __device__ __forceinline__ float w_hi(Wide<float> a) { return a.hi; }
 __device__ __forceinline__ Wide<double> w_add(Wide<double> a, Wide<double> b) { return {a.v + b.v}; }
 __device__ __forceinline__ Wide<double> w_sub(Wide<double> a, Wide<double> b) { return {a.v - b.v}; }
-__device__ __forceinline__ Wide<double> w_mul(Wide<double> a, Wide<double> b) { return {a.v * b.v}; }
+__device__ __forceinline__ Wide<double> w_mul(Wide<double> a, Wide<double> b) { return {__dmul_rn(a.v, b.v)}; }
 __device__ __forceinline__ Wide<double> w_div(Wide<double> a, Wide<double> b) { return {a.v / b.v}; }
-__device__ __forceinline__ Wide<double> w_scale(Wide<double> a, double c) { return {a.v * c}; }
+__device__ __forceinline__ Wide<double> w_scale(Wide<double> a, double c) { return {__dmul_rn(a.v, c)}; }
 
 __device__ __forceinline__ Wide<float> w_norm(float s, float e) {  // |s| >= |e|
     const float hi = s + e;
@@ -253,14 +290,14 @@ __device__ __forceinline__ Wide<float> w_add(Wide<float> a, Wide<float> b) {
 }
 __device__ __forceinline__ Wide<float> w_sub(Wide<float> a, Wide<float> b) { return w_add(a, {-b.hi, -b.lo}); }
 __device__ __forceinline__ Wide<float> w_mul(Wide<float> a, Wide<float> b) {
-    const float p = a.hi * b.hi;
+    const float p = __fmul_rn(a.hi, b.hi);
     float e = fmaf(a.hi, b.hi, -p);
     e = fmaf(a.hi, b.lo, e);
     e = fmaf(a.lo, b.hi, e);
     return w_norm(p, e);
 }
 __device__ __forceinline__ Wide<float> w_scale(Wide<float> a, float c) {
-    const float p = a.hi * c;
+    const float p = __fmul_rn(a.hi, c);
     const float e = fmaf(a.lo, c, fmaf(a.hi, c, -p));
     return w_norm(p, e);
 }
@@ -320,29 +357,6 @@ __device__ __forceinline__ T warp_sum16_transposed(const T (&v)[16], int lane) {
     const T send = b1 ? w2[0] : w2[1], keep = b1 ? w2[1] : w2[0];
     const T w1 = keep + __shfl_xor_sync(0xffffffffu, send, 2);
     return w1 + __shfl_xor_sync(0xffffffffu, w1, 1);
-}
-
-// Five-point derivative stencil in the mapped coordinate (gradients of Eq. j1): fourth-order
-// central in the interior, one-sided fourth-order at the two cells next to each wall.
-template <typename R>
-__device__ __forceinline__ void stencil5(int c, int N, int* idx, R* w) {
-    const R k = R(1) / R(12);
-    if (c >= 2 && c <= N - 3) {
-        idx[0] = c - 2; idx[1] = c - 1; idx[2] = c; idx[3] = c + 1; idx[4] = c + 2;
-        w[0] = k; w[1] = -8 * k; w[2] = 0; w[3] = 8 * k; w[4] = -k;
-    } else if (c == 0) {
-        for (int q = 0; q < 5; ++q) idx[q] = q;
-        w[0] = -25 * k; w[1] = 48 * k; w[2] = -36 * k; w[3] = 16 * k; w[4] = -3 * k;
-    } else if (c == 1) {
-        for (int q = 0; q < 5; ++q) idx[q] = q;
-        w[0] = -3 * k; w[1] = -10 * k; w[2] = 18 * k; w[3] = -6 * k; w[4] = k;
-    } else if (c == N - 2) {
-        for (int q = 0; q < 5; ++q) idx[q] = N - 1 - q;
-        w[0] = 3 * k; w[1] = 10 * k; w[2] = -18 * k; w[3] = 6 * k; w[4] = -k;
-    } else {
-        for (int q = 0; q < 5; ++q) idx[q] = N - 1 - q;
-        w[0] = 25 * k; w[1] = -48 * k; w[2] = 36 * k; w[3] = -16 * k; w[4] = 3 * k;
-    }
 }
 
 }  // namespace fdlb

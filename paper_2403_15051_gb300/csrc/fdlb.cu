@@ -84,8 +84,8 @@ struct Solver {
     int use_bulk = 0;
     int closure_cells = 4, closure_threads = 128;  // own cells per closure item (<= kClosureCells)
     int closure_batch = 0;  // the closure as two launches over all items (items of kClosureCells cells)
-    int grid_cbatch = 1;
-    size_t cbatch_smem = 0;
+    ClosureBatchShape cbatch{};
+    int wall_parts = kWallParts;  // closure work items per wall
     int autotune_mode = 1;  // 0 off; 1 tune on the first step of a batch; 2 also of a single instance
     int stall_checks = 0;   // run_to_steady: checks without halving the best residual before an instance stops
     int stage_minb = 1;     // register bound of the stage kernel (1; 3, 2 or 5 blocks per SM where built)
@@ -357,6 +357,8 @@ int plan_solver(const fdlb_params* ps, int n, Solver& S) try {
     S.n2 = p0.Q_2;
     S.n3 = S.reduced ? 2 : p0.Q_3;
     S.Np = S.nR * S.n2 * S.n3;
+    // a thread of a wall item per outgoing momentum (half of them; of the reduced pair, phi's)
+    S.wall_parts = std::clamp((S.nR / 2 * S.n2 * (S.reduced ? 1 : S.n3) + 127) / 128, 1, kWallParts);
     S.setup.resize(n);
     for (int q = 0; q < n; ++q) {
         rc = build_instance(ps[q], S.aR, S.setup[q]);
@@ -484,6 +486,7 @@ int plan_step_kernel(Solver& S, int n_items) {
     for (int q = 0; q < S.n_inst; ++q)
         wst = std::max(wst, std::min(S.setup[q].p.n_cells, S.max_tile + 4) * S.setup[q].band.width);
     wst = (int)std::min<size_t>((size_t)wst, (limit - base) / S.tsize);
+    wst = wst / 4 * 4;  // as in upload_items
     S.step_wst = wst;
     S.step_clo_off = (int)clo_off;
     S.smem_step = clo_off + closure_smem(S.nR, S.n2, S.n3, S.max_union, wst, (int)S.tsize);
@@ -505,6 +508,11 @@ int upload_items(Solver& S) {
                      [&](int a, int b) { return S.setup[a].p.n_cells > S.setup[b].p.n_cells; });
     std::vector<int4> si, ci;
     const int slices = S.n3 / S.KS;
+    // batch form: items of 28 cells where there are warps enough (8 per SM), else of 12 (16 cells with
+    // the reach): half the bands and equilibrium vectors per warp
+    long long act_cells = 0;
+    for (int q : order) act_cells += S.setup[q].p.n_cells;
+    const int batch_cells = act_cells >= 8LL * kClosureCells * S.n_sm ? kClosureCells : 12;
     for (int q : order) {
         const int N = S.setup[q].p.n_cells;
         int nt = (N + S.B - 1) / S.B;
@@ -525,15 +533,24 @@ int upload_items(Solver& S) {
         }
         // the wall densities first (their blocks read four cells of populations), then the cells
         for (int side = 0; side < 2; ++side)
-            for (int part = 0; part < kWallParts; ++part) ci.push_back(make_int4(q, side ? N - 1 : 0, part, 1 + side));
-        const int cc = S.closure_batch ? kClosureCells : S.closure_cells;
-        for (int c = 0; c < N; c += cc) ci.push_back(make_int4(q, c, std::min(cc, N - c), 0));
+            for (int part = 0; part < S.wall_parts; ++part) ci.push_back(make_int4(q, side ? N - 1 : 0, part, 1 + side));
+        // items of equal size (differing by at most one cell): in the batch form a warp's time is that
+        // of its widest item
+        const int cc = S.closure_batch ? batch_cells : S.closure_cells, nci = (N + cc - 1) / cc;
+        for (int k = 0, c = 0; k < nci; ++k) {
+            const int cnt = N / nci + (k < N % nci ? 1 : 0);
+            ci.push_back(make_int4(q, c, cnt, 0));
+            c += cnt;
+        }
     }
     if ((int)si.size() > S.max_sitems || (int)ci.size() > S.max_citems) return FDLB_EINVAL;
     // the batch closure's band jobs: two band rows of an item at a time (instances with chi at the
     // local density have none), or a wall part; geometry only, so formed here once per work list
     std::vector<BandPair> bp;
-    if (S.closure_batch) {
+    int widest = 0;
+    for (int q : order) widest = std::max(widest, S.inst_h[q].chi_local ? 0 : S.setup[q].band.width);
+    const bool inline_band = widest <= kInlineBandMax;
+    if (S.closure_batch && !inline_band) {
         for (const int4& w : ci) {
             const InstanceSetup& I = S.setup[w.x];
             const InstDev& D = S.inst_h[w.x];
@@ -609,12 +626,11 @@ int upload_items(Solver& S) {
         const size_t target = S.smem_per_sm / closure_bps;
         wst = target > base + 1024 ? (int)std::min<size_t>((size_t)wst, (target - base - 1024) / S.tsize) : 0;
     }
+    wst = wst / 4 * 4;  // the tables behind the band rows start on a 16-byte boundary
     S.closure_wst = wst;
     S.closure_smem = closure_smem(S.nR, S.n2, S.n3, max_union, wst, (int)S.tsize);
     S.grid_closure = std::max(1, std::min(nc, S.n_sm * (throughput ? closure_bps : 8)));
-    // the batch form: the tables only, as many blocks as reside
-    S.cbatch_smem = closure_smem(S.nR, S.n2, S.n3, 0, 0, (int)S.tsize);
-    S.grid_cbatch = std::max(1, std::min(nc, S.n_sm * closure_batch_blocks_per_sm((int)S.tsize, S.cbatch_smem)));
+    S.cbatch = closure_batch_shape((int)S.tsize, S.nR, S.n2, S.n3, nc, nbp, !inline_band ? 0 : widest <= 64 ? 2 : 4, S.n_sm);
     S.grid_stream = std::max(1, ns);
     return plan_step_kernel(S, ns);
 }
@@ -770,23 +786,20 @@ int launch_closure_buf(Solver& S, int buf, int write_ca) {
     A.geoT = S.geoT;
     A.slices = S.M.slices;
     A.max_union = S.max_union;
-    A.wall_parts = kWallParts;
+    A.wall_parts = S.wall_parts;
     A.wst_elems = S.closure_wst;
     A.err = S.err;
     A.programmatic = S.programmatic;
     A.pairs = S.bpairs;
     A.n_pairs = S.n_bpairs;
     if (S.closure_batch) {
-        if (S.precision == FDLB_FP32)
-            launch_closure_batch<float>(A, S.M, S.grid_cbatch, S.cbatch_smem, S.stream);
-        else
-            launch_closure_batch<double>(A, S.M, S.grid_cbatch, S.cbatch_smem, S.stream);
-        S.launches += 2;
+        FDLB_CUDA(S.precision == FDLB_FP32 ? launch_closure_batch<float>(A, S.M, S.cbatch, S.stream)
+                                           : launch_closure_batch<double>(A, S.M, S.cbatch, S.stream));
+        S.launches += S.cbatch.inline_band ? 1 : 2;
     } else {
-        if (S.precision == FDLB_FP32)
-            launch_closure<float>(A, S.M, S.grid_closure, S.closure_threads, S.closure_smem, S.stream);
-        else
-            launch_closure<double>(A, S.M, S.grid_closure, S.closure_threads, S.closure_smem, S.stream);
+        FDLB_CUDA(S.precision == FDLB_FP32
+                      ? launch_closure<float>(A, S.M, S.grid_closure, S.closure_threads, S.closure_smem, S.stream)
+                      : launch_closure<double>(A, S.M, S.grid_closure, S.closure_threads, S.closure_smem, S.stream));
         S.launches++;
     }
     if (write_ca) {
@@ -877,7 +890,7 @@ int launch_stream_only(Solver& S, int in, int fn, int out, double a, double b, i
     A.rec = S.rec;
     A.rec_stride = record_stride(S.nR, S.n2, S.n3);
     A.nwp = S.nwp;
-    A.wall_parts = kWallParts;
+    A.wall_parts = S.wall_parts;
     A.sums_out = S.sums[out];
     A.sumsw_out = S.sumsw[out];
     A.dens_out = S.dens[out];
@@ -1019,7 +1032,7 @@ int launch_steps_fused(Solver& S, int64_t n) {
     A.rec = S.rec;
     A.rec_stride = record_stride(S.nR, S.n2, S.n3);
     A.nwp = S.nwp;
-    A.wall_parts = kWallParts;
+    A.wall_parts = S.wall_parts;
     A.items = S.sitems;
     A.n_items = S.n_sitems;
     A.inst = S.inst_d;
@@ -1046,7 +1059,7 @@ int launch_steps_fused(Solver& S, int64_t n) {
     C.geoT = S.geoT;
     C.slices = S.M.slices;
     C.max_union = S.max_union;
-    C.wall_parts = kWallParts;
+    C.wall_parts = S.wall_parts;
     C.wst_elems = S.step_wst;
     C.err = S.err;
     for (int b = 0; b < 3; ++b) {
@@ -1236,7 +1249,7 @@ int do_steps(Solver& S, int64_t n) {
         if (rc) return rc;
         while (n - done >= S.graph_steps) {
             FDLB_CUDA(cudaGraphLaunch(S.gexec, S.stream));
-            S.launches += (int64_t)S.graph_steps * 3 * ((S.krg_on ? 1 : 0) + (S.k3_on ? 1 : 0) + (S.closure_batch ? 2 : 1) + 1);
+            S.launches += (int64_t)S.graph_steps * 3 * ((S.krg_on ? 1 : 0) + (S.k3_on ? 1 : 0) + (S.closure_batch && !S.cbatch.inline_band ? 2 : 1) + 1);
             done += S.graph_steps;
         }
     }
@@ -1645,7 +1658,7 @@ int fdlb_get_closure(fdlb_handle h, int instance, double* nbar, double* chi, dou
     if (rc) return rc;
     const int N = S->setup[instance].p.n_cells;
     std::vector<double> ca((size_t)N * fdlb::kCA);
-    const int P = fdlb::kWallParts;
+    const int P = S->wall_parts;
     std::vector<unsigned char> parts((size_t)2 * P * S->tsize);
     FDLB_CUDA(cudaMemcpyAsync(ca.data(), S->ca + (size_t)S->cell_off[instance] * fdlb::kCA, ca.size() * 8,
                               cudaMemcpyDeviceToHost, S->stream));

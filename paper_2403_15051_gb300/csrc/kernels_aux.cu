@@ -116,10 +116,18 @@ __global__ void __launch_bounds__(kClosureThreads) closure_kernel(ClosureArgs A,
         fence_mbar_init();
     }
     __syncthreads();
-    pdl_wait();  // everything below reads what the previous kernels wrote
-    // the successor (the stage kernel) may start now: it requests the rows of the stage input,
-    // written by the kernel this one has just waited for
-    pdl_trigger();
+    // A block's first item is looked up and its constants (band extents and rows, geometry) are requested
+    // before the wait on the previous kernel; work lists, instances and bands are not written by kernels.
+    // The successor (the stage kernel) may start after the wait: it requests the rows of the stage input,
+    // written by the kernel this one has just waited for.
+    bool waited = false;
+    auto wait = [&]() {
+        if (!waited) {
+            pdl_wait();
+            pdl_trigger();
+            waited = true;
+        }
+    };
     const T* fin_all = reinterpret_cast<const T*>(A.f_in);
     T* rec_all = reinterpret_cast<T*>(A.rec);
     T* nwp = reinterpret_cast<T*>(A.nwp);
@@ -130,6 +138,7 @@ __global__ void __launch_bounds__(kClosureThreads) closure_kernel(ClosureArgs A,
         const InstDev I = A.inst[w.x];
         if (w.w != 0) {
             // ---- one part of the outgoing flux through a wall
+            wait();
             const int side = w.w - 1, part = w.z, P = A.wall_parts;
             const T* wall = fin_all + I.f_off + (side == 0 ? 0LL : (long long)(I.n_cells - 1) * M.Np);
             T acc = wall_flux_partial<T>(wall, side == 0 ? (long long)M.Np : -(long long)M.Np, M, tb, side, part, P, tid);
@@ -141,19 +150,20 @@ __global__ void __launch_bounds__(kClosureThreads) closure_kernel(ClosureArgs A,
             continue;
         }
         T* recb = rec_all + (long long)(I.cell_off + w.y) * A.rec_stride;
-        if (!closure_cells<T>(A, M, tb, I, w.y, w.z, recb, wst, nbuf, &cbar, phase, NoExtra{}, NoAfterLoads{})) return;
+        if (!closure_cells<T>(A, M, tb, I, w.y, w.z, recb, wst, nbuf, &cbar, phase, NoExtra{}, wait, NoHook{})) return;
     }
+    wait();
 }
 
 // ------------------------------------------------------------------------------ batch closure
-// The closure of a batch as two launches over all items instead of one item chain per block.  With
-// many more items than co-resident blocks the chain form is bound by how many items are in flight:
-// most of its phases run one lane per reach cell while the other lanes wait at its barriers, and
-// its FM band rows are read one item at a time.  Here closure_band_kernel gives every band row of
-// every item to a warp of its own (the band sum of Eq. fm, then chi and nbar into A.cw) and takes
-// the wall items, with no block barrier; closure_records_kernel then forms each item's records from
-// the raw sums of its reach and the band results, every phase spread over the whole block.  Both
-// are made of the chain's per-cell functions (closure_item.cuh), so the records are the chain's.
+// The closure of a batch with a warp for each job and no block barrier.  With many more items than
+// co-resident blocks the chain form is bound by how many items are in flight: most of its phases run one
+// lane per reach cell while the other warps wait at its barriers, and its FM band rows are read one item
+// at a time.  Here closure_band_kernel gives every pair of band rows to a warp (the band sum of Eq. fm,
+// then chi and nbar into A.cw) and takes the wall parts; closure_records_kernel gives every item (28 own
+// cells, 32 with its reach) to a warp, a lane per cell.  Where the bands are short (kInlineBand columns)
+// the records kernel sums them itself and takes the wall parts, and the first launch goes.  All are made
+// of the chain's per-cell functions (closure_item.cuh), so the records are the chain's.
 
 // A warp per job of the host-formed list A.pairs: two band rows summed together by clo_band_row2
 // with the loads of both in flight, then chi and nbar of the two cells; or one part of the
@@ -178,18 +188,9 @@ __global__ void __launch_bounds__(kClosureThreads, sizeof(T) == 4 ? 8 : 4) closu
     for (int v = gw; v < np; v += nw) {
         const BandPair P = A.pairs[v];
         if (P.kmaxA < 0) {
-            // one part of the outgoing flux through a wall, by one warp in the order of the chain
-            // form's block of kClosureThreads threads: lane L takes the momenta of its threads
-            // L, L + 32, L + 64, L + 96 and the four warp sums are combined as there
-            const InstDev I = A.inst[P.q];
-            const int side = -1 - P.kmaxA, part = P.kmaxB, WP = A.wall_parts;
-            const T* wall = fin_all + I.f_off + (side == 0 ? 0LL : (long long)(I.n_cells - 1) * M.Np);
-            T r[kClosureWarps];
-#pragma unroll
-            for (int vw = 0; vw < kClosureWarps; ++vw)
-                r[vw] = warp_sum(wall_flux_partial<T>(wall, side == 0 ? (long long)M.Np : -(long long)M.Np, M, tb, side,
-                                                      part, WP, 32 * vw + lane));
-            if (lane == 0) nwp[((long long)P.q * 2 + side) * WP + part] = wall_part_sum(r);
+            const int side = -1 - P.kmaxA, part = P.kmaxB;
+            const T x = wall_part_of_warp<T>(fin_all, M, tb, A.inst[P.q], side, part, A.wall_parts, lane);
+            if (lane == 0) nwp[((long long)P.q * 2 + side) * A.wall_parts + part] = x;
             continue;
         }
         const T* ndA = dens + P.dA * slices;
@@ -222,112 +223,154 @@ __global__ void __launch_bounds__(kClosureThreads, sizeof(T) == 4 ? 8 : 4) closu
     }
 }
 
+// What a warp of the records kernel shares among its lanes: an item's reach cells, pair terms and
+// expansion coefficients.
 template <typename T>
-__global__ void __launch_bounds__(kClosureThreads, sizeof(T) == 4 ? 8 : 4) closure_records_kernel(ClosureArgs A, MomSet M) {
+struct WarpReach {
+    Wide<T> n[32], Tc[32], u[3][32];
+    T nb[32], gp[5][32], nf[32];
+    EqCoeffs<T> ecs;
+};
+
+// Bound by the latency of one item's chain of phases, with 8 to 16 warps per SM to hide it; every phase
+// but the equilibrium vectors has a lane per cell, so its instructions are shared by up to 32 cells (in
+// FP64, where an instruction costs the same however few lanes take it, that is the point).  kBand: the
+// widest band in units of 32 columns, rounded up to 2 or 4 (0: closure_band_kernel sums the bands).
+template <typename T, int kBand>
+__global__ void __launch_bounds__(kClosureThreads, sizeof(T) == 4 ? 4 : 2) closure_records_kernel(ClosureArgs A, MomSet M) {
     using W = Wide<T>;
-    __shared__ W sw_n[32], sw_T[32], sw_u[3][32];  // reach cells
-    __shared__ T s_chi[32], snb[32];
-    __shared__ T sq[kClosureCells][3], sgeo[kClosureCells][2];  // own cells
-    __shared__ T ecs[kClosureCells][4][kMaxE];
-    __shared__ T sgp[kClosureCells][5][5];
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x;
-    const ClosureTabs<T> tb = closure_tables<T>(reinterpret_cast<T*>(smem_raw), A.tabT, M, tid, NT);
-    __syncthreads();
-    pdl_wait();  // the band results of closure_band_kernel
-    pdl_trigger();
-    T* cw = reinterpret_cast<T*>(A.cw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wpb = blockDim.x >> 5;
+    WarpReach<T>& R = reinterpret_cast<WarpReach<T>*>(smem_raw)[warp];
+    const ClosureTabs<T> tb = closure_tables<T>(reinterpret_cast<T*>(smem_raw + wpb * sizeof(WarpReach<T>)), A.tabT, M, tid, blockDim.x);
     const T* geoT = reinterpret_cast<const T*>(A.geoT);
+    const T* band = reinterpret_cast<const T*>(A.band);
+    const T* dens = reinterpret_cast<const T*>(A.dens);
+    T* cw = reinterpret_cast<T*>(A.cw);
     T* rec_all = reinterpret_cast<T*>(A.rec);
-    const int rs = A.rec_stride, ng = M.nR + M.n2 + M.n3;
-    const ReachView<T> RV{sw_n, sw_T, {sw_u[0], sw_u[1], sw_u[2]}, s_chi, snb};
-    const int nit = *A.n_items;
-    for (int it = blockIdx.x; it < nit; it += gridDim.x) {
+    const int rs = A.rec_stride, slices = A.slices;
+    const ReachView<T> RV{R.n, R.Tc, {R.u[0], R.u[1], R.u[2]}, R.nb};
+    const int nit = *A.n_items, nw = gridDim.x * wpb;
+    __syncthreads();
+    bool waited = false;
+    auto wait = [&]() {
+        if (!waited) {
+            pdl_wait();  // the band results, or the previous stage's sums
+            pdl_trigger();
+            waited = true;
+        }
+    };
+    for (int it = blockIdx.x * wpb + warp; it < nit; it += nw) {
         const int4 w = A.items[it];
-        if (w.w != 0) continue;  // wall items: closure_band_kernel
+        if (!kBand && w.w != 0) continue;  // wall items: closure_band_kernel
         const InstDev I = A.inst[w.x];
+        if (w.w != 0) {
+            wait();
+            const int side = w.w - 1, part = w.z;
+            const T x = wall_part_of_warp<T>(reinterpret_cast<const T*>(A.f_in), M, tb, I, side, part, A.wall_parts, lane);
+            if (lane == 0) reinterpret_cast<T*>(A.nwp)[((long long)w.x * 2 + side) * A.wall_parts + part] = x;
+            continue;
+        }
         const int c0 = w.y, cnt = w.z, N = I.n_cells;
         int h0, h1;
         clo_reach(c0, cnt, N, h0, h1);
-        const int nh = h1 - h0;
-        T* recb = rec_all + (long long)(I.cell_off + c0) * rs;
+        const int nh = h1 - h0, t = h0 + lane - c0;  // this lane's reach cell, and as an own cell
+        const long long gc = (long long)I.cell_off + h0 + min(lane, nh - 1);
+        const bool own = t >= 0 && t < cnt && lane < nh;
+        T* recb = rec_all + ((long long)I.cell_off + c0) * rs;
+        T ct[kCellScalars];
         const T etaf = inst_param<T>(I.etafac, I.f_etafac);
-        // ---- the reach's n, u, T from the raw sums (thread per reach cell), chi and nbar from the
-        // band kernel or, for chi at the local density, here; the own cells' q and geometry
-        for (int e = tid; e < nh; e += NT) {
-            const long long gc = (long long)I.cell_off + h0 + e;
-            W sv[kSums];
-            clo_load_sums<T>(A, gc, sv);
-            W n, u[3], Tc;
-            T q[3];
-            clo_fields<T>(sv, n, u, Tc, q);
-            sw_n[e] = n;
-            sw_u[0][e] = u[0];
-            sw_u[1][e] = u[1];
-            sw_u[2][e] = u[2];
-            sw_T[e] = Tc;
-            const int t = h0 + e - c0;
-            if (I.chi_local) {
-                s_chi[e] = clo_chi<T>(etaf, w_hi(n));
-                snb[e] = w_hi(n);
-                if (t >= 0 && t < cnt) {
-                    cw[gc * 2] = s_chi[e];
-                    cw[gc * 2 + 1] = snb[e];
+        const T geo0 = geoT[gc * kGeo], geo1 = geoT[gc * kGeo + 1];
+        int2 bl = make_int2(0, 0);
+        if (kBand && !I.chi_local) bl = reinterpret_cast<const int2*>(A.band_lo)[gc];
+        wait();
+        // ---- n, u, T of the reach cells, nbar (the band kernel's, or summed here, or local)
+        W sv[kSums];
+        clo_load_sums<T>(A, gc, sv);
+        if (kBand && !I.chi_local) {
+            constexpr int kRows = kBand == 2 ? 8 : 4;
+            for (int r0 = 0; r0 < nh; r0 += kRows) {
+                const T *Wr[kRows], *nd[kRows];
+                int km[kRows];
+                T tot[kRows];
+#pragma unroll
+                for (int r = 0; r < kRows; ++r) {
+                    const int rr = min(r0 + r, nh - 1);
+                    const int lo = __shfl_sync(0xffffffffu, bl.x, rr), ext = __shfl_sync(0xffffffffu, bl.y, rr);
+                    Wr[r] = band + I.band_off + (long long)(h0 + rr) * I.band_w;
+                    nd[r] = dens + ((long long)I.cell_off + lo) * slices;
+                    km[r] = r0 + r < nh ? min(ext, N - lo) : 0;
                 }
-            } else {
-                s_chi[e] = cw[gc * 2];
-                snb[e] = cw[gc * 2 + 1];
-            }
-            if (t >= 0 && t < cnt) {
-                sq[t][0] = q[0];
-                sq[t][1] = q[1];
-                sq[t][2] = q[2];
-                const T* g = geoT + gc * kGeo;
-                sgeo[t][0] = g[0];
-                sgeo[t][1] = g[1];
-            }
-        }
-        __syncthreads();
-        // ---- gradient terms (thread per own cell and stencil position)
-        for (int e = tid; e < cnt * 5; e += NT) {
-            const int t = e / 5, q = e % 5, c = c0 + t;
-            int cq;
-            T wq;
-            stencil5_at<T>(c, N, q, cq, wq);
-            T g[5];
-            clo_grad_terms<T>(RV, cq - h0, c - h0, wq, etaf, I.chi_local != 0, g);
+                clo_band_rows<T, kRows, kBand ? kBand : 4>(Wr, nd, km, slices, lane, tot);
+                // lane 0's sums (every lane ends the butterfly with the total, each in its own order)
+                if (lane == 0)
 #pragma unroll
-            for (int v = 0; v < 5; ++v) sgp[t][v][q] = g[v];
-        }
-        __syncthreads();
-        // ---- expansion coefficients (warp = job, lane = own cell); the last warp, whose job (the
-        // third axis) is the shortest, then the record scalars
-        if (lane < cnt) {
-            const int t = lane, job = warp, lt = c0 + t - h0;
-            const T cT = w_hi(sw_T[lt]);
-            const T tm1 = w_hi(w_sub(sw_T[lt], w_from_t(T(1))));  // T - 1 without cancellation
-            T ev[kMaxE + 1];
-            clo_eq_coeffs<T>(job, cT, tm1, w_hi(sw_u[0][lt]), w_hi(sw_u[job == 2 ? 1 : 2][lt]), tb, M, ev);
-#pragma unroll
-            for (int l = 0; l < kMaxE; ++l) ecs[t][job][l] = ev[l];
-            if (warp == kClosureWarps - 1) {
-                const T q[3] = {sq[t][0], sq[t][1], sq[t][2]};
-                clo_record_scalars<T>(recb + (long long)t * rs, RV, lt, sgp[t], sgeo[t][0], sgeo[t][1], q, I);
+                    for (int r = 0; r < kRows; ++r)
+                        if (r0 + r < nh) R.nb[r0 + r] = tot[r];
             }
         }
-        __syncthreads();
-        // ---- per-axis equilibrium vectors
-        for (int e = tid; e < cnt * ng; e += NT) {
-            const int t = e / ng, k = e % ng;
-            int dst;
-            const T g = clo_g_entry<T>(k, ecs[t], w_hi(sw_T[c0 + t - h0]), tb, M, dst);
-            recb[(long long)t * rs + dst] = g;
+        W n, u[3], Tc;
+        T q[3];
+        clo_fields<T>(sv, n, u, Tc, q);
+        R.n[lane] = n;
+        R.Tc[lane] = Tc;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) R.u[a][lane] = u[a];
+        __syncwarp();
+        if (I.chi_local)
+            R.nb[lane] = w_hi(n);
+        else if (!kBand)
+            R.nb[lane] = cw[gc * 2 + 1];
+        __syncwarp();
+        // ---- the pair terms; of the own cells the expansion coefficients and the transport scalars
+        if (lane < nh - 1) {
+            T d[5];
+            clo_pair_terms<T>(RV, lane, etaf, I.chi_local != 0, d);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) R.gp[v][lane] = d[v];
         }
-        __syncthreads();
-        // ---- discrete mass of the stored equilibrium (a thread per own cell)
-        for (int t = tid; t < cnt; t += NT) clo_mass_normalise<T>(recb + (long long)t * rs, sw_n[c0 + t - h0], M);
-        __syncthreads();  // shared arrays are reused by the next item
+        const T cT = w_hi(Tc), cu0 = w_hi(u[0]), cu1 = w_hi(u[1]), cu2 = w_hi(u[2]);
+        if (own) {
+            const T tm1 = w_hi(w_sub(Tc, w_from_t(T(1))));  // T - 1 without cancellation
+#pragma unroll
+            for (int job = 0; job < 4; ++job) {
+                T ev[kMaxE + 1];
+                clo_eq_coeffs<T>(job, cT, tm1, cu0, job == 2 ? cu1 : cu2, tb, M, ev);
+#pragma unroll
+                for (int l = 0; l < kMaxE; ++l) R.ecs.v[job][l][t] = ev[l];
+            }
+            const T nb = R.nb[lane], chi = clo_chi<T>(etaf, nb);
+            if (kBand || I.chi_local) {
+                cw[gc * 2] = chi;
+                cw[gc * 2 + 1] = nb;
+            }
+            clo_record_transport<T>(ct, n, cu0, cu1, cu2, cT, chi, q, I);
+        }
+        __syncwarp();
+        if (own) clo_record_gradients<T>(ct, c0 + t, N, h0, R.gp, cu0, cu1, cu2, cT, geo0, geo1, I);
+        // ---- the equilibrium vectors and the normalised density (eight lanes per own cell), then the
+        // scalars with it
+        for (int e = lane; e < (8 * cnt + 31) / 32 * 32; e += 32) {
+            const int tt = min(e >> 3, cnt - 1), lt = c0 + tt - h0;
+            const bool on = (e >> 3) < cnt;
+            const T nf = clo_equilibrium<T>(on, e & 7, recb + (long long)tt * rs, R.n[lt], w_hi(R.Tc[lt]), R.ecs, tt, tb, M);
+            if (on && (e & 7) == 0) R.nf[tt] = nf;
+        }
+        __syncwarp();
+        if (own) {
+            ct[0] = R.nf[t];
+            T* dst = recb + (long long)t * rs;
+#pragma unroll
+            for (int k = 0; k < kCellScalars; k += 16 / (int)sizeof(T)) {  // 16-byte stores
+                if constexpr (sizeof(T) == 4)
+                    *reinterpret_cast<float4*>(dst + k) = make_float4(ct[k], ct[k + 1], ct[k + 2], ct[k + 3]);
+                else
+                    *reinterpret_cast<double2*>(dst + k) = make_double2(ct[k], ct[k + 1]);
+            }
+        }
+        __syncwarp();  // the shared arrays are reused by the next item
     }
+    wait();
 }
 
 // ------------------------------------------------------------------------------ state change
@@ -507,33 +550,58 @@ void launch_dens_from_sums(const double* sums, T* dens, long long n, cudaStream_
 }
 
 template <typename T>
-void launch_closure(const ClosureArgs& A, const MomSet& M, int grid, int threads, size_t smem, cudaStream_t s) {
+cudaError_t launch_closure(const ClosureArgs& A, const MomSet& M, int grid, int threads, size_t smem, cudaStream_t s) {
+    if (A.wst_elems % 4) return cudaErrorInvalidValue;  // vector loads of the tables behind the band rows
     if (smem > 32 * 1024) cudaFuncSetAttribute(closure_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_maybe_programmatic(closure_kernel<T>, grid, threads, smem, s, A.programmatic, A, M);
+    return launch_maybe_programmatic(closure_kernel<T>, grid, threads, smem, s, A.programmatic, A, M);
+}
+
+size_t closure_records_smem(int nR, int n2, int n3, int warps, int tsize) {
+    return (size_t)warps * (tsize == 4 ? sizeof(WarpReach<float>) : sizeof(WarpReach<double>)) +
+           (size_t)closure_tab_elems(nR, n2, n3) * tsize + 16;
 }
 
 template <typename T>
-void launch_closure_batch(const ClosureArgs& A, const MomSet& M, int grid, size_t smem, cudaStream_t s) {
-    launch_maybe_programmatic(closure_band_kernel<T>, grid, kClosureThreads, smem, s, A.programmatic, A, M);
-    launch_maybe_programmatic(closure_records_kernel<T>, grid, kClosureThreads, smem, s, A.programmatic, A, M);
+auto closure_records(int inline_band) {
+    return inline_band == 2 ? closure_records_kernel<T, 2> : inline_band ? closure_records_kernel<T, 4> : closure_records_kernel<T, 0>;
 }
 
-int closure_batch_blocks_per_sm(int tsize, size_t smem) {
-    int a = 0, b = 0;
-    cudaError_t e1, e2;
-    if (tsize == 4) {
-        e1 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, closure_band_kernel<float>, kClosureThreads, smem);
-        e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, closure_records_kernel<float>, kClosureThreads, smem);
-    } else {
-        e1 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, closure_band_kernel<double>, kClosureThreads, smem);
-        e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, closure_records_kernel<double>, kClosureThreads, smem);
-    }
-    if (e1 != cudaSuccess || e2 != cudaSuccess) {
-        cudaGetLastError();
-        return 4;
-    }
-    const int n = a < b ? a : b;
-    return n > 0 ? n : 1;
+template <typename T>
+cudaError_t launch_closure_batch(const ClosureArgs& A, const MomSet& M, const ClosureBatchShape& B, cudaStream_t s) {
+    auto rec = closure_records<T>(B.inline_band);
+    const size_t smem = closure_records_smem(M.nR, M.n2, M.n3, B.warps, (int)sizeof(T));
+    cudaError_t e = cudaFuncSetAttribute(rec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && !B.inline_band)
+        e = launch_maybe_programmatic(closure_band_kernel<T>, B.grid_band, kClosureThreads,
+                                      closure_smem_bytes(M.nR, M.n2, M.n3, 0, 0, (int)sizeof(T)), s, A.programmatic, A, M);
+    if (e == cudaSuccess) e = launch_maybe_programmatic(rec, B.grid, 32 * B.warps, smem, s, A.programmatic, A, M);
+    return e;
+}
+
+// Launch shape of the batch form for a work list of `items` items and `pairs` band jobs: as many blocks
+// as reside; fewer warps per block where the items would otherwise leave SMs without one.
+ClosureBatchShape closure_batch_shape(int tsize, int nR, int n2, int n3, int items, int pairs, int inline_band, int n_sm) {
+    ClosureBatchShape B{};
+    B.inline_band = inline_band;
+    B.warps = kClosureWarps;
+    while (B.warps > 1 && items < 2 * B.warps * n_sm) B.warps /= 2;
+    const size_t smem = closure_records_smem(nR, n2, n3, B.warps, tsize);
+    auto resident = [](const void* k, int threads, size_t sm) {
+        int n = 0;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, sm) != cudaSuccess) {
+            cudaGetLastError();
+            return 4;
+        }
+        return n > 0 ? n : 1;
+    };
+    const void* rec = tsize == 4 ? (const void*)closure_records<float>(inline_band) : (const void*)closure_records<double>(inline_band);
+    const void* bk = tsize == 4 ? (const void*)closure_band_kernel<float> : (const void*)closure_band_kernel<double>;
+    auto clamp = [](long long need, long long most) { return (int)(need < 1 ? 1 : need < most ? need : most); };
+    B.grid = clamp((items + B.warps - 1) / B.warps, (long long)n_sm * resident(rec, 32 * B.warps, smem));
+    B.grid_band = clamp((pairs + kClosureWarps - 1) / kClosureWarps,
+                        (long long)n_sm * resident(bk, kClosureThreads, closure_smem_bytes(nR, n2, n3, 0, 0, tsize)));
+    return B;
 }
 
 int closure_blocks_per_sm(int tsize, size_t smem) {
@@ -625,9 +693,9 @@ template void launch_moments<float>(const float*, double*, float*, void*, long l
                                     cudaStream_t);
 template void launch_moments<double>(const double*, double*, double*, void*, long long, int, const double*,
                                      const MomSet&, cudaStream_t);
-template void launch_closure<float>(const ClosureArgs&, const MomSet&, int, int, size_t, cudaStream_t);
-template void launch_closure<double>(const ClosureArgs&, const MomSet&, int, int, size_t, cudaStream_t);
-template void launch_closure_batch<float>(const ClosureArgs&, const MomSet&, int, size_t, cudaStream_t);
-template void launch_closure_batch<double>(const ClosureArgs&, const MomSet&, int, size_t, cudaStream_t);
+template cudaError_t launch_closure<float>(const ClosureArgs&, const MomSet&, int, int, size_t, cudaStream_t);
+template cudaError_t launch_closure<double>(const ClosureArgs&, const MomSet&, int, int, size_t, cudaStream_t);
+template cudaError_t launch_closure_batch<float>(const ClosureArgs&, const MomSet&, const ClosureBatchShape&, cudaStream_t);
+template cudaError_t launch_closure_batch<double>(const ClosureArgs&, const MomSet&, const ClosureBatchShape&, cudaStream_t);
 
 }  // namespace fdlb

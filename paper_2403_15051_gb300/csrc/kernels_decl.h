@@ -100,17 +100,21 @@ template <typename T>
 void launch_dens_from_sums(const double* sums, T* dens, long long n, cudaStream_t s);
 
 template <typename T>
-void launch_closure(const ClosureArgs& A, const MomSet& M, int grid, int threads, size_t smem, cudaStream_t s);
+cudaError_t launch_closure(const ClosureArgs& A, const MomSet& M, int grid, int threads, size_t smem, cudaStream_t s);
 
 size_t closure_smem(int nR, int n2, int n3, int max_union, int wst_elems, int tsize);
 // Blocks of the closure kernel that fit on an SM with `smem` bytes of dynamic shared memory each.
 int closure_blocks_per_sm(int tsize, size_t smem);
-// The batch form of the closure (closure_band_kernel, then closure_records_kernel; items of at
-// most kClosureCells cells), and the blocks of either that reside on one SM.
+// The batch form of the closure: closure_records_kernel, a warp per item of at most kClosureCells
+// cells, after closure_band_kernel unless the bands are short enough for it to sum them itself.
+constexpr int kInlineBandMax = 128;  // columns of the widest band the records kernel sums
+struct ClosureBatchShape {
+    int inline_band;             // columns of the widest band / 32, 2 or 4, when the records kernel sums the bands; 0
+    int warps, grid, grid_band;  // warps per block of the records kernel; grids of the two kernels
+};
+ClosureBatchShape closure_batch_shape(int tsize, int nR, int n2, int n3, int items, int pairs, int inline_band, int n_sm);
 template <typename T>
-void launch_closure_batch(const ClosureArgs& A, const MomSet& M, int grid, size_t smem, cudaStream_t s);
-int closure_batch_blocks_per_sm(int tsize, size_t smem);
-
+cudaError_t launch_closure_batch(const ClosureArgs& A, const MomSet& M, const ClosureBatchShape& B, cudaStream_t s);
 
 #define FDLB_STREAM_DECL(T, G)                                                                             \
     cudaError_t launch_stream_##T##_##G(const StreamCfg& cfg, const StageArgs& A, const MomSet& M, int grid, \

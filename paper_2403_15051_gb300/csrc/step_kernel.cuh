@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(512, 1) step_kernel(StepArgs S, MomSet M) {
 
     uint32_t sphase = 0, cphase = 0;
     unsigned nbar = 0;
-    const int nit = *S.st.n_items;
+    const int nit = *S.st.n_items, WP = S.cl.wall_parts;
     for (int step = 0; step < S.n_steps; ++step) {
         for (int stage = 0; stage < 3; ++stage) {
             // f1 = f + dt L(f); f2 = 3/4 f + 1/4 (f1 + dt L(f1)); f^{n+1} = 1/3 f + 2/3 (f2 + dt L(f2))
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(512, 1) step_kernel(StepArgs S, MomSet M) {
                         if (lane == 0) atomicOr(A.err, 1);  // the stage's own wait reports it too
                         return;
                     }
-                    const int nv = ((wl ? 1 : 0) + (wr ? 1 : 0)) * kWallParts * kClosureWarps;
+                    const int nv = ((wl ? 1 : 0) + (wr ? 1 : 0)) * WP * kClosureWarps;
                     // four virtual warps at a time: independent chains in flight together
                     for (int v0 = w; v0 < nv; v0 += 4 * nw) {
                         T acc[4];
@@ -140,19 +140,19 @@ __global__ void __launch_bounds__(512, 1) step_kernel(StepArgs S, MomSet M) {
                             const int v = v0 + u * nw;
                             acc[u] = T(0);
                             if (v < nv) {
-                                const int side = (wl && v < kWallParts * kClosureWarps) ? 0 : 1;
-                                const int r = v % (kWallParts * kClosureWarps), part = r / kClosureWarps;
+                                const int side = (wl && v < WP * kClosureWarps) ? 0 : 1;
+                                const int r = v % (WP * kClosureWarps), part = r / kClosureWarps;
                                 const T* wall = fs + (long long)((side == 0 ? 0 : N - 1) - wi.y + 3) * Ms;
                                 acc[u] = wall_flux_partial<T>(wall, side == 0 ? (long long)Ms : -(long long)Ms, M, tb, side,
-                                                              part, kWallParts, (r % kClosureWarps) * 32 + lane);
+                                                              part, WP, (r % kClosureWarps) * 32 + lane);
                             }
                         }
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
                             const int v = v0 + u * nw;
                             if (v < nv) {  // warp-uniform
-                                const int side = (wl && v < kWallParts * kClosureWarps) ? 0 : 1;
-                                const int r = v % (kWallParts * kClosureWarps);
+                                const int side = (wl && v < WP * kClosureWarps) ? 0 : 1;
+                                const int r = v % (WP * kClosureWarps);
                                 const T a = warp_sum(acc[u]);
                                 if (lane == 0) wred[side][r / kClosureWarps][r % kClosureWarps] = a;
                             }
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(512, 1) step_kernel(StepArgs S, MomSet M) {
                 // 1. the rows of the stage input, requested after the closure's loads (the
                 // records come from the closure)
                 auto rows = [&]() { stream_issue<T, GEOM, VW, NV, NR_, N2_, N3_>(A, M, wi, I, false); };
-                if (!closure_cells<T>(C, M, tb, I, wi.y, wi.z, cellT, wst, nbuf, &cbar, cphase, walls, rows)) {
+                if (!closure_cells<T>(C, M, tb, I, wi.y, wi.z, cellT, wst, nbuf, &cbar, cphase, walls, NoHook{}, rows)) {
                     stream_wait<T, GEOM, VW, NV, NR_, N2_, N3_>(A, M, sphase);  // the rows still in flight
                     return;
                 }
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(512, 1) step_kernel(StepArgs S, MomSet M) {
                 for (int side = 0; side < 2; ++side) {
                     if (side == 0 ? !wl : !wr) continue;
                     T sum = T(0);
-                    for (int p = 0; p < kWallParts; ++p) sum += wall_part_sum(wred[side][p]);
+                    for (int p = 0; p < WP; ++p) sum += wall_part_sum(wred[side][p]);
                     const T iden = sizeof(T) == 4 ? (T)I.f_nw_iden[side] : (T)I.nw_iden[side];
                     nw[side] = sum * iden;
                 }

@@ -481,7 +481,7 @@ __device__ __forceinline__ void stream_compute(const StageArgs& A, const MomSet&
                 ld_pairs<T, VW>(b + 4 * Ms, r4);
 #pragma unroll
                 for (int h = 0; h < NP; ++h)
-                    vl_[g][h] = weno5_pair<T>(r0[h], r1[h], r2[h], r3[h], r4[h], s3, ns3, dL, dR, e4w_[g][h]);
+                    vl_[g][h] = weno5_pair(r0[h], r1[h], r2[h], r3[h], r4[h], s3, ns3, dL, dR, e4w_[g][h]);
             }
         }
     }
@@ -554,7 +554,7 @@ __device__ __forceinline__ void stream_compute(const StageArgs& A, const MomSet&
                     ld_pairs<T, VW>(b + 4 * Ms, r4);
 #pragma unroll
                     for (int h = 0; h < NP; ++h)
-                        vr[h] = weno5_pair<T>(r0[h], r1[h], r2[h], r3[h], r4[h], s3, ns3, dL, dR, e4w_[g][h]);
+                        vr[h] = weno5_pair(r0[h], r1[h], r2[h], r3[h], r4[h], s3, ns3, dL, dR, e4w_[g][h]);
                 }
                 // curvature force: K^h along i (one column shared by the vector), K_2 along j; each
                 // output sums its terms in the order of the contracted index
