@@ -258,7 +258,7 @@ const char* fdlb_error_string(int code);
  * for handles of more than 64 cells per SM.
  *
  * fdlb_autotune times candidate tile shapes on the device and keeps the fastest: the cells per
- * stream tile (2 .. 32) under each register bound of the stage kernel that is built for the shape
+ * stream item (2 .. 64) under each register bound of the stage kernel that is built for the shape
  * (the compiled arithmetic is the same), then the closure's form and its own cells per item (2, 4,
  * 8, 16), each candidate over three stages written to the stage-1 scratch buffers (the state, its
  * sums and the step count are not touched).  Only these regrouping knobs are searched, so a tuned

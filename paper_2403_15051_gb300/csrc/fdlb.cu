@@ -81,6 +81,9 @@ struct Solver {
     int B = 16, KS = 1, threads = 0;
     StreamCfg scfg{1, 4, 0};
     size_t smem_stream = 0;
+    int march_G = 2, teams = 1;   // cells per group of the stage's march; warps of a block that walk items of their own
+    int tiles = 0;                // the stage kernel stages whole tiles
+    int step_B = 0;               // persistent step kernel: cells of its staged tiles
     int use_bulk = 0;
     int closure_cells = 4, closure_threads = 128;  // own cells per closure item (<= kClosureCells)
     int closure_batch = 0;  // the closure as two launches over all items (items of kClosureCells cells)
@@ -466,6 +469,18 @@ cudaError_t launch_step_dispatch(const Solver& S, const StepArgs* P, int* blocks
                          : launch_step_double_1(S.scfg, P, S.M, S.grid_step, S.threads, S.smem_step, S.stream, blocks_per_sm);
 }
 
+// The stage kernel of the current configuration: its launch, or with `blocks_per_sm` its occupancy.
+cudaError_t launch_stage_kernel(const Solver& S, const StageArgs& A, int grid, int* blocks_per_sm) {
+    const int threads = S.threads * S.teams;
+    if (S.precision == FDLB_FP32)
+        return S.geometry == FDLB_CYL
+                   ? launch_stream_float_0(S.scfg, A, S.M, grid, threads, S.smem_stream, S.stream, blocks_per_sm)
+                   : launch_stream_float_1(S.scfg, A, S.M, grid, threads, S.smem_stream, S.stream, blocks_per_sm);
+    return S.geometry == FDLB_CYL
+               ? launch_stream_double_0(S.scfg, A, S.M, grid, threads, S.smem_stream, S.stream, blocks_per_sm)
+               : launch_stream_double_1(S.scfg, A, S.M, grid, threads, S.smem_stream, S.stream, blocks_per_sm);
+}
+
 // Whether the persistent step kernel runs the current configuration, and its launch shape: the
 // compile-time shapes, one momentum slice, the bulk staging, tiles within the closure's reach,
 // at least one warp beyond the closure's four, and a co-resident grid (every block owns the
@@ -478,7 +493,8 @@ int plan_step_kernel(Solver& S, int n_items) {
         return FDLB_OK;
     // shared memory: the stage's plan, then [staged band rows | closure tables | band-union
     // densities]; static shared memory of the closure (< 16 KB) stays below the opt-in limit
-    const size_t clo_off = (S.smem_stream + 15) / 16 * 16;
+    S.step_B = S.max_tile;
+    const size_t clo_off = (stream_smem_plan(S.step_B, S.M.Ms, S.nR, S.n2, S.n3, S.threads / 32, (int)S.tsize, S.mma_on, 0).total + 15) / 16 * 16;
     const size_t base = clo_off + closure_smem(S.nR, S.n2, S.n3, S.max_union, 0, (int)S.tsize);
     const size_t limit = S.smem_optin > 16384 ? S.smem_optin - 16384 : 0;
     if (base > limit) return FDLB_OK;
@@ -523,6 +539,9 @@ int upload_items(Solver& S) {
             const int per_wave = S.n_sm;
             const int r = (nt * slices + per_wave - 1) / per_wave * per_wave / slices;
             if (r >= nt && r * slices % per_wave == 0 && N / r >= 2) nt = r;
+            // fewer cells than SMs: one to a tile (each computes both its faces, half as much again, on
+            // twice the SMs: the FP64 stage of 64 cells x 128 momenta took 48.8 us in tiles of four)
+            if (!S.fused && !S.tiles && N * slices <= S.n_sm && N * slices <= S.max_sitems) nt = N;
         }
         const int base = N / nt, rem = N % nt;
         int c0 = 0;
@@ -548,7 +567,8 @@ int upload_items(Solver& S) {
     // local density have none), or a wall part; geometry only, so formed here once per work list
     std::vector<BandPair> bp;
     int widest = 0;
-    for (int q : order) widest = std::max(widest, S.inst_h[q].chi_local ? 0 : S.setup[q].band.width);
+    // (over every instance: a captured graph keeps its kernels while instances retire)
+    for (int q = 0; q < S.n_inst; ++q) widest = std::max(widest, S.inst_h[q].chi_local ? 0 : S.setup[q].band.width);
     const bool inline_band = widest <= kInlineBandMax;
     if (S.closure_batch && !inline_band) {
         for (const int4& w : ci) {
@@ -631,7 +651,29 @@ int upload_items(Solver& S) {
     S.closure_smem = closure_smem(S.nR, S.n2, S.n3, max_union, wst, (int)S.tsize);
     S.grid_closure = std::max(1, std::min(nc, S.n_sm * (throughput ? closure_bps : 8)));
     S.cbatch = closure_batch_shape((int)S.tsize, S.nR, S.n2, S.n3, nc, nbp, !inline_band ? 0 : widest <= 64 ? 2 : 4, S.n_sm);
-    S.grid_stream = std::max(1, ns);
+    // The stage: as many blocks as reside, each walking its items one after another with one copy of the
+    // tables.  Generic kernels whose momentum set fits a warp walk an item per warp; up to eight warps share a
+    // block, fewer where the items would otherwise leave SMs without one.
+    S.teams = 1;
+    if (!S.tiles) {
+        const MarchSmem P = march_smem_plan(S.march_G, S.M.Ms, S.nR, S.n2, S.n3, S.threads / 32, (int)S.tsize, S.krg_on ? 1 : 0);
+        if (!S.scfg.spec && S.threads == 32) {
+            // the warps per block that leave the fullest SM the fewest warps (the largest such block)
+            auto most = [&](int t) { return ((ns + t - 1) / t + S.n_sm - 1) / S.n_sm * t; };
+            for (int t = 2; t <= 8; ++t)
+                if (P.teams + (size_t)t * P.team_bytes <= S.smem_optin / 2 && most(t) <= most(S.teams)) S.teams = t;
+        }
+        S.smem_stream = P.teams + (size_t)S.teams * P.team_bytes;
+    }
+    int bps = 0;
+    StageArgs A{};
+    A.mma = S.mma_on;
+    if (launch_stage_kernel(S, A, 0, &bps) != cudaSuccess || bps < 1) {
+        cudaGetLastError();
+        bps = 1;
+    }
+    // (tiles: a block each, placed as blocks finish; their tables cost less than an uneven share of tiles)
+    S.grid_stream = std::max(1, S.tiles ? ns : std::min((ns + S.teams - 1) / S.teams, bps * S.n_sm));
     return plan_step_kernel(S, ns);
 }
 
@@ -672,11 +714,11 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
     StreamCfg cfg{};
     if (S.tsize == 4)
         cfg.vw = S.n2 % 4 == 0 ? 4 : (S.n2 % 2 == 0 ? 2 : 1);
-    else
-        cfg.vw = S.n2 % 2 == 0 ? 2 : 1;
+    else  // (four FP64 momenta per thread: blocks of up to 256 threads, for their registers)
+        cfg.vw = S.n2 % 4 == 0 && Ms <= 1024 ? 4 : (S.n2 % 2 == 0 ? 2 : 1);
     cfg.spec = ((S.geometry == FDLB_CYL && S.nR == 16 && S.n2 == 8 && S.n3 == 8) ||
                 (S.geometry == FDLB_SPH && S.nR == 24 && S.n2 == 12 && S.n3 == 12)) &&
-               cfg.vw == (S.tsize == 4 ? 4 : 2);
+               cfg.vw == (S.tsize == 4 || S.geometry == FDLB_CYL ? 4 : 2);
     const int cap = threads > 0 ? threads : 256;
     // the cylinder's FP32 shape in blocks of at most 128 threads: a thread per whole p_2 row (8
     // momenta; per-vector and per-cell work spread over twice the momenta, half the warps per cell)
@@ -689,11 +731,13 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
     } else if (cfg.spec) {
         // vectors per thread fixed by the instantiation: the smaller count whose block fits the cap
         const int na = S.geometry == FDLB_CYL ? 1 : 2, nb = 2 * na;
-        cfg.nv = ((Vs + na - 1) / na + 31) / 32 * 32 <= std::max(cap, 32) ? na : nb;
+        cfg.nv = cfg.vw * S.tsize == 32 || ((Vs + na - 1) / na + 31) / 32 * 32 <= std::max(cap, 32) ? na : nb;
         nt = ((Vs + cfg.nv - 1) / cfg.nv + 31) / 32 * 32;
     } else {
-        cfg.nv = cfg.vw == 4 ? 2 : 4;  // the most a thread holds; fewer when the block has room
-        nt = (std::min(Vs, cap) + 31) / 32 * 32;
+        // the most a thread holds; fewer when the block has room, except that two vectors per thread
+        // keep up to 64 of them in one warp
+        cfg.nv = cfg.vw == 4 ? (S.tsize == 4 && Vs > 32 ? 2 : 1) : 4;
+        nt = Vs <= 32 * cfg.nv ? 32 : (std::min(Vs, cap) + 31) / 32 * 32;
         if ((long long)nt * cfg.nv < Vs) nt = ((Vs + cfg.nv - 1) / cfg.nv + 31) / 32 * 32;
     }
     if (nt > 512 || (long long)nt * cfg.nv < Vs) return FDLB_EINVAL;
@@ -704,17 +748,25 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
     S.scfg = cfg;
     S.threads = nt;
     S.mma_on = S.tensor && cfg.spec && cfg.vw == 4 && S.tsize == 4 && S.nR % 8 == 0 && !S.krg_on;
-    // shrink the tile until it fits in shared memory
-    for (;;) {
-        StreamSmem P = stream_smem_plan(S.B, Ms, S.nR, S.n2, S.n3, nt / 32, (int)S.tsize, S.mma_on ? 1 : 0,
-                                        S.krg_on ? 1 : 0);
-        if ((size_t)P.total <= S.smem_optin || S.B <= 2) {
+    // the march's ring does not depend on the cells per item; where whole tiles are staged (also by the
+    // persistent step kernel) the tile shrinks until it fits in shared memory
+    S.tiles = stage_tiles((int)S.tsize, cfg.spec) ? 1 : 0;
+    S.B = std::min(S.B, 4096);
+    if (S.tiles || S.fused) {
+        for (;;) {
+            StreamSmem P = stream_smem_plan(S.B, Ms, S.nR, S.n2, S.n3, nt / 32, (int)S.tsize, S.mma_on ? 1 : 0,
+                                            S.krg_on ? 1 : 0);
             S.smem_stream = P.total;
-            break;
+            if ((size_t)P.total <= S.smem_optin || S.B <= 2) break;
+            S.B = std::max(2, S.B / 2);
         }
-        S.B = std::max(2, S.B / 2);
+        if (S.tiles && S.smem_stream > S.smem_optin) return FDLB_EINVAL;
     }
-    if (S.smem_stream > S.smem_optin) return FDLB_EINVAL;
+    for (S.march_G = 2; !S.tiles && S.march_G >= 1; --S.march_G) {
+        const MarchSmem P = march_smem_plan(S.march_G, Ms, S.nR, S.n2, S.n3, nt / 32, (int)S.tsize, S.krg_on ? 1 : 0);
+        if ((size_t)(P.teams + P.team_bytes) <= S.smem_optin) break;
+    }
+    if (S.march_G < 1) return FDLB_EINVAL;
     S.use_bulk = ((size_t)Ms * S.tsize % 16 == 0 && (size_t)S.Np * S.tsize % 16 == 0) ? 1 : 0;
     if (S.gexec) {
         cudaGraphExecDestroy(S.gexec);
@@ -908,20 +960,17 @@ int launch_stream_only(Solver& S, int in, int fn, int out, double a, double b, i
     A.fb = (float)b;
     A.mode = mode;
     A.B = S.B;
+    A.G = S.march_G;
+    A.teams = S.teams;
+    if (S.n2 == kK2Order)
+        for (int e = 0; e < S.n2 * S.n2; ++e) A.K2[(e % S.n2) * S.n2 + e / S.n2] = (float)S.tab_h[S.M.o_K2 + e];
     A.use_bulk = S.use_bulk;
     A.programmatic = S.programmatic;
     A.mma = S.mma_on;
     A.tx_extra = S.test_tx_extra;
     A.krf = S.krg_on ? S.krf : nullptr;
     A.k3f = S.k3_on ? S.k3f : nullptr;
-    cudaError_t e;
-    const int g = S.geometry;
-    if (S.precision == FDLB_FP32)
-        e = g == FDLB_CYL ? launch_stream_float_0(S.scfg, A, S.M, S.grid_stream, S.threads, S.smem_stream, S.stream)
-                          : launch_stream_float_1(S.scfg, A, S.M, S.grid_stream, S.threads, S.smem_stream, S.stream);
-    else
-        e = g == FDLB_CYL ? launch_stream_double_0(S.scfg, A, S.M, S.grid_stream, S.threads, S.smem_stream, S.stream)
-                          : launch_stream_double_1(S.scfg, A, S.M, S.grid_stream, S.threads, S.smem_stream, S.stream);
+    const cudaError_t e = launch_stage_kernel(S, A, S.grid_stream, nullptr);
     S.launches++;
     return cuda_status(e);
 }
@@ -1042,7 +1091,9 @@ int launch_steps_fused(Solver& S, int64_t n) {
     A.gwT = S.gwT;
     A.err = S.err;
     A.mode = 0;
-    A.B = S.B;
+    A.B = S.step_B;
+    A.G = S.march_G;
+    A.teams = 1;
     A.use_bulk = S.use_bulk;
     A.mma = S.mma_on;
     ClosureArgs& C = P.cl;
@@ -1170,7 +1221,7 @@ int run_autotune(Solver& S, bool use_cache) {
     int bestB = S.B, bestC = S.closure_cells, bestM = S.stage_minb, bestBatch = S.closure_batch;
     float best = time_stages(S, e0, e1);
     if (best < 0.f) best = 1e30f;
-    const int Bs[] = {2, 3, 4, 6, 8, 12, 16, 24, 32};
+    const int Bs[] = {2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
     // the register bound of the stage kernel: three blocks per SM where that variant is built, and
     // for the row kernel also two and five
     const bool minb_choice = S.scfg.spec && S.tsize == 4 && S.geometry == FDLB_CYL && S.threads <= 256;

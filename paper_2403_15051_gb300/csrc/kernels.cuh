@@ -64,6 +64,8 @@ struct MomSet {
     int o_pR, o_wR, o_p2, o_w2, o_p3, o_w3, o_KR, o_K2, o_K3, o_GR, o_G2, o_G3, o_ha, o_hb, o_h0;
 };
 
+constexpr int kK2Order = 8;         // second-axis order whose K_2 travels with the stage's launch
+
 struct StageArgs {
     const void* f_in;
     const void* f_n;
@@ -86,13 +88,16 @@ struct StageArgs {
     float fa, fb;                  // the same in FP32
     int wall_parts;
     int mode;                      // 0: RK stage; 1: write L(f_in) to f_out
-    int B;                         // cells per tile
+    int B;                         // cells per tile (staged tiles)
+    int G;                         // cells per group of the march
+    int teams;                     // > 1: every warp of the block walks an item of its own
     int use_bulk;                  // stage the tile with cp.async.bulk
     int programmatic;              // launched with programmatic stream serialization
     int mma;                       // K^h contraction on the tensor cores (FP32 compile-time shapes)
     int tx_extra;                  // test hook: bytes the staged-copy barrier waits for beyond the copy
     const void* krf;               // K^h f of f_in from the contraction kernel (T, layout of f), or
                                    // null: the stage contracts from the K^h table in shared memory
+    float K2[kK2Order * kK2Order]; // K_2 transposed, [b][j], where the second axis has that order
     const void* k3f;               // sphere: K_3 f of f_in (T, layout of f) when the momenta are
                                    // sliced along p_3, or null: contracted from the staged rows
 };

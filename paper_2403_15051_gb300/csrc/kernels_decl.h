@@ -47,7 +47,7 @@ struct StreamSmem {
     int fs, rec, tabs, geo, red, kr, total;
 };
 
-// Shared-memory plan of the stream kernel (byte offsets), shared with the host: the staged rows
+// Shared-memory plan of a staged tile (byte offsets), shared with the host: the staged rows
 // of cells c0-3 .. c0+B+2, the tile's collision records, the tables (the p_2 nodes, K_2
 // transposed, then K^h with row stride kr_stride(nR), K_3 with row stride n3+1, the other nodes
 // and the weights, the wall Maxwellians), the cell geometry and the per-warp partial sums.
@@ -71,6 +71,41 @@ __host__ __device__ inline StreamSmem stream_smem_plan(int B, int Ms, int nR, in
     s.kr = off;  // K^h f of the tile's own cells (tensor-core path)
     if (mma) off += al((long long)B * Ms * tsize);
     s.total = off;
+    return s;
+}
+
+// Whether the stage kernel of a shape stages whole tiles of cells (else it walks a ring of rows): the
+// compile-time shapes in FP32.
+inline __host__ __device__ constexpr bool stage_tiles(int tsize, bool spec) { return tsize == 4 && spec; }
+
+// Rows in the ring of a team that walks groups of G cells: a group's stencils span G + 5 rows, and the
+// next group's G rows are on their way meanwhile; the first face also needs row c0 - 3 of the first G + 6.
+__host__ __device__ inline int march_ring(int G) { return 2 * G + 5; }
+
+struct MarchSmem {
+    int teams, fs, rec, gw, geo, red, team_bytes;  // teams: byte offset of the first team's region; the rest within one
+};
+// Shared-memory plan of the stream kernel: the block's tables, then per team the copy barrier and wall
+// densities, the ring of rows, two groups' records, the wall Maxwellians, two groups' geometry and per-warp
+// sums.
+__host__ __device__ inline MarchSmem march_smem_plan(int G, int Ms, int nR, int n2, int n3, int nwarps, int tsize, int krg) {
+    auto al = [](long long x) { return (int)((x + 15) & ~15LL); };
+    MarchSmem s;
+    // (no K^h table when K^h f comes from the contraction kernel: krg)
+    s.teams = al((long long)(p2_span(n2) + 2 * (nR + n3) + n2 + (krg ? 0 : nR) * kr_stride(nR) + kr_offset(n2, tsize) +
+                             n3 * (n3 + 1)) * tsize);
+    int off = 32;
+    s.fs = off;
+    off += al((long long)march_ring(G) * Ms * tsize);
+    s.rec = off;
+    off += al(2LL * G * record_stride(nR, n2, n3) * tsize);
+    s.gw = off;
+    off += al(2LL * (nR + n2 + n3) * tsize);
+    s.geo = off;
+    off += al(2LL * G * 3 * tsize);
+    s.red = off;
+    off += al(2LL * G * nwarps * 16 * tsize);
+    s.team_bytes = off;
     return s;
 }
 
@@ -118,7 +153,7 @@ cudaError_t launch_closure_batch(const ClosureArgs& A, const MomSet& M, const Cl
 
 #define FDLB_STREAM_DECL(T, G)                                                                             \
     cudaError_t launch_stream_##T##_##G(const StreamCfg& cfg, const StageArgs& A, const MomSet& M, int grid, \
-                                        int threads, size_t smem, cudaStream_t s);
+                                        int threads, size_t smem, cudaStream_t s, int* blocks_per_sm);
 FDLB_STREAM_DECL(float, 0)
 FDLB_STREAM_DECL(float, 1)
 FDLB_STREAM_DECL(double, 0)

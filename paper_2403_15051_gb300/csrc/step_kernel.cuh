@@ -8,7 +8,7 @@
 //      their collision records straight into the shared record array; on a tile near a wall,
 //      the warps beyond the closure's four sum the outgoing wall flux meanwhile, in the closure
 //      kernel's order of the sums;
-//   3. the stage's populations and raw sums (stream_compute, the code of the stage kernel).
+//   3. the stage's populations and raw sums (stage_cell, the code of the stage kernel).
 // Between stages a grid barrier: the next closure reads the raw sums and slice densities of the
 // cells of other blocks.  The records, wall densities and results are those of the closure and
 // stage kernels, bit for bit; what goes away is two launches and two table loads per stage.
@@ -59,23 +59,22 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target) {
 }
 
 template <typename T, int GEOM, int VW, int NV, int NR_, int N2_, int N3_>
-__global__ void __launch_bounds__(512, 1) step_kernel(StepArgs S, MomSet M) {
+__global__ void __launch_bounds__(stage_max_threads<T, VW, 1>(), 1) step_kernel(StepArgs S, MomSet M) {
     __shared__ T wred[2][kWallParts][kClosureWarps];  // wall flux: warp sums per side and part
     __shared__ __align__(8) uint64_t cbar;            // completion of the band-row copy
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31;
     const int nR = NR_ ? NR_ : M.nR, n2 = N2_ ? N2_ : M.n2, n3 = N3_ ? N3_ : M.n3;
     const int KS = M.KS;  // the sphere runs here with one slice (KS = n3)
-    const StreamSmem P = stream_smem_plan(S.st.B, nR * n2 * KS, nR, n2, n3, (int)(blockDim.x >> 5), (int)sizeof(T),
-                                          (sizeof(T) == 4 && S.st.mma) ? 1 : 0);
-    T* cellT = reinterpret_cast<T*>(smem_raw + P.rec);
-    T* fs = reinterpret_cast<T*>(smem_raw + P.fs);
-    uint64_t* sbar = reinterpret_cast<uint64_t*>(smem_raw);  // the stage's copy barrier
+    const StagePtrs<T> SP = tile_ptrs<T, GEOM, VW, NV, NR_, N2_, N3_>(smem_raw, S.st, M);
+    T* cellT = SP.rec;
+    T* fs = SP.fs;
+    uint64_t* sbar = SP.bar;  // the stage's copy barrier
     const int Ms = nR * n2 * KS;
     // closure region: [staged band rows | tables | band-union densities]
     T* wst = reinterpret_cast<T*>(smem_raw + S.clo_off);
     T* ctab = wst + S.cl.wst_elems;
-    stream_tables<T, GEOM, VW, NV, NR_, N2_, N3_>(S.st, M);
+    stage_tables<T, GEOM, VW, NV, NR_, N2_, N3_>(SP, S.st, M);
     const ClosureTabs<T> tb = closure_tables<T>(ctab, S.cl.tabT, M, tid, blockDim.x);
     T* nbuf = ctab + closure_tab_elems(M.nR, M.n2, M.n3);
     if (tid == 0) {
@@ -161,12 +160,16 @@ __global__ void __launch_bounds__(512, 1) step_kernel(StepArgs S, MomSet M) {
                 };
                 // 1. the rows of the stage input, requested after the closure's loads (the
                 // records come from the closure)
-                auto rows = [&]() { stream_issue<T, GEOM, VW, NV, NR_, N2_, N3_>(A, M, wi, I, false); };
+                auto rows = [&]() { tile_request<T, GEOM, VW, NV, NR_, N2_, N3_>(SP, wi, I, false, 3, A, M); };
                 if (!closure_cells<T>(C, M, tb, I, wi.y, wi.z, cellT, wst, nbuf, &cbar, cphase, walls, NoHook{}, rows)) {
-                    stream_wait<T, GEOM, VW, NV, NR_, N2_, N3_>(A, M, sphase);  // the rows still in flight
+                    stage_wait<T, GEOM, VW, NV, NR_, N2_, N3_>(SP, A, M, sphase);  // the rows still in flight
                     return;
                 }
-                stream_statics<T, GEOM, VW, NV, NR_, N2_, N3_>(A, M, wi, I);
+                tile_geometry<T, GEOM, VW, NV, NR_, N2_, N3_>(SP, wi, I, A, M);
+                {
+                    const T* gwi = reinterpret_cast<const T*>(A.gwT) + (long long)wi.x * 2 * (nR + n2 + n3);
+                    for (int e = tid; e < 2 * (nR + n2 + n3); e += blockDim.x) SP.gw[e] = gwi[e];
+                }
                 // the wall densities as the stage kernel forms them from the parts
                 T nw[2] = {T(0), T(0)};
 #pragma unroll
@@ -175,12 +178,12 @@ __global__ void __launch_bounds__(512, 1) step_kernel(StepArgs S, MomSet M) {
                     T sum = T(0);
                     for (int p = 0; p < WP; ++p) sum += wall_part_sum(wred[side][p]);
                     const T iden = sizeof(T) == 4 ? (T)I.f_nw_iden[side] : (T)I.nw_iden[side];
-                    nw[side] = sum * iden;
+                    nw[side] = mul_rn(sum, iden);
                 }
                 // (the wait ends with a block-wide vote: the barrier after the copy and the statics)
-                if (!stream_wait<T, GEOM, VW, NV, NR_, N2_, N3_>(A, M, sphase)) return;
+                if (!stage_wait<T, GEOM, VW, NV, NR_, N2_, N3_>(SP, A, M, sphase)) return;
                 // 3. the stage
-                stream_compute<T, GEOM, VW, NV, NR_, N2_, N3_, true>(A, M, wi, I, nw[0], nw[1]);
+                tile_compute<T, GEOM, VW, NV, NR_, N2_, N3_, true>(SP, wi, I, nw[0], nw[1], A, M);
             }
         }
     }
@@ -218,7 +221,7 @@ cudaError_t step_occupancy_t(int threads, size_t smem, int* blocks_per_sm) {
 template <typename T, int G>
 cudaError_t step_dispatch(const StreamCfg& cfg, const StepArgs* S, const MomSet& M, int grid, int threads, size_t smem,
                           cudaStream_t s, int* blocks_per_sm) {
-    constexpr int VS = sizeof(T) == 4 ? 4 : 2;
+    constexpr int VS = sizeof(T) == 4 || G == 0 ? 4 : 2;
     constexpr int SR = G == 0 ? 16 : 24, S2 = G == 0 ? 8 : 12, S3 = G == 0 ? 8 : 12;
     constexpr int NA = G == 0 ? 1 : 2, NB = 2 * NA;
     if (!cfg.spec || cfg.vw != VS) return cudaErrorInvalidValue;
@@ -226,6 +229,7 @@ cudaError_t step_dispatch(const StreamCfg& cfg, const StepArgs* S, const MomSet&
         if (blocks_per_sm) return step_occupancy_t<T, G, VS, NA, SR, S2, S3>(threads, smem, blocks_per_sm);
         return launch_step_t<T, G, VS, NA, SR, S2, S3>(*S, M, grid, threads, smem, s);
     }
+    if constexpr (sizeof(T) == 4 || G == 1)
     if (cfg.nv == NB) {
         if (blocks_per_sm) return step_occupancy_t<T, G, VS, NB, SR, S2, S3>(threads, smem, blocks_per_sm);
         return launch_step_t<T, G, VS, NB, SR, S2, S3>(*S, M, grid, threads, smem, s);
