@@ -7,10 +7,18 @@
 // complex W x W mixing, G the truncated inverse) -> GELU(v P1 + c1) (hidden H) -> P2 + c2 ->
 // 4 output channels (normalised n, u_2, T, q_R profiles).
 //
-// Precision: FP32 master weights (Adam), BF16 copies of every weight matrix used as GEMM
-// operands, FP32 activations and FP32 accumulation in every product.  The products with a BF16
-// weight operand run on the tensor cores (mma.sync BF16, the activations as two BF16 parts); the
-// products of two FP32 operands (the DFT pair, the weight gradients) on the FP32 pipe.
+// Precision: FP32 master weights (Adam), BF16 copies of every weight matrix used as operands of the
+// products, FP32 activations and FP32 accumulation in every product (a BF16 weight is exact in FP32: one
+// rounding per fused multiply-add).
+//
+// A batch is a few thousand rows of at most a few hundred channels, so a product is microseconds of work
+// and the passes over memory and launches around it are what counts.  A layer is two launches: the
+// spectral path of each (sample, mode) in one block, then the pointwise product, the inverse transform,
+// bias and GELU of 64 rows in one block; the head with the loss is one; the backward pass has the same
+// shape, with GELU's derivative in the epilogue that forms its input; the gradients of every weight
+// matrix but the spectral ones are one launch, split over the rows so that they fill the device (as one
+// product after another, each a single block of 64 x 64 outputs over all rows, they were 6.2 of the
+// 7.0 ms of a training batch of 32), with a second that adds the splits in a fixed order.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -21,7 +29,9 @@
 #include <utility>
 #include <vector>
 
+#include "device_common.cuh"
 #include "internal.h"
+#include "kernels_decl.h"
 
 namespace fdlb {
 namespace {
@@ -32,219 +42,499 @@ constexpr int kCin = 6, kCout = 4;
 __device__ __forceinline__ float to_f(float x) { return x; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
 
-// C[z] = alpha op(A[z]) op(B[z]) + beta C[z], row-major, batch z = blockIdx.z.  64 x 64 tiles,
-// 256 threads, 4 x 4 outputs per thread, K in slices of 16 staged in shared memory, FP32 FMA.
-template <typename TB>
-__global__ void __launch_bounds__(256) gemm_kernel(int M, int N, int K, const float* __restrict__ A, int lda, int tA,
-                                                   long long sA, const TB* __restrict__ Bm, int ldb, int tB,
-                                                   long long sB, float* __restrict__ C, int ldc, long long sC,
-                                                   float alpha, float beta) {
-    __shared__ float As[16][64 + 4];
-    __shared__ float Bs[16][64 + 4];
-    const int z = blockIdx.z;
-    A += z * sA;
-    Bm += z * sB;
-    C += z * sC;
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-            const int kk = e >> 6, mm = e & 63;
-            const int gm = m0 + mm, gk = k0 + kk;
-            float va = 0.f;
-            if (gm < M && gk < K) va = tA ? A[(long long)gk * lda + gm] : A[(long long)gm * lda + gk];
-            As[kk][mm] = va;
-            const int gn = n0 + mm;
-            float vb = 0.f;
-            if (gn < N && gk < K) vb = to_f(tB ? Bm[(long long)gn * ldb + gk] : Bm[(long long)gk * ldb + gn]);
-            Bs[kk][mm] = vb;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * b[j];
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int gm = m0 + ty * 4 + i, gn = n0 + tx * 4 + j;
-            if (gm < M && gn < N) {
-                float* c = C + (long long)gm * ldc + gn;
-                *c = alpha * acc[i][j] + (beta != 0.f ? beta * *c : 0.f);
-            }
-        }
-}
-
-// The products with a BF16 weight operand on the tensor cores: C[z] = alpha A[z] op(B[z]) + beta C[z]
-// with mma.sync m16n8k16 (BF16 operands, FP32 accumulation).  The FP32 activations A are split into
-// two BF16 parts, a = a_hi + a_lo (a_hi = bf16(a), a_lo = bf16(a - a_hi)), and both parts multiply the
-// (exactly BF16) weights: the product keeps ~2^-17 of a's relative accuracy, as the FP32 FMA form does
-// to within that.  64 x 64 output tiles, 128 threads (four warps of 32 x 32: 2 x 4 MMA tiles of
-// 16 x 8), K in slices of 16 staged in shared memory as [row][k] BF16.
-// Fragment ownership of m16n8k16 (g = lane / 4, t = lane % 4; pairs of BF16 per 32-bit register, the
-// lower index in the low half): A a0 (g, 2t..2t+1), a1 (g+8, 2t..), a2 (g, 2t+8..), a3 (g+8, 2t+8..);
-// B b0 (k 2t..2t+1, n g), b1 (k 2t+8..2t+9, n g); D d0 (g, 2t), d1 (g, 2t+1), d2 (g+8, 2t), d3 (g+8, 2t+1).
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-__global__ void __launch_bounds__(128) gemm_bf16_kernel(int M, int N, int K, const float* __restrict__ A, int lda, int tA,
-                                                        long long sA, const __nv_bfloat16* __restrict__ Bm, int ldb, int tB,
-                                                        long long sB, float* __restrict__ C, int ldc, long long sC,
-                                                        float alpha, float beta) {
-    constexpr int KP = 16 + 8;  // padded row: 48 bytes, pairs stay 4-byte aligned
-    __shared__ __align__(16) __nv_bfloat16 Ah[64][KP], Al[64][KP], Bs[64][KP];
-    const int z = blockIdx.z;
-    A += z * sA;
-    Bm += z * sB;
-    C += z * sC;
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-    float acc[2][4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int e = threadIdx.x; e < 64 * 16; e += 128) {
-            const int r = e >> 4, kk = e & 15, gk = k0 + kk;
-            const int gm = m0 + r;
-            float va = 0.f;
-            if (gm < M && gk < K) va = tA ? A[(long long)gk * lda + gm] : A[(long long)gm * lda + gk];
-            const __nv_bfloat16 hi = __float2bfloat16_rn(va);
-            Ah[r][kk] = hi;
-            Al[r][kk] = __float2bfloat16_rn(va - __bfloat162float(hi));
-            const int gn = n0 + r;
-            __nv_bfloat16 vb = __float2bfloat16_rn(0.f);
-            if (gn < N && gk < K) vb = tB ? Bm[(long long)gn * ldb + gk] : Bm[(long long)gk * ldb + gn];
-            Bs[r][kk] = vb;
-        }
-        __syncthreads();
-        uint32_t ah[2][4], al[2][4];
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-            const int r = wm + mt * 16 + g;
-            ah[mt][0] = *reinterpret_cast<const uint32_t*>(&Ah[r][2 * t]);
-            ah[mt][1] = *reinterpret_cast<const uint32_t*>(&Ah[r + 8][2 * t]);
-            ah[mt][2] = *reinterpret_cast<const uint32_t*>(&Ah[r][2 * t + 8]);
-            ah[mt][3] = *reinterpret_cast<const uint32_t*>(&Ah[r + 8][2 * t + 8]);
-            al[mt][0] = *reinterpret_cast<const uint32_t*>(&Al[r][2 * t]);
-            al[mt][1] = *reinterpret_cast<const uint32_t*>(&Al[r + 8][2 * t]);
-            al[mt][2] = *reinterpret_cast<const uint32_t*>(&Al[r][2 * t + 8]);
-            al[mt][3] = *reinterpret_cast<const uint32_t*>(&Al[r + 8][2 * t + 8]);
-        }
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int c = wn + nt * 8 + g;
-            const uint32_t b0 = *reinterpret_cast<const uint32_t*>(&Bs[c][2 * t]);
-            const uint32_t b1 = *reinterpret_cast<const uint32_t*>(&Bs[c][2 * t + 8]);
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-                mma_bf16(acc[mt][nt], al[mt], b0, b1);
-                mma_bf16(acc[mt][nt], ah[mt], b0, b1);
-            }
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int gm = m0 + wm + mt * 16 + g + ((q & 2) ? 8 : 0), gn = n0 + wn + nt * 8 + 2 * t + (q & 1);
-                if (gm < M && gn < N) {
-                    float* c = C + (long long)gm * ldc + gn;
-                    *c = alpha * acc[mt][nt][q] + (beta != 0.f ? beta * *c : 0.f);
-                }
-            }
-}
-
 __device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad_f(float x) {
     return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.39894228040143267794f;
 }
 
-// u <- u + bias (per column); v = GELU(u) when v != nullptr.
-__global__ void bias_act_kernel(float* __restrict__ u, const float* __restrict__ bias, float* __restrict__ v,
-                                long long rows, int cols) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < rows * cols;
-         e += (long long)gridDim.x * blockDim.x) {
-        const float x = u[e] + bias[e % cols];
-        u[e] = x;
-        if (v) v[e] = gelu_f(x);
+constexpr int kT = 64;        // rows and columns of an output tile
+constexpr int kKc = 32;       // contraction values staged at a time
+constexpr int kLd = kT + 4;   // row stride of a staged chunk [k][64]
+constexpr int kNT = 256;      // threads: 16 x 16, 4 x 4 outputs each
+constexpr int kMaxSplits = 64;  // row splits of the weight gradients
+
+// Every kernel here may start while its predecessor drains and waits before it reads anything.
+__device__ __forceinline__ void nn_begin() {
+    pdl_trigger();
+    pdl_wait();
+}
+
+struct Tile {
+    float2 a[4][2];  // 4 rows x 4 columns
+};
+__device__ __forceinline__ void tile_zero(Tile& t) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t.a[i][0] = t.a[i][1] = make_float2(0.f, 0.f);
+}
+// t += X^T Y over the staged chunk: per k two vector loads and eight packed fused multiply-adds.
+__device__ __forceinline__ void tile_mma(Tile& t, const float* X, const float* Y, float sign = 1.f) {
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll 8
+    for (int k = 0; k < kKc; ++k) {
+        const float4 x = *reinterpret_cast<const float4*>(X + k * kLd + ty * 4);
+        const float4 y = *reinterpret_cast<const float4*>(Y + k * kLd + tx * 4);
+        const float xs[4] = {sign * x.x, sign * x.y, sign * x.z, sign * x.w};
+        const float2 y0 = make_float2(y.x, y.y), y1 = make_float2(y.z, y.w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            t.a[i][0] = __ffma2_rn(p_splat(xs[i]), y0, t.a[i][0]);
+            t.a[i][1] = __ffma2_rn(p_splat(xs[i]), y1, t.a[i][1]);
+        }
+    }
+}
+__device__ __forceinline__ float tile_at(const Tile& t, int i, int j) {
+    return j == 0 ? t.a[i][0].x : j == 1 ? t.a[i][0].y : j == 2 ? t.a[i][1].x : t.a[i][1].y;
+}
+
+// dst[k][c] = src[(k0 + k) ld + c0 + c], zero outside k0 + k < kn, c0 + c < cn.
+template <typename TS>
+__device__ __forceinline__ void stage_rows(float* dst, const TS* src, long long ld, long long k0, long long kn, int c0, int cn) {
+    if constexpr (sizeof(TS) == 4) {
+        if ((ld & 3) == 0 && (cn & 3) == 0) {  // (rows start on 16-byte boundaries: the buffers do)
+#pragma unroll
+            for (int e = threadIdx.x; e < kKc * kT / 4; e += kNT) {
+                const int k = e / (kT / 4), c = e % (kT / 4) * 4;
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (k0 + k < kn && c0 + c < cn) v = *reinterpret_cast<const float4*>(src + (k0 + k) * ld + c0 + c);
+                *reinterpret_cast<float4*>(dst + k * kLd + c) = v;
+            }
+            return;
+        }
+    }
+#pragma unroll
+    for (int e = threadIdx.x; e < kKc * kT; e += kNT) {
+        const int k = e / kT, c = e % kT;
+        dst[k * kLd + c] = (k0 + k < kn && c0 + c < cn) ? to_f(src[(k0 + k) * ld + c0 + c]) : 0.f;
+    }
+}
+// dst[k][r] = src[(r0 + r) ld + k0 + k], zero outside r0 + r < rn, k0 + k < kn (a transposed chunk).
+template <typename TS>
+__device__ __forceinline__ void stage_cols(float* dst, const TS* src, long long ld, long long r0, long long rn, int k0, int kn) {
+#pragma unroll
+    for (int e = threadIdx.x; e < kKc * kT; e += kNT) {
+        const int r = e / kKc, k = e % kKc;
+        dst[k * kLd + r] = (r0 + r < rn && k0 + k < kn) ? to_f(src[(r0 + r) * ld + k0 + k]) : 0.f;
     }
 }
 
-// d <- d * GELU'(u)
-__global__ void gelu_back_kernel(float* __restrict__ d, const float* __restrict__ u, long long n) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
-        d[e] *= gelu_grad_f(u[e]);
-}
-
-// column sums of a [rows][cols] array into out[cols] (one block per column, fixed order)
-__global__ void colsum_kernel(const float* __restrict__ x, long long rows, int cols, float* __restrict__ out) {
-    __shared__ float red[32];
-    const int c = blockIdx.x;
-    float s = 0.f;
-    for (long long r = threadIdx.x; r < rows; r += blockDim.x) s += x[r * cols + c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        out[c] = t;
-    }
-}
-
-// Input channels: the five parameters, normalised, broadcast over x, then x / (P - 1).
+// Input channels (the five parameters, normalised, then x / (P - 1)) and the lift, v = a W + b.
 // Normalisation: (log10 Kn + 1), (eta0 - 0.155)/0.145, (ratio - 3.1)/1.9, (u_w - 0.15)/0.15,
 // (T_ratio - 1.15)/0.15 (the ranges of the parameter sweep mapped to about [-1, 1]).
-__global__ void features_kernel(const float* __restrict__ raw, int B, int P, float* __restrict__ a) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < B * P; e += gridDim.x * blockDim.x) {
-        const int b = e / P, x = e % P;
+__global__ void lift_kernel(const float* __restrict__ raw, int B, int P, int W, const __nv_bfloat16* __restrict__ w,
+                            const float* __restrict__ bias, float* __restrict__ a, float* __restrict__ v) {
+    nn_begin();
+    const long long n = (long long)B * P * W;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+        const long long row = e / W;
+        const int c = (int)(e % W), b = (int)(row / P), x = (int)(row % P);
         const float* r = raw + b * 5;
-        float* o = a + (long long)e * kCin;
-        o[0] = log10f(r[0]) + 1.f;
-        o[1] = (r[1] - 0.155f) / 0.145f;
-        o[2] = (r[2] - 3.1f) / 1.9f;
-        o[3] = (r[3] - 0.15f) / 0.15f;
-        o[4] = (r[4] - 1.15f) / 0.15f;
-        o[5] = (float)x / (float)(P - 1);
+        const float f[kCin] = {log10f(r[0]) + 1.f,         (r[1] - 0.155f) / 0.145f, (r[2] - 3.1f) / 1.9f,
+                               (r[3] - 0.15f) / 0.15f, (r[4] - 1.15f) / 0.15f,   (float)x / (float)(P - 1)};
+        float s = bias[c];
+#pragma unroll
+        for (int i = 0; i < kCin; ++i) s = fmaf(f[i], to_f(w[i * W + c]), s);
+        v[e] = s;
+        if (c == 0)
+#pragma unroll
+            for (int i = 0; i < kCin; ++i) a[row * kCin + i] = f[i];
     }
 }
 
-// MSE loss and its gradient: loss = mean (out - t)^2, dout = 2 (out - t) / count.  One block,
-// fixed-order reduction.
-__global__ void mse_kernel(const float* __restrict__ out, const float* __restrict__ t, long long n,
-                           float* __restrict__ dout, float* __restrict__ loss) {
-    __shared__ double red[32];
-    double s = 0.0;
-    for (long long e = threadIdx.x; e < n; e += blockDim.x) {
-        const float d = out[e] - t[e];
-        dout[e] = 2.f * d / (float)n;
-        s += (double)d * d;
+// The spectral path of one sample and mode (block (k, b)).  Forward: vh = F v (rows k and m + k of the DFT)
+// and the mode's complex mixing yh = vh R.  Backward: dyh = G^T du and dvh = dyh R^H in the same form (re, im
+// = columns k, m + k): dre = dyre Rre^T + dyim Rim^T, dim = dyim Rre^T - dyre Rim^T.  Sums over x by groups of
+// threads, in group order; src [P][W] of the sample, hat and mix [2m][W] of the sample.
+template <bool kBack>
+__global__ void __launch_bounds__(kNT) spectral_kernel(const float* __restrict__ src, const float* __restrict__ basis, int P, int W,
+                                                       int m, const __nv_bfloat16* __restrict__ Rre,
+                                                       const __nv_bfloat16* __restrict__ Rim, float* __restrict__ hat,
+                                                       float* __restrict__ mix) {
+    extern __shared__ float sh[];  // [groups][2][W] partial sums, then [2][W]
+    nn_begin();
+    const int k = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+    const float* s = src + (long long)b * P * W;
+    hat += (long long)b * 2 * m * W;
+    mix += (long long)b * 2 * m * W;
+    Rre += (long long)k * W * W;
+    Rim += (long long)k * W * W;
+    const int groups = W <= kNT ? kNT / W : 1;
+    float* tot = sh + 2 * (size_t)groups * W;
+    if (tid < groups * W || W > kNT) {
+        const int g = W <= kNT ? tid / W : 0;
+        for (int c = W <= kNT ? tid % W : tid; c < W; c += kNT) {
+            float re = 0.f, im = 0.f;
+#pragma unroll 8
+            for (int x = g; x < P; x += groups) {
+                const float v = s[(long long)x * W + c];
+                re = fmaf(kBack ? basis[x * 2 * m + k] : basis[k * P + x], v, re);
+                im = fmaf(kBack ? basis[x * 2 * m + m + k] : basis[(m + k) * P + x], v, im);
+            }
+            sh[(g * 2) * W + c] = re;
+            sh[(g * 2 + 1) * W + c] = im;
+        }
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-        *loss = (float)(tot / (double)n);
+    for (int e = tid; e < 2 * W; e += kNT) {
+        float t = 0.f;
+        for (int g = 0; g < groups; ++g) t += sh[g * 2 * W + e];
+        tot[e] = t;
+        hat[(long long)(e < W ? k : m + k) * W + e % W] = t;
     }
+    __syncthreads();
+    const float *tr = tot, *ti = tot + W;
+    if constexpr (!kBack) {
+        // yre = re Rre - im Rim, yim = re Rim + im Rre: a thread per output and group of inputs
+        if (tid < groups * W || W > kNT) {
+            const int g = W <= kNT ? tid / W : 0;
+            for (int o = W <= kNT ? tid % W : tid; o < W; o += kNT) {
+                float yr = 0.f, yi = 0.f;
+#pragma unroll 8
+                for (int i = g; i < W; i += groups) {
+                    const float a = to_f(Rre[i * W + o]), c = to_f(Rim[i * W + o]);
+                    yr = fmaf(tr[i], a, fmaf(-ti[i], c, yr));
+                    yi = fmaf(tr[i], c, fmaf(ti[i], a, yi));
+                }
+                sh[(g * 2) * W + o] = yr;
+                sh[(g * 2 + 1) * W + o] = yi;
+            }
+        }
+        __syncthreads();
+        for (int e = tid; e < 2 * W; e += kNT) {
+            float t = 0.f;
+            for (int g = 0; g < groups; ++g) t += sh[g * 2 * W + e];
+            mix[(long long)(e < W ? k : m + k) * W + e % W] = t;
+        }
+    } else {
+        // a warp per input row of R, its lanes over the outputs
+        const int lane = tid & 31;
+#pragma unroll 2
+        for (int i = tid >> 5; i < W; i += kNT / 32) {
+            float dr = 0.f, di = 0.f;
+            for (int o = lane; o < W; o += 32) {
+                const float a = to_f(Rre[i * W + o]), c = to_f(Rim[i * W + o]);
+                dr = fmaf(tr[o], a, fmaf(ti[o], c, dr));
+                di = fmaf(ti[o], a, fmaf(-tr[o], c, di));
+            }
+            dr = warp_sum(dr);
+            di = warp_sum(di);
+            if (lane == 0) {
+                mix[(long long)k * W + i] = dr;
+                mix[(long long)(m + k) * W + i] = di;
+            }
+        }
+    }
+}
+
+// 64 rows of one sample (grid: row tiles, samples, column tiles) through a layer.
+// Forward: u = v W + b + G yh, vout = GELU(u).
+__global__ void __launch_bounds__(kNT) layer_kernel(const float* __restrict__ v, int P, int W, int m,
+                                                    const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
+                                                    const float* __restrict__ G, const float* __restrict__ yh,
+                                                    float* __restrict__ u, float* __restrict__ vout) {
+    __shared__ __align__(16) float X[kKc * kLd], Y[kKc * kLd];
+    nn_begin();
+    const int r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT;
+    const float* vb = v + (long long)b * P * W;
+    Tile t;
+    tile_zero(t);
+    for (int k0 = 0; k0 < W; k0 += kKc) {
+        stage_cols(X, vb, W, r0, P, k0, W);
+        stage_rows(Y, w, W, k0, W, n0, W);
+        __syncthreads();
+        tile_mma(t, X, Y);
+        __syncthreads();
+    }
+    for (int k0 = 0; k0 < 2 * m; k0 += kKc) {
+        stage_cols(X, G, 2 * m, r0, P, k0, 2 * m);
+        stage_rows(Y, yh + (long long)b * 2 * m * W, W, k0, 2 * m, n0, W);
+        __syncthreads();
+        tile_mma(t, X, Y);
+        __syncthreads();
+    }
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int x = r0 + ty * 4 + i, c = n0 + tx * 4 + j;
+            if (x < P && c < W) {
+                const long long e = ((long long)b * P + x) * W + c;
+                const float s = tile_at(t, i, j) + bias[c];
+                u[e] = s;
+                vout[e] = gelu_f(s);
+            }
+        }
+}
+
+// Backward: dv = du W^T + F^T dvh, and into `out` dv GELU'(u) (in place of u, the layer below's du), or dv
+// itself where u is null.
+__global__ void __launch_bounds__(kNT) layer_back_kernel(const float* __restrict__ du, int P, int W, int m,
+                                                         const __nv_bfloat16* __restrict__ w, const float* __restrict__ F,
+                                                         const float* __restrict__ dvh, const float* u, float* out) {
+    __shared__ __align__(16) float X[kKc * kLd], Y[kKc * kLd];
+    nn_begin();
+    const int r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT;
+    Tile t;
+    tile_zero(t);
+    for (int k0 = 0; k0 < W; k0 += kKc) {
+        stage_cols(X, du + (long long)b * P * W, W, r0, P, k0, W);
+        stage_cols(Y, w, W, n0, W, k0, W);
+        __syncthreads();
+        tile_mma(t, X, Y);
+        __syncthreads();
+    }
+    for (int k0 = 0; k0 < 2 * m; k0 += kKc) {
+        stage_rows(X, F, P, k0, 2 * m, r0, P);
+        stage_rows(Y, dvh + (long long)b * 2 * m * W, W, k0, 2 * m, n0, W);
+        __syncthreads();
+        tile_mma(t, X, Y);
+        __syncthreads();
+    }
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int x = r0 + ty * 4 + i, c = n0 + tx * 4 + j;
+            if (x < P && c < W) {
+                const long long e = ((long long)b * P + x) * W + c;
+                out[e] = u ? tile_at(t, i, j) * gelu_grad_f(u[e]) : tile_at(t, i, j);
+            }
+        }
+}
+
+// The head for 64 rows: z1 = v P1 + c1, h = GELU(z1), out = h P2 + c2, hidden units 64 at a time; z1 and h
+// are kept where not null (the backward pass).  With targets also the loss: dout = 2 (out - t) / count and
+// the block's sum of (out - t)^2.
+__global__ void __launch_bounds__(kNT) head_kernel(const float* __restrict__ v, long long rows, int W, int H,
+                                                   const __nv_bfloat16* __restrict__ p1, const float* __restrict__ c1,
+                                                   const __nv_bfloat16* __restrict__ p2, const float* __restrict__ c2,
+                                                   float* __restrict__ z1, float* __restrict__ h, float* __restrict__ out,
+                                                   const float* __restrict__ tgt, float* __restrict__ dout,
+                                                   double* __restrict__ loss_part) {
+    __shared__ __align__(16) float X[kKc * kLd], Y[kKc * kLd];
+    __shared__ float hs[kT][kT + 1], w2[kT][kCout];
+    __shared__ double red[kNT / 32];
+    nn_begin();
+    const long long r0 = (long long)blockIdx.x * kT;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int orow = threadIdx.x / kCout, oc = threadIdx.x % kCout;  // this thread's output
+    float o = 0.f;
+    for (int n0 = 0; n0 < H; n0 += kT) {
+        Tile t;
+        tile_zero(t);
+        for (int k0 = 0; k0 < W; k0 += kKc) {
+            stage_cols(X, v, W, r0, rows, k0, W);
+            stage_rows(Y, p1, H, k0, W, n0, H);
+            __syncthreads();
+            tile_mma(t, X, Y);
+            __syncthreads();
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = n0 + tx * 4 + j;
+                const long long r = r0 + ty * 4 + i;
+                float hv = 0.f;
+                if (r < rows && c < H) {
+                    const float z = tile_at(t, i, j) + c1[c];
+                    hv = gelu_f(z);
+                    if (z1) {
+                        z1[r * H + c] = z;
+                        h[r * H + c] = hv;
+                    }
+                }
+                hs[ty * 4 + i][tx * 4 + j] = hv;
+            }
+        for (int e = threadIdx.x; e < kT * kCout; e += kNT)
+            w2[e / kCout][e % kCout] = n0 + e / kCout < H ? to_f(p2[(n0 + e / kCout) * kCout + e % kCout]) : 0.f;
+        __syncthreads();
+#pragma unroll 16
+        for (int j = 0; j < kT; ++j) o = fmaf(hs[orow][j], w2[j][oc], o);
+        __syncthreads();
+    }
+    o += c2[oc];
+    const long long r = r0 + orow;
+    double d2 = 0.0;
+    if (r < rows) {
+        out[r * kCout + oc] = o;
+        if (tgt) {
+            const float d = o - tgt[r * kCout + oc];
+            dout[r * kCout + oc] = 2.f * d / (float)(rows * kCout);
+            d2 = (double)d * d;
+        }
+    }
+    if (tgt) {
+        d2 = warp_sum(d2);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = d2;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int w = 0; w < kNT / 32; ++w) s += red[w];
+            loss_part[blockIdx.x] = s;
+        }
+    }
+}
+static_assert(kT * kCout == kNT, "a thread per output of the head's tile");
+
+// The head backwards for 64 rows: dz1 = (dout P2^T) GELU'(z1) (in place of z1), then dv = dz1 P1^T and
+// du = dv GELU'(u) of the last layer (in place of u).  Column tiles beyond the first leave z1 as it is and
+// are launched after it: they read dz1.
+__global__ void __launch_bounds__(kNT) head_back_kernel(const float* __restrict__ dout, long long rows, int W, int H,
+                                                        const __nv_bfloat16* __restrict__ p1,
+                                                        const __nv_bfloat16* __restrict__ p2, float* z1, float* u, int n0) {
+    __shared__ __align__(16) float X[kKc * kLd], Y[kKc * kLd];
+    nn_begin();
+    const long long r0 = (long long)blockIdx.x * kT;
+    Tile t;
+    tile_zero(t);
+    for (int k0 = 0; k0 < H; k0 += kKc) {
+        for (int e = threadIdx.x; e < kKc * kT; e += kNT) {
+            const int rr = e / kKc, k = e % kKc;
+            const long long r = r0 + rr;
+            float d = 0.f;
+            if (r < rows && k0 + k < H) {
+                const long long q = r * H + k0 + k;
+                if (n0 == 0) {
+                    const float* dr = dout + r * kCout;
+                    const __nv_bfloat16* p = p2 + (k0 + k) * kCout;
+                    float s = 0.f;
+#pragma unroll
+                    for (int c = 0; c < kCout; ++c) s = fmaf(dr[c], to_f(p[c]), s);
+                    d = s * gelu_grad_f(z1[q]);
+                    z1[q] = d;
+                } else {
+                    d = z1[q];
+                }
+            }
+            X[k * kLd + rr] = d;
+        }
+        stage_cols(Y, p1, H, n0, W, k0, H);
+        __syncthreads();
+        tile_mma(t, X, Y);
+        __syncthreads();
+    }
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const long long r = r0 + ty * 4 + i;
+            const int c = n0 + tx * 4 + j;
+            if (r < rows && c < W) u[r * W + c] = tile_at(t, i, j) * gelu_grad_f(u[r * W + c]);
+        }
+}
+
+// ---- gradients of the weights that act on rows: C = X^T Y over the rows of one split (blockIdx.y), with
+// the column sums of Y (the bias gradients) from the tiles of the first 64 rows of C.  A task is one weight
+// matrix; its tiles are consecutive blocks.  The splits' results go to part[split][.], the tasks' matrices
+// and biases one after another as in the parameter vector without the spectral weights.
+struct GradTask {
+    const float *X, *Y;
+    int M, N;        // columns of X and Y
+    int tile0;       // first tile
+    long long out;   // the matrix in part; the bias follows it
+};
+constexpr int kMaxTasks = 19;  // 16 layers, the lift, the head's two
+struct GradTasks {
+    GradTask t[kMaxTasks];
+    int n;
+};
+__global__ void __launch_bounds__(kNT) grad_kernel(GradTasks T, long long rows, int splits, float* __restrict__ part, long long stride) {
+    __shared__ __align__(16) float X[kKc * kLd], Y[kKc * kLd];
+    nn_begin();
+    int q = 0;
+    while (q + 1 < T.n && (int)blockIdx.x >= T.t[q + 1].tile0) ++q;
+    const GradTask g = T.t[q];
+    const int nt = (g.N + kT - 1) / kT, tile = blockIdx.x - g.tile0, m0 = tile / nt * kT, n0 = tile % nt * kT;
+    const long long lo = rows * blockIdx.y / splits, hi = rows * (blockIdx.y + 1) / splits;
+    Tile t;
+    tile_zero(t);
+    float cs = 0.f;
+    for (long long k0 = lo; k0 < hi; k0 += kKc) {
+        stage_rows(X, g.X, g.M, k0, hi, m0, g.M);
+        stage_rows(Y, g.Y, g.N, k0, hi, n0, g.N);
+        __syncthreads();
+        tile_mma(t, X, Y);
+        if (m0 == 0 && threadIdx.x < kT)
+#pragma unroll 8
+            for (int k = 0; k < kKc; ++k) cs += Y[k * kLd + threadIdx.x];
+        __syncthreads();
+    }
+    float* C = part + blockIdx.y * stride + g.out;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int a = m0 + ty * 4 + i, c = n0 + tx * 4 + j;
+            if (a < g.M && c < g.N) C[(long long)a * g.N + c] = tile_at(t, i, j);
+        }
+    if (m0 == 0 && threadIdx.x < kT && n0 + threadIdx.x < g.N) C[(long long)g.M * g.N + n0 + threadIdx.x] = cs;
+}
+
+// Gradients of the spectral weights: block (l m + k, row tile, column tile): dRre = re^T dyre + im^T dyim,
+// dRim = re^T dyim - im^T dyre over the samples.
+__global__ void __launch_bounds__(kNT) grad_spectral_kernel(const float* __restrict__ vh, const float* __restrict__ dyh, int B, int W,
+                                                            int m, float* __restrict__ g, long long o_rre, long long layer_stride) {
+    __shared__ __align__(16) float Xr[kKc * kLd], Xi[kKc * kLd], Yr[kKc * kLd], Yi[kKc * kLd];
+    nn_begin();
+    const int l = blockIdx.x / m, k = blockIdx.x % m, i0 = blockIdx.y * kT, n0 = blockIdx.z * kT;
+    const long long ld = 2LL * m * W;
+    const float* x = vh + l * B * ld + (long long)k * W;
+    const float* y = dyh + l * B * ld + (long long)k * W;
+    Tile tr, ti;
+    tile_zero(tr);
+    tile_zero(ti);
+    for (int k0 = 0; k0 < B; k0 += kKc) {
+        stage_rows(Xr, x, ld, k0, B, i0, W);
+        stage_rows(Xi, x + (long long)m * W, ld, k0, B, i0, W);
+        stage_rows(Yr, y, ld, k0, B, n0, W);
+        stage_rows(Yi, y + (long long)m * W, ld, k0, B, n0, W);
+        __syncthreads();
+        tile_mma(tr, Xr, Yr);
+        tile_mma(tr, Xi, Yi);
+        tile_mma(ti, Xr, Yi);
+        tile_mma(ti, Xi, Yr, -1.f);
+        __syncthreads();
+    }
+    float* gr = g + o_rre + l * layer_stride + (long long)k * W * W;
+    float* gi = gr + (long long)m * W * W;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int a = i0 + ty * 4 + i, c = n0 + tx * 4 + j;
+            if (a < W && c < W) {
+                gr[(long long)a * W + c] = tile_at(tr, i, j);
+                gi[(long long)a * W + c] = tile_at(ti, i, j);
+            }
+        }
+}
+
+// The splits added in order into the gradient (compact index to parameter: the lift, each layer's W and b
+// behind its spectral weights, the head), and the loss from the head's blocks.
+__global__ void __launch_bounds__(kNT) grad_sum_kernel(const float* __restrict__ part, long long stride, int splits, long long n_lift,
+                                                       long long per_layer, int L, long long spectral, float* __restrict__ g,
+                                                       const double* __restrict__ loss_part, int blocks, double count,
+                                                       float* __restrict__ loss) {
+    nn_begin();
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        double s = 0.0;
+        for (int i = threadIdx.x; i < blocks; i += 32) s += loss_part[i];
+        s = warp_sum(s);
+        if (threadIdx.x == 0) *loss = (float)(s / count);
+    }
+    const long long e = blockIdx.x * (long long)kNT + threadIdx.x;
+    if (e >= stride) return;
+    float s = 0.f;
+#pragma unroll 8
+    for (int q = 0; q < splits; ++q) s += part[q * stride + e];
+    // (spectral weights before this entry: those of its layer and the layers below)
+    const long long layers = e < n_lift ? 0 : min((e - n_lift) / per_layer + 1, (long long)L);
+    g[e + layers * spectral] = s;
 }
 
 // Adam (beta1 0.9, beta2 0.999, eps 1e-8) on the FP32 master weights, then the BF16 copy.
@@ -283,111 +573,89 @@ struct NNet {
     float *w = nullptr, *g = nullptr, *m1 = nullptr, *m2 = nullptr;
     __nv_bfloat16* wb = nullptr;
     float *F = nullptr, *G = nullptr;
-    float *raw = nullptr, *a = nullptr, *vs = nullptr, *us = nullptr, *vh = nullptr, *yh = nullptr, *s = nullptr;
-    float *z1 = nullptr, *h = nullptr, *out = nullptr, *tgt = nullptr, *dout = nullptr, *dh = nullptr;
-    float *dv = nullptr, *dv2 = nullptr, *du = nullptr, *dyh = nullptr, *dvh = nullptr, *loss = nullptr;
+    float *raw = nullptr, *a = nullptr, *vs = nullptr, *us = nullptr, *vh = nullptr, *yh = nullptr;
+    float *z1 = nullptr, *h = nullptr, *out = nullptr, *tgt = nullptr, *dout = nullptr;
+    float *dv = nullptr, *dyh = nullptr, *dvh = nullptr, *loss = nullptr, *part = nullptr;
+    double* loss_part = nullptr;
+    long long n_rows_params = 0;  // parameters without the spectral weights
     int step = 0;
 };
 
 namespace {
 
-template <typename TB>
-cudaError_t gemm(NNet& n, int M, int N, int K, const float* A, int lda, int tA, long long sA, const TB* B, int ldb,
-                 int tB, long long sB, float* C, int ldc, long long sC, int batch, float alpha, float beta) {
-    dim3 grid((N + 63) / 64, (M + 63) / 64, batch);
-    if constexpr (std::is_same<TB, __nv_bfloat16>::value)
-        gemm_bf16_kernel<<<grid, 128, 0, n.stream>>>(M, N, K, A, lda, tA, sA, B, ldb, tB, sB, C, ldc, sC, alpha, beta);
-    else
-        gemm_kernel<TB><<<grid, 256, 0, n.stream>>>(M, N, K, A, lda, tA, sA, B, ldb, tB, sB, C, ldc, sC, alpha, beta);
-    return cudaGetLastError();
-}
-
 int grid_for(long long n) { return (int)std::min<long long>((n + 255) / 256, 4096); }
 
-// Forward pass for B samples whose raw parameters are in n.raw; leaves every activation the
-// backward pass needs.
-int forward(NNet& n, int B) {
+// Launches with programmatic stream serialization (nn_begin); the last error is read by the caller.
+template <typename... KA, typename... A>
+void nn_launch(NNet& n, void (*kern)(KA...), dim3 grid, size_t smem, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kNT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = n.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, KA(args)...);
+}
+
+unsigned tiles(long long n) { return (unsigned)((n + kT - 1) / kT); }
+size_t spectral_smem(int W) { return (size_t)(W <= kNT ? kNT / W + 1 : 2) * 2 * W * sizeof(float); }
+int grad_splits(long long rows) { return (int)std::min<long long>((rows + 127) / 128, kMaxSplits); }
+
+// Forward pass for B samples whose raw parameters are in n.raw; for training (targets in n.tgt) leaves every
+// activation the backward pass needs, dout and the loss's parts.
+int forward(NNet& n, int B, bool train) {
     const int W = n.W, m = n.m, P = n.P, H = n.H;
     const long long rows = (long long)B * P;
-    features_kernel<<<grid_for(rows), 256, 0, n.stream>>>(n.raw, B, P, n.a);
-    float* v0 = n.vs;
-    gemm(n, (int)rows, W, kCin, n.a, kCin, 0, 0, n.wb + n.o_lw, W, 0, 0, v0, W, 0, 1, 1.f, 0.f);
-    bias_act_kernel<<<grid_for(rows * W), 256, 0, n.stream>>>(v0, n.w + n.o_lb, nullptr, rows, W);
+    nn_launch(n, lift_kernel, dim3(grid_for(rows * W)), 0, n.raw, B, P, W, n.wb + n.o_lw, n.w + n.o_lb, n.a, n.vs);
     for (int l = 0; l < n.L; ++l) {
         float* v = n.vs + (long long)l * rows * W;
-        float* vn = n.vs + (long long)(l + 1) * rows * W;
-        float* u = n.us + (long long)l * rows * W;
         float* vh = n.vh + (long long)l * B * 2 * m * W;
-        // spectral path: vh[b] = F v[b]; per mode k: yre = re Rre - im Rim, yim = re Rim + im Rre;
-        // s[b] = G yh[b]
-        gemm(n, 2 * m, W, P, n.F, P, 0, 0, v, W, 0, (long long)P * W, vh, W, (long long)2 * m * W, B, 1.f, 0.f);
-        const __nv_bfloat16* rre = n.wb + n.o_rre[l];
-        const __nv_bfloat16* rim = n.wb + n.o_rim[l];
-        const int ld = 2 * m * W;
-        gemm(n, B, W, W, vh, ld, 0, W, rre, W, 0, (long long)W * W, n.yh, ld, W, m, 1.f, 0.f);
-        gemm(n, B, W, W, vh + m * W, ld, 0, W, rim, W, 0, (long long)W * W, n.yh, ld, W, m, -1.f, 1.f);
-        gemm(n, B, W, W, vh, ld, 0, W, rim, W, 0, (long long)W * W, n.yh + m * W, ld, W, m, 1.f, 0.f);
-        gemm(n, B, W, W, vh + m * W, ld, 0, W, rre, W, 0, (long long)W * W, n.yh + m * W, ld, W, m, 1.f, 1.f);
-        gemm(n, P, W, 2 * m, n.G, 2 * m, 0, 0, n.yh, W, 0, (long long)2 * m * W, u, W, (long long)P * W, B, 1.f, 0.f);
-        // pointwise path and activation: u = s + v W_l + b_l, v' = GELU(u)
-        gemm(n, (int)rows, W, W, v, W, 0, 0, n.wb + n.o_w[l], W, 0, 0, u, W, 0, 1, 1.f, 1.f);
-        bias_act_kernel<<<grid_for(rows * W), 256, 0, n.stream>>>(u, n.w + n.o_b[l], vn, rows, W);
+        nn_launch(n, spectral_kernel<false>, dim3(m, B), spectral_smem(W), v, n.F, P, W, m, n.wb + n.o_rre[l], n.wb + n.o_rim[l], vh,
+                  n.yh);
+        nn_launch(n, layer_kernel, dim3(tiles(P), B, tiles(W)), 0, v, P, W, m, n.wb + n.o_w[l], n.w + n.o_b[l], n.G, n.yh,
+                  n.us + (long long)l * rows * W, v + rows * W);
     }
-    const float* vL = n.vs + (long long)n.L * rows * W;
-    gemm(n, (int)rows, H, W, vL, W, 0, 0, n.wb + n.o_p1w, H, 0, 0, n.z1, H, 0, 1, 1.f, 0.f);
-    bias_act_kernel<<<grid_for(rows * H), 256, 0, n.stream>>>(n.z1, n.w + n.o_p1b, n.h, rows, H);
-    gemm(n, (int)rows, kCout, H, n.h, H, 0, 0, n.wb + n.o_p2w, kCout, 0, 0, n.out, kCout, 0, 1, 1.f, 0.f);
-    bias_act_kernel<<<grid_for(rows * kCout), 256, 0, n.stream>>>(n.out, n.w + n.o_p2b, nullptr, rows, kCout);
+    nn_launch(n, head_kernel, dim3(tiles(rows)), 0, n.vs + (long long)n.L * rows * W, rows, W, H, n.wb + n.o_p1w, n.w + n.o_p1b,
+              n.wb + n.o_p2w, n.w + n.o_p2b, train ? n.z1 : nullptr, n.h, n.out, train ? n.tgt : nullptr, n.dout, n.loss_part);
     return cudaGetLastError() == cudaSuccess ? FDLB_OK : FDLB_ECUDA;
 }
 
-// Backward pass from n.dout into n.g (reverse order of `forward`).
+// Backward pass from n.dout into n.g (reverse order of `forward`), and the loss.
 int backward(NNet& n, int B) {
-    const int W = n.W, m = n.m, P = n.P, H = n.H;
-    const long long rows = (long long)B * P;
-    float* g = n.g;
-    gemm(n, H, kCout, (int)rows, n.h, H, 1, 0, n.dout, kCout, 0, 0, g + n.o_p2w, kCout, 0, 1, 1.f, 0.f);
-    colsum_kernel<<<kCout, 256, 0, n.stream>>>(n.dout, rows, kCout, g + n.o_p2b);
-    gemm(n, (int)rows, H, kCout, n.dout, kCout, 0, 0, n.wb + n.o_p2w, kCout, 1, 0, n.dh, H, 0, 1, 1.f, 0.f);
-    gelu_back_kernel<<<grid_for(rows * H), 256, 0, n.stream>>>(n.dh, n.z1, rows * H);
-    const float* vL = n.vs + (long long)n.L * rows * W;
-    gemm(n, W, H, (int)rows, vL, W, 1, 0, n.dh, H, 0, 0, g + n.o_p1w, H, 0, 1, 1.f, 0.f);
-    colsum_kernel<<<H, 256, 0, n.stream>>>(n.dh, rows, H, g + n.o_p1b);
-    gemm(n, (int)rows, W, H, n.dh, H, 0, 0, n.wb + n.o_p1w, H, 1, 0, n.dv, W, 0, 1, 1.f, 0.f);
-    const int ld = 2 * m * W;
-    for (int l = n.L - 1; l >= 0; --l) {
-        const float* v = n.vs + (long long)l * rows * W;
-        const float* u = n.us + (long long)l * rows * W;
-        const float* vh = n.vh + (long long)l * B * 2 * m * W;
-        const __nv_bfloat16* rre = n.wb + n.o_rre[l];
-        const __nv_bfloat16* rim = n.wb + n.o_rim[l];
-        // du = dv GELU'(u) (in place in dv)
-        gelu_back_kernel<<<grid_for(rows * W), 256, 0, n.stream>>>(n.dv, u, rows * W);
-        float* du = n.dv;
-        gemm(n, W, W, (int)rows, v, W, 1, 0, du, W, 0, 0, g + n.o_w[l], W, 0, 1, 1.f, 0.f);
-        colsum_kernel<<<W, 256, 0, n.stream>>>(du, rows, W, g + n.o_b[l]);
-        gemm(n, (int)rows, W, W, du, W, 0, 0, n.wb + n.o_w[l], W, 1, 0, n.dv2, W, 0, 1, 1.f, 0.f);
-        // spectral path: dyh[b] = G^T du[b]
-        gemm(n, 2 * m, W, P, n.G, 2 * m, 1, 0, du, W, 0, (long long)P * W, n.dyh, W, (long long)2 * m * W, B, 1.f,
-             0.f);
-        // dRre[k] = re^T dyre + im^T dyim ; dRim[k] = re^T dyim - im^T dyre
-        gemm(n, W, W, B, vh, ld, 1, W, n.dyh, ld, 0, W, g + n.o_rre[l], W, (long long)W * W, m, 1.f, 0.f);
-        gemm(n, W, W, B, vh + m * W, ld, 1, W, n.dyh + m * W, ld, 0, W, g + n.o_rre[l], W, (long long)W * W, m, 1.f,
-             1.f);
-        gemm(n, W, W, B, vh, ld, 1, W, n.dyh + m * W, ld, 0, W, g + n.o_rim[l], W, (long long)W * W, m, 1.f, 0.f);
-        gemm(n, W, W, B, vh + m * W, ld, 1, W, n.dyh, ld, 0, W, g + n.o_rim[l], W, (long long)W * W, m, -1.f, 1.f);
-        // dre = dyre Rre^T + dyim Rim^T ; dim = -dyre Rim^T + dyim Rre^T
-        gemm(n, B, W, W, n.dyh, ld, 0, W, rre, W, 1, (long long)W * W, n.dvh, ld, W, m, 1.f, 0.f);
-        gemm(n, B, W, W, n.dyh + m * W, ld, 0, W, rim, W, 1, (long long)W * W, n.dvh, ld, W, m, 1.f, 1.f);
-        gemm(n, B, W, W, n.dyh, ld, 0, W, rim, W, 1, (long long)W * W, n.dvh + m * W, ld, W, m, -1.f, 0.f);
-        gemm(n, B, W, W, n.dyh + m * W, ld, 0, W, rre, W, 1, (long long)W * W, n.dvh + m * W, ld, W, m, 1.f, 1.f);
-        // dv = du W^T + F^T dvh[b]
-        gemm(n, P, W, 2 * m, n.F, P, 1, 0, n.dvh, W, 0, (long long)2 * m * W, n.dv2, W, (long long)P * W, B, 1.f,
-             1.f);
-        std::swap(n.dv, n.dv2);
+    const int W = n.W, m = n.m, P = n.P, H = n.H, L = n.L;
+    const long long rows = (long long)B * P, hat = (long long)B * 2 * m * W;
+    auto us = [&](int l) { return n.us + (long long)l * rows * W; };  // u of layer l, then du in its place
+    for (int n0 = 0; n0 < W; n0 += kT)
+        nn_launch(n, head_back_kernel, dim3(tiles(rows)), 0, n.dout, rows, W, H, n.wb + n.o_p1w, n.wb + n.o_p2w, n.z1, us(L - 1), n0);
+    for (int l = L - 1; l >= 0; --l) {
+        nn_launch(n, spectral_kernel<true>, dim3(m, B), spectral_smem(W), us(l), n.G, P, W, m, n.wb + n.o_rre[l], n.wb + n.o_rim[l],
+                  n.dyh + l * hat, n.dvh);
+        nn_launch(n, layer_back_kernel, dim3(tiles(P), B, tiles(W)), 0, us(l), P, W, m, n.wb + n.o_w[l], n.F, n.dvh,
+                  l > 0 ? us(l - 1) : nullptr, l > 0 ? us(l - 1) : n.dv);
     }
-    gemm(n, kCin, W, (int)rows, n.a, kCin, 1, 0, n.dv, W, 0, 0, g + n.o_lw, W, 0, 1, 1.f, 0.f);
-    colsum_kernel<<<W, 256, 0, n.stream>>>(n.dv, rows, W, g + n.o_lb);
+    GradTasks T{};
+    int tile = 0;
+    long long out = 0;
+    auto task = [&](const float* X, int M, const float* Y, int N) {
+        T.t[T.n++] = GradTask{X, Y, M, N, tile, out};
+        tile += (int)(tiles(M) * tiles(N));
+        out += (long long)M * N + N;
+    };
+    task(n.a, kCin, n.dv, W);
+    for (int l = 0; l < L; ++l) task(n.vs + (long long)l * rows * W, W, us(l), W);
+    task(n.vs + (long long)L * rows * W, W, n.z1, H);
+    task(n.h, H, n.dout, kCout);
+    const int splits = grad_splits(rows);
+    nn_launch(n, grad_kernel, dim3(tile, splits), 0, T, rows, splits, n.part, n.n_rows_params);
+    const long long spectral = 2LL * m * W * W, per_layer = (long long)W * W + W;
+    nn_launch(n, grad_spectral_kernel, dim3(L * m, tiles(W), tiles(W)), 0, n.vh, n.dyh, B, W, m, n.g, n.o_rre[0],
+              spectral + per_layer);
+    nn_launch(n, grad_sum_kernel, dim3((unsigned)((n.n_rows_params + kNT - 1) / kNT)), 0, n.part, n.n_rows_params, splits,
+              (long long)(kCin + 1) * W, per_layer, L, spectral, n.g, n.loss_part, (int)tiles(rows), (double)(rows * kCout), n.loss);
     return cudaGetLastError() == cudaSuccess ? FDLB_OK : FDLB_ECUDA;
 }
 
@@ -440,6 +708,7 @@ int fdlb_nn_create(int width, int modes, int layers, int hidden, int n_points, i
     n->o_p2w = take((long long)hidden * fdlb::kCout);
     n->o_p2b = take(fdlb::kCout);
     n->n_params = off;
+    n->n_rows_params = off - 2LL * layers * modes * W * W;
     // workspace
     const long long rows = (long long)max_batch * n_points;
     const long long np = n->n_params;
@@ -451,10 +720,10 @@ int fdlb_nn_create(int width, int modes, int layers, int hidden, int n_points, i
         {(void**)&n->us, (size_t)layers * rows * W * 4}, {(void**)&n->vh, (size_t)layers * max_batch * 2 * modes * W * 4},
         {(void**)&n->yh, (size_t)max_batch * 2 * modes * W * 4}, {(void**)&n->z1, rows * hidden * 4},
         {(void**)&n->h, rows * hidden * 4}, {(void**)&n->out, rows * fdlb::kCout * 4},
-        {(void**)&n->tgt, rows * fdlb::kCout * 4}, {(void**)&n->dout, rows * fdlb::kCout * 4},
-        {(void**)&n->dh, rows * hidden * 4}, {(void**)&n->dv, rows * W * 4}, {(void**)&n->dv2, rows * W * 4},
-        {(void**)&n->dyh, (size_t)max_batch * 2 * modes * W * 4}, {(void**)&n->dvh, (size_t)max_batch * 2 * modes * W * 4},
-        {(void**)&n->loss, 256}};
+        {(void**)&n->tgt, rows * fdlb::kCout * 4}, {(void**)&n->dout, rows * fdlb::kCout * 4}, {(void**)&n->dv, rows * W * 4},
+        {(void**)&n->dyh, (size_t)layers * max_batch * 2 * modes * W * 4}, {(void**)&n->dvh, (size_t)max_batch * 2 * modes * W * 4},
+        {(void**)&n->part, (size_t)fdlb::grad_splits(rows) * n->n_rows_params * 4},
+        {(void**)&n->loss_part, (size_t)((rows + fdlb::kT - 1) / fdlb::kT) * 8}, {(void**)&n->loss, 256}};
     size_t total = 0;
     for (auto& b : bufs) total += (b.second + 255) / 256 * 256;
     if (cudaMalloc(&n->ws, total) != cudaSuccess) {
@@ -563,7 +832,7 @@ int fdlb_nn_forward(fdlb_nn_handle h, const float* raw_params, int batch, float*
     NNet* n = reinterpret_cast<NNet*>(h);
     if (!n || !raw_params || !out_host || batch < 1 || batch > n->Bmax) return FDLB_EINVAL;
     int rc = fdlb::upload_inputs(*n, raw_params, nullptr, batch);
-    if (!rc) rc = fdlb::forward(*n, batch);
+    if (!rc) rc = fdlb::forward(*n, batch, false);
     if (rc) return rc;
     if (cudaMemcpyAsync(out_host, n->out, (size_t)batch * n->P * fdlb::kCout * 4, cudaMemcpyDeviceToHost, n->stream) !=
         cudaSuccess)
@@ -576,11 +845,8 @@ int fdlb_nn_loss_grad(fdlb_nn_handle h, const float* raw_params, const float* ta
     NNet* n = reinterpret_cast<NNet*>(h);
     if (!n || !raw_params || !targets || batch < 1 || batch > n->Bmax) return FDLB_EINVAL;
     int rc = fdlb::upload_inputs(*n, raw_params, targets, batch);
-    if (!rc) rc = fdlb::forward(*n, batch);
-    if (rc) return rc;
-    const long long cnt = (long long)batch * n->P * fdlb::kCout;
-    fdlb::mse_kernel<<<1, 1024, 0, n->stream>>>(n->out, n->tgt, cnt, n->dout, n->loss);
-    rc = fdlb::backward(*n, batch);
+    if (!rc) rc = fdlb::forward(*n, batch, true);
+    if (!rc) rc = fdlb::backward(*n, batch);
     if (rc) return rc;
     if (loss && cudaMemcpyAsync(loss, n->loss, 4, cudaMemcpyDeviceToHost, n->stream) != cudaSuccess) return FDLB_ECUDA;
     if (grad_host &&
