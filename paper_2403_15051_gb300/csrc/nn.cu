@@ -12,13 +12,15 @@
 // rounding per fused multiply-add).
 //
 // A batch is a few thousand rows of at most a few hundred channels, so a product is microseconds of work
-// and the passes over memory and launches around it are what counts.  A layer is two launches: the
-// spectral path of each (sample, mode) in one block, then the pointwise product, the inverse transform,
-// bias and GELU of 64 rows in one block; the head with the loss is one; the backward pass has the same
-// shape, with GELU's derivative in the epilogue that forms its input; the gradients of every weight
-// matrix but the spectral ones are one launch, split over the rows so that they fill the device (as one
-// product after another, each a single block of 64 x 64 outputs over all rows, they were 6.2 of the
-// 7.0 ms of a training batch of 32), with a second that adds the splits in a fixed order.
+// and the passes over memory and launches around it are what counts.  A layer is one launch: 64 rows of a
+// sample to a block, which forms the sample's spectral coefficients from the row tiles' partial transforms
+// (left by the launch before), mixes them, adds the inverse transform to the pointwise product, applies
+// bias and GELU and leaves its own rows' partial transform for the next layer.  The head with the loss is
+// one launch; the backward pass has the same shape, with GELU's derivative in the epilogue that forms its
+// input; the gradients of every weight matrix but the spectral ones are one launch, split over the rows so
+// that they fill the device (as one product after another, each a single block of 64 x 64 outputs over all
+// rows, they were 6.2 of the 7.0 ms of a training batch of 32), with a second that adds the splits in a
+// fixed order.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -48,7 +50,8 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
 }
 
 constexpr int kT = 64;        // rows and columns of an output tile
-constexpr int kKc = 32;       // contraction values staged at a time
+constexpr int kKc = 64;       // contraction values staged at a time
+constexpr int kModes = kKc / 2;  // modes (real and imaginary row) of a chunk
 constexpr int kLd = kT + 4;   // row stride of a staged chunk [k][64]
 constexpr int kNT = 256;      // threads: 16 x 16, 4 x 4 outputs each
 constexpr int kMaxSplits = 64;  // row splits of the weight gradients
@@ -67,10 +70,10 @@ __device__ __forceinline__ void tile_zero(Tile& t) {
     for (int i = 0; i < 4; ++i) t.a[i][0] = t.a[i][1] = make_float2(0.f, 0.f);
 }
 // t += X^T Y over the staged chunk: per k two vector loads and eight packed fused multiply-adds.
-__device__ __forceinline__ void tile_mma(Tile& t, const float* X, const float* Y, float sign = 1.f) {
+__device__ __forceinline__ void tile_mma(Tile& t, const float* X, const float* Y, float sign = 1.f, int n = kKc) {
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll 8
-    for (int k = 0; k < kKc; ++k) {
+    for (int k = 0; k < n; ++k) {
         const float4 x = *reinterpret_cast<const float4*>(X + k * kLd + ty * 4);
         const float4 y = *reinterpret_cast<const float4*>(Y + k * kLd + tx * 4);
         const float xs[4] = {sign * x.x, sign * x.y, sign * x.z, sign * x.w};
@@ -117,138 +120,206 @@ __device__ __forceinline__ void stage_cols(float* dst, const TS* src, long long 
     }
 }
 
-// Input channels (the five parameters, normalised, then x / (P - 1)) and the lift, v = a W + b.
-// Normalisation: (log10 Kn + 1), (eta0 - 0.155)/0.145, (ratio - 3.1)/1.9, (u_w - 0.15)/0.15,
-// (T_ratio - 1.15)/0.15 (the ranges of the parameter sweep mapped to about [-1, 1]).
-__global__ void lift_kernel(const float* __restrict__ raw, int B, int P, int W, const __nv_bfloat16* __restrict__ w,
-                            const float* __restrict__ bias, float* __restrict__ a, float* __restrict__ v) {
-    nn_begin();
-    const long long n = (long long)B * P * W;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const long long row = e / W;
-        const int c = (int)(e % W), b = (int)(row / P), x = (int)(row % P);
-        const float* r = raw + b * 5;
-        const float f[kCin] = {log10f(r[0]) + 1.f,         (r[1] - 0.155f) / 0.145f, (r[2] - 3.1f) / 1.9f,
-                               (r[3] - 0.15f) / 0.15f, (r[4] - 1.15f) / 0.15f,   (float)x / (float)(P - 1)};
-        float s = bias[c];
-#pragma unroll
-        for (int i = 0; i < kCin; ++i) s = fmaf(f[i], to_f(w[i * W + c]), s);
-        v[e] = s;
-        if (c == 0)
-#pragma unroll
-            for (int i = 0; i < kCin; ++i) a[row * kCin + i] = f[i];
+// Shared memory of the tile kernels: two staged chunks, X and Y, and behind them the spectral
+// coefficients of a chunk of modes, [2 kModes][W].  An output tile takes X's place, [row][kLd].
+__device__ __forceinline__ float* chunk_y(float* sm) { return sm + kKc * kLd; }
+__device__ __forceinline__ float* hats_of(float* sm) { return sm + 2 * kKc * kLd; }
+
+// The block's output tile T[row][column] (`rows` of 64, zero-filled columns) into its partial transform:
+// part[k][n0 + c] = sum over the rows of basis(k, row) T[row][c] for the 2m rows of the basis; basis(k, row)
+// at basis[k sk + row sr].  part: [2m][W] of this row tile.
+__device__ __forceinline__ void partial_transform(const float* T, const float* basis, long long sk, long long sr, int m2, int rows,
+                                                  int n0, int W, float* bs, float* part) {
+    const int c = threadIdx.x % kT, g = threadIdx.x / kT;
+    for (int k0 = 0; k0 < m2; k0 += kKc) {
+        const int nk = min(kKc, m2 - k0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < nk * kT; e += kNT) {
+            const int k = e / kT, r = e % kT;
+            bs[k * kT + r] = r < rows ? basis[(k0 + k) * sk + r * sr] : 0.f;
+        }
+        __syncthreads();
+        for (int k = g; k < nk; k += kNT / kT) {
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll 8
+            for (int r = 0; r < kT; r += 2) {
+                s0 = fmaf(bs[k * kT + r], T[r * kLd + c], s0);
+                s1 = fmaf(bs[k * kT + r + 1], T[(r + 1) * kLd + c], s1);
+            }
+            if (n0 + c < W) part[(long long)(k0 + k) * W + n0 + c] = s0 + s1;
+        }
     }
 }
 
-// The spectral path of one sample and mode (block (k, b)).  Forward: vh = F v (rows k and m + k of the DFT)
-// and the mode's complex mixing yh = vh R.  Backward: dyh = G^T du and dvh = dyh R^H in the same form (re, im
-// = columns k, m + k): dre = dyre Rre^T + dyim Rim^T, dim = dyim Rre^T - dyre Rim^T.  Sums over x by groups of
-// threads, in group order; src [P][W] of the sample, hat and mix [2m][W] of the sample.
-template <bool kBack>
-__global__ void __launch_bounds__(kNT) spectral_kernel(const float* __restrict__ src, const float* __restrict__ basis, int P, int W,
-                                                       int m, const __nv_bfloat16* __restrict__ Rre,
-                                                       const __nv_bfloat16* __restrict__ Rim, float* __restrict__ hat,
-                                                       float* __restrict__ mix) {
-    extern __shared__ float sh[];  // [groups][2][W] partial sums, then [2][W]
-    nn_begin();
-    const int k = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-    const float* s = src + (long long)b * P * W;
-    hat += (long long)b * 2 * m * W;
-    mix += (long long)b * 2 * m * W;
-    Rre += (long long)k * W * W;
-    Rim += (long long)k * W * W;
-    const int groups = W <= kNT ? kNT / W : 1;
-    float* tot = sh + 2 * (size_t)groups * W;
-    if (tid < groups * W || W > kNT) {
-        const int g = W <= kNT ? tid / W : 0;
-        for (int c = W <= kNT ? tid % W : tid; c < W; c += kNT) {
-            float re = 0.f, im = 0.f;
-#pragma unroll 8
-            for (int x = g; x < P; x += groups) {
-                const float v = s[(long long)x * W + c];
-                re = fmaf(kBack ? basis[x * 2 * m + k] : basis[k * P + x], v, re);
-                im = fmaf(kBack ? basis[x * 2 * m + m + k] : basis[(m + k) * P + x], v, im);
-            }
-            sh[(g * 2) * W + c] = re;
-            sh[(g * 2 + 1) * W + c] = im;
+// The spectral coefficients of `nm` modes from k0 on, summed over the row tiles' partial transforms in
+// order: hats[q][i] = sum_t part[t][mode row][i], rows q < kModes the real, q >= kModes the imaginary parts;
+// kept in `keep` ([2m][W]) where not null.
+__device__ __forceinline__ void sum_hats(float* hats, const float* part, int nt, int m, int W, int k0, int nm, float* keep) {
+    for (int e = threadIdx.x; e < 2 * nm * W; e += kNT) {
+        const int q = e / W, i = e % W, im = q >= nm, row = (im ? m : 0) + k0 + (im ? q - nm : q);
+        float s = 0.f;
+#pragma unroll 4
+        for (int t = 0; t < nt; ++t) s += part[((long long)t * 2 * m + row) * W + i];
+        hats[((im ? kModes : 0) + (im ? q - nm : q)) * W + i] = s;
+        if (keep) keep[(long long)row * W + i] = s;
+    }
+}
+
+// The modes' complex mixing into the chunk Y: rows 0 .. nm-1 the real, nm .. 2 nm - 1 the imaginary parts of
+// column n0 + c.  yre = re Rre - im Rim, yim = re Rim + im Rre: a thread per column and quarter of the inputs,
+// the quarters added through `scratch` ([4][2 nm][64], over X and Y; the caller has synchronised).
+__device__ __forceinline__ void mix_forward(float* Y, float* scratch, const float* hats, const __nv_bfloat16* Rre,
+                                            const __nv_bfloat16* Rim, int W, int k0, int nm, int n0) {
+    const int c = threadIdx.x % kT, g = threadIdx.x / kT, col = min(n0 + c, W - 1);
+    // (four quarters of 2 nm rows fit over the chunks for nm <= 17: at most 16 modes at a time)
+    for (int q = 0; q < nm; ++q) {
+        const __nv_bfloat16* a = Rre + (long long)(k0 + q) * W * W + col;
+        const __nv_bfloat16* b = Rim + (long long)(k0 + q) * W * W + col;
+        float yr = 0.f, yi = 0.f;
+#pragma unroll 16
+        for (int i = g; i < W; i += 4) {
+            const float ra = to_f(a[(long long)i * W]), rb = to_f(b[(long long)i * W]);
+            const float re = hats[q * W + i], im = hats[(kModes + q) * W + i];
+            yr = fmaf(re, ra, fmaf(-im, rb, yr));
+            yi = fmaf(re, rb, fmaf(im, ra, yi));
+        }
+        scratch[(g * 2 * nm + q) * kT + c] = yr;
+        scratch[(g * 2 * nm + nm + q) * kT + c] = yi;
+    }
+    __syncthreads();
+    float v[2 * kModes * kT / kNT];
+#pragma unroll
+    for (int h = 0; h < 2 * kModes * kT / kNT; ++h) {
+        const int e = threadIdx.x + h * kNT;
+        if (e < 2 * nm * kT) {
+            const int st = 2 * nm * kT;
+            v[h] = (scratch[e] + scratch[st + e]) + (scratch[2 * st + e] + scratch[3 * st + e]);
         }
     }
     __syncthreads();
-    for (int e = tid; e < 2 * W; e += kNT) {
-        float t = 0.f;
-        for (int g = 0; g < groups; ++g) t += sh[g * 2 * W + e];
-        tot[e] = t;
-        hat[(long long)(e < W ? k : m + k) * W + e % W] = t;
+#pragma unroll
+    for (int h = 0; h < 2 * kModes * kT / kNT; ++h) {
+        const int e = threadIdx.x + h * kNT;
+        if (e < 2 * nm * kT) Y[e / kT * kLd + e % kT] = n0 + e % kT < W ? v[h] : 0.f;
     }
-    __syncthreads();
-    const float *tr = tot, *ti = tot + W;
-    if constexpr (!kBack) {
-        // yre = re Rre - im Rim, yim = re Rim + im Rre: a thread per output and group of inputs
-        if (tid < groups * W || W > kNT) {
-            const int g = W <= kNT ? tid / W : 0;
-            for (int o = W <= kNT ? tid % W : tid; o < W; o += kNT) {
-                float yr = 0.f, yi = 0.f;
-#pragma unroll 8
-                for (int i = g; i < W; i += groups) {
-                    const float a = to_f(Rre[i * W + o]), c = to_f(Rim[i * W + o]);
-                    yr = fmaf(tr[i], a, fmaf(-ti[i], c, yr));
-                    yi = fmaf(tr[i], c, fmaf(ti[i], a, yi));
-                }
-                sh[(g * 2) * W + o] = yr;
-                sh[(g * 2 + 1) * W + o] = yi;
-            }
-        }
-        __syncthreads();
-        for (int e = tid; e < 2 * W; e += kNT) {
-            float t = 0.f;
-            for (int g = 0; g < groups; ++g) t += sh[g * 2 * W + e];
-            mix[(long long)(e < W ? k : m + k) * W + e % W] = t;
-        }
-    } else {
-        // a warp per input row of R, its lanes over the outputs
-        const int lane = tid & 31;
+}
+
+// The backward mixing into Y: dre = dyre Rre^T + dyim Rim^T, dim = dyim Rre^T - dyre Rim^T, column n0 + c
+// being row n0 + c of R: eight lanes per row, eight outputs a lane at a time.
+__device__ __forceinline__ void mix_backward(float* Y, const float* hats, const __nv_bfloat16* Rre, const __nv_bfloat16* Rim, int W,
+                                             int k0, int nm, int n0) {
+    const int sub = threadIdx.x & 7;
+    for (int e0 = 0; e0 < nm * kT; e0 += kNT / 8) {
+        const int e = e0 + (threadIdx.x >> 3), q = min(e / kT, nm - 1), c = e % kT;
+        float dr = 0.f, di = 0.f;
+        if (e < nm * kT && n0 + c < W) {
+            const __nv_bfloat16* a = Rre + ((long long)(k0 + q) * W + n0 + c) * W;
+            const __nv_bfloat16* b = Rim + ((long long)(k0 + q) * W + n0 + c) * W;
+            const float *re = hats + q * W, *im = hats + (kModes + q) * W;
+            if (W % 8 == 0) {  // (rows of eight BF16 values start on 16-byte boundaries)
 #pragma unroll 2
-        for (int i = tid >> 5; i < W; i += kNT / 32) {
-            float dr = 0.f, di = 0.f;
-            for (int o = lane; o < W; o += 32) {
-                const float a = to_f(Rre[i * W + o]), c = to_f(Rim[i * W + o]);
-                dr = fmaf(tr[o], a, fmaf(ti[o], c, dr));
-                di = fmaf(ti[o], a, fmaf(-tr[o], c, di));
-            }
-            dr = warp_sum(dr);
-            di = warp_sum(di);
-            if (lane == 0) {
-                mix[(long long)k * W + i] = dr;
-                mix[(long long)(m + k) * W + i] = di;
+                for (int o = sub * 8; o < W; o += 64) {
+                    const uint4 xa = *reinterpret_cast<const uint4*>(a + o), xb = *reinterpret_cast<const uint4*>(b + o);
+                    const uint32_t ua[4] = {xa.x, xa.y, xa.z, xa.w}, ub[4] = {xb.x, xb.y, xb.z, xb.w};
+#pragma unroll
+                    for (int h = 0; h < 8; ++h) {
+                        const float fa = __uint_as_float(h & 1 ? ua[h / 2] & 0xFFFF0000u : ua[h / 2] << 16);
+                        const float fb = __uint_as_float(h & 1 ? ub[h / 2] & 0xFFFF0000u : ub[h / 2] << 16);
+                        dr = fmaf(re[o + h], fa, fmaf(im[o + h], fb, dr));
+                        di = fmaf(im[o + h], fa, fmaf(-re[o + h], fb, di));
+                    }
+                }
+            } else {
+                for (int o = sub; o < W; o += 8) {
+                    const float fa = to_f(a[o]), fb = to_f(b[o]);
+                    dr = fmaf(re[o], fa, fmaf(im[o], fb, dr));
+                    di = fmaf(im[o], fa, fmaf(-re[o], fb, di));
+                }
             }
         }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            dr += __shfl_xor_sync(0xffffffffu, dr, o);
+            di += __shfl_xor_sync(0xffffffffu, di, o);
+        }
+        if (sub == 0 && e < nm * kT) {
+            Y[q * kLd + c] = dr;
+            Y[(nm + q) * kLd + c] = di;
+        }
     }
+}
+
+// Input channels (the five parameters, normalised, then x / (P - 1)), the lift v = a W + b and its partial
+// transform; grid as layer_kernel.
+// Normalisation: (log10 Kn + 1), (eta0 - 0.155)/0.145, (ratio - 3.1)/1.9, (u_w - 0.15)/0.15,
+// (T_ratio - 1.15)/0.15 (the ranges of the parameter sweep mapped to about [-1, 1]).
+__global__ void __launch_bounds__(kNT) lift_kernel(const float* __restrict__ raw, int P, int W, int m,
+                                                   const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
+                                                   const float* __restrict__ F, float* __restrict__ a, float* __restrict__ v,
+                                                   float* __restrict__ part) {
+    extern __shared__ __align__(16) float sm[];
+    nn_begin();
+    const int r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT, rows = min(kT, P - r0);
+    const float* r = raw + b * 5;
+    float f[kCin] = {log10f(r[0]) + 1.f, (r[1] - 0.155f) / 0.145f, (r[2] - 3.1f) / 1.9f, (r[3] - 0.15f) / 0.15f,
+                     (r[4] - 1.15f) / 0.15f, 0.f};
+    const int c = threadIdx.x % kT, col = n0 + c;
+    float wc[kCin], bc = 0.f;
+#pragma unroll
+    for (int i = 0; i < kCin; ++i) wc[i] = col < W ? to_f(w[i * W + col]) : 0.f;
+    if (col < W) bc = bias[col];
+    for (int rr = threadIdx.x / kT; rr < kT; rr += kNT / kT) {
+        float s = 0.f;
+        if (rr < rows && col < W) {
+            f[5] = (float)(r0 + rr) / (float)(P - 1);
+            s = bc;
+#pragma unroll
+            for (int i = 0; i < kCin; ++i) s = fmaf(f[i], wc[i], s);
+            v[((long long)b * P + r0 + rr) * W + col] = s;
+        }
+        sm[rr * kLd + c] = s;
+    }
+    if (blockIdx.z == 0)
+        for (int e = threadIdx.x; e < rows * kCin; e += kNT) {
+            const int rr = e / kCin, i = e % kCin;
+            a[((long long)b * P + r0) * kCin + e] = i == 5 ? (float)(r0 + rr) / (float)(P - 1) : f[i];
+        }
+    partial_transform(sm, F + r0, P, 1, 2 * m, rows, n0, W, chunk_y(sm), part + ((long long)b * gridDim.x + blockIdx.x) * 2 * m * W);
 }
 
 // 64 rows of one sample (grid: row tiles, samples, column tiles) through a layer.
-// Forward: u = v W + b + G yh, vout = GELU(u).
-__global__ void __launch_bounds__(kNT) layer_kernel(const float* __restrict__ v, int P, int W, int m,
+// Forward: u = v W + b + G yh, vout = GELU(u); hat: the layer's spectral coefficients, kept for the
+// gradients; part_out (or null): the partial transform of vout.
+__global__ void __launch_bounds__(kNT) layer_kernel(const float* __restrict__ v, const float* __restrict__ part_in, int P, int W, int m,
                                                     const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
-                                                    const float* __restrict__ G, const float* __restrict__ yh,
-                                                    float* __restrict__ u, float* __restrict__ vout) {
-    __shared__ __align__(16) float X[kKc * kLd], Y[kKc * kLd];
+                                                    const __nv_bfloat16* __restrict__ Rre, const __nv_bfloat16* __restrict__ Rim,
+                                                    const float* __restrict__ F, const float* __restrict__ G, float* __restrict__ hat,
+                                                    float* __restrict__ u, float* __restrict__ vout, float* __restrict__ part_out) {
+    extern __shared__ __align__(16) float sm[];
+    float *X = sm, *Y = chunk_y(sm), *hats = hats_of(sm);
     nn_begin();
-    const int r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT;
-    const float* vb = v + (long long)b * P * W;
+    const int nt = gridDim.x, r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT;
     Tile t;
     tile_zero(t);
     for (int k0 = 0; k0 < W; k0 += kKc) {
-        stage_cols(X, vb, W, r0, P, k0, W);
+        stage_cols(X, v + (long long)b * P * W, W, r0, P, k0, W);
         stage_rows(Y, w, W, k0, W, n0, W);
         __syncthreads();
         tile_mma(t, X, Y);
         __syncthreads();
     }
-    for (int k0 = 0; k0 < 2 * m; k0 += kKc) {
-        stage_cols(X, G, 2 * m, r0, P, k0, 2 * m);
-        stage_rows(Y, yh + (long long)b * 2 * m * W, W, k0, 2 * m, n0, W);
+    for (int k0 = 0; k0 < m; k0 += 16) {
+        const int nm = min(16, m - k0);
+        sum_hats(hats, part_in + (long long)b * nt * 2 * m * W, nt, m, W, k0, nm,
+                 blockIdx.x == 0 && blockIdx.z == 0 ? hat + (long long)b * 2 * m * W : nullptr);
         __syncthreads();
-        tile_mma(t, X, Y);
+        mix_forward(Y, sm, hats, Rre, Rim, W, k0, nm, n0);
+        for (int e = threadIdx.x; e < 2 * nm * kT; e += kNT) {
+            const int q = e % (2 * nm), r = e / (2 * nm), col = q < nm ? k0 + q : m + k0 + q - nm;
+            X[q * kLd + r] = r0 + r < P ? G[(long long)(r0 + r) * 2 * m + col] : 0.f;
+        }
+        __syncthreads();
+        tile_mma(t, X, Y, 1.f, 2 * nm);
         __syncthreads();
     }
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -257,23 +328,32 @@ __global__ void __launch_bounds__(kNT) layer_kernel(const float* __restrict__ v,
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int x = r0 + ty * 4 + i, c = n0 + tx * 4 + j;
+            float g = 0.f;
             if (x < P && c < W) {
                 const long long e = ((long long)b * P + x) * W + c;
                 const float s = tile_at(t, i, j) + bias[c];
+                g = gelu_f(s);
                 u[e] = s;
-                vout[e] = gelu_f(s);
+                vout[e] = g;
             }
+            X[(ty * 4 + i) * kLd + tx * 4 + j] = g;
         }
+    if (part_out)
+        partial_transform(X, F + r0, P, 1, 2 * m, min(kT, P - r0), n0, W, Y, part_out + ((long long)b * nt + blockIdx.x) * 2 * m * W);
 }
 
-// Backward: dv = du W^T + F^T dvh, and into `out` dv GELU'(u) (in place of u, the layer below's du), or dv
-// itself where u is null.
-__global__ void __launch_bounds__(kNT) layer_back_kernel(const float* __restrict__ du, int P, int W, int m,
-                                                         const __nv_bfloat16* __restrict__ w, const float* __restrict__ F,
-                                                         const float* __restrict__ dvh, const float* u, float* out) {
-    __shared__ __align__(16) float X[kKc * kLd], Y[kKc * kLd];
+// Backward: dv = du W^T + F^T dvh, and into `out` dv GELU'(u) (in place of u, the layer below's du) with its
+// partial transform by G^T, or dv itself where u is null.
+__global__ void __launch_bounds__(kNT) layer_back_kernel(const float* __restrict__ du, const float* __restrict__ part_in, int P, int W,
+                                                         int m, const __nv_bfloat16* __restrict__ w,
+                                                         const __nv_bfloat16* __restrict__ Rre, const __nv_bfloat16* __restrict__ Rim,
+                                                         const float* __restrict__ F, const float* __restrict__ G,
+                                                         float* __restrict__ hat, const float* u, float* out,
+                                                         float* __restrict__ part_out) {
+    extern __shared__ __align__(16) float sm[];
+    float *X = sm, *Y = chunk_y(sm), *hats = hats_of(sm);
     nn_begin();
-    const int r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT;
+    const int nt = gridDim.x, r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT;
     Tile t;
     tile_zero(t);
     for (int k0 = 0; k0 < W; k0 += kKc) {
@@ -283,11 +363,18 @@ __global__ void __launch_bounds__(kNT) layer_back_kernel(const float* __restrict
         tile_mma(t, X, Y);
         __syncthreads();
     }
-    for (int k0 = 0; k0 < 2 * m; k0 += kKc) {
-        stage_rows(X, F, P, k0, 2 * m, r0, P);
-        stage_rows(Y, dvh + (long long)b * 2 * m * W, W, k0, 2 * m, n0, W);
+    for (int k0 = 0; k0 < m; k0 += 16) {
+        const int nm = min(16, m - k0);
+        sum_hats(hats, part_in + (long long)b * nt * 2 * m * W, nt, m, W, k0, nm,
+                 blockIdx.x == 0 && blockIdx.z == 0 ? hat + (long long)b * 2 * m * W : nullptr);
         __syncthreads();
-        tile_mma(t, X, Y);
+        mix_backward(Y, hats, Rre, Rim, W, k0, nm, n0);
+        for (int e = threadIdx.x; e < 2 * nm * kT; e += kNT) {
+            const int q = e / kT, r = e % kT, row = q < nm ? k0 + q : m + k0 + q - nm;
+            X[q * kLd + r] = r0 + r < P ? F[(long long)row * P + r0 + r] : 0.f;
+        }
+        __syncthreads();
+        tile_mma(t, X, Y, 1.f, 2 * nm);
         __syncthreads();
     }
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -296,11 +383,17 @@ __global__ void __launch_bounds__(kNT) layer_back_kernel(const float* __restrict
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int x = r0 + ty * 4 + i, c = n0 + tx * 4 + j;
+            float d = 0.f;
             if (x < P && c < W) {
                 const long long e = ((long long)b * P + x) * W + c;
-                out[e] = u ? tile_at(t, i, j) * gelu_grad_f(u[e]) : tile_at(t, i, j);
+                d = u ? tile_at(t, i, j) * gelu_grad_f(u[e]) : tile_at(t, i, j);
+                out[e] = d;
             }
+            X[(ty * 4 + i) * kLd + tx * 4 + j] = d;
         }
+    if (part_out)
+        partial_transform(X, G + (long long)r0 * 2 * m, 1, 2 * m, 2 * m, min(kT, P - r0), n0, W, Y,
+                          part_out + ((long long)b * nt + blockIdx.x) * 2 * m * W);
 }
 
 // The head for 64 rows: z1 = v P1 + c1, h = GELU(z1), out = h P2 + c2, hidden units 64 at a time; z1 and h
@@ -312,9 +405,10 @@ __global__ void __launch_bounds__(kNT) head_kernel(const float* __restrict__ v, 
                                                    float* __restrict__ z1, float* __restrict__ h, float* __restrict__ out,
                                                    const float* __restrict__ tgt, float* __restrict__ dout,
                                                    double* __restrict__ loss_part) {
-    __shared__ __align__(16) float X[kKc * kLd], Y[kKc * kLd];
-    __shared__ float hs[kT][kT + 1], w2[kT][kCout];
+    extern __shared__ __align__(16) float sm[];
+    __shared__ float w2[kT][kCout];
     __shared__ double red[kNT / 32];
+    float *X = sm, *Y = chunk_y(sm);
     nn_begin();
     const long long r0 = (long long)blockIdx.x * kT;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -324,7 +418,7 @@ __global__ void __launch_bounds__(kNT) head_kernel(const float* __restrict__ v, 
         Tile t;
         tile_zero(t);
         for (int k0 = 0; k0 < W; k0 += kKc) {
-            stage_cols(X, v, W, r0, rows, k0, W);
+            if (W > kKc || n0 == 0) stage_cols(X, v, W, r0, rows, k0, W);  // (one chunk: staged once)
             stage_rows(Y, p1, H, k0, W, n0, H);
             __syncthreads();
             tile_mma(t, X, Y);
@@ -345,13 +439,13 @@ __global__ void __launch_bounds__(kNT) head_kernel(const float* __restrict__ v, 
                         h[r * H + c] = hv;
                     }
                 }
-                hs[ty * 4 + i][tx * 4 + j] = hv;
+                Y[(ty * 4 + i) * kLd + tx * 4 + j] = hv;
             }
         for (int e = threadIdx.x; e < kT * kCout; e += kNT)
             w2[e / kCout][e % kCout] = n0 + e / kCout < H ? to_f(p2[(n0 + e / kCout) * kCout + e % kCout]) : 0.f;
         __syncthreads();
 #pragma unroll 16
-        for (int j = 0; j < kT; ++j) o = fmaf(hs[orow][j], w2[j][oc], o);
+        for (int j = 0; j < kT; ++j) o = fmaf(Y[orow * kLd + j], w2[j][oc], o);
         __syncthreads();
     }
     o += c2[oc];
@@ -378,35 +472,33 @@ __global__ void __launch_bounds__(kNT) head_kernel(const float* __restrict__ v, 
 }
 static_assert(kT * kCout == kNT, "a thread per output of the head's tile");
 
-// The head backwards for 64 rows: dz1 = (dout P2^T) GELU'(z1) (in place of z1), then dv = dz1 P1^T and
-// du = dv GELU'(u) of the last layer (in place of u).  Column tiles beyond the first leave z1 as it is and
-// are launched after it: they read dz1.
-__global__ void __launch_bounds__(kNT) head_back_kernel(const float* __restrict__ dout, long long rows, int W, int H,
-                                                        const __nv_bfloat16* __restrict__ p1,
-                                                        const __nv_bfloat16* __restrict__ p2, float* z1, float* u, int n0) {
-    __shared__ __align__(16) float X[kKc * kLd], Y[kKc * kLd];
+// The head backwards for 64 rows of a sample (grid as layer_kernel): dz = (dout P2^T) GELU'(z1), kept by the
+// first column tile's blocks, then dv = dz P1^T and du = dv GELU'(u) of the last layer (in place of u) with its
+// partial transform by G^T.
+__global__ void __launch_bounds__(kNT) head_back_kernel(const float* __restrict__ dout, int P, int W, int H, int m,
+                                                        const __nv_bfloat16* __restrict__ p1, const __nv_bfloat16* __restrict__ p2,
+                                                        const float* __restrict__ z1, float* __restrict__ dz,
+                                                        const float* __restrict__ G, float* u, float* __restrict__ part_out) {
+    extern __shared__ __align__(16) float sm[];
+    float *X = sm, *Y = chunk_y(sm);
     nn_begin();
-    const long long r0 = (long long)blockIdx.x * kT;
+    const int nt = gridDim.x, r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT, rows = min(kT, P - r0);
+    const long long base = (long long)b * P + r0;
     Tile t;
     tile_zero(t);
     for (int k0 = 0; k0 < H; k0 += kKc) {
+#pragma unroll 4
         for (int e = threadIdx.x; e < kKc * kT; e += kNT) {
             const int rr = e / kKc, k = e % kKc;
-            const long long r = r0 + rr;
             float d = 0.f;
-            if (r < rows && k0 + k < H) {
-                const long long q = r * H + k0 + k;
-                if (n0 == 0) {
-                    const float* dr = dout + r * kCout;
-                    const __nv_bfloat16* p = p2 + (k0 + k) * kCout;
-                    float s = 0.f;
+            if (rr < rows && k0 + k < H) {
+                const float* dr = dout + (base + rr) * kCout;
+                const __nv_bfloat16* p = p2 + (k0 + k) * kCout;
+                float s = 0.f;
 #pragma unroll
-                    for (int c = 0; c < kCout; ++c) s = fmaf(dr[c], to_f(p[c]), s);
-                    d = s * gelu_grad_f(z1[q]);
-                    z1[q] = d;
-                } else {
-                    d = z1[q];
-                }
+                for (int c = 0; c < kCout; ++c) s = fmaf(dr[c], to_f(p[c]), s);
+                d = s * gelu_grad_f(z1[(base + rr) * H + k0 + k]);
+                if (blockIdx.z == 0) dz[(base + rr) * H + k0 + k] = d;
             }
             X[k * kLd + rr] = d;
         }
@@ -420,10 +512,16 @@ __global__ void __launch_bounds__(kNT) head_back_kernel(const float* __restrict_
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const long long r = r0 + ty * 4 + i;
-            const int c = n0 + tx * 4 + j;
-            if (r < rows && c < W) u[r * W + c] = tile_at(t, i, j) * gelu_grad_f(u[r * W + c]);
+            const int rr = ty * 4 + i, c = n0 + tx * 4 + j;
+            float d = 0.f;
+            if (rr < rows && c < W) {
+                d = tile_at(t, i, j) * gelu_grad_f(u[(base + rr) * W + c]);
+                u[(base + rr) * W + c] = d;
+            }
+            X[rr * kLd + tx * 4 + j] = d;
         }
+    partial_transform(X, G + (long long)r0 * 2 * m, 1, 2 * m, 2 * m, rows, n0, W, Y,
+                      part_out + ((long long)b * nt + blockIdx.x) * 2 * m * W);
 }
 
 // ---- gradients of the weights that act on rows: C = X^T Y over the rows of one split (blockIdx.y), with
@@ -442,7 +540,8 @@ struct GradTasks {
     int n;
 };
 __global__ void __launch_bounds__(kNT) grad_kernel(GradTasks T, long long rows, int splits, float* __restrict__ part, long long stride) {
-    __shared__ __align__(16) float X[kKc * kLd], Y[kKc * kLd];
+    extern __shared__ __align__(16) float sm[];
+    float *X = sm, *Y = chunk_y(sm);
     nn_begin();
     int q = 0;
     while (q + 1 < T.n && (int)blockIdx.x >= T.t[q + 1].tile0) ++q;
@@ -478,7 +577,8 @@ __global__ void __launch_bounds__(kNT) grad_kernel(GradTasks T, long long rows, 
 // dRim = re^T dyim - im^T dyre over the samples.
 __global__ void __launch_bounds__(kNT) grad_spectral_kernel(const float* __restrict__ vh, const float* __restrict__ dyh, int B, int W,
                                                             int m, float* __restrict__ g, long long o_rre, long long layer_stride) {
-    __shared__ __align__(16) float Xr[kKc * kLd], Xi[kKc * kLd], Yr[kKc * kLd], Yi[kKc * kLd];
+    extern __shared__ __align__(16) float sm[];
+    float *Xr = sm, *Xi = sm + kKc * kLd, *Yr = sm + 2 * kKc * kLd, *Yi = sm + 3 * kKc * kLd;
     nn_begin();
     const int l = blockIdx.x / m, k = blockIdx.x % m, i0 = blockIdx.y * kT, n0 = blockIdx.z * kT;
     const long long ld = 2LL * m * W;
@@ -493,10 +593,11 @@ __global__ void __launch_bounds__(kNT) grad_spectral_kernel(const float* __restr
         stage_rows(Yr, y, ld, k0, B, n0, W);
         stage_rows(Yi, y + (long long)m * W, ld, k0, B, n0, W);
         __syncthreads();
-        tile_mma(tr, Xr, Yr);
-        tile_mma(tr, Xi, Yi);
-        tile_mma(ti, Xr, Yi);
-        tile_mma(ti, Xi, Yr, -1.f);
+        const int n = min(kKc, B - k0);
+        tile_mma(tr, Xr, Yr, 1.f, n);
+        tile_mma(tr, Xi, Yi, 1.f, n);
+        tile_mma(ti, Xr, Yi, 1.f, n);
+        tile_mma(ti, Xi, Yr, -1.f, n);
         __syncthreads();
     }
     float* gr = g + o_rre + l * layer_stride + (long long)k * W * W;
@@ -573,9 +674,10 @@ struct NNet {
     float *w = nullptr, *g = nullptr, *m1 = nullptr, *m2 = nullptr;
     __nv_bfloat16* wb = nullptr;
     float *F = nullptr, *G = nullptr;
-    float *raw = nullptr, *a = nullptr, *vs = nullptr, *us = nullptr, *vh = nullptr, *yh = nullptr;
-    float *z1 = nullptr, *h = nullptr, *out = nullptr, *tgt = nullptr, *dout = nullptr;
-    float *dv = nullptr, *dyh = nullptr, *dvh = nullptr, *loss = nullptr, *part = nullptr;
+    float *raw = nullptr, *a = nullptr, *vs = nullptr, *us = nullptr, *vh = nullptr;
+    float *z1 = nullptr, *dz = nullptr, *h = nullptr, *out = nullptr, *tgt = nullptr, *dout = nullptr;
+    float *dv = nullptr, *dyh = nullptr, *loss = nullptr, *part = nullptr;
+    float* hat_part[2] = {nullptr, nullptr};  // the row tiles' partial transforms, of a layer and the next
     double* loss_part = nullptr;
     long long n_rows_params = 0;  // parameters without the spectral weights
     int step = 0;
@@ -602,7 +704,8 @@ void nn_launch(NNet& n, void (*kern)(KA...), dim3 grid, size_t smem, A... args) 
 }
 
 unsigned tiles(long long n) { return (unsigned)((n + kT - 1) / kT); }
-size_t spectral_smem(int W) { return (size_t)(W <= kNT ? kNT / W + 1 : 2) * 2 * W * sizeof(float); }
+constexpr size_t kChunks = 2 * (size_t)kKc * kLd * sizeof(float);  // shared memory of two staged chunks
+size_t layer_smem(int W) { return kChunks + 2 * (size_t)kModes * W * sizeof(float); }
 int grad_splits(long long rows) { return (int)std::min<long long>((rows + 127) / 128, kMaxSplits); }
 
 // Forward pass for B samples whose raw parameters are in n.raw; for training (targets in n.tgt) leaves every
@@ -610,16 +713,15 @@ int grad_splits(long long rows) { return (int)std::min<long long>((rows + 127) /
 int forward(NNet& n, int B, bool train) {
     const int W = n.W, m = n.m, P = n.P, H = n.H;
     const long long rows = (long long)B * P;
-    nn_launch(n, lift_kernel, dim3(grid_for(rows * W)), 0, n.raw, B, P, W, n.wb + n.o_lw, n.w + n.o_lb, n.a, n.vs);
+    const dim3 grid(tiles(P), B, tiles(W));
+    nn_launch(n, lift_kernel, grid, kChunks, n.raw, P, W, m, n.wb + n.o_lw, n.w + n.o_lb, n.F, n.a, n.vs, n.hat_part[0]);
     for (int l = 0; l < n.L; ++l) {
         float* v = n.vs + (long long)l * rows * W;
-        float* vh = n.vh + (long long)l * B * 2 * m * W;
-        nn_launch(n, spectral_kernel<false>, dim3(m, B), spectral_smem(W), v, n.F, P, W, m, n.wb + n.o_rre[l], n.wb + n.o_rim[l], vh,
-                  n.yh);
-        nn_launch(n, layer_kernel, dim3(tiles(P), B, tiles(W)), 0, v, P, W, m, n.wb + n.o_w[l], n.w + n.o_b[l], n.G, n.yh,
-                  n.us + (long long)l * rows * W, v + rows * W);
+        nn_launch(n, layer_kernel, grid, layer_smem(W), v, n.hat_part[l & 1], P, W, m, n.wb + n.o_w[l], n.w + n.o_b[l],
+                  n.wb + n.o_rre[l], n.wb + n.o_rim[l], n.F, n.G, n.vh + (long long)l * B * 2 * m * W,
+                  n.us + (long long)l * rows * W, v + rows * W, l + 1 < n.L ? n.hat_part[(l + 1) & 1] : nullptr);
     }
-    nn_launch(n, head_kernel, dim3(tiles(rows)), 0, n.vs + (long long)n.L * rows * W, rows, W, H, n.wb + n.o_p1w, n.w + n.o_p1b,
+    nn_launch(n, head_kernel, dim3(tiles(rows)), kChunks, n.vs + (long long)n.L * rows * W, rows, W, H, n.wb + n.o_p1w, n.w + n.o_p1b,
               n.wb + n.o_p2w, n.w + n.o_p2b, train ? n.z1 : nullptr, n.h, n.out, train ? n.tgt : nullptr, n.dout, n.loss_part);
     return cudaGetLastError() == cudaSuccess ? FDLB_OK : FDLB_ECUDA;
 }
@@ -629,13 +731,14 @@ int backward(NNet& n, int B) {
     const int W = n.W, m = n.m, P = n.P, H = n.H, L = n.L;
     const long long rows = (long long)B * P, hat = (long long)B * 2 * m * W;
     auto us = [&](int l) { return n.us + (long long)l * rows * W; };  // u of layer l, then du in its place
-    for (int n0 = 0; n0 < W; n0 += kT)
-        nn_launch(n, head_back_kernel, dim3(tiles(rows)), 0, n.dout, rows, W, H, n.wb + n.o_p1w, n.wb + n.o_p2w, n.z1, us(L - 1), n0);
+    const dim3 grid(tiles(P), B, tiles(W));
+    nn_launch(n, head_back_kernel, grid, kChunks, n.dout, P, W, H, m, n.wb + n.o_p1w, n.wb + n.o_p2w, n.z1, n.dz, n.G, us(L - 1),
+              n.hat_part[(L - 1) & 1]);
     for (int l = L - 1; l >= 0; --l) {
-        nn_launch(n, spectral_kernel<true>, dim3(m, B), spectral_smem(W), us(l), n.G, P, W, m, n.wb + n.o_rre[l], n.wb + n.o_rim[l],
-                  n.dyh + l * hat, n.dvh);
-        nn_launch(n, layer_back_kernel, dim3(tiles(P), B, tiles(W)), 0, us(l), P, W, m, n.wb + n.o_w[l], n.F, n.dvh,
-                  l > 0 ? us(l - 1) : nullptr, l > 0 ? us(l - 1) : n.dv);
+        float* below = l > 0 ? us(l - 1) : nullptr;
+        nn_launch(n, layer_back_kernel, grid, layer_smem(W), us(l), n.hat_part[l & 1], P, W, m, n.wb + n.o_w[l], n.wb + n.o_rre[l],
+                  n.wb + n.o_rim[l], n.F, n.G, n.dyh + l * hat, below, l > 0 ? below : n.dv,
+                  l > 0 ? n.hat_part[(l - 1) & 1] : nullptr);
     }
     GradTasks T{};
     int tile = 0;
@@ -647,12 +750,12 @@ int backward(NNet& n, int B) {
     };
     task(n.a, kCin, n.dv, W);
     for (int l = 0; l < L; ++l) task(n.vs + (long long)l * rows * W, W, us(l), W);
-    task(n.vs + (long long)L * rows * W, W, n.z1, H);
+    task(n.vs + (long long)L * rows * W, W, n.dz, H);
     task(n.h, H, n.dout, kCout);
     const int splits = grad_splits(rows);
-    nn_launch(n, grad_kernel, dim3(tile, splits), 0, T, rows, splits, n.part, n.n_rows_params);
+    nn_launch(n, grad_kernel, dim3(tile, splits), kChunks, T, rows, splits, n.part, n.n_rows_params);
     const long long spectral = 2LL * m * W * W, per_layer = (long long)W * W + W;
-    nn_launch(n, grad_spectral_kernel, dim3(L * m, tiles(W), tiles(W)), 0, n.vh, n.dyh, B, W, m, n.g, n.o_rre[0],
+    nn_launch(n, grad_spectral_kernel, dim3(L * m, tiles(W), tiles(W)), 2 * kChunks, n.vh, n.dyh, B, W, m, n.g, n.o_rre[0],
               spectral + per_layer);
     nn_launch(n, grad_sum_kernel, dim3((unsigned)((n.n_rows_params + kNT - 1) / kNT)), 0, n.part, n.n_rows_params, splits,
               (long long)(kCin + 1) * W, per_layer, L, spectral, n.g, n.loss_part, (int)tiles(rows), (double)(rows * kCout), n.loss);
@@ -718,10 +821,12 @@ int fdlb_nn_create(int width, int modes, int layers, int hidden, int n_points, i
         {(void**)&n->G, (size_t)2 * modes * n_points * 4}, {(void**)&n->raw, (size_t)max_batch * 5 * 4},
         {(void**)&n->a, rows * fdlb::kCin * 4}, {(void**)&n->vs, (size_t)(layers + 1) * rows * W * 4},
         {(void**)&n->us, (size_t)layers * rows * W * 4}, {(void**)&n->vh, (size_t)layers * max_batch * 2 * modes * W * 4},
-        {(void**)&n->yh, (size_t)max_batch * 2 * modes * W * 4}, {(void**)&n->z1, rows * hidden * 4},
+        {(void**)&n->hat_part[0], (size_t)max_batch * fdlb::tiles(n_points) * 2 * modes * W * 4},
+        {(void**)&n->hat_part[1], (size_t)max_batch * fdlb::tiles(n_points) * 2 * modes * W * 4},
+        {(void**)&n->z1, rows * hidden * 4}, {(void**)&n->dz, rows * hidden * 4},
         {(void**)&n->h, rows * hidden * 4}, {(void**)&n->out, rows * fdlb::kCout * 4},
         {(void**)&n->tgt, rows * fdlb::kCout * 4}, {(void**)&n->dout, rows * fdlb::kCout * 4}, {(void**)&n->dv, rows * W * 4},
-        {(void**)&n->dyh, (size_t)layers * max_batch * 2 * modes * W * 4}, {(void**)&n->dvh, (size_t)max_batch * 2 * modes * W * 4},
+        {(void**)&n->dyh, (size_t)layers * max_batch * 2 * modes * W * 4},
         {(void**)&n->part, (size_t)fdlb::grad_splits(rows) * n->n_rows_params * 4},
         {(void**)&n->loss_part, (size_t)((rows + fdlb::kT - 1) / fdlb::kT) * 8}, {(void**)&n->loss, 256}};
     size_t total = 0;
@@ -734,6 +839,15 @@ int fdlb_nn_create(int width, int modes, int layers, int hidden, int n_points, i
     for (auto& b : bufs) {
         *b.first = n->ws + o;
         o += (b.second + 255) / 256 * 256;
+    }
+    // dynamic shared memory beyond the default limit
+    const int layer_sm = (int)fdlb::layer_smem(W), two = (int)(2 * fdlb::kChunks);
+    if (cudaFuncSetAttribute(fdlb::layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, layer_sm) != cudaSuccess ||
+        cudaFuncSetAttribute(fdlb::layer_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, layer_sm) != cudaSuccess ||
+        cudaFuncSetAttribute(fdlb::grad_spectral_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, two) != cudaSuccess) {
+        cudaFree(n->ws);
+        delete n;
+        return FDLB_ECUDA;
     }
     n->stream = (cudaStream_t)cuda_stream;
     if (!n->stream) {
