@@ -22,9 +22,13 @@ namespace {
 
 constexpr double kPiH = 3.14159265358979323846;
 constexpr size_t kAlign = 256;
-// Radial node counts from which the K^h contraction runs as its own kernel (the fused stage then
-// reads K^h f; below, the stage contracts from a K^h table in shared memory).
+// Radial node counts from which the K^h contraction can run as its own kernel (the fused stage then
+// reads K^h f), and from which it does by default: below, the stage contracts from a K^h table in shared
+// memory.  At 40 nodes the kernel's launch and its pass over f cost more than the 40 multiply-adds it
+// takes off the stage: KRCMP.  Beyond 48 nodes the table itself and,
+// in FP32, the range of K^h (entries as sqrt(w_i / w_a), the weights below 1e-30) speak for the kernel.
 constexpr int kKrKernelMinNodes = 32;
+constexpr int kKrKernelDefaultNodes = 50;
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -539,6 +543,8 @@ int upload_items(Solver& S) {
             const int per_wave = S.n_sm;
             const int r = (nt * slices + per_wave - 1) / per_wave * per_wave / slices;
             if (r >= nt && r * slices % per_wave == 0 && N / r >= 2) nt = r;
+            // not that many: tiles of two cells where they still find an SM each
+            else if (nt * slices < per_wave && N / 2 * slices <= per_wave && N / 2 > nt && !S.fused) nt = N / 2;
             // fewer cells than SMs: one to a tile (each computes both its faces, half as much again, on
             // twice the SMs: the FP64 stage of 64 cells x 128 momenta took 48.8 us in tiles of four)
             if (!S.fused && !S.tiles && N * slices <= S.n_sm && N * slices <= S.max_sitems) nt = N;
@@ -716,6 +722,8 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
         cfg.vw = S.n2 % 4 == 0 ? 4 : (S.n2 % 2 == 0 ? 2 : 1);
     else  // (four FP64 momenta per thread: blocks of up to 256 threads, for their registers)
         cfg.vw = S.n2 % 4 == 0 && Ms <= 1024 ? 4 : (S.n2 % 2 == 0 ? 2 : 1);
+    // rows of eight per thread over many cells, as for the compile-time shape below
+    const bool rows8 = S.tsize == 4 && S.n2 == 8 && Ms / 8 <= 512 && (long long)S.total_cells * S.Np > (long long)S.n_sm * 65536;
     cfg.spec = ((S.geometry == FDLB_CYL && S.nR == 16 && S.n2 == 8 && S.n3 == 8) ||
                 (S.geometry == FDLB_SPH && S.nR == 24 && S.n2 == 12 && S.n3 == 12)) &&
                cfg.vw == (S.tsize == 4 || S.geometry == FDLB_CYL ? 4 : 2);
@@ -723,6 +731,7 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
     // the cylinder's FP32 shape in blocks of at most 128 threads: a thread per whole p_2 row (8
     // momenta; per-vector and per-cell work spread over twice the momenta, half the warps per cell)
     if (cfg.spec && S.tsize == 4 && S.geometry == FDLB_CYL && cap <= 128 && Ms / 8 <= 128) cfg.vw = 8;
+    if (!cfg.spec && rows8) cfg.vw = 8;
     const int Vs = Ms / cfg.vw;
     int nt = 0;
     if (cfg.vw == 8) {
@@ -741,7 +750,7 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
         if ((long long)nt * cfg.nv < Vs) nt = ((Vs + cfg.nv - 1) / cfg.nv + 31) / 32 * 32;
     }
     if (nt > 512 || (long long)nt * cfg.nv < Vs) return FDLB_EINVAL;
-    if (cfg.vw == 8)
+    if (cfg.vw == 8 && cfg.spec)
         cfg.minb = (S.stage_minb == 2 || S.stage_minb == 3 || S.stage_minb == 5) ? S.stage_minb : 1;
     else
         cfg.minb = (S.stage_minb == 3 && cfg.spec && S.tsize == 4 && S.geometry == FDLB_CYL && nt <= 256) ? 3 : 1;
@@ -962,8 +971,12 @@ int launch_stream_only(Solver& S, int in, int fn, int out, double a, double b, i
     A.B = S.B;
     A.G = S.march_G;
     A.teams = S.teams;
-    if (S.n2 == kK2Order)
-        for (int e = 0; e < S.n2 * S.n2; ++e) A.K2[(e % S.n2) * S.n2 + e / S.n2] = (float)S.tab_h[S.M.o_K2 + e];
+    if ((size_t)S.n2 * S.n2 * S.tsize <= (size_t)kK2Bytes)
+        for (int e = 0; e < S.n2 * S.n2; ++e) {
+            const int t = (e % S.n2) * S.n2 + e / S.n2;
+            if (S.precision == FDLB_FP32) A.K2.f[t] = (float)S.tab_h[S.M.o_K2 + e];
+            else A.K2.d[t] = S.tab_h[S.M.o_K2 + e];
+        }
     A.use_bulk = S.use_bulk;
     A.programmatic = S.programmatic;
     A.mma = S.mma_on;
@@ -1225,7 +1238,7 @@ int run_autotune(Solver& S, bool use_cache) {
     // the register bound of the stage kernel: three blocks per SM where that variant is built, and
     // for the row kernel also two and five
     const bool minb_choice = S.scfg.spec && S.tsize == 4 && S.geometry == FDLB_CYL && S.threads <= 256;
-    const bool rows = S.scfg.vw == 8;
+    const bool rows = S.scfg.vw == 8 && S.scfg.spec;
     int rc = FDLB_OK;
     for (int mb : {1, 3, 2, 5}) {
         if (mb == 3 && !minb_choice) continue;
@@ -1379,16 +1392,16 @@ int solver_create(const fdlb_params* ps, int n, void* stream, void* workspace, s
     R.rprev = (double*)(R.ws + L.rprev);
     R.rout = (double*)(R.ws + L.rout);
     R.krf = R.nR >= kKrKernelMinNodes ? (void*)(R.ws + L.krf) : nullptr;
-    R.krg_on = R.krf != nullptr;
+    R.krg_on = R.krf != nullptr && R.nR >= kKrKernelDefaultNodes;
     FDLB_CUDA(cudaMemsetAsync(R.ws, 0, L.total, R.stream));
-    if (R.krg_on && R.precision == FDLB_FP32) {
+    if (R.krf && R.precision == FDLB_FP32) {
         // K^h as TF32 pairs for the tensor-core contraction (after the workspace is cleared)
         R.krB = (float*)(R.ws + L.krB);
         const std::vector<float> kb = kr_split_table(R.tab_h, R.M.o_KR, R.M.o_wR, R.nR);
         FDLB_CUDA(cudaMemcpyAsync(R.krB, kb.data(), kb.size() * sizeof(float), cudaMemcpyHostToDevice, R.stream));
         FDLB_CUDA(cudaStreamSynchronize(R.stream));
-        R.tensor = 1;  // the tensor-core contraction by default
-        R.kr_tc = 1;
+        R.tensor = R.krg_on;  // the contraction kernel on the tensor cores
+        R.kr_tc = R.krg_on;
     }
     // tables, instances, geometry, walls, FM band
     FDLB_CUDA(cudaMemcpyAsync(R.tab, R.tab_h.data(), R.tab_h.size() * 8, cudaMemcpyHostToDevice, R.stream));
@@ -2160,14 +2173,20 @@ int fdlb_set_tensor_contraction(fdlb_handle h, int enable, int* in_use) try {
     Solver* S = SOL(h);
     if (!S) return FDLB_EINVAL;
     S->tensor = enable ? 1 : 0;
-    if (S->krg_on) {
-        // large radial orders: the contraction kernel on the tensor cores (FP32) or the CUDA cores
+    if (S->krf) {
+        // radial orders with a contraction kernel: on the tensor cores (FP32); else, where the stage contracts
+        // by default, in the stage, beyond on the CUDA cores
+        const int by_kernel = S->nR >= fdlb::kKrKernelDefaultNodes || (S->tensor && S->krB) ? 1 : 0;
         S->kr_tc = S->tensor && S->krB ? 1 : 0;
+        if (in_use) *in_use = S->kr_tc;
+        if (by_kernel != S->krg_on) {
+            S->krg_on = by_kernel;
+            return fdlb::configure_tiling(*S, S->B, S->KS, S->threads);
+        }
         if (S->gexec) {
             cudaGraphExecDestroy(S->gexec);
             S->gexec = nullptr;
         }
-        if (in_use) *in_use = S->kr_tc;
         return FDLB_OK;
     }
     const int rc = fdlb::configure_tiling(*S, S->B, S->KS, S->threads);

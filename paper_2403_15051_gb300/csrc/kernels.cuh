@@ -64,7 +64,7 @@ struct MomSet {
     int o_pR, o_wR, o_p2, o_w2, o_p3, o_w3, o_KR, o_K2, o_K3, o_GR, o_G2, o_G3, o_ha, o_hb, o_h0;
 };
 
-constexpr int kK2Order = 8;         // second-axis order whose K_2 travels with the stage's launch
+constexpr int kK2Bytes = 256;       // K_2 travels with the stage's launch where it is at most this large
 
 struct StageArgs {
     const void* f_in;
@@ -97,7 +97,10 @@ struct StageArgs {
     int tx_extra;                  // test hook: bytes the staged-copy barrier waits for beyond the copy
     const void* krf;               // K^h f of f_in from the contraction kernel (T, layout of f), or
                                    // null: the stage contracts from the K^h table in shared memory
-    float K2[kK2Order * kK2Order]; // K_2 transposed, [b][j], where the second axis has that order
+    union {
+        float f[kK2Bytes / 4];
+        double d[kK2Bytes / 8];
+    } K2;                          // K_2 transposed, [b][j], in T, where it fits
     const void* k3f;               // sphere: K_3 f of f_in (T, layout of f) when the momenta are
                                    // sliced along p_3, or null: contracted from the staged rows
 };

@@ -402,7 +402,9 @@ __device__ __forceinline__ void stage_ghosts(const StageWalk<T, VW, NV>& W, cons
 
 // Whether K_2's coefficients come with the launch (StageArgs::K2).
 template <typename T, int VW, int N2_>
-constexpr bool kK2Const = sizeof(T) == 4 && VW == N2_ && N2_ == kK2Order;
+constexpr bool kK2Const = VW == N2_ && N2_ * N2_ * sizeof(T) <= kK2Bytes;
+__device__ __forceinline__ float2 k2_pair(const StageArgs& A, int e, float) { return make_float2(A.K2.f[e], A.K2.f[e + 1]); }
+__device__ __forceinline__ double2 k2_pair(const StageArgs& A, int e, double) { return make_double2(A.K2.d[e], A.K2.d[e + 1]); }
 
 // Cell c of the walk: advection, force, collision, RK combination and store of the thread's vectors, the
 // warp's raw sums to red[0 .. 15].  o[0 .. 5]: element offsets in fs of the rows of cells c-2 .. c+3
@@ -488,14 +490,16 @@ __device__ __forceinline__ void stage_cell(StageWalk<T, VW, NV>& W, const StageP
         } else {
             const T* col = fc + kk * nR * n2 + jb * VW;
             const T* kr = S.KR + i * krs;
-            if constexpr (sizeof(T) == 4 && NR_ > 0 && NR_ % 4 == 0) {
-                // four entries of the K^h row per vector load
+            if constexpr (sizeof(T) == 4) {
+                // four entries of the K^h row per vector load (the rows' stride is a multiple of four)
 #pragma unroll 2
-                for (int a4 = 0; a4 < NR_; a4 += 4) {
+                for (int a4 = 0; a4 < nR; a4 += 4) {
                     T kq[4];
                     ld_vec<T, 4>(kr + a4, kq);
 #pragma unroll
                     for (int t = 0; t < 4; ++t) {
+                        if (NR_ % 4 != 0 || NR_ == 0)
+                            if (a4 + t >= nR) break;
                         V2 cv[NP];
                         ld_pairs<T, VW>(col + (a4 + t) * n2, cv);
                         const V2 kv = p_splat(kq[t]);
@@ -529,7 +533,7 @@ __device__ __forceinline__ void stage_cell(StageWalk<T, VW, NV>& W, const StageP
                     const V2 fv1 = p_splat(rv[b]);
 #pragma unroll
                     for (int h = 0; h < NP; ++h)
-                        K2f[h] = p_fma(p_make((T)A.K2[b * VW + 2 * h], (T)A.K2[b * VW + 2 * h + 1]), fv1, K2f[h]);
+                        K2f[h] = p_fma(k2_pair(A, b * VW + 2 * h, T(0)), fv1, K2f[h]);
                 }
             } else
 #pragma unroll 2
@@ -1130,6 +1134,16 @@ cudaError_t launch_stream_dispatch(const StreamCfg& cfg, const StageArgs& A, con
         if constexpr (sizeof(T) == 4 || G == 1)
             if (cfg.nv == NB) return launch_stream_t<T, G, VS, NB, SR, S2, S3>(A, M, grid, threads, smem, s, bps);
         return cudaErrorInvalidValue;
+    }
+    // second-axis orders 4 and 8 at compile time: a whole row per thread or half of one
+    if (cfg.vw == 4 && M.n2 == 4) {
+        if (cfg.nv == 1) return launch_stream_t<T, G, 4, 1, 0, 4, 0>(A, M, grid, threads, smem, s, bps);
+        if constexpr (sizeof(T) == 4)
+            if (cfg.nv == 2) return launch_stream_t<T, G, 4, 2, 0, 4, 0>(A, M, grid, threads, smem, s, bps);
+    }
+    if constexpr (sizeof(T) == 4) {
+        if (cfg.vw == 8 && cfg.nv == 1 && M.n2 == 8) return launch_stream_t<T, G, 8, 1, 0, 8, 0>(A, M, grid, threads, smem, s, bps);
+        if (cfg.vw == 4 && cfg.nv == 2 && M.n2 == 8) return launch_stream_t<T, G, 4, 2, 0, 8, 0>(A, M, grid, threads, smem, s, bps);
     }
     if (cfg.vw == 1 && cfg.nv == 4) return launch_stream_t<T, G, 1, 4, 0, 0, 0>(A, M, grid, threads, smem, s, bps);
     if (cfg.vw == 2 && cfg.nv == 4) return launch_stream_t<T, G, 2, 4, 0, 0, 0>(A, M, grid, threads, smem, s, bps);
