@@ -136,14 +136,20 @@ __device__ T wall_flux_partial(const T* wall, long long st, const MomSet& M, con
                 for (int r = 0; r < 4; ++r) fv[u][r] = wall[m + r * st];
             }
         }
-#pragma unroll
+#pragma unroll 1
         for (int u = 0; u < 4; ++u) {
             const int mo = m0 + u * NT;
-            if (mo >= mhi) continue;
+            if (mo >= mhi) break;
             const int k = mo / (QR * n2), rem = mo % (QR * n2), i = (side == 0 ? QR : 0) + rem / n2, j = rem % n2;
             const T wm = mul_rn(mul_rn(tb.wRt[i], tb.w3t[k]), tb.w2t[j]), ew = mul_rn(mul_rn(T(4e-6), wm), wm);
             const T e4 = sizeof(T) == 4 ? fmax(ew, T(1e-37)) : ew;
-            const T f0 = fv[u][0], f1 = fv[u][1], f2 = fv[u][2], f3 = fv[u][3];
+            const T f0 = fv[0][0], f1 = fv[0][1], f2 = fv[0][2], f3 = fv[0][3];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {  // the next pass's populations move up
+                fv[0][r] = fv[1][r];
+                fv[1][r] = fv[2][r];
+                fv[2][r] = fv[3][r];
+            }
             const T g1 = fma(T(4), f0, fma(T(-6), f1, fma(T(4), f2, -f3)));
             const T g2 = fma(T(10), f0, fma(T(-20), f1, fma(T(15), f2, mul_rn(T(-4), f3))));
             const T vh = side == 0 ? weno5_one(g2, g1, f0, f1, f2, sg, dL, dR, e4) : weno5_one(f2, f1, f0, g1, g2, sg, dL, dR, e4);
@@ -166,11 +172,16 @@ template <typename T>
 __device__ T wall_part_of_warp(const T* fin, const MomSet& M, const ClosureTabs<T>& tb, const InstDev& I, int side, int part,
                                int P, int lane) {
     const T* wall = fin + I.f_off + (side == 0 ? 0LL : (long long)(I.n_cells - 1) * M.Np);
-    T r[kClosureWarps];
-#pragma unroll
-    for (int vw = 0; vw < kClosureWarps; ++vw)
-        r[vw] = warp_sum(wall_flux_partial<T>(wall, side == 0 ? (long long)M.Np : -(long long)M.Np, M, tb, side, part, P,
-                                              32 * vw + lane));
+    T r0 = T(0), r1 = T(0), r2 = T(0), r3 = T(0);
+#pragma unroll 1
+    for (int vw = 0; vw < kClosureWarps; ++vw) {
+        r0 = r1;
+        r1 = r2;
+        r2 = r3;
+        r3 = warp_sum(wall_flux_partial<T>(wall, side == 0 ? (long long)M.Np : -(long long)M.Np, M, tb, side, part, P,
+                                           32 * vw + lane));
+    }
+    const T r[kClosureWarps] = {r0, r1, r2, r3};
     return wall_part_sum(r);
 }
 

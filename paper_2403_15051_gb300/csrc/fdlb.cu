@@ -772,7 +772,8 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
         }
         if (S.tiles && S.smem_stream > S.smem_optin) return FDLB_EINVAL;
     }
-    for (S.march_G = 2; !S.tiles && S.march_G >= 1; --S.march_G) {
+    // (a warp's rows are short: groups of four cells halve what a group costs beside its cells)
+    for (S.march_G = nt == 32 ? 4 : 2; !S.tiles && S.march_G >= 1; --S.march_G) {
         const MarchSmem P = march_smem_plan(S.march_G, Ms, S.nR, S.n2, S.n3, nt / 32, (int)S.tsize, S.krg_on ? 1 : 0);
         if ((size_t)(P.teams + P.team_bytes) <= S.smem_optin) break;
     }

@@ -332,7 +332,9 @@ __global__ void __launch_bounds__(kClosureThreads, sizeof(T) == 4 ? 4 : 2) closu
         const T cT = w_hi(Tc), cu0 = w_hi(u[0]), cu1 = w_hi(u[1]), cu2 = w_hi(u[2]);
         if (own) {
             const T tm1 = w_hi(w_sub(Tc, w_from_t(T(1))));  // T - 1 without cancellation
-#pragma unroll
+            // (a launch runs most of this code once per warp: the loop stays a loop, the kernel small, since fetching
+            // its instructions is a good part of a short launch)
+#pragma unroll 1
             for (int job = 0; job < 4; ++job) {
                 T ev[kMaxE + 1];
                 clo_eq_coeffs<T>(job, cT, tm1, cu0, job == 2 ? cu1 : cu2, tb, M, ev);
