@@ -474,6 +474,16 @@ cudaError_t launch_step_dispatch(const Solver& S, const StepArgs* P, int* blocks
                          : launch_step_double_1(S.scfg, P, S.M, S.grid_step, S.threads, S.smem_step, S.stream, blocks_per_sm);
 }
 
+// K_2 among the launch's constants, where it fits.
+void set_k2(const Solver& S, StageArgs& A) {
+    if ((size_t)S.n2 * S.n2 * S.tsize <= (size_t)kK2Bytes)
+        for (int e = 0; e < S.n2 * S.n2; ++e) {
+            const int t = (e % S.n2) * S.n2 + e / S.n2;
+            if (S.precision == FDLB_FP32) A.K2.f[t] = (float)S.tab_h[S.M.o_K2 + e];
+            else A.K2.d[t] = S.tab_h[S.M.o_K2 + e];
+        }
+}
+
 // The stage kernel of the current configuration: its launch, or with `blocks_per_sm` its occupancy.
 cudaError_t launch_stage_kernel(const Solver& S, const StageArgs& A, int grid, int* blocks_per_sm) {
     const int threads = S.threads * S.teams;
@@ -733,9 +743,13 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
     // momenta; per-vector and per-cell work spread over twice the momenta, half the warps per cell)
     if (cfg.spec && S.tsize == 4 && S.geometry == FDLB_CYL && cap <= 128 && Ms / 8 <= 128) cfg.vw = 8;
     if (!cfg.spec && rows8) cfg.vw = 8;
+    // the sphere's FP32 shape: a thread per row of twelve.  The stage is bound by the shared-memory data unit (four
+    // momenta per thread: 86 vector loads per vector, 69% of its rate at 81 us on 2048 cells); a whole row shares
+    // the coefficients of K^h and K_3, and K_2's are launch constants.  Not for the mma.sync form, built for four
+    if (cfg.spec && S.tsize == 4 && S.geometry == FDLB_SPH && !S.tensor) cfg.vw = 12;
     const int Vs = Ms / cfg.vw;
     int nt = 0;
-    if (cfg.vw == 8) {
+    if (cfg.vw == 8 || cfg.vw == 12) {
         cfg.nv = 1;
         nt = (Vs + 31) / 32 * 32;
     } else if (cfg.spec) {
@@ -973,12 +987,7 @@ int launch_stream_only(Solver& S, int in, int fn, int out, double a, double b, i
     A.B = S.B;
     A.G = S.march_G;
     A.teams = S.teams;
-    if ((size_t)S.n2 * S.n2 * S.tsize <= (size_t)kK2Bytes)
-        for (int e = 0; e < S.n2 * S.n2; ++e) {
-            const int t = (e % S.n2) * S.n2 + e / S.n2;
-            if (S.precision == FDLB_FP32) A.K2.f[t] = (float)S.tab_h[S.M.o_K2 + e];
-            else A.K2.d[t] = S.tab_h[S.M.o_K2 + e];
-        }
+    set_k2(S, A);
     A.use_bulk = S.use_bulk;
     A.programmatic = S.programmatic;
     A.mma = S.mma_on;
@@ -1107,6 +1116,7 @@ int launch_steps_fused(Solver& S, int64_t n) {
     A.err = S.err;
     A.mode = 0;
     A.B = S.step_B;
+    set_k2(S, A);
     A.G = S.march_G;
     A.teams = 1;
     A.use_bulk = S.use_bulk;

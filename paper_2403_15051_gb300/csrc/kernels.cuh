@@ -64,7 +64,7 @@ struct MomSet {
     int o_pR, o_wR, o_p2, o_w2, o_p3, o_w3, o_KR, o_K2, o_K3, o_GR, o_G2, o_G3, o_ha, o_hb, o_h0;
 };
 
-constexpr int kK2Bytes = 256;       // K_2 travels with the stage's launch where it is at most this large
+constexpr int kK2Bytes = 576;       // K_2 travels with the stage's launch where it is at most this large
 
 struct StageArgs {
     const void* f_in;

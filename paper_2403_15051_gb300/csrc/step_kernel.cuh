@@ -224,6 +224,11 @@ cudaError_t step_dispatch(const StreamCfg& cfg, const StepArgs* S, const MomSet&
     constexpr int VS = sizeof(T) == 4 || G == 0 ? 4 : 2;
     constexpr int SR = G == 0 ? 16 : 24, S2 = G == 0 ? 8 : 12, S3 = G == 0 ? 8 : 12;
     constexpr int NA = G == 0 ? 1 : 2, NB = 2 * NA;
+    if constexpr (sizeof(T) == 4 && G == 1)
+        if (cfg.spec && cfg.vw == 12 && cfg.nv == 1) {
+            if (blocks_per_sm) return step_occupancy_t<T, G, 12, 1, SR, S2, S3>(threads, smem, blocks_per_sm);
+            return launch_step_t<T, G, 12, 1, SR, S2, S3>(*S, M, grid, threads, smem, s);
+        }
     if (!cfg.spec || cfg.vw != VS) return cudaErrorInvalidValue;
     if (cfg.nv == NA) {
         if (blocks_per_sm) return step_occupancy_t<T, G, VS, NA, SR, S2, S3>(threads, smem, blocks_per_sm);

@@ -46,12 +46,12 @@ __device__ __forceinline__ void wall_ghosts(T f0, T f1, T f2, T f3, T& g1, T& g2
 // VW consecutive elements (16-byte aligned for VW * sizeof(T) >= 16; 8-byte for float2).
 template <typename T, int VW>
 __device__ __forceinline__ void ld_vec(const T* p, T (&o)[VW]) {
-    if constexpr (sizeof(T) == 4 && VW == 4) {
-        const float4 x = *reinterpret_cast<const float4*>(p);
-        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
-    } else if constexpr (sizeof(T) == 4 && VW == 8) {
-        const float4 x = reinterpret_cast<const float4*>(p)[0], y = reinterpret_cast<const float4*>(p)[1];
-        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w; o[4] = y.x; o[5] = y.y; o[6] = y.z; o[7] = y.w;
+    if constexpr (sizeof(T) == 4 && VW % 4 == 0) {
+#pragma unroll
+        for (int h = 0; h < VW / 4; ++h) {
+            const float4 x = reinterpret_cast<const float4*>(p)[h];
+            o[4 * h] = x.x; o[4 * h + 1] = x.y; o[4 * h + 2] = x.z; o[4 * h + 3] = x.w;
+        }
     } else if constexpr (sizeof(T) == 4 && VW == 2) {
         const float2 x = *reinterpret_cast<const float2*>(p);
         o[0] = x.x; o[1] = x.y;
@@ -69,12 +69,12 @@ __device__ __forceinline__ void ld_vec(const T* p, T (&o)[VW]) {
 
 template <typename T, int VW>
 __device__ __forceinline__ void ldg_vec(const T* p, T (&o)[VW]) {
-    if constexpr (sizeof(T) == 4 && VW == 4) {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(p));
-        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
-    } else if constexpr (sizeof(T) == 4 && VW == 8) {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(p)), y = __ldg(reinterpret_cast<const float4*>(p) + 1);
-        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w; o[4] = y.x; o[5] = y.y; o[6] = y.z; o[7] = y.w;
+    if constexpr (sizeof(T) == 4 && VW % 4 == 0) {
+#pragma unroll
+        for (int h = 0; h < VW / 4; ++h) {
+            const float4 x = __ldg(reinterpret_cast<const float4*>(p) + h);
+            o[4 * h] = x.x; o[4 * h + 1] = x.y; o[4 * h + 2] = x.z; o[4 * h + 3] = x.w;
+        }
     } else if constexpr (sizeof(T) == 4 && VW == 2) {
         const float2 x = __ldg(reinterpret_cast<const float2*>(p));
         o[0] = x.x; o[1] = x.y;
@@ -93,12 +93,12 @@ __device__ __forceinline__ void ldg_vec(const T* p, T (&o)[VW]) {
 // The same through L2 only (data written earlier in the same launch by other blocks).
 template <typename T, int VW>
 __device__ __forceinline__ void ldcg_vec(const T* p, T (&o)[VW]) {
-    if constexpr (sizeof(T) == 4 && VW == 4) {
-        const float4 x = __ldcg(reinterpret_cast<const float4*>(p));
-        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
-    } else if constexpr (sizeof(T) == 4 && VW == 8) {
-        const float4 x = __ldcg(reinterpret_cast<const float4*>(p)), y = __ldcg(reinterpret_cast<const float4*>(p) + 1);
-        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w; o[4] = y.x; o[5] = y.y; o[6] = y.z; o[7] = y.w;
+    if constexpr (sizeof(T) == 4 && VW % 4 == 0) {
+#pragma unroll
+        for (int h = 0; h < VW / 4; ++h) {
+            const float4 x = __ldcg(reinterpret_cast<const float4*>(p) + h);
+            o[4 * h] = x.x; o[4 * h + 1] = x.y; o[4 * h + 2] = x.z; o[4 * h + 3] = x.w;
+        }
     } else if constexpr (sizeof(T) == 4 && VW == 2) {
         const float2 x = __ldcg(reinterpret_cast<const float2*>(p));
         o[0] = x.x; o[1] = x.y;
@@ -116,11 +116,10 @@ __device__ __forceinline__ void ldcg_vec(const T* p, T (&o)[VW]) {
 
 template <typename T, int VW>
 __device__ __forceinline__ void st_vec(T* p, const T (&o)[VW]) {
-    if constexpr (sizeof(T) == 4 && VW == 4) {
-        *reinterpret_cast<float4*>(p) = make_float4(o[0], o[1], o[2], o[3]);
-    } else if constexpr (sizeof(T) == 4 && VW == 8) {
-        reinterpret_cast<float4*>(p)[0] = make_float4(o[0], o[1], o[2], o[3]);
-        reinterpret_cast<float4*>(p)[1] = make_float4(o[4], o[5], o[6], o[7]);
+    if constexpr (sizeof(T) == 4 && VW % 4 == 0) {
+#pragma unroll
+        for (int h = 0; h < VW / 4; ++h)
+            reinterpret_cast<float4*>(p)[h] = make_float4(o[4 * h], o[4 * h + 1], o[4 * h + 2], o[4 * h + 3]);
     } else if constexpr (sizeof(T) == 4 && VW == 2) {
         *reinterpret_cast<float2*>(p) = make_float2(o[0], o[1]);
     } else if constexpr (sizeof(T) == 8 && VW >= 2) {
@@ -1075,13 +1074,14 @@ __device__ __forceinline__ void tile_body(const StageArgs& A, const MomSet& M) {
 }
 
 // The stage kernel; MINB = the blocks per SM the register allocation is bounded for: 1 (up to 512
-// threads, 128 registers each; 256 threads where four FP64 momenta per thread need more) or, for blocks of
+// threads, 128 registers each; 256 threads where four FP64 momenta per thread need more, 288 for the
+// sphere's rows of twelve) or, for blocks of
 // at most 256 threads, 3 (at most 85 registers each); for the row kernel (VW = 8, blocks of at most 128
 // threads) 5, 3 or 2 (at most 102, 170 or 255 registers each).  The arithmetic and its order are the same
 // in all.
 template <typename T, int VW, int MINB>
 constexpr int stage_max_threads() {
-    return VW == 8 ? (MINB == 1 ? 512 : 128) : (sizeof(T) == 8 && VW == 4) || MINB > 1 ? 256 : 512;
+    return VW == 12 ? 288 : VW == 8 ? (MINB == 1 ? 512 : 128) : (sizeof(T) == 8 && VW == 4) || MINB > 1 ? 256 : 512;
 }
 template <typename T, int GEOM, int VW, int NV, int NR_, int N2_, int N3_, int MINB>
 __global__ void __launch_bounds__(stage_max_threads<T, VW, MINB>(), MINB) stream_kernel(StageArgs A, MomSet M) {
@@ -1123,6 +1123,10 @@ cudaError_t launch_stream_dispatch(const StreamCfg& cfg, const StageArgs& A, con
                 if (cfg.minb == 2) return launch_stream_t<T, G, 8, 1, SR, S2, S3, 2>(A, M, grid, threads, smem, s, bps);
                 return launch_stream_t<T, G, 8, 1, SR, S2, S3>(A, M, grid, threads, smem, s, bps);
             }
+        }
+        if constexpr (sizeof(T) == 4 && G == 1) {
+            // the sphere's as one whole p_2 row (12 momenta) per thread
+            if (cfg.vw == 12 && cfg.nv == 1) return launch_stream_t<T, G, 12, 1, SR, S2, S3>(A, M, grid, threads, smem, s, bps);
         }
         if (cfg.vw != VS) return cudaErrorInvalidValue;
         if constexpr (sizeof(T) == 4 && G == 0) {
