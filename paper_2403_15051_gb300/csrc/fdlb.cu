@@ -733,6 +733,15 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
         cfg.vw = S.n2 % 4 == 0 ? 4 : (S.n2 % 2 == 0 ? 2 : 1);
     else  // (four FP64 momenta per thread: blocks of up to 256 threads, for their registers)
         cfg.vw = S.n2 % 4 == 0 && Ms <= 1024 ? 4 : (S.n2 % 2 == 0 ? 2 : 1);
+    // FP64 over few cells: each of an SM's four partitions takes an FP64 warp instruction every 64 cycles, so a cell
+    // whose momenta fit one warp has a quarter of its SM.  Fewer momenta per thread then, as long as cells and warps
+    // together do not fill the partitions (one cell's face and update: 41000 cycles by one warp)
+    bool spread = false;
+    if (S.tsize == 8)
+        while (cfg.vw > 1 && Ms / cfg.vw < 128 && (long long)S.total_cells * ((Ms / cfg.vw + 31) / 32) < 4LL * S.n_sm) {
+            cfg.vw /= 2;
+            spread = true;
+        }
     // rows of eight per thread over many cells, as for the compile-time shape below
     const bool rows8 = S.tsize == 4 && S.n2 == 8 && Ms / 8 <= 512 && (long long)S.total_cells * S.Np > (long long)S.n_sm * 65536;
     cfg.spec = ((S.geometry == FDLB_CYL && S.nR == 16 && S.n2 == 8 && S.n3 == 8) ||
@@ -760,8 +769,8 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
     } else {
         // the most a thread holds; fewer when the block has room, except that two vectors per thread
         // keep up to 64 of them in one warp
-        cfg.nv = cfg.vw == 4 ? (S.tsize == 4 && Vs > 32 ? 2 : 1) : 4;
-        nt = Vs <= 32 * cfg.nv ? 32 : (std::min(Vs, cap) + 31) / 32 * 32;
+        cfg.nv = cfg.vw == 4 ? (S.tsize == 4 && Vs > 32 ? 2 : 1) : spread ? 1 : 4;
+        nt = spread ? (Vs + 31) / 32 * 32 : Vs <= 32 * cfg.nv ? 32 : (std::min(Vs, cap) + 31) / 32 * 32;
         if ((long long)nt * cfg.nv < Vs) nt = ((Vs + cfg.nv - 1) / cfg.nv + 31) / 32 * 32;
     }
     if (nt > 512 || (long long)nt * cfg.nv < Vs) return FDLB_EINVAL;

@@ -166,10 +166,7 @@ __global__ void __launch_bounds__(stage_max_threads<T, VW, 1>(), 1) step_kernel(
                     return;
                 }
                 tile_geometry<T, GEOM, VW, NV, NR_, N2_, N3_>(SP, wi, I, A, M);
-                {
-                    const T* gwi = reinterpret_cast<const T*>(A.gwT) + (long long)wi.x * 2 * (nR + n2 + n3);
-                    for (int e = tid; e < 2 * (nR + n2 + n3); e += blockDim.x) SP.gw[e] = gwi[e];
-                }
+                stage_maxwellians<T, GEOM, VW, NV, NR_, N2_, N3_>(SP, wi.x, A, M);
                 // the wall densities as the stage kernel forms them from the parts
                 T nw[2] = {T(0), T(0)};
 #pragma unroll

@@ -728,13 +728,18 @@ __device__ __forceinline__ void stage_sums(const T* red, const InstDev& I, int c
     }
 }
 
-// The wall Maxwellians of an item's instance and its wall densities (from the parts of the outgoing
-// fluxes) into shared memory; the caller synchronises.
+// The wall Maxwellians of an item's instance into shared memory; the caller synchronises.
 template <typename T, int GEOM, int VW, int NV, int NR_, int N2_, int N3_>
-__device__ __forceinline__ void stage_walls(const StagePtrs<T>& S, int q, const InstDev& I, const StageArgs& A, const MomSet& M) {
+__device__ __forceinline__ void stage_maxwellians(const StagePtrs<T>& S, int q, const StageArgs& A, const MomSet& M) {
     FDLB_STAGE_SIZES;
     const T* gwi = reinterpret_cast<const T*>(A.gwT) + (long long)q * 2 * gwstride;
     for (int e = tid; e < 2 * gwstride; e += NT) S.gw[e] = gwi[e];
+}
+
+// Its wall densities, from the parts of the outgoing fluxes.
+template <typename T, int GEOM, int VW, int NV, int NR_, int N2_, int N3_>
+__device__ __forceinline__ void stage_walls(const StagePtrs<T>& S, int q, const InstDev& I, const StageArgs& A, const MomSet& M) {
+    FDLB_STAGE_SIZES;
     if (tid < 2) {
         const T* pp = reinterpret_cast<const T*>(A.nwp) + ((long long)q * 2 + tid) * A.wall_parts;
         T part[kWallParts], sum = T(0);  // every load in flight; summed in order
@@ -846,27 +851,39 @@ __device__ __forceinline__ void march_body(const StageArgs& A, const MomSet& M) 
         const int c0 = wi.y, cg = min(G, wi.z);
         march_request<T, GEOM, VW, NV, NR_, N2_, N3_>(S, I, wi.w, c0 - 3, R, c0 - 3, c0 + cg + 3, c0, cg, S.rec, c0, c0 + cg, part, A, M);
     };
+    // What an item needs of the constants: the geometry of the G cells from c0 + cl on, the wall
+    // Maxwellians and the threads' vectors; of the first item also before the wait.
+    auto geometry = [&](int4 wi, const InstDev& I, int cl, T* dst) {
+        const T* geoT = reinterpret_cast<const T*>(A.geoT) + (long long)(I.cell_off + wi.y) * kGeo;
+        for (int e = tid; e < 3 * min(G, wi.z - cl); e += NT) dst[e] = geoT[(long long)(cl + e / 3) * kGeo + 2 + e % 3];
+    };
+    StageWalk<T, VW, NV> W;
+    auto constants = [&](int4 wi, const InstDev& I) {
+        geometry(wi, I, 0, S.geo);
+        stage_maxwellians<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi.x, A, M);
+        stage_walk_init<T, GEOM, VW, NV, NR_, N2_, N3_>(W, S, wi.w, A, M);
+    };
+    int4 wi = make_int4(0, 0, 0, 0);
+    InstDev I;
     const bool early = A.use_bulk && it0 < nit;
-    if (early) {
-        const int4 wi = A.items[it0];
-        first(wi, A.inst[wi.x], 1);
+    if (it0 < nit) {
+        wi = A.items[it0];
+        I = A.inst[wi.x];
+        if (early) first(wi, I, 1);
+        constants(wi, I);
     }
     pdl_trigger();
     pdl_wait();  // everything below reads what the previous kernels wrote
     uint32_t phase = 0;
-    StageWalk<T, VW, NV> W;
     for (int it = it0; it < nit; it += gridDim.x * teams) {
-        const int4 wi = A.items[it];
-        const InstDev I = A.inst[wi.x];
+        if (it != it0) {
+            wi = A.items[it];
+            I = A.inst[wi.x];
+        }
         const int N = I.n_cells, c0 = wi.y, Be = wi.z, sl = wi.w, c1 = c0 + Be;
         first(wi, I, early && it == it0 ? 2 : 3);
-        const T* geoT = reinterpret_cast<const T*>(A.geoT) + (long long)(I.cell_off + c0) * kGeo;
-        auto geometry = [&](int cl, T* dst) {  // of the G cells from c0 + cl on
-            for (int e = tid; e < 3 * min(G, Be - cl); e += NT) dst[e] = geoT[(long long)(cl + e / 3) * kGeo + 2 + e % 3];
-        };
         stage_walls<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi.x, I, A, M);
-        geometry(0, S.geo);
-        stage_walk_init<T, GEOM, VW, NV, NR_, N2_, N3_>(W, S, sl, A, M);
+        if (it != it0) constants(wi, I);
         if (!stage_wait<T, GEOM, VW, NV, NR_, N2_, N3_>(S, A, M, phase)) return;
         const T nwL = S.nw[0], nwR = S.nw[1];
         // ring slot of cell r, as an element offset
@@ -898,7 +915,7 @@ __device__ __forceinline__ void march_body(const StageArgs& A, const MomSet& M) 
             if (cn > 0) {
                 march_request<T, GEOM, VW, NV, NR_, N2_, N3_>(S, I, sl, c0 - 3, R, c + cg + 3, c + cg + cn + 3, c + cg, cn,
                                                               S.rec + (buf ^ 1) * G * rs, c + cg, c + cg + cn, 3, A, M);
-                geometry(cl + G, S.geo + (buf ^ 1) * 3 * G);
+                geometry(wi, I, cl + G, S.geo + (buf ^ 1) * 3 * G);
             }
             if (A.mode == 0 && prev > 0)
                 stage_sums<T, GEOM, VW, NV, NR_, N2_, N3_>(S.red + (buf ^ 1) * G * nwarps * 16, I, c - prev, prev, sl, A, M);
@@ -1066,7 +1083,9 @@ __device__ __forceinline__ void tile_body(const StageArgs& A, const MomSet& M) {
         const int4 wi = A.items[it];
         const InstDev I = A.inst[wi.x];
         tile_request<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi, I, true, early && it == (int)blockIdx.x ? 2 : 3, A, M);
+        // (here, where they overlap the copy: before the wait they cost the tile kernels 4%)
         tile_geometry<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi, I, A, M);
+        stage_maxwellians<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi.x, A, M);
         stage_walls<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi.x, I, A, M);
         if (!stage_wait<T, GEOM, VW, NV, NR_, N2_, N3_>(S, A, M, phase)) return;
         tile_compute<T, GEOM, VW, NV, NR_, N2_, N3_, false>(S, wi, I, snw[0], snw[1], A, M);
@@ -1148,6 +1167,10 @@ cudaError_t launch_stream_dispatch(const StreamCfg& cfg, const StageArgs& A, con
     if constexpr (sizeof(T) == 4) {
         if (cfg.vw == 8 && cfg.nv == 1 && M.n2 == 8) return launch_stream_t<T, G, 8, 1, 0, 8, 0>(A, M, grid, threads, smem, s, bps);
         if (cfg.vw == 4 && cfg.nv == 2 && M.n2 == 8) return launch_stream_t<T, G, 4, 2, 0, 8, 0>(A, M, grid, threads, smem, s, bps);
+    }
+    if constexpr (sizeof(T) == 8) {
+        if (cfg.vw == 1 && cfg.nv == 1) return launch_stream_t<T, G, 1, 1, 0, 0, 0>(A, M, grid, threads, smem, s, bps);
+        if (cfg.vw == 2 && cfg.nv == 1) return launch_stream_t<T, G, 2, 1, 0, 0, 0>(A, M, grid, threads, smem, s, bps);
     }
     if (cfg.vw == 1 && cfg.nv == 4) return launch_stream_t<T, G, 1, 4, 0, 0, 0>(A, M, grid, threads, smem, s, bps);
     if (cfg.vw == 2 && cfg.nv == 4) return launch_stream_t<T, G, 2, 4, 0, 0, 0>(A, M, grid, threads, smem, s, bps);
