@@ -51,12 +51,15 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
 
 constexpr int kT = 64;        // rows and columns of an output tile
 constexpr int kKc = 64;       // contraction values staged at a time
-constexpr int kModes = kKc / 2;  // modes (real and imaginary row) of a chunk
+constexpr int kModes = 16;    // modes (real and imaginary row) mixed at a time
+constexpr int kBasis = 32;    // basis rows staged at a time
 constexpr int kLd = kT + 4;   // row stride of a staged chunk [k][64]
 constexpr int kNT = 256;      // threads: 16 x 16, 4 x 4 outputs each
 constexpr int kMaxSplits = 64;  // row splits of the weight gradients
+constexpr int kMaxWidth = 512;
 
-// Every kernel here may start while its predecessor drains and waits before it reads anything.
+// Every kernel here may start while its predecessor drains: it requests weights and bases, which no kernel
+// of a pass writes, and waits before it reads anything else.
 __device__ __forceinline__ void nn_begin() {
     pdl_trigger();
     pdl_wait();
@@ -120,33 +123,47 @@ __device__ __forceinline__ void stage_cols(float* dst, const TS* src, long long 
     }
 }
 
-// Shared memory of the tile kernels: two staged chunks, X and Y, and behind them the spectral
-// coefficients of a chunk of modes, [2 kModes][W].  An output tile takes X's place, [row][kLd].
+// Shared memory of the tile kernels: two staged chunks, X and Y, the rows of the basis of the partial
+// transform, [kBasis][64], those of the inverse transform's, [2 kModes][kLd], and the spectral coefficients of a
+// chunk of modes, [2 kModes][W].  An output tile takes X's place, [row][kLd].
 __device__ __forceinline__ float* chunk_y(float* sm) { return sm + kKc * kLd; }
-__device__ __forceinline__ float* hats_of(float* sm) { return sm + 2 * kKc * kLd; }
+__device__ __forceinline__ float* basis_of(float* sm) { return sm + 2 * kKc * kLd; }
+__device__ __forceinline__ float* inverse_of(float* sm) { return basis_of(sm) + kBasis * kT; }
+__device__ __forceinline__ float* hats_of(float* sm) { return inverse_of(sm) + 2 * kModes * kLd; }
+
+// Rows k0 .. k0 + nk - 1 of a basis at the tile's rows into bs[k][row]: basis(k, row) at basis[k sk + row sr].
+__device__ __forceinline__ void stage_basis(float* bs, const float* basis, long long sk, long long sr, int k0, int nk, int rows) {
+#pragma unroll 4
+    for (int e = threadIdx.x; e < nk * kT; e += kNT) {
+        const int k = sk == 1 ? e % nk : e / kT, r = sk == 1 ? e / nk : e % kT;  // (along the basis in memory)
+        bs[k * kT + r] = r < rows ? basis[(k0 + k) * sk + r * sr] : 0.f;
+    }
+}
 
 // The block's output tile T[row][column] (`rows` of 64, zero-filled columns) into its partial transform:
-// part[k][n0 + c] = sum over the rows of basis(k, row) T[row][c] for the 2m rows of the basis; basis(k, row)
-// at basis[k sk + row sr].  part: [2m][W] of this row tile.
+// part[k][n0 + c] = sum over the rows of basis(k, row) T[row][c] for the 2m rows of the basis, the first chunk
+// of which is in bs.  part: [2m][W] of this row tile.
 __device__ __forceinline__ void partial_transform(const float* T, const float* basis, long long sk, long long sr, int m2, int rows,
                                                   int n0, int W, float* bs, float* part) {
     const int c = threadIdx.x % kT, g = threadIdx.x / kT;
-    for (int k0 = 0; k0 < m2; k0 += kKc) {
-        const int nk = min(kKc, m2 - k0);
+    for (int k0 = 0; k0 < m2; k0 += kBasis) {
+        const int nk = min(kBasis, m2 - k0);
         __syncthreads();
-        for (int e = threadIdx.x; e < nk * kT; e += kNT) {
-            const int k = e / kT, r = e % kT;
-            bs[k * kT + r] = r < rows ? basis[(k0 + k) * sk + r * sr] : 0.f;
+        if (k0 > 0) {
+            stage_basis(bs, basis, sk, sr, k0, nk, rows);
+            __syncthreads();
         }
-        __syncthreads();
         for (int k = g; k < nk; k += kNT / kT) {
-            float s0 = 0.f, s1 = 0.f;
-#pragma unroll 8
-            for (int r = 0; r < kT; r += 2) {
-                s0 = fmaf(bs[k * kT + r], T[r * kLd + c], s0);
-                s1 = fmaf(bs[k * kT + r + 1], T[(r + 1) * kLd + c], s1);
+            float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
+#pragma unroll 4
+            for (int r = 0; r < kT; r += 4) {
+                const float4 x = *reinterpret_cast<const float4*>(bs + k * kT + r);
+                p0 = fmaf(x.x, T[r * kLd + c], p0);
+                p1 = fmaf(x.y, T[(r + 1) * kLd + c], p1);
+                p2 = fmaf(x.z, T[(r + 2) * kLd + c], p2);
+                p3 = fmaf(x.w, T[(r + 3) * kLd + c], p3);
             }
-            if (n0 + c < W) part[(long long)(k0 + k) * W + n0 + c] = s0 + s1;
+            if (n0 + c < W) part[(long long)(k0 + k) * W + n0 + c] = (p0 + p1) + (p2 + p3);
         }
     }
 }
@@ -155,11 +172,18 @@ __device__ __forceinline__ void partial_transform(const float* T, const float* b
 // order: hats[q][i] = sum_t part[t][mode row][i], rows q < kModes the real, q >= kModes the imaginary parts;
 // kept in `keep` ([2m][W]) where not null.
 __device__ __forceinline__ void sum_hats(float* hats, const float* part, int nt, int m, int W, int k0, int nm, float* keep) {
+#pragma unroll 4
     for (int e = threadIdx.x; e < 2 * nm * W; e += kNT) {
         const int q = e / W, i = e % W, im = q >= nm, row = (im ? m : 0) + k0 + (im ? q - nm : q);
+        const float* p = part + (long long)row * W + i;
+        const long long st = 2LL * m * W;
         float s = 0.f;
-#pragma unroll 4
-        for (int t = 0; t < nt; ++t) s += part[((long long)t * 2 * m + row) * W + i];
+        int t = 0;
+        for (; t + 4 <= nt; t += 4) {
+            const float a = p[t * st], b = p[(t + 1) * st], c = p[(t + 2) * st], d = p[(t + 3) * st];
+            s = (((s + a) + b) + c) + d;
+        }
+        for (; t < nt; ++t) s += p[t * st];
         hats[((im ? kModes : 0) + (im ? q - nm : q)) * W + i] = s;
         if (keep) keep[(long long)row * W + i] = s;
     }
@@ -172,16 +196,28 @@ __device__ __forceinline__ void mix_forward(float* Y, float* scratch, const floa
                                             const __nv_bfloat16* Rim, int W, int k0, int nm, int n0) {
     const int c = threadIdx.x % kT, g = threadIdx.x / kT, col = min(n0 + c, W - 1);
     // (four quarters of 2 nm rows fit over the chunks for nm <= 17: at most 16 modes at a time)
+#pragma unroll 2
     for (int q = 0; q < nm; ++q) {
         const __nv_bfloat16* a = Rre + (long long)(k0 + q) * W * W + col;
         const __nv_bfloat16* b = Rim + (long long)(k0 + q) * W * W + col;
         float yr = 0.f, yi = 0.f;
-#pragma unroll 16
-        for (int i = g; i < W; i += 4) {
-            const float ra = to_f(a[(long long)i * W]), rb = to_f(b[(long long)i * W]);
-            const float re = hats[q * W + i], im = hats[(kModes + q) * W + i];
-            yr = fmaf(re, ra, fmaf(-im, rb, yr));
-            yi = fmaf(re, rb, fmaf(im, ra, yi));
+        for (int i0 = g; i0 < W; i0 += kT) {
+            __nv_bfloat16 ra[kT / 4], rb[kT / 4];
+#pragma unroll
+            for (int u = 0; u < kT / 4; ++u) {
+                const int i = min(i0 + 4 * u, W - 1);
+                ra[u] = a[(long long)i * W];
+                rb[u] = b[(long long)i * W];
+            }
+#pragma unroll
+            for (int u = 0; u < kT / 4; ++u) {
+                const int i = i0 + 4 * u;
+                if (i < W) {
+                    const float re = hats[q * W + i], im = hats[(kModes + q) * W + i], fa = to_f(ra[u]), fb = to_f(rb[u]);
+                    yr = fmaf(re, fa, fmaf(-im, fb, yr));
+                    yi = fmaf(re, fb, fmaf(im, fa, yi));
+                }
+            }
         }
         scratch[(g * 2 * nm + q) * kT + c] = yr;
         scratch[(g * 2 * nm + nm + q) * kT + c] = yi;
@@ -258,8 +294,9 @@ __global__ void __launch_bounds__(kNT) lift_kernel(const float* __restrict__ raw
                                                    const float* __restrict__ F, float* __restrict__ a, float* __restrict__ v,
                                                    float* __restrict__ part) {
     extern __shared__ __align__(16) float sm[];
-    nn_begin();
     const int r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT, rows = min(kT, P - r0);
+    stage_basis(basis_of(sm), F + r0, P, 1, 0, min(kBasis, 2 * m), rows);
+    nn_begin();
     const float* r = raw + b * 5;
     float f[kCin] = {log10f(r[0]) + 1.f, (r[1] - 0.155f) / 0.145f, (r[2] - 3.1f) / 1.9f, (r[3] - 0.15f) / 0.15f,
                      (r[4] - 1.15f) / 0.15f, 0.f};
@@ -284,7 +321,7 @@ __global__ void __launch_bounds__(kNT) lift_kernel(const float* __restrict__ raw
             const int rr = e / kCin, i = e % kCin;
             a[((long long)b * P + r0) * kCin + e] = i == 5 ? (float)(r0 + rr) / (float)(P - 1) : f[i];
         }
-    partial_transform(sm, F + r0, P, 1, 2 * m, rows, n0, W, chunk_y(sm), part + ((long long)b * gridDim.x + blockIdx.x) * 2 * m * W);
+    partial_transform(sm, F + r0, P, 1, 2 * m, rows, n0, W, basis_of(sm), part + ((long long)b * gridDim.x + blockIdx.x) * 2 * m * W);
 }
 
 // 64 rows of one sample (grid: row tiles, samples, column tiles) through a layer.
@@ -296,30 +333,36 @@ __global__ void __launch_bounds__(kNT) layer_kernel(const float* __restrict__ v,
                                                     const float* __restrict__ F, const float* __restrict__ G, float* __restrict__ hat,
                                                     float* __restrict__ u, float* __restrict__ vout, float* __restrict__ part_out) {
     extern __shared__ __align__(16) float sm[];
-    float *X = sm, *Y = chunk_y(sm), *hats = hats_of(sm);
-    nn_begin();
+    float *X = sm, *Y = chunk_y(sm), *Gs = inverse_of(sm), *hats = hats_of(sm);
     const int nt = gridDim.x, r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT;
+    stage_rows(Y, w, W, 0, W, n0, W);
+    if (part_out) stage_basis(basis_of(sm), F + r0, P, 1, 0, min(kBasis, 2 * m), min(kT, P - r0));
+    auto inverse_basis = [&](int k0, int nm) {
+        for (int e = threadIdx.x; e < 2 * nm * kT; e += kNT) {
+            const int q = e % (2 * nm), r = e / (2 * nm), col = q < nm ? k0 + q : m + k0 + q - nm;
+            Gs[q * kLd + r] = r0 + r < P ? G[(long long)(r0 + r) * 2 * m + col] : 0.f;
+        }
+    };
+    inverse_basis(0, min(kModes, m));
+    nn_begin();
     Tile t;
     tile_zero(t);
     for (int k0 = 0; k0 < W; k0 += kKc) {
         stage_cols(X, v + (long long)b * P * W, W, r0, P, k0, W);
-        stage_rows(Y, w, W, k0, W, n0, W);
+        if (k0 > 0) stage_rows(Y, w, W, k0, W, n0, W);
         __syncthreads();
         tile_mma(t, X, Y);
         __syncthreads();
     }
-    for (int k0 = 0; k0 < m; k0 += 16) {
-        const int nm = min(16, m - k0);
+    for (int k0 = 0; k0 < m; k0 += kModes) {
+        const int nm = min(kModes, m - k0);
         sum_hats(hats, part_in + (long long)b * nt * 2 * m * W, nt, m, W, k0, nm,
                  blockIdx.x == 0 && blockIdx.z == 0 ? hat + (long long)b * 2 * m * W : nullptr);
+        if (k0 > 0) inverse_basis(k0, nm);
         __syncthreads();
         mix_forward(Y, sm, hats, Rre, Rim, W, k0, nm, n0);
-        for (int e = threadIdx.x; e < 2 * nm * kT; e += kNT) {
-            const int q = e % (2 * nm), r = e / (2 * nm), col = q < nm ? k0 + q : m + k0 + q - nm;
-            X[q * kLd + r] = r0 + r < P ? G[(long long)(r0 + r) * 2 * m + col] : 0.f;
-        }
         __syncthreads();
-        tile_mma(t, X, Y, 1.f, 2 * nm);
+        tile_mma(t, Gs, Y, 1.f, 2 * nm);
         __syncthreads();
     }
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -339,7 +382,8 @@ __global__ void __launch_bounds__(kNT) layer_kernel(const float* __restrict__ v,
             X[(ty * 4 + i) * kLd + tx * 4 + j] = g;
         }
     if (part_out)
-        partial_transform(X, F + r0, P, 1, 2 * m, min(kT, P - r0), n0, W, Y, part_out + ((long long)b * nt + blockIdx.x) * 2 * m * W);
+        partial_transform(X, F + r0, P, 1, 2 * m, min(kT, P - r0), n0, W, basis_of(sm),
+                          part_out + ((long long)b * nt + blockIdx.x) * 2 * m * W);
 }
 
 // Backward: dv = du W^T + F^T dvh, and into `out` dv GELU'(u) (in place of u, the layer below's du) with its
@@ -351,30 +395,36 @@ __global__ void __launch_bounds__(kNT) layer_back_kernel(const float* __restrict
                                                          float* __restrict__ hat, const float* u, float* out,
                                                          float* __restrict__ part_out) {
     extern __shared__ __align__(16) float sm[];
-    float *X = sm, *Y = chunk_y(sm), *hats = hats_of(sm);
-    nn_begin();
+    float *X = sm, *Y = chunk_y(sm), *Fs = inverse_of(sm), *hats = hats_of(sm);
     const int nt = gridDim.x, r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT;
+    stage_cols(Y, w, W, n0, W, 0, W);
+    if (part_out) stage_basis(basis_of(sm), G + (long long)r0 * 2 * m, 1, 2 * m, 0, min(kBasis, 2 * m), min(kT, P - r0));
+    auto inverse_basis = [&](int k0, int nm) {
+        for (int e = threadIdx.x; e < 2 * nm * kT; e += kNT) {
+            const int q = e / kT, r = e % kT, row = q < nm ? k0 + q : m + k0 + q - nm;
+            Fs[q * kLd + r] = r0 + r < P ? F[(long long)row * P + r0 + r] : 0.f;
+        }
+    };
+    inverse_basis(0, min(kModes, m));
+    nn_begin();
     Tile t;
     tile_zero(t);
     for (int k0 = 0; k0 < W; k0 += kKc) {
         stage_cols(X, du + (long long)b * P * W, W, r0, P, k0, W);
-        stage_cols(Y, w, W, n0, W, k0, W);
+        if (k0 > 0) stage_cols(Y, w, W, n0, W, k0, W);
         __syncthreads();
         tile_mma(t, X, Y);
         __syncthreads();
     }
-    for (int k0 = 0; k0 < m; k0 += 16) {
-        const int nm = min(16, m - k0);
+    for (int k0 = 0; k0 < m; k0 += kModes) {
+        const int nm = min(kModes, m - k0);
         sum_hats(hats, part_in + (long long)b * nt * 2 * m * W, nt, m, W, k0, nm,
                  blockIdx.x == 0 && blockIdx.z == 0 ? hat + (long long)b * 2 * m * W : nullptr);
+        if (k0 > 0) inverse_basis(k0, nm);
         __syncthreads();
         mix_backward(Y, hats, Rre, Rim, W, k0, nm, n0);
-        for (int e = threadIdx.x; e < 2 * nm * kT; e += kNT) {
-            const int q = e / kT, r = e % kT, row = q < nm ? k0 + q : m + k0 + q - nm;
-            X[q * kLd + r] = r0 + r < P ? F[(long long)row * P + r0 + r] : 0.f;
-        }
         __syncthreads();
-        tile_mma(t, X, Y, 1.f, 2 * nm);
+        tile_mma(t, Fs, Y, 1.f, 2 * nm);
         __syncthreads();
     }
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -392,7 +442,7 @@ __global__ void __launch_bounds__(kNT) layer_back_kernel(const float* __restrict
             X[(ty * 4 + i) * kLd + tx * 4 + j] = d;
         }
     if (part_out)
-        partial_transform(X, G + (long long)r0 * 2 * m, 1, 2 * m, 2 * m, min(kT, P - r0), n0, W, Y,
+        partial_transform(X, G + (long long)r0 * 2 * m, 1, 2 * m, 2 * m, min(kT, P - r0), n0, W, basis_of(sm),
                           part_out + ((long long)b * nt + blockIdx.x) * 2 * m * W);
 }
 
@@ -409,6 +459,7 @@ __global__ void __launch_bounds__(kNT) head_kernel(const float* __restrict__ v, 
     __shared__ float w2[kT][kCout];
     __shared__ double red[kNT / 32];
     float *X = sm, *Y = chunk_y(sm);
+    stage_rows(Y, p1, H, 0, W, 0, H);
     nn_begin();
     const long long r0 = (long long)blockIdx.x * kT;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -419,7 +470,7 @@ __global__ void __launch_bounds__(kNT) head_kernel(const float* __restrict__ v, 
         tile_zero(t);
         for (int k0 = 0; k0 < W; k0 += kKc) {
             if (W > kKc || n0 == 0) stage_cols(X, v, W, r0, rows, k0, W);  // (one chunk: staged once)
-            stage_rows(Y, p1, H, k0, W, n0, H);
+            if (n0 > 0 || k0 > 0) stage_rows(Y, p1, H, k0, W, n0, H);
             __syncthreads();
             tile_mma(t, X, Y);
             __syncthreads();
@@ -480,29 +531,37 @@ __global__ void __launch_bounds__(kNT) head_back_kernel(const float* __restrict_
                                                         const float* __restrict__ z1, float* __restrict__ dz,
                                                         const float* __restrict__ G, float* u, float* __restrict__ part_out) {
     extern __shared__ __align__(16) float sm[];
+    __shared__ float ds[kT][kCout];
     float *X = sm, *Y = chunk_y(sm);
-    nn_begin();
     const int nt = gridDim.x, r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT, rows = min(kT, P - r0);
     const long long base = (long long)b * P + r0;
+    stage_cols(Y, p1, H, n0, W, 0, H);
+    stage_basis(basis_of(sm), G + (long long)r0 * 2 * m, 1, 2 * m, 0, min(kBasis, 2 * m), rows);
+    nn_begin();
+    ds[threadIdx.x / kCout][threadIdx.x % kCout] = (int)threadIdx.x / kCout < rows ? dout[base * kCout + threadIdx.x] : 0.f;
+    __syncthreads();
     Tile t;
     tile_zero(t);
     for (int k0 = 0; k0 < H; k0 += kKc) {
+        // a thread's hidden unit is the same in all its rows
+        const int k = threadIdx.x % kKc, col = k0 + k;
+        float pc[kCout];
+#pragma unroll
+        for (int c = 0; c < kCout; ++c) pc[c] = col < H ? to_f(p2[col * kCout + c]) : 0.f;
 #pragma unroll 4
-        for (int e = threadIdx.x; e < kKc * kT; e += kNT) {
-            const int rr = e / kKc, k = e % kKc;
+        for (int rr = threadIdx.x / kKc; rr < kT; rr += kNT / kKc) {
             float d = 0.f;
-            if (rr < rows && k0 + k < H) {
-                const float* dr = dout + (base + rr) * kCout;
-                const __nv_bfloat16* p = p2 + (k0 + k) * kCout;
+            if (rr < rows && col < H) {
+                const float z = z1[(base + rr) * H + col];
                 float s = 0.f;
 #pragma unroll
-                for (int c = 0; c < kCout; ++c) s = fmaf(dr[c], to_f(p[c]), s);
-                d = s * gelu_grad_f(z1[(base + rr) * H + k0 + k]);
-                if (blockIdx.z == 0) dz[(base + rr) * H + k0 + k] = d;
+                for (int c = 0; c < kCout; ++c) s = fmaf(ds[rr][c], pc[c], s);
+                d = s * gelu_grad_f(z);
+                if (blockIdx.z == 0) dz[(base + rr) * H + col] = d;
             }
             X[k * kLd + rr] = d;
         }
-        stage_cols(Y, p1, H, n0, W, k0, H);
+        if (k0 > 0) stage_cols(Y, p1, H, n0, W, k0, H);
         __syncthreads();
         tile_mma(t, X, Y);
         __syncthreads();
@@ -520,7 +579,7 @@ __global__ void __launch_bounds__(kNT) head_back_kernel(const float* __restrict_
             }
             X[rr * kLd + tx * 4 + j] = d;
         }
-    partial_transform(X, G + (long long)r0 * 2 * m, 1, 2 * m, 2 * m, rows, n0, W, Y,
+    partial_transform(X, G + (long long)r0 * 2 * m, 1, 2 * m, 2 * m, rows, n0, W, basis_of(sm),
                       part_out + ((long long)b * nt + blockIdx.x) * 2 * m * W);
 }
 
@@ -556,9 +615,9 @@ __global__ void __launch_bounds__(kNT) grad_kernel(GradTasks T, long long rows, 
         stage_rows(Y, g.Y, g.N, k0, hi, n0, g.N);
         __syncthreads();
         tile_mma(t, X, Y);
-        if (m0 == 0 && threadIdx.x < kT)
+        if (m0 == 0)  // (four groups of threads, a quarter of the rows each)
 #pragma unroll 8
-            for (int k = 0; k < kKc; ++k) cs += Y[k * kLd + threadIdx.x];
+            for (int k = threadIdx.x / kT; k < kKc; k += kNT / kT) cs += Y[k * kLd + threadIdx.x % kT];
         __syncthreads();
     }
     float* C = part + blockIdx.y * stride + g.out;
@@ -570,7 +629,12 @@ __global__ void __launch_bounds__(kNT) grad_kernel(GradTasks T, long long rows, 
             const int a = m0 + ty * 4 + i, c = n0 + tx * 4 + j;
             if (a < g.M && c < g.N) C[(long long)a * g.N + c] = tile_at(t, i, j);
         }
-    if (m0 == 0 && threadIdx.x < kT && n0 + threadIdx.x < g.N) C[(long long)g.M * g.N + n0 + threadIdx.x] = cs;
+    if (m0 == 0) {
+        X[threadIdx.x] = cs;
+        __syncthreads();
+        if (threadIdx.x < kT && n0 + threadIdx.x < g.N)
+            C[(long long)g.M * g.N + n0 + threadIdx.x] = (X[threadIdx.x] + X[kT + threadIdx.x]) + (X[2 * kT + threadIdx.x] + X[3 * kT + threadIdx.x]);
+    }
 }
 
 // Gradients of the spectral weights: block (l m + k, row tile, column tile): dRre = re^T dyre + im^T dyim,
@@ -705,7 +769,8 @@ void nn_launch(NNet& n, void (*kern)(KA...), dim3 grid, size_t smem, A... args) 
 
 unsigned tiles(long long n) { return (unsigned)((n + kT - 1) / kT); }
 constexpr size_t kChunks = 2 * (size_t)kKc * kLd * sizeof(float);  // shared memory of two staged chunks
-size_t layer_smem(int W) { return kChunks + 2 * (size_t)kModes * W * sizeof(float); }
+constexpr size_t kTileSmem = kChunks + (size_t)kBasis * kT * sizeof(float);
+size_t layer_smem(int W) { return kTileSmem + 2 * (size_t)kModes * (kLd + W) * sizeof(float); }
 int grad_splits(long long rows) { return (int)std::min<long long>((rows + 127) / 128, kMaxSplits); }
 
 // Forward pass for B samples whose raw parameters are in n.raw; for training (targets in n.tgt) leaves every
@@ -714,7 +779,7 @@ int forward(NNet& n, int B, bool train) {
     const int W = n.W, m = n.m, P = n.P, H = n.H;
     const long long rows = (long long)B * P;
     const dim3 grid(tiles(P), B, tiles(W));
-    nn_launch(n, lift_kernel, grid, kChunks, n.raw, P, W, m, n.wb + n.o_lw, n.w + n.o_lb, n.F, n.a, n.vs, n.hat_part[0]);
+    nn_launch(n, lift_kernel, grid, kTileSmem, n.raw, P, W, m, n.wb + n.o_lw, n.w + n.o_lb, n.F, n.a, n.vs, n.hat_part[0]);
     for (int l = 0; l < n.L; ++l) {
         float* v = n.vs + (long long)l * rows * W;
         nn_launch(n, layer_kernel, grid, layer_smem(W), v, n.hat_part[l & 1], P, W, m, n.wb + n.o_w[l], n.w + n.o_b[l],
@@ -732,7 +797,7 @@ int backward(NNet& n, int B) {
     const long long rows = (long long)B * P, hat = (long long)B * 2 * m * W;
     auto us = [&](int l) { return n.us + (long long)l * rows * W; };  // u of layer l, then du in its place
     const dim3 grid(tiles(P), B, tiles(W));
-    nn_launch(n, head_back_kernel, grid, kChunks, n.dout, P, W, H, m, n.wb + n.o_p1w, n.wb + n.o_p2w, n.z1, n.dz, n.G, us(L - 1),
+    nn_launch(n, head_back_kernel, grid, kTileSmem, n.dout, P, W, H, m, n.wb + n.o_p1w, n.wb + n.o_p2w, n.z1, n.dz, n.G, us(L - 1),
               n.hat_part[(L - 1) & 1]);
     for (int l = L - 1; l >= 0; --l) {
         float* below = l > 0 ? us(l - 1) : nullptr;
@@ -779,7 +844,7 @@ extern "C" {
 
 int fdlb_nn_create(int width, int modes, int layers, int hidden, int n_points, int max_batch, void* cuda_stream,
                    fdlb_nn_handle* out) try {
-    if (!out || width < 1 || width > 512 || modes < 1 || 2 * modes > n_points || layers < 1 || layers > 16 ||
+    if (!out || width < 1 || width > fdlb::kMaxWidth || modes < 1 || 2 * modes > n_points || layers < 1 || layers > 16 ||
         hidden < 1 || n_points < 8 || n_points > 4096 || max_batch < 1 || max_batch > 4096)
         return FDLB_EINVAL;
     int ndev = 0;
@@ -840,8 +905,8 @@ int fdlb_nn_create(int width, int modes, int layers, int hidden, int n_points, i
         *b.first = n->ws + o;
         o += (b.second + 255) / 256 * 256;
     }
-    // dynamic shared memory beyond the default limit
-    const int layer_sm = (int)fdlb::layer_smem(W), two = (int)(2 * fdlb::kChunks);
+    // dynamic shared memory beyond the default limit (a function's limit is the process's: the widest network's)
+    const int layer_sm = (int)fdlb::layer_smem(fdlb::kMaxWidth), two = (int)(2 * fdlb::kChunks);
     if (cudaFuncSetAttribute(fdlb::layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, layer_sm) != cudaSuccess ||
         cudaFuncSetAttribute(fdlb::layer_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, layer_sm) != cudaSuccess ||
         cudaFuncSetAttribute(fdlb::grad_spectral_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, two) != cudaSuccess) {
