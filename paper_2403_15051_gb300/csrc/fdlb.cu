@@ -42,6 +42,8 @@ struct Layout {
 
 }  // namespace
 
+constexpr int kWhole = 2;  // the whole work list among its ranges (Solver::Range)
+
 struct Solver {
     int n_inst = 0, geometry = 0, precision = 0;
     int reduced = 0;  // FDLB_CYL_Z: the cylinder's kernels on the pair (phi, chi) as the third index
@@ -92,21 +94,29 @@ struct Solver {
     int use_bulk = 0;
     int closure_cells = 4, closure_threads = 128;  // own cells per closure item (<= kClosureCells)
     int closure_batch = 0;  // the closure as two launches over all items (items of kClosureCells cells)
-    ClosureBatchShape cbatch{};
     int wall_parts = kWallParts;  // closure work items per wall
     int autotune_mode = 1;  // 0 off; 1 tune on the first step of a batch; 2 also of a single instance
     int stall_checks = 0;   // run_to_steady: checks without halving the best residual before an instance stops
     int stage_minb = 1;     // register bound of the stage kernel (1; 3, 2 or 5 blocks per SM where built)
     bool tuned = false;     // the tuner has run (or its cached choice was applied) for this handle
     int closure_wst = 0;                           // staged band-row elements per closure block
-    int grid_stream = 1, grid_closure = 1;
+    // Launch shapes for the ranges of the work lists: the two lanes (launch_steps) and the whole list.  The device
+    // holds each list's ranges as three pairs (first, end).
+    struct Range {
+        int grid_stream = 1, grid_closure = 1;
+        ClosureBatchShape cbatch{};
+    } range[3];
+    bool lanes_on = false;
+    cudaStream_t side = nullptr;  // the second lane's stream
+    cudaEvent_t fork = nullptr, join = nullptr;
+    bool joined = false;  // the last launches were the lanes'
     size_t closure_smem = 0;
     int max_union = 1;
     std::vector<char> active;
     std::vector<int64_t> inst_steps;
     std::vector<double> last_res;
     cudaGraphExec_t gexec = nullptr;
-    int64_t launches = 0, last_launches = 0;
+    int64_t launches = 0, last_launches = 0, graph_launches = 0;
     bool prev_valid = false;
     int graph_steps = 20;
     // per-kernel timing (events around each launch, direct launches)
@@ -294,7 +304,7 @@ Layout make_layout(const Solver& S) {
     L.mpk = take((size_t)S.total_cells * kNmom * sizeof(double));  // the moments query's rows
     L.bpairs = take((size_t)S.max_citems * sizeof(BandPair));   // the batch closure's band jobs
     L.k3f = take(S.geometry == FDLB_SPH ? S.f_elems * S.tsize : 0);  // sphere: K_3 f of the stage input
-    L.n_bpairs = take(sizeof(int));
+    L.n_bpairs = take(6 * sizeof(int));
     L.cw = take((size_t)S.total_cells * 2 * S.tsize);
     L.rec = take((size_t)S.total_cells * record_stride(S.nR, S.n2, S.n3) * S.tsize);
     L.tab = take(S.tab_h.size() * sizeof(double));
@@ -307,9 +317,9 @@ Layout make_layout(const Solver& S) {
     L.band = take(S.band_elems * S.tsize);
     L.band_lo = take((size_t)S.total_cells * 2 * sizeof(int));  // (first column, extent) per cell
     L.sitems = take((size_t)S.max_sitems * sizeof(int4));
-    L.n_sitems = take(sizeof(int));
+    L.n_sitems = take(6 * sizeof(int));
     L.citems = take((size_t)S.max_citems * sizeof(int4));
-    L.n_citems = take(sizeof(int));
+    L.n_citems = take(6 * sizeof(int));
     L.nwp = take((size_t)S.n_inst * 2 * kWallParts * S.tsize);
     L.err = take(sizeof(int));
     L.gbar = take(64);  // grid barrier counter of the persistent step kernel
@@ -485,15 +495,15 @@ void set_k2(const Solver& S, StageArgs& A) {
 }
 
 // The stage kernel of the current configuration: its launch, or with `blocks_per_sm` its occupancy.
-cudaError_t launch_stage_kernel(const Solver& S, const StageArgs& A, int grid, int* blocks_per_sm) {
+cudaError_t launch_stage_kernel(const Solver& S, const StageArgs& A, int grid, int* blocks_per_sm, cudaStream_t st) {
     const int threads = S.threads * S.teams;
     if (S.precision == FDLB_FP32)
         return S.geometry == FDLB_CYL
-                   ? launch_stream_float_0(S.scfg, A, S.M, grid, threads, S.smem_stream, S.stream, blocks_per_sm)
-                   : launch_stream_float_1(S.scfg, A, S.M, grid, threads, S.smem_stream, S.stream, blocks_per_sm);
+                   ? launch_stream_float_0(S.scfg, A, S.M, grid, threads, S.smem_stream, st, blocks_per_sm)
+                   : launch_stream_float_1(S.scfg, A, S.M, grid, threads, S.smem_stream, st, blocks_per_sm);
     return S.geometry == FDLB_CYL
-               ? launch_stream_double_0(S.scfg, A, S.M, grid, threads, S.smem_stream, S.stream, blocks_per_sm)
-               : launch_stream_double_1(S.scfg, A, S.M, grid, threads, S.smem_stream, S.stream, blocks_per_sm);
+               ? launch_stream_double_0(S.scfg, A, S.M, grid, threads, S.smem_stream, st, blocks_per_sm)
+               : launch_stream_double_1(S.scfg, A, S.M, grid, threads, S.smem_stream, st, blocks_per_sm);
 }
 
 // Whether the persistent step kernel runs the current configuration, and its launch shape: the
@@ -537,6 +547,24 @@ int upload_items(Solver& S) {
         if (S.active[q]) order.push_back(q);
     std::stable_sort(order.begin(), order.end(),
                      [&](int a, int b) { return S.setup[a].p.n_cells > S.setup[b].p.n_cells; });
+    // Two lanes of about equal cells, each from the largest instance to the smallest, for every batch whose stage
+    // stages whole tiles.  (The march's blocks stay for the whole launch, so that a lane's launch only queues behind
+    // the other's: 91.4 and 91.1 us per step on 256 instances of 64 cells, 365 and 363 on 48 in FP64)
+    S.lanes_on = order.size() > 1 && S.tiles && !S.fused && !S.krg_on && !S.k3_on;
+    size_t lane1 = order.size();  // the first instance of the second lane
+    if (S.lanes_on) {
+        std::vector<int> lane[2];
+        long long cells[2] = {0, 0};
+        for (int q : order) {
+            const int l = cells[1] < cells[0];
+            lane[l].push_back(q);
+            cells[l] += S.setup[q].p.n_cells;
+        }
+        lane1 = lane[0].size();
+        order = lane[0];
+        order.insert(order.end(), lane[1].begin(), lane[1].end());
+    }
+    int s1 = 0, k1 = 0, p1 = 0;  // the second lane's first stage item, closure item and band job
     std::vector<int4> si, ci;
     const int slices = S.n3 / S.KS;
     // batch form: items of 28 cells where there are warps enough (8 per SM), else of 12 (16 cells with
@@ -544,8 +572,12 @@ int upload_items(Solver& S) {
     long long act_cells = 0;
     for (int q : order) act_cells += S.setup[q].p.n_cells;
     const int batch_cells = act_cells >= 8LL * kClosureCells * S.n_sm ? kClosureCells : 12;
-    for (int q : order) {
-        const int N = S.setup[q].p.n_cells;
+    for (size_t o = 0; o < order.size(); ++o) {
+        const int q = order[o], N = S.setup[q].p.n_cells;
+        if (o == lane1) {
+            s1 = (int)si.size();
+            k1 = (int)ci.size();
+        }
         int nt = (N + S.B - 1) / S.B;
         if (S.n_inst == 1 && S.n_sm > 0) {
             // one instance: a multiple of the SM count of tiles (one or more full waves; every
@@ -579,6 +611,10 @@ int upload_items(Solver& S) {
             c += cnt;
         }
     }
+    if (lane1 >= order.size()) {
+        s1 = (int)si.size();
+        k1 = (int)ci.size();
+    }
     if ((int)si.size() > S.max_sitems || (int)ci.size() > S.max_citems) return FDLB_EINVAL;
     // the batch closure's band jobs: two band rows of an item at a time (instances with chi at the
     // local density have none), or a wall part; geometry only, so formed here once per work list
@@ -588,7 +624,9 @@ int upload_items(Solver& S) {
     for (int q = 0; q < S.n_inst; ++q) widest = std::max(widest, S.inst_h[q].chi_local ? 0 : S.setup[q].band.width);
     const bool inline_band = widest <= kInlineBandMax;
     if (S.closure_batch && !inline_band) {
-        for (const int4& w : ci) {
+        for (size_t e = 0; e < ci.size(); ++e) {
+            const int4 w = ci[e];
+            if ((int)e == k1) p1 = (int)bp.size();
             const InstanceSetup& I = S.setup[w.x];
             const InstDev& D = S.inst_h[w.x];
             if (w.w != 0) {
@@ -615,13 +653,16 @@ int upload_items(Solver& S) {
         if ((int)bp.size() > S.max_citems) return FDLB_EINVAL;
     }
     const int nbp = (int)bp.size();
+    if (k1 >= (int)ci.size()) p1 = nbp;
     if (nbp) FDLB_CUDA(cudaMemcpyAsync(S.bpairs, bp.data(), nbp * sizeof(BandPair), cudaMemcpyHostToDevice, S.stream));
-    FDLB_CUDA(cudaMemcpyAsync(S.n_bpairs, &nbp, sizeof(int), cudaMemcpyHostToDevice, S.stream));
     const int ns = (int)si.size(), nc = (int)ci.size();
     if (ns) FDLB_CUDA(cudaMemcpyAsync(S.sitems, si.data(), ns * sizeof(int4), cudaMemcpyHostToDevice, S.stream));
     if (nc) FDLB_CUDA(cudaMemcpyAsync(S.citems, ci.data(), nc * sizeof(int4), cudaMemcpyHostToDevice, S.stream));
-    FDLB_CUDA(cudaMemcpyAsync(S.n_sitems, &ns, sizeof(int), cudaMemcpyHostToDevice, S.stream));
-    FDLB_CUDA(cudaMemcpyAsync(S.n_citems, &nc, sizeof(int), cudaMemcpyHostToDevice, S.stream));
+    // (first, end) of the ranges: the lanes, the whole list
+    const int rs[6] = {0, s1, s1, ns, 0, ns}, rc[6] = {0, k1, k1, nc, 0, nc}, rp[6] = {0, p1, p1, nbp, 0, nbp};
+    FDLB_CUDA(cudaMemcpyAsync(S.n_sitems, rs, sizeof(rs), cudaMemcpyHostToDevice, S.stream));
+    FDLB_CUDA(cudaMemcpyAsync(S.n_citems, rc, sizeof(rc), cudaMemcpyHostToDevice, S.stream));
+    FDLB_CUDA(cudaMemcpyAsync(S.n_bpairs, rp, sizeof(rp), cudaMemcpyHostToDevice, S.stream));
     FDLB_CUDA(cudaStreamSynchronize(S.stream));  // host vectors go out of scope
     // closure shared memory: the tables and the union of the FM bands of one item's reach (the
     // closure kernel's items and, for the persistent step kernel, the tiles)
@@ -666,8 +707,12 @@ int upload_items(Solver& S) {
     wst = wst / 4 * 4;  // the tables behind the band rows start on a 16-byte boundary
     S.closure_wst = wst;
     S.closure_smem = closure_smem(S.nR, S.n2, S.n3, max_union, wst, (int)S.tsize);
-    S.grid_closure = std::max(1, std::min(nc, S.n_sm * (throughput ? closure_bps : 8)));
-    S.cbatch = closure_batch_shape((int)S.tsize, S.nR, S.n2, S.n3, nc, nbp, !inline_band ? 0 : widest <= 64 ? 2 : 4, S.n_sm);
+    for (int l = 0; l < 3; ++l) {
+        const int n_c = rc[2 * l + 1] - rc[2 * l], n_p = rp[2 * l + 1] - rp[2 * l];
+        S.range[l].grid_closure = std::max(1, std::min(n_c, S.n_sm * (throughput ? closure_bps : 8)));
+        S.range[l].cbatch =
+            closure_batch_shape((int)S.tsize, S.nR, S.n2, S.n3, n_c, n_p, !inline_band ? 0 : widest <= 64 ? 2 : 4, S.n_sm);
+    }
     // The stage: as many blocks as reside, each walking its items one after another with one copy of the
     // tables.  Generic kernels whose momentum set fits a warp walk an item per warp; up to eight warps share a
     // block, fewer where the items would otherwise leave SMs without one.
@@ -685,12 +730,15 @@ int upload_items(Solver& S) {
     int bps = 0;
     StageArgs A{};
     A.mma = S.mma_on;
-    if (launch_stage_kernel(S, A, 0, &bps) != cudaSuccess || bps < 1) {
+    if (launch_stage_kernel(S, A, 0, &bps, S.stream) != cudaSuccess || bps < 1) {
         cudaGetLastError();
         bps = 1;
     }
     // (tiles: a block each, placed as blocks finish; their tables cost less than an uneven share of tiles)
-    S.grid_stream = std::max(1, S.tiles ? ns : std::min((ns + S.teams - 1) / S.teams, bps * S.n_sm));
+    for (int l = 0; l < 3; ++l) {
+        const int n_s = rs[2 * l + 1] - rs[2 * l];
+        S.range[l].grid_stream = std::max(1, S.tiles ? n_s : std::min((n_s + S.teams - 1) / S.teams, bps * S.n_sm));
+    }
     return plan_step_kernel(S, ns);
 }
 
@@ -853,7 +901,7 @@ int launch_moments_all(Solver& S, int buf) {
     return cuda_status(cudaGetLastError());
 }
 
-int launch_closure_buf(Solver& S, int buf, int write_ca) {
+int launch_closure_buf(Solver& S, int buf, int write_ca, int lane, int programmatic) {
     ClosureArgs A{};
     A.sums = S.sums[buf];
     A.sumsw = S.sumsw[buf];
@@ -864,7 +912,7 @@ int launch_closure_buf(Solver& S, int buf, int write_ca) {
     A.rec_stride = record_stride(S.nR, S.n2, S.n3);
     A.nwp = S.nwp;
     A.items = S.citems;
-    A.n_items = S.n_citems;
+    A.n_items = S.n_citems + 2 * lane;
     A.inst = S.inst_d;
     A.band = S.band;
     A.band_lo = S.band_lo;
@@ -875,17 +923,19 @@ int launch_closure_buf(Solver& S, int buf, int write_ca) {
     A.wall_parts = S.wall_parts;
     A.wst_elems = S.closure_wst;
     A.err = S.err;
-    A.programmatic = S.programmatic;
+    A.programmatic = programmatic;
     A.pairs = S.bpairs;
-    A.n_pairs = S.n_bpairs;
+    A.n_pairs = S.n_bpairs + 2 * lane;
+    const Solver::Range& G = S.range[lane];
+    const cudaStream_t st = lane == 1 ? S.side : S.stream;
     if (S.closure_batch) {
-        FDLB_CUDA(S.precision == FDLB_FP32 ? launch_closure_batch<float>(A, S.M, S.cbatch, S.stream)
-                                           : launch_closure_batch<double>(A, S.M, S.cbatch, S.stream));
-        S.launches += S.cbatch.inline_band ? 1 : 2;
+        FDLB_CUDA(S.precision == FDLB_FP32 ? launch_closure_batch<float>(A, S.M, G.cbatch, st)
+                                           : launch_closure_batch<double>(A, S.M, G.cbatch, st));
+        S.launches += G.cbatch.inline_band ? 1 : 2;
     } else {
         FDLB_CUDA(S.precision == FDLB_FP32
-                      ? launch_closure<float>(A, S.M, S.grid_closure, S.closure_threads, S.closure_smem, S.stream)
-                      : launch_closure<double>(A, S.M, S.grid_closure, S.closure_threads, S.closure_smem, S.stream));
+                      ? launch_closure<float>(A, S.M, G.grid_closure, S.closure_threads, S.closure_smem, st)
+                      : launch_closure<double>(A, S.M, G.grid_closure, S.closure_threads, S.closure_smem, st));
         S.launches++;
     }
     if (write_ca) {
@@ -899,22 +949,22 @@ int launch_closure_buf(Solver& S, int buf, int write_ca) {
     return cuda_status(cudaGetLastError());
 }
 
-int launch_stream_only(Solver& S, int in, int fn, int out, double a, double b, int mode);
+int launch_stream_only(Solver& S, int in, int fn, int out, double a, double b, int mode, int lane, int programmatic);
 
 // K^h f of buffer `in` by the contraction kernel (large radial orders).
 int launch_kr_buf(Solver& S, int in) {
-    const int grid = std::max(1, std::min(S.grid_stream, S.n_sm * 8));
+    const int grid = std::max(1, std::min(S.range[kWhole].grid_stream, S.n_sm * 8));
     cudaError_t e;
     const float* isw = S.krB ? S.krB + kr_split_floats(S.nR) : nullptr;
     const float* sw = isw ? isw + S.nR : nullptr;
     if (S.kr_tc)
-        e = launch_kr_contract_tc((const float*)S.f[in], (float*)S.krf, S.sitems, S.n_sitems, S.inst_d, S.krB, isw, sw,
-                                  S.M, kr_npad(S.nR), S.err, std::max(1, std::min(S.grid_stream, S.n_sm)), S.stream);
+        e = launch_kr_contract_tc((const float*)S.f[in], (float*)S.krf, S.sitems, S.n_sitems + 2 * kWhole + 1, S.inst_d, S.krB, isw, sw,
+                                  S.M, kr_npad(S.nR), S.err, std::max(1, std::min(S.range[kWhole].grid_stream, S.n_sm)), S.stream);
     else if (S.precision == FDLB_FP32)  // the weight-scaled form, as the tensor-core kernel
-        e = launch_kr_contract<float>((const float*)S.f[in], (float*)S.krf, S.sitems, S.n_sitems, S.inst_d, sw + S.nR,
+        e = launch_kr_contract<float>((const float*)S.f[in], (float*)S.krf, S.sitems, S.n_sitems + 2 * kWhole + 1, S.inst_d, sw + S.nR,
                                       isw, sw, S.M, grid, S.stream);
     else
-        e = launch_kr_contract<double>((const double*)S.f[in], (double*)S.krf, S.sitems, S.n_sitems, S.inst_d,
+        e = launch_kr_contract<double>((const double*)S.f[in], (double*)S.krf, S.sitems, S.n_sitems + 2 * kWhole + 1, S.inst_d,
                                        (const double*)S.tabT + S.M.o_KR, nullptr, nullptr, S.M, grid, S.stream);
     S.launches++;
     return cuda_status(e);
@@ -922,13 +972,13 @@ int launch_kr_buf(Solver& S, int in) {
 
 // Sphere with momenta sliced along p_3: K_3 f of buffer `in` by its contraction kernel.
 int launch_k3_buf(Solver& S, int in) {
-    const int grid = std::max(1, std::min(S.grid_stream, S.n_sm * 8));
+    const int grid = std::max(1, std::min(S.range[kWhole].grid_stream, S.n_sm * 8));
     cudaError_t e;
     if (S.precision == FDLB_FP32)
-        e = launch_k3_contract<float>((const float*)S.f[in], (float*)S.k3f, S.sitems, S.n_sitems, S.inst_d,
+        e = launch_k3_contract<float>((const float*)S.f[in], (float*)S.k3f, S.sitems, S.n_sitems + 2 * kWhole + 1, S.inst_d,
                                       (const float*)S.tabT + S.M.o_K3, S.M, grid, S.stream);
     else
-        e = launch_k3_contract<double>((const double*)S.f[in], (double*)S.k3f, S.sitems, S.n_sitems, S.inst_d,
+        e = launch_k3_contract<double>((const double*)S.f[in], (double*)S.k3f, S.sitems, S.n_sitems + 2 * kWhole + 1, S.inst_d,
                                        (const double*)S.tabT + S.M.o_K3, S.M, grid, S.stream);
     S.launches++;
     return cuda_status(e);
@@ -947,10 +997,10 @@ int launch_stage(Solver& S, int in, int fn, int out, double a, double b, int mod
     }
     if (S.timing) {
         FDLB_CUDA(cudaEventRecord(S.tev[0], S.stream));
-        int rc = launch_closure_buf(S, in, write_ca);
+        int rc = launch_closure_buf(S, in, write_ca, kWhole, S.programmatic);
         if (rc) return rc;
         FDLB_CUDA(cudaEventRecord(S.tev[1], S.stream));
-        rc = launch_stream_only(S, in, fn, out, a, b, mode);
+        rc = launch_stream_only(S, in, fn, out, a, b, mode, kWhole, S.programmatic);
         if (rc) return rc;
         FDLB_CUDA(cudaEventRecord(S.tev[2], S.stream));
         FDLB_CUDA(cudaEventSynchronize(S.tev[2]));
@@ -963,12 +1013,15 @@ int launch_stage(Solver& S, int in, int fn, int out, double a, double b, int mod
         S.n_stream_t++;
         return FDLB_OK;
     }
-    int rc = launch_closure_buf(S, in, write_ca);
+    // (the first launch after the lanes' join follows an event, not a kernel)
+    const int first = S.joined ? 0 : S.programmatic;
+    S.joined = false;
+    int rc = launch_closure_buf(S, in, write_ca, kWhole, first);
     if (rc) return rc;
-    return launch_stream_only(S, in, fn, out, a, b, mode);
+    return launch_stream_only(S, in, fn, out, a, b, mode, kWhole, S.programmatic);
 }
 
-int launch_stream_only(Solver& S, int in, int fn, int out, double a, double b, int mode) {
+int launch_stream_only(Solver& S, int in, int fn, int out, double a, double b, int mode, int lane, int programmatic) {
     StageArgs A{};
     A.f_in = S.f[in];
     A.f_n = S.f[fn];
@@ -981,7 +1034,7 @@ int launch_stream_only(Solver& S, int in, int fn, int out, double a, double b, i
     A.sumsw_out = S.sumsw[out];
     A.dens_out = S.dens[out];
     A.items = S.sitems;
-    A.n_items = S.n_sitems;
+    A.n_items = S.n_sitems + 2 * lane;
     A.inst = S.inst_d;
     A.tab = S.tab;
     A.tabT = S.tabT;
@@ -998,12 +1051,12 @@ int launch_stream_only(Solver& S, int in, int fn, int out, double a, double b, i
     A.teams = S.teams;
     set_k2(S, A);
     A.use_bulk = S.use_bulk;
-    A.programmatic = S.programmatic;
+    A.programmatic = programmatic;
     A.mma = S.mma_on;
     A.tx_extra = S.test_tx_extra;
     A.krf = S.krg_on ? S.krf : nullptr;
     A.k3f = S.k3_on ? S.k3f : nullptr;
-    const cudaError_t e = launch_stage_kernel(S, A, S.grid_stream, nullptr);
+    const cudaError_t e = launch_stage_kernel(S, A, S.range[lane].grid_stream, nullptr, lane == 1 ? S.side : S.stream);
     S.launches++;
     return cuda_status(e);
 }
@@ -1014,6 +1067,40 @@ int launch_step(Solver& S) {
     int rc = launch_stage(S, 0, 0, 1, 0.0, 1.0, 0);
     if (!rc) rc = launch_stage(S, 1, 0, 2, 0.75, 0.25, 0);
     if (!rc) rc = launch_stage(S, 2, 0, 0, 1.0 / 3.0, 2.0 / 3.0, 0);
+    return rc;
+}
+
+// n steps.  In a batch with lanes (upload_items) the two halves of the instances, which never meet, have a chain of
+// launches each, on S.stream and on S.side: the closure of one, bound by latency, and the last, uneven wave of its
+// stage's tiles run beside the stage of the other.  Per step, one chain and two: 251 and 223 us (12 instances of
+// 128 to 2048 cells, 16 x 8 x 8), 2510 and 2375 (128 of them), 64.5 and 62.7 (3 of 64 to 1024), 27.6 and 27.4
+// (2 of 64).
+int launch_steps(Solver& S, int64_t n) {
+    if (n < 1) return FDLB_OK;
+    int rc = FDLB_OK;
+    if (!S.lanes_on || S.timing) {
+        for (int64_t s = 0; s < n && !rc; ++s) rc = launch_step(S);
+        return rc;
+    }
+    if (!S.side) {
+        FDLB_CUDA(cudaEventCreateWithFlags(&S.fork, cudaEventDisableTiming));
+        FDLB_CUDA(cudaEventCreateWithFlags(&S.join, cudaEventDisableTiming));
+        FDLB_CUDA(cudaStreamCreateWithFlags(&S.side, cudaStreamNonBlocking));
+    }
+    FDLB_CUDA(cudaEventRecord(S.fork, S.stream));
+    FDLB_CUDA(cudaStreamWaitEvent(S.side, S.fork, 0));
+    for (int64_t s = 0; s < 3 * n && !rc; ++s) {
+        const int k = (int)(s % 3), in = k, out = k == 2 ? 0 : k + 1;
+        const double a = k == 0 ? 0.0 : k == 1 ? 0.75 : 1.0 / 3.0, b = k == 0 ? 1.0 : k == 1 ? 0.25 : 2.0 / 3.0;
+        // (a lane's first launch follows an event, not a kernel)
+        for (int l = 0; l < 2 && !rc; ++l) {
+            rc = launch_closure_buf(S, in, 0, l, s ? S.programmatic : 0);
+            if (!rc) rc = launch_stream_only(S, in, 0, out, a, b, 0, l, S.programmatic);
+        }
+    }
+    FDLB_CUDA(cudaEventRecord(S.join, S.side));
+    FDLB_CUDA(cudaStreamWaitEvent(S.stream, S.join, 0));
+    S.joined = true;
     return rc;
 }
 
@@ -1094,7 +1181,8 @@ int ensure_graph(Solver& S) {
     const int64_t before = S.launches;
     FDLB_CUDA(cudaStreamBeginCapture(S.stream, cudaStreamCaptureModeThreadLocal));
     int rc = FDLB_OK;
-    for (int s = 0; s < S.graph_steps && !rc; ++s) rc = launch_step(S);
+    rc = launch_steps(S, S.graph_steps);
+    S.graph_launches = S.launches - before;
     cudaError_t e = cudaStreamEndCapture(S.stream, &graph);
     S.launches = before;
     if (rc) {
@@ -1116,7 +1204,7 @@ int launch_steps_fused(Solver& S, int64_t n) {
     A.nwp = S.nwp;
     A.wall_parts = S.wall_parts;
     A.items = S.sitems;
-    A.n_items = S.n_sitems;
+    A.n_items = S.n_sitems + 2 * kWhole;
     A.inst = S.inst_d;
     A.tab = S.tab;
     A.tabT = S.tabT;
@@ -1136,7 +1224,7 @@ int launch_steps_fused(Solver& S, int64_t n) {
     C.rec_stride = A.rec_stride;
     C.nwp = S.nwp;
     C.items = S.sitems;
-    C.n_items = S.n_sitems;
+    C.n_items = S.n_sitems + 2 * kWhole;
     C.inst = S.inst_d;
     C.band = S.band;
     C.band_lo = S.band_lo;
@@ -1334,14 +1422,11 @@ int do_steps(Solver& S, int64_t n) {
         if (rc) return rc;
         while (n - done >= S.graph_steps) {
             FDLB_CUDA(cudaGraphLaunch(S.gexec, S.stream));
-            S.launches += (int64_t)S.graph_steps * 3 * ((S.krg_on ? 1 : 0) + (S.k3_on ? 1 : 0) + (S.closure_batch && !S.cbatch.inline_band ? 2 : 1) + 1);
+            S.launches += S.graph_launches;
             done += S.graph_steps;
         }
     }
-    for (; done < n; ++done) {
-        int rc = launch_step(S);
-        if (rc) return rc;
-    }
+    if (const int rc = launch_steps(S, n - done)) return rc;
     for (int q = 0; q < S.n_inst; ++q)
         if (S.active[q]) S.inst_steps[q] += n;
     S.last_launches = S.launches - before;
@@ -1569,6 +1654,9 @@ void fdlb_destroy(fdlb_handle h) {
     if (S->own_ws && S->ws) cudaFree(S->ws);
     for (cudaEvent_t e : S->tev)
         if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : {S->fork, S->join})
+        if (e) cudaEventDestroy(e);
+    if (S->side) cudaStreamDestroy(S->side);
     if (S->own_stream) cudaStreamDestroy(S->stream);
     delete S;
 }

@@ -77,7 +77,7 @@ struct StageArgs {
     void* sumsw_out;               // the same as double-float pairs (FP32 populations), [cell][slice][13]
     void* dens_out;                // per-slice densities of f_out (T), [cell][slice]
     const int4* items;             // (instance, first cell, cells, slice)
-    const int* n_items;
+    const int* n_items;            // (first, end) of the launch's items
     const InstDev* inst;
     const double* tab;
     const void* tabT;              // the same tables in T
@@ -124,7 +124,7 @@ struct ClosureArgs {
     int rec_stride;
     void* nwp;                     // [instance][2][kWallParts] outgoing wall fluxes (T)
     const int4* items;             // (instance, first cell, cells, 0) or (instance, -, part, 1 + side)
-    const int* n_items;
+    const int* n_items;            // (first, end) of the launch's items
     const InstDev* inst;
     const void* band;              // FM band values (T)
     const int* band_lo;            // per global cell: first column, stored extent
@@ -137,7 +137,7 @@ struct ClosureArgs {
     int programmatic;              // launched with programmatic stream serialization
     int* err;                      // set when a bulk copy never completes
     const BandPair* pairs;         // batch form: the band kernel's jobs
-    const int* n_pairs;
+    const int* n_pairs;            // (first, end) of the launch's jobs
 };
 
 struct StepArgs {

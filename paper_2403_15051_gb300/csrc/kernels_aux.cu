@@ -132,8 +132,8 @@ __global__ void __launch_bounds__(kClosureThreads) closure_kernel(ClosureArgs A,
     T* rec_all = reinterpret_cast<T*>(A.rec);
     T* nwp = reinterpret_cast<T*>(A.nwp);
     uint32_t phase = 0;
-    const int nit = *A.n_items;
-    for (int it = blockIdx.x; it < nit; it += gridDim.x) {
+    const int nit = A.n_items[1];
+    for (int it = A.n_items[0] + blockIdx.x; it < nit; it += gridDim.x) {
         const int4 w = A.items[it];
         const InstDev I = A.inst[w.x];
         if (w.w != 0) {
@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(kClosureThreads, sizeof(T) == 4 ? 8 : 4) closu
     T* nwp = reinterpret_cast<T*>(A.nwp);
     T* cw = reinterpret_cast<T*>(A.cw);
     const int slices = A.slices;
-    const int np = *A.n_pairs;
-    const int gw = blockIdx.x * kClosureWarps + warp, nw = gridDim.x * kClosureWarps;
+    const int np = A.n_pairs[1];
+    const int gw = A.n_pairs[0] + blockIdx.x * kClosureWarps + warp, nw = gridDim.x * kClosureWarps;
     for (int v = gw; v < np; v += nw) {
         const BandPair P = A.pairs[v];
         if (P.kmaxA < 0) {
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kClosureThreads, sizeof(T) == 4 ? 4 : 2) closu
     T* rec_all = reinterpret_cast<T*>(A.rec);
     const int rs = A.rec_stride, slices = A.slices;
     const ReachView<T> RV{R.n, R.Tc, {R.u[0], R.u[1], R.u[2]}, R.nb};
-    const int nit = *A.n_items, nw = gridDim.x * wpb;
+    const int nit = A.n_items[1], nw = gridDim.x * wpb;
     __syncthreads();
     bool waited = false;
     auto wait = [&]() {
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kClosureThreads, sizeof(T) == 4 ? 4 : 2) closu
             waited = true;
         }
     };
-    for (int it = blockIdx.x * wpb + warp; it < nit; it += nw) {
+    for (int it = A.n_items[0] + blockIdx.x * wpb + warp; it < nit; it += nw) {
         const int4 w = A.items[it];
         if (!kBand && w.w != 0) continue;  // wall items: closure_band_kernel
         const InstDev I = A.inst[w.x];
@@ -572,7 +572,9 @@ template <typename T>
 cudaError_t launch_closure_batch(const ClosureArgs& A, const MomSet& M, const ClosureBatchShape& B, cudaStream_t s) {
     auto rec = closure_records<T>(B.inline_band);
     const size_t smem = closure_records_smem(M.nR, M.n2, M.n3, B.warps, (int)sizeof(T));
-    cudaError_t e = cudaFuncSetAttribute(rec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the limit is the function's: that of the largest block, whichever the launch)
+    cudaError_t e = cudaFuncSetAttribute(rec, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)closure_records_smem(M.nR, M.n2, M.n3, kClosureWarps, (int)sizeof(T)));
     if (e == cudaSuccess && !B.inline_band)
         e = launch_maybe_programmatic(closure_band_kernel<T>, B.grid_band, kClosureThreads,
                                       closure_smem_bytes(M.nR, M.n2, M.n3, 0, 0, (int)sizeof(T)), s, A.programmatic, A, M);

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(stage_max_threads<T, VW, 1>(), 1) step_kernel(
 
     uint32_t sphase = 0, cphase = 0;
     unsigned nbar = 0;
-    const int nit = *S.st.n_items, WP = S.cl.wall_parts;
+    const int nit = S.st.n_items[1], WP = S.cl.wall_parts;
     for (int step = 0; step < S.n_steps; ++step) {
         for (int stage = 0; stage < 3; ++stage) {
             // f1 = f + dt L(f); f2 = 3/4 f + 1/4 (f1 + dt L(f1)); f^{n+1} = 1/3 f + 2/3 (f2 + dt L(f2))

@@ -840,8 +840,8 @@ __device__ __forceinline__ void march_body(const StageArgs& A, const MomSet& M) 
     const StagePtrs<T> S = march_ptrs<T, GEOM, VW, NV, NR_, N2_, N3_>(smem_raw, A, M);
     const int G = A.G, R = march_ring(G);
     stage_tables<T, GEOM, VW, NV, NR_, N2_, N3_>(S, A, M);
-    const int nit = *A.n_items, teams = warps_apart ? A.teams : 1;
-    const int it0 = blockIdx.x * teams + (warps_apart ? (int)threadIdx.x >> 5 : 0);
+    const int nit = A.n_items[1], teams = warps_apart ? A.teams : 1;
+    const int it0 = A.n_items[0] + blockIdx.x * teams + (warps_apart ? (int)threadIdx.x >> 5 : 0);
     __syncthreads();
     // An item's first request: rows c0-3 .. c0+G+2, the records and f_n of its first group.  The rows of the
     // first item are requested before the wait: they are the output of the stage kernel two launches
@@ -1068,21 +1068,21 @@ __device__ __forceinline__ void tile_body(const StageArgs& A, const MomSet& M) {
     StagePtrs<T> S = tile_ptrs<T, GEOM, VW, NV, NR_, N2_, N3_>(smem_raw, A, M);
     S.nw = snw;
     stage_tables<T, GEOM, VW, NV, NR_, N2_, N3_>(S, A, M);
-    const int nit = *A.n_items;
+    const int it0 = A.n_items[0] + blockIdx.x, nit = A.n_items[1];
     __syncthreads();
     // (the first tile's rows before the wait, as in march_body)
-    const bool early = A.use_bulk && (int)blockIdx.x < nit;
+    const bool early = A.use_bulk && it0 < nit;
     if (early) {
-        const int4 wi = A.items[blockIdx.x];
+        const int4 wi = A.items[it0];
         tile_request<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi, A.inst[wi.x], true, 1, A, M);
     }
     pdl_trigger();
     pdl_wait();  // everything below reads what the previous kernels wrote
     uint32_t phase = 0;
-    for (int it = blockIdx.x; it < nit; it += gridDim.x) {
+    for (int it = it0; it < nit; it += gridDim.x) {
         const int4 wi = A.items[it];
         const InstDev I = A.inst[wi.x];
-        tile_request<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi, I, true, early && it == (int)blockIdx.x ? 2 : 3, A, M);
+        tile_request<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi, I, true, early && it == it0 ? 2 : 3, A, M);
         // (here, where they overlap the copy: before the wait they cost the tile kernels 4%)
         tile_geometry<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi, I, A, M);
         stage_maxwellians<T, GEOM, VW, NV, NR_, N2_, N3_>(S, wi.x, A, M);
