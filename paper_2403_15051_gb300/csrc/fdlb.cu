@@ -790,12 +790,15 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
             cfg.vw /= 2;
             spread = true;
         }
-    // rows of eight per thread over many cells, as for the compile-time shape below
-    const bool rows8 = S.tsize == 4 && S.n2 == 8 && Ms / 8 <= 512 && (long long)S.total_cells * S.Np > (long long)S.n_sm * 65536;
+    const int cap = threads > 0 ? threads : 256;
+    // rows of eight per thread over many cells, as for the compile-time shape below, and where a block of four
+    // momenta per thread would hold two vectors each: the same threads, half the instructions beside the arithmetic
+    // (40 x 8 x 8 on 240 cells: 22.2 and 20.5 us)
+    const bool rows8 = S.tsize == 4 && S.n2 == 8 && Ms / 8 <= 512 &&
+                       ((long long)S.total_cells * S.Np > (long long)S.n_sm * 65536 || Ms / 4 > cap);
     cfg.spec = ((S.geometry == FDLB_CYL && S.nR == 16 && S.n2 == 8 && S.n3 == 8) ||
                 (S.geometry == FDLB_SPH && S.nR == 24 && S.n2 == 12 && S.n3 == 12)) &&
                cfg.vw == (S.tsize == 4 || S.geometry == FDLB_CYL ? 4 : 2);
-    const int cap = threads > 0 ? threads : 256;
     // the cylinder's FP32 shape in blocks of at most 128 threads: a thread per whole p_2 row (8
     // momenta; per-vector and per-cell work spread over twice the momenta, half the warps per cell)
     if (cfg.spec && S.tsize == 4 && S.geometry == FDLB_CYL && cap <= 128 && Ms / 8 <= 128) cfg.vw = 8;

@@ -1,7 +1,7 @@
 """The stage kernel's walk along the radius at the sizes where its ring of rows, its groups of cells and
 its teams change: the smallest instances, items of one cell (fewer cells than SMs), of two, of an odd count
 and of the whole instance, items that start one or two cells from a wall; momentum sets of one warp (one
-vector or two per thread), of a whole block, and whose rows the bulk engine cannot copy (plain loads).
+vector or two per thread), of a whole block (in FP32 also rows of eight per thread), and whose rows the bulk engine cannot copy (plain loads).
 A cell's results do not depend on its item, so every tiling steps bit for bit alike; one of them is
 compared with the oracle (the tolerances of the parity tests)."""
 import numpy as np
@@ -25,7 +25,7 @@ def _built():
 
 
 SETS = [(wl.CYL, (4, 4, 4)), (wl.SPH, (4, 4, 4)), (wl.CYL, (4, 4, 8)), (wl.CYL, (3, 5, 3)), (wl.SPH, (5, 6, 4)),
-        (wl.CYL, (8, 8, 8)), (wl.CYL, (1, 1, 1))]
+        (wl.CYL, (8, 8, 8)), (wl.CYL, (9, 8, 8)), (wl.CYL, (1, 1, 1))]
 
 
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
