@@ -1085,11 +1085,6 @@ int launch_steps(Solver& S, int64_t n) {
         for (int64_t s = 0; s < n && !rc; ++s) rc = launch_step(S);
         return rc;
     }
-    if (!S.side) {
-        FDLB_CUDA(cudaEventCreateWithFlags(&S.fork, cudaEventDisableTiming));
-        FDLB_CUDA(cudaEventCreateWithFlags(&S.join, cudaEventDisableTiming));
-        FDLB_CUDA(cudaStreamCreateWithFlags(&S.side, cudaStreamNonBlocking));
-    }
     FDLB_CUDA(cudaEventRecord(S.fork, S.stream));
     FDLB_CUDA(cudaStreamWaitEvent(S.side, S.fork, 0));
     for (int64_t s = 0; s < 3 * n && !rc; ++s) {
@@ -1599,8 +1594,16 @@ int solver_create(const fdlb_params* ps, int n, void* stream, void* workspace, s
     R.closure_batch = R.total_cells / kClosureCells > R.n_sm * 4 ? 1 : 0;
     if (!rc) rc = upload_items(R);
     for (int q = 0; q < n && !rc; ++q) rc = fdlb_init_uniform(reinterpret_cast<fdlb_handle>(S.get()), q, 0.0, 0.0);
+    if (!rc && n > 1 &&
+        (cudaStreamCreateWithFlags(&R.side, cudaStreamNonBlocking) != cudaSuccess ||
+         cudaEventCreateWithFlags(&R.fork, cudaEventDisableTiming) != cudaSuccess ||
+         cudaEventCreateWithFlags(&R.join, cudaEventDisableTiming) != cudaSuccess))
+        rc = FDLB_ECUDA;
     if (rc) {
         if (R.own_ws) cudaFree(R.ws);
+        for (cudaEvent_t e : {R.fork, R.join})
+            if (e) cudaEventDestroy(e);
+        if (R.side) cudaStreamDestroy(R.side);
         if (R.own_stream) cudaStreamDestroy(R.stream);
         return rc;
     }
