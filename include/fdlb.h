@@ -291,7 +291,9 @@ int fdlb_set_stage_min_blocks(fdlb_handle h, int min_blocks, int* in_use);
  * TF32 products with FP32 accumulation, FP32-level accuracy) with mma.sync m16n8k8, for FP32
  * populations on the 16 x 8 x 8 and 24 x 12 x 12 quadratures; elsewhere the CUDA-core path
  * stays.  *in_use (may be NULL) tells whether it applies to this handle.  On GB300 these
- * contractions are too small to pay for the splitting: the default is the CUDA-core path. */
+ * contractions are too small to pay for the splitting: the default is the CUDA-core path.
+ * For 2Q_R >= 32 radial nodes it selects the contraction kernel of its own (FP32: on the tensor
+ * cores), the default from 2Q_R = 50 on; below, the stage contracts from shared memory. */
 int fdlb_set_tensor_contraction(fdlb_handle h, int enable, int* in_use);
 
 /* Whole SSP-RK3 steps in one persistent launch (default off): each block owns tiles of cells
@@ -335,11 +337,11 @@ int fdlb_set_closure_cells(fdlb_handle h, int cells);
 
 /* Form of the closure (Eqs. fm, chi, j1, tau, prandtl and the equilibria of Sec. III.C, once per
  * stage).  form 0, the chain: one launch, each block runs an item of a few cells through the whole
- * closure (short, latency-bound: one instance).  form 1, the batch form: two launches over items
- * of 28 cells, the first giving every FM band row a warp of its own (the band sum, chi), the
- * second forming the records of each item from the raw sums of its reach and the band results
- * (throughput-bound: batches and long instances; the default when the items of 28 cells are more
- * than four times the SM count).  The records are the same bit for bit either way.
+ * closure (short, latency-bound: one instance).  form 1, the batch form: a warp takes an item of 28
+ * cells (of 12 where there are fewer than eight such items per SM) from the raw sums of its reach to
+ * the records; bands of up to 128 columns are summed in the same launch, wider ones in a launch before
+ * it that gives every pair of band rows a warp (batches and long instances; the default when the
+ * items of 28 cells are more than four times the SM count).  The records are the same bit for bit either way.
  * form -1 changes nothing.  *in_use (may be NULL) = the form in use.  FDLB_EINVAL for another
  * form. */
 int fdlb_set_closure_form(fdlb_handle h, int form, int* in_use);
