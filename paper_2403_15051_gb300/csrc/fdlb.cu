@@ -1073,33 +1073,37 @@ int launch_step(Solver& S) {
     return rc;
 }
 
-// n steps.  In a batch with lanes (upload_items) the two halves of the instances, which never meet, have a chain of
-// launches each, on S.stream and on S.side: the closure of one, bound by latency, and the last, uneven wave of its
-// stage's tiles run beside the stage of the other.  Per step, one chain and two: 251 and 223 us (12 instances of
-// 128 to 2048 cells, 16 x 8 x 8), 2510 and 2375 (128 of them), 64.5 and 62.7 (3 of 64 to 1024), 27.6 and 27.4
-// (2 of 64).
-int launch_steps(Solver& S, int64_t n) {
-    if (n < 1) return FDLB_OK;
+// n stages on the two lanes of a batch (upload_items), stage(s, lane, programmatic) launching one.  The two halves
+// of the instances, which never meet, have a chain of launches each, on S.stream and on S.side: the closure of one,
+// bound by latency, and the last, uneven wave of its stage's tiles run beside the stage of the other.  Per step, one
+// chain and two: 251 and 220 us (12 instances of 128 to 2048 cells, 16 x 8 x 8), 2510 and 2375 (128 of them), 102
+// and 91 (8 of 64 to 1024), 64.5 and 57.3 (3 of them), 28 and 28 (2 of 64).
+template <typename F>
+int on_lanes(Solver& S, int64_t n, const F& stage) {
     int rc = FDLB_OK;
-    if (!S.lanes_on || S.timing) {
-        for (int64_t s = 0; s < n && !rc; ++s) rc = launch_step(S);
-        return rc;
-    }
     FDLB_CUDA(cudaEventRecord(S.fork, S.stream));
     FDLB_CUDA(cudaStreamWaitEvent(S.side, S.fork, 0));
-    for (int64_t s = 0; s < 3 * n && !rc; ++s) {
-        const int k = (int)(s % 3), in = k, out = k == 2 ? 0 : k + 1;
-        const double a = k == 0 ? 0.0 : k == 1 ? 0.75 : 1.0 / 3.0, b = k == 0 ? 1.0 : k == 1 ? 0.25 : 2.0 / 3.0;
-        // (a lane's first launch follows an event, not a kernel)
-        for (int l = 0; l < 2 && !rc; ++l) {
-            rc = launch_closure_buf(S, in, 0, l, s ? S.programmatic : 0);
-            if (!rc) rc = launch_stream_only(S, in, 0, out, a, b, 0, l, S.programmatic);
-        }
-    }
+    for (int64_t s = 0; s < n && !rc; ++s)  // (a lane's first launch follows an event, not a kernel)
+        for (int l = 0; l < 2 && !rc; ++l) rc = stage(s, l, s ? S.programmatic : 0);
     FDLB_CUDA(cudaEventRecord(S.join, S.side));
     FDLB_CUDA(cudaStreamWaitEvent(S.stream, S.join, 0));
     S.joined = true;
     return rc;
+}
+
+int launch_steps(Solver& S, int64_t n) {
+    if (n < 1) return FDLB_OK;
+    if (!S.lanes_on || S.timing) {
+        int rc = FDLB_OK;
+        for (int64_t s = 0; s < n && !rc; ++s) rc = launch_step(S);
+        return rc;
+    }
+    return on_lanes(S, 3 * n, [&](int64_t s, int l, int programmatic) {
+        const int k = (int)(s % 3), in = k, out = k == 2 ? 0 : k + 1;
+        const double a = k == 0 ? 0.0 : k == 1 ? 0.75 : 1.0 / 3.0, b = k == 0 ? 1.0 : k == 1 ? 0.25 : 2.0 / 3.0;
+        const int rc = launch_closure_buf(S, in, 0, l, programmatic);
+        return rc ? rc : launch_stream_only(S, in, 0, out, a, b, 0, l, S.programmatic);
+    });
 }
 
 int upload_state(Solver& S, int q, const double* f_host) {
@@ -1265,7 +1269,7 @@ int launch_steps_fused(Solver& S, int64_t n) {
 // knobs that regroup cells without changing any cell's arithmetic (the per-cell results and the
 // order of every sum stay those of the default, so tuning changes no result bit); the block size
 // and the momentum slicing, which do reorder the sums, stay as configured.  Each candidate is
-// timed over three stages (closure + fused stage, the second RK stage's form, written to the
+// timed over three stages (closure + fused stage, on the lanes where the steps run there, the second RK stage's form, written to the
 // stage-1 buffers, which every step overwrites before reading) after one warm-up stage; B is
 // tuned first at the current closure grouping, then the closure grouping at the best B.  The
 // choice is cached per process for the momentum set, precision, block size, slicing and the
@@ -1309,10 +1313,19 @@ int set_closure_grouping(Solver& S, int cells, int batch = -1) {
 
 // Time of three stages of the current tiling (ms), or a negative value if a launch failed.
 float time_stages(Solver& S, cudaEvent_t e0, cudaEvent_t e1) {
-    if (launch_stage(S, 0, 0, 1, 0.75, 0.25, 0) != FDLB_OK) return -1.f;
+    auto stages = [&](int n) {
+        if (S.lanes_on)
+            return on_lanes(S, n, [&](int64_t, int l, int programmatic) {
+                const int rc = launch_closure_buf(S, 0, 0, l, programmatic);
+                return rc ? rc : launch_stream_only(S, 0, 0, 1, 0.75, 0.25, 0, l, S.programmatic);
+            });
+        int rc = FDLB_OK;
+        for (int r = 0; r < n && !rc; ++r) rc = launch_stage(S, 0, 0, 1, 0.75, 0.25, 0);
+        return rc;
+    };
+    if (stages(1) != FDLB_OK) return -1.f;
     cudaEventRecord(e0, S.stream);
-    for (int r = 0; r < 3; ++r)
-        if (launch_stage(S, 0, 0, 1, 0.75, 0.25, 0) != FDLB_OK) return -1.f;
+    if (stages(3) != FDLB_OK) return -1.f;
     cudaEventRecord(e1, S.stream);
     if (cudaEventSynchronize(e1) != cudaSuccess) return -1.f;
     float ms = 0.f;
