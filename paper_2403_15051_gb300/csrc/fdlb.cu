@@ -591,6 +591,11 @@ int upload_items(Solver& S) {
             // fewer cells than SMs: one to a tile (each computes both its faces, half as much again, on
             // twice the SMs: the FP64 stage of 64 cells x 128 momenta took 48.8 us in tiles of four)
             if (!S.fused && !S.tiles && N * slices <= S.n_sm && N * slices <= S.max_sitems) nt = N;
+            // the march's blocks share an SM: items of two cells up to 16 warps per SM (per step, items of four and
+            // two: 256 momenta by two warps on 499 cells 43.8 and 33.6 us, 1000 54.4 and 42.4; 1000 momenta by eight
+            // warps on 499 cells 52.5 and 45.4, but on 1000, beyond the line, 59.5 and 72.0)
+            else if (!S.fused && !S.tiles && nt < (N + 1) / 2 && (N + 1LL) / 2 * slices * (S.threads / 32) <= 16LL * S.n_sm)
+                nt = (N + 1) / 2;
         }
         const int base = N / nt, rem = N % nt;
         int c0 = 0;
@@ -821,6 +826,11 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
         // the most a thread holds; fewer when the block has room, except that two vectors per thread
         // keep up to 64 of them in one warp
         cfg.nv = cfg.vw == 4 ? (S.tsize == 4 && Vs > 32 ? 2 : 1) : spread ? 1 : 4;
+        // (over few cells the second warp is free: 256 momenta on 499 cells 62.2 us per step by one warp, 43.8 by two)
+        if (cfg.nv == 2 && Vs <= 64 && 2LL * S.total_cells <= 16LL * S.n_sm) {
+            cfg.nv = 1;
+            spread = true;
+        }
         nt = spread ? (Vs + 31) / 32 * 32 : Vs <= 32 * cfg.nv ? 32 : (std::min(Vs, cap) + 31) / 32 * 32;
         if ((long long)nt * cfg.nv < Vs) nt = ((Vs + cfg.nv - 1) / cfg.nv + 31) / 32 * 32;
     }

@@ -55,9 +55,11 @@ def test_items_of_every_size_agree_and_match_oracle(n_cells, geom, Q, precision)
             assert np.all(np.isfinite(f)) and np.array_equal(f, ref), cells
 
 
-def test_many_items_share_blocks():
-    # more items than SMs: several warps of a block walk items of their own, blocks take several items
-    ds = [small_case(precision="fp32", n_cells=n, R=(1.0, 2.0 + 0.01 * q)) for q, n in enumerate([64, 33, 50] * 40)]
+@pytest.mark.parametrize("Q", [(4, 4, 4), (4, 4, 8)])
+def test_many_items_share_blocks(Q):
+    # more items than SMs: several warps of a block walk items of their own, blocks take several items; a thread of
+    # one vector, and of two (256 momenta over many cells)
+    ds = [small_case(precision="fp32", n_cells=n, Q=Q, R=(1.0, 2.0 + 0.01 * q)) for q, n in enumerate([64, 33, 50] * 40)]
     out = []
     for cells in (2, 7, 64):
         with fdlb.Solver(ds) as S:
