@@ -395,15 +395,45 @@ struct ReachView {
     const T* nb;
 };
 
+// Whether one of four values is below -1/8, on the bits: negative values order like their bit patterns, above
+// the positive ones (an FP64 comparison would be another dependent FP64 operation).  A NaN may fall on either side.
+__device__ __forceinline__ bool steep_drop(float a, float b, float c, float d) {
+    return max(max(__float_as_uint(a), __float_as_uint(b)), max(__float_as_uint(c), __float_as_uint(d))) > 0xBE000000u;
+}
+__device__ __forceinline__ bool steep_drop(double a, double b, double c, double d) {
+    return max(max((unsigned)__double2hiint(a), (unsigned)__double2hiint(b)),
+               max((unsigned)__double2hiint(c), (unsigned)__double2hiint(d))) >= 0xBFC00000u;
+}
+
+// ln(n'^2 chi' T') - ln(n^2 chi T) factor by factor, each logarithm as that of a rise (beside the code of the usual
+// case, whose instructions a short launch fetches cold).  n1, T1: the second cell's; dn, dT, deta: the differences.
+template <typename T>
+__device__ __noinline__ T clo_steep_log(T n0, T n1, T dn, T T0, T T1, T dT, T eta, T deta) {
+    T sum = T(0);
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        // n and 1 / (1 - eta) enter with their powers, T and 2 - eta once
+        const T p = k == 0 ? n0 : k == 1 ? T0 : k == 2 ? T(2) - eta : T(1) - eta;
+        const T s = k == 0 ? n1 : k == 1 ? T1 : p - deta;
+        const T dv = k == 0 ? dn : k == 1 ? dT : -deta;
+        const T r = dv < T(0) ? log1p(ratio_fast(-dv, s)) : -log1p(ratio_fast(dv, p));  // ln(p / s)
+        sum = fma(k == 0 ? T(-2) : k == 3 ? T(3) : T(-1), r, sum);
+    }
+    return sum;
+}
+
 // The terms of the J1 gradients (Eq. j1) of the neighbouring reach cells lt and lt + 1: the
 // differences of ln(n^2 chi T), ln T and the three velocities.  A derivative stencil is a weighted sum
 // of four such differences (stencil5_pairs), so each is formed once per pair of cells instead of once
 // per cell and stencil position, with two logarithms instead of four: the ratio of n^2 chi T is the
 // product of 1 + x over the factors' relative differences, and its deviation from one is carried as
-// E <- E + x + E x (every factor is formed from a difference of the wide values, so nothing cancels);
-// ln chi(eta) = ln(2 - eta) - ln 2 - 3 ln(1 - eta) from the packing-fraction difference alone (no
-// rounding noise of chi itself).  The gradients of two cells' closure in FP64 took 20800 cycles with
-// twenty logarithms per cell, a third of the whole chain in FP32.
+// E <- E + x + E x; ln chi(eta) = ln(2 - eta) - ln 2 - 3 ln(1 - eta) from the packing-fraction difference
+// alone (no rounding noise of chi itself).  The factors' differences are taken in the wide type, but a
+// product well below one leaves E near -1, known to the absolute accuracy of one only (FP32: 1.3e-2 of
+// the logarithm at a density ratio of 1e-3, minus infinity from 2e-4 on).  So where a factor drops by
+// more than an eighth (the product of the rest is then above 0.39, and the error within three roundings),
+// and where one is negative, the factors' logarithms are taken one by one, each as that of a rise.  The gradients of two cells'
+// closure in FP64 took 20800 cycles with twenty logarithms per cell, a third of the whole chain in FP32.
 template <typename T>
 __device__ __forceinline__ void clo_pair_terms(const ReachView<T>& R, int lt, T etaf, bool chi_local, T (&d)[5]) {
     const Wide<T> nw = R.n[lt], Tw = R.Tc[lt];
@@ -421,6 +451,9 @@ __device__ __forceinline__ void clo_pair_terms(const ReachView<T>& R, int lt, T 
     E = fma(E, y, E + y);
     d[0] = log1p(E);
     d[1] = log1p(b);
+    if (__builtin_expect(steep_drop(a, b, x, y), 0)) {
+        d[0] = clo_steep_log<T>(w_hi(nw), w_hi(R.n[lt + 1]), dn, w_hi(Tw), w_hi(R.Tc[lt + 1]), w_hi(w_sub(R.Tc[lt + 1], Tw)), eta, deta);
+    }
     d[2] = w_hi(w_sub(R.u[0][lt + 1], R.u[0][lt]));
     d[3] = w_hi(w_sub(R.u[1][lt + 1], R.u[1][lt]));
     d[4] = w_hi(w_sub(R.u[2][lt + 1], R.u[2][lt]));
