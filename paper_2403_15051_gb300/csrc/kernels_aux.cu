@@ -554,7 +554,8 @@ void launch_dens_from_sums(const double* sums, T* dens, long long n, cudaStream_
 template <typename T>
 cudaError_t launch_closure(const ClosureArgs& A, const MomSet& M, int grid, int threads, size_t smem, cudaStream_t s) {
     if (A.wst_elems % 4) return cudaErrorInvalidValue;  // vector loads of the tables behind the band rows
-    if (smem > 32 * 1024) cudaFuncSetAttribute(closure_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_dynamic_smem((const void*)closure_kernel<T>, smem);
+    if (e != cudaSuccess) return e;
     return launch_maybe_programmatic(closure_kernel<T>, grid, threads, smem, s, A.programmatic, A, M);
 }
 
@@ -572,12 +573,11 @@ template <typename T>
 cudaError_t launch_closure_batch(const ClosureArgs& A, const MomSet& M, const ClosureBatchShape& B, cudaStream_t s) {
     auto rec = closure_records<T>(B.inline_band);
     const size_t smem = closure_records_smem(M.nR, M.n2, M.n3, B.warps, (int)sizeof(T));
-    // (the limit is the function's: that of the largest block, whichever the launch)
-    cudaError_t e = cudaFuncSetAttribute(rec, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)closure_records_smem(M.nR, M.n2, M.n3, kClosureWarps, (int)sizeof(T)));
+    const size_t band_smem = closure_smem_bytes(M.nR, M.n2, M.n3, 0, 0, (int)sizeof(T));
+    cudaError_t e = allow_dynamic_smem((const void*)rec, smem);
+    if (e == cudaSuccess && !B.inline_band) e = allow_dynamic_smem((const void*)closure_band_kernel<T>, band_smem);
     if (e == cudaSuccess && !B.inline_band)
-        e = launch_maybe_programmatic(closure_band_kernel<T>, B.grid_band, kClosureThreads,
-                                      closure_smem_bytes(M.nR, M.n2, M.n3, 0, 0, (int)sizeof(T)), s, A.programmatic, A, M);
+        e = launch_maybe_programmatic(closure_band_kernel<T>, B.grid_band, kClosureThreads, band_smem, s, A.programmatic, A, M);
     if (e == cudaSuccess) e = launch_maybe_programmatic(rec, B.grid, 32 * B.warps, smem, s, A.programmatic, A, M);
     return e;
 }
@@ -592,7 +592,7 @@ ClosureBatchShape closure_batch_shape(int tsize, int nR, int n2, int n3, int ite
     const size_t smem = closure_records_smem(nR, n2, n3, B.warps, tsize);
     auto resident = [](const void* k, int threads, size_t sm) {
         int n = 0;
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
+        if (allow_dynamic_smem(k, sm) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, sm) != cudaSuccess) {
             cudaGetLastError();
             return 4;
@@ -651,10 +651,10 @@ cudaError_t launch_fm_band(int tsize, const double* Rc, int rc_stride, const dou
                            int width, const int2* blo, void* W, const FmRule& rule, int grid, cudaStream_t s) {
     const size_t smem = (size_t)(width + 1) * sizeof(double);
     if (tsize == 4) {
-        cudaFuncSetAttribute(fm_band_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (const cudaError_t e = allow_dynamic_smem((const void*)fm_band_kernel<float>, smem)) return e;
         fm_band_kernel<float><<<grid, 128, smem, s>>>(Rc, rc_stride, Rf, N, sphere, sigma, width, blo, (float*)W, rule);
     } else {
-        cudaFuncSetAttribute(fm_band_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (const cudaError_t e = allow_dynamic_smem((const void*)fm_band_kernel<double>, smem)) return e;
         fm_band_kernel<double><<<grid, 128, smem, s>>>(Rc, rc_stride, Rf, N, sphere, sigma, width, blo, (double*)W, rule);
     }
     return cudaPeekAtLastError();

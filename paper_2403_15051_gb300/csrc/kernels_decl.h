@@ -17,6 +17,22 @@ inline __host__ __device__ int rec_off_g2() { return kCellScalars; }
 inline __host__ __device__ int rec_off_gR(int n2) { return kCellScalars + n2; }
 inline __host__ __device__ int rec_off_g3(int nR, int n2) { return kCellScalars + n2 + nR; }
 
+// Lets `kern` be launched with `smem` bytes of dynamic shared memory.  A function's limit is the process's,
+// shared by every handle and thread: it is never set to one launch's size (a handle with a smaller momentum
+// set would then make another's next launch fail) but raised, where the launch needs more than it allows, to
+// what the device offers beside the function's static shared memory.
+inline cudaError_t allow_dynamic_smem(const void* kern, size_t smem) {
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, kern);
+    if (e != cudaSuccess || smem <= (size_t)a.maxDynamicSharedSizeBytes) return e;
+    int dev = 0, optin = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+    const size_t most = (size_t)optin > a.sharedSizeBytes ? (size_t)optin - a.sharedSizeBytes : 0;
+    if (smem > most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Launch with programmatic stream serialization when `programmatic` (see pdl_wait), else the
 // ordinary way.
 template <typename... Args>

@@ -390,7 +390,7 @@ cudaError_t launch_kr_contract_tc(const float* f, float* out, const int4* items,
                                   const float* Bsplit, const float* isw, const float* sw, const MomSet& M, int Npad,
                                   int* err, int grid, cudaStream_t s) {
     const size_t smem = kr_tc_smem_bytes(Npad);
-    cudaError_t e = cudaFuncSetAttribute(kr_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem((const void*)kr_tc_kernel, smem);
     if (e != cudaSuccess) return e;
     kr_tc_kernel<<<grid, 128, smem, s>>>(f, out, items, n_items, inst, Bsplit, isw, sw, M, Npad, err);
     return cudaPeekAtLastError();

@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(stage_max_threads<T, VW, 1>(), 1) step_kernel(
 template <typename T, int GEOM, int VW, int NV, int NR_, int N2_, int N3_>
 cudaError_t launch_step_t(const StepArgs& S, const MomSet& M, int grid, int threads, size_t smem, cudaStream_t s) {
     auto kern = step_kernel<T, GEOM, VW, NV, NR_, N2_, N3_>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
@@ -207,7 +207,7 @@ cudaError_t launch_step_t(const StepArgs& S, const MomSet& M, int grid, int thre
 template <typename T, int GEOM, int VW, int NV, int NR_, int N2_, int N3_>
 cudaError_t step_occupancy_t(int threads, size_t smem, int* blocks_per_sm) {
     auto kern = step_kernel<T, GEOM, VW, NV, NR_, N2_, N3_>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, threads, smem);
 }

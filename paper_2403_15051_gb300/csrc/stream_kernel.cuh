@@ -1114,7 +1114,7 @@ __global__ void __launch_bounds__(stage_max_threads<T, VW, MINB>(), MINB) stream
 template <typename... Args>
 cudaError_t stage_launch(void (*kern)(Args...), const StageArgs& A, const MomSet& M, int grid, int threads, size_t smem,
                          cudaStream_t s, int* blocks_per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     if (blocks_per_sm) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, threads, smem);
     return launch_maybe_programmatic(kern, grid, threads, smem, s, A.programmatic, A, M);
