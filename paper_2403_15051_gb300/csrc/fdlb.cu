@@ -86,6 +86,7 @@ struct Solver {
     MomSet M{};
     // tiling of the stream kernel
     int B = 16, KS = 1, threads = 0;
+    int block_cap = 256;  // threads per block asked for; `threads` follows from it and the shape
     StreamCfg scfg{1, 4, 0};
     size_t smem_stream = 0;
     int march_G = 2, teams = 1;   // cells per group of the stage's march; warps of a block that walk items of their own
@@ -749,10 +750,14 @@ int upload_items(Solver& S) {
 
 int launch_moments_all(Solver& S, int buf);
 
+// The tiling and the stage kernel of a handle; 0 keeps a value.  The kernel is chosen by the block size asked
+// for, never by the one that came out of it, so that applying a handle's own configuration again (the tuner, the
+// setters of other options) selects the same kernel, with the same order of the moment sums.
 int configure_tiling(Solver& S, int B, int KS, int threads) {
     const int old_slices = S.M.slices;
     if (B > 0) S.B = std::max(2, B);
     if (KS > 0) S.KS = KS;
+    if (threads > 0) S.block_cap = threads;
     // the sphere's force couples every axis: slices narrower than the p_3 axis take K_3 f from its
     // own contraction kernel
     if (S.geometry == FDLB_SPH && !S.k3f) S.KS = S.n3;
@@ -795,7 +800,7 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
             cfg.vw /= 2;
             spread = true;
         }
-    const int cap = threads > 0 ? threads : 256;
+    const int cap = S.block_cap;
     // rows of eight per thread over many cells, as for the compile-time shape below, and where a block of four
     // momenta per thread would hold two vectors each: the same threads, half the instructions beside the arithmetic
     // (40 x 8 x 8 on 240 cells: 22.2 and 20.5 us)
@@ -1285,11 +1290,11 @@ int launch_steps_fused(Solver& S, int64_t n) {
 // choice is cached per process for the momentum set, precision, block size, slicing and the
 // size class of the handle (log2 of its cells and of its instances).
 struct TuneKey {
-    int geometry, precision, nR, n2, n3, KS, threads, cells_log2, inst_log2;
+    int geometry, precision, nR, n2, n3, KS, threads, vw, nv, cells_log2, inst_log2;
     bool operator<(const TuneKey& o) const {
-        const int a[9] = {geometry, precision, nR, n2, n3, KS, threads, cells_log2, inst_log2};
-        const int b[9] = {o.geometry, o.precision, o.nR, o.n2, o.n3, o.KS, o.threads, o.cells_log2, o.inst_log2};
-        return std::lexicographical_compare(a, a + 9, b, b + 9);
+        const int a[11] = {geometry, precision, nR, n2, n3, KS, threads, vw, nv, cells_log2, inst_log2};
+        const int b[11] = {o.geometry, o.precision, o.nR, o.n2, o.n3, o.KS, o.threads, o.vw, o.nv, o.cells_log2, o.inst_log2};
+        return std::lexicographical_compare(a, a + 11, b, b + 11);
     }
 };
 struct TuneVal {
@@ -1308,7 +1313,7 @@ int ilog2(long long x) {
 }
 
 TuneKey tune_key(const Solver& S) {
-    return TuneKey{S.geometry, S.precision, S.nR, S.n2, S.n3, S.KS, S.threads, ilog2(S.total_cells), ilog2(S.n_inst)};
+    return TuneKey{S.geometry, S.precision, S.nR, S.n2, S.n3, S.KS, S.threads, S.scfg.vw, S.scfg.nv, ilog2(S.total_cells), ilog2(S.n_inst)};
 }
 
 int set_closure_grouping(Solver& S, int cells, int batch = -1) {
@@ -1351,7 +1356,7 @@ int run_autotune(Solver& S, bool use_cache) {
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) {
             S.stage_minb = it->second.minb;
-            int rc = configure_tiling(S, it->second.B, S.KS, S.threads);
+            int rc = configure_tiling(S, it->second.B, 0, 0);
             return rc ? rc : set_closure_grouping(S, it->second.closure_cells, it->second.batch);
         }
     }
@@ -1360,7 +1365,6 @@ int run_autotune(Solver& S, bool use_cache) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     FDLB_CUDA(cudaEventCreate(&e0));
     FDLB_CUDA(cudaEventCreate(&e1));
-    const int KS = S.KS, threads = S.threads;
     int bestB = S.B, bestC = S.closure_cells, bestM = S.stage_minb, bestBatch = S.closure_batch;
     float best = time_stages(S, e0, e1);
     if (best < 0.f) best = 1e30f;
@@ -1376,7 +1380,7 @@ int run_autotune(Solver& S, bool use_cache) {
         S.stage_minb = mb;
         for (int B : Bs) {
             if (B == bestB && mb == bestM) continue;
-            if (configure_tiling(S, B, KS, threads) != FDLB_OK || S.B != B) continue;
+            if (configure_tiling(S, B, 0, 0) != FDLB_OK || S.B != B) continue;
             const float ms = time_stages(S, e0, e1);
             if (ms >= 0.f && ms < best) {
                 best = ms;
@@ -1386,7 +1390,7 @@ int run_autotune(Solver& S, bool use_cache) {
         }
     }
     S.stage_minb = bestM;
-    rc = configure_tiling(S, bestB, KS, threads);
+    rc = configure_tiling(S, bestB, 0, 0);
     // the closure: the chain form with items of C cells, or the batch form (two launches)
     const int Cs[] = {2, 4, 8, 16};
     for (int C : Cs) {
@@ -2319,7 +2323,7 @@ int fdlb_set_tensor_contraction(fdlb_handle h, int enable, int* in_use) try {
         if (in_use) *in_use = S->kr_tc;
         if (by_kernel != S->krg_on) {
             S->krg_on = by_kernel;
-            return fdlb::configure_tiling(*S, S->B, S->KS, S->threads);
+            return fdlb::configure_tiling(*S, 0, 0, 0);
         }
         if (S->gexec) {
             cudaGraphExecDestroy(S->gexec);
@@ -2327,7 +2331,7 @@ int fdlb_set_tensor_contraction(fdlb_handle h, int enable, int* in_use) try {
         }
         return FDLB_OK;
     }
-    const int rc = fdlb::configure_tiling(*S, S->B, S->KS, S->threads);
+    const int rc = fdlb::configure_tiling(*S, 0, 0, 0);
     if (in_use) *in_use = S->mma_on;
     return rc;
 } FDLB_HOST_CATCH
@@ -2340,7 +2344,7 @@ int fdlb_set_persistent_step(fdlb_handle h, int enable, int* in_use) try {
         return FDLB_OK;
     }
     S->fused = enable ? 1 : 0;
-    const int rc = fdlb::configure_tiling(*S, S->B, S->KS, S->threads);
+    const int rc = fdlb::configure_tiling(*S, 0, 0, 0);
     if (in_use) *in_use = S->fused_on;
     return rc;
 } FDLB_HOST_CATCH
@@ -2406,11 +2410,11 @@ int fdlb_set_stage_min_blocks(fdlb_handle h, int min_blocks, int* in_use) try {
     if (min_blocks > 0) {
         const int old = S->stage_minb;
         S->stage_minb = min_blocks;
-        int rc = fdlb::configure_tiling(*S, S->B, S->KS, S->threads);
+        int rc = fdlb::configure_tiling(*S, 0, 0, 0);
         if (rc == FDLB_OK && S->scfg.minb != min_blocks) rc = FDLB_EINVAL;  // not built for this shape
         if (rc) {
             S->stage_minb = old;
-            fdlb::configure_tiling(*S, S->B, S->KS, S->threads);
+            fdlb::configure_tiling(*S, 0, 0, 0);
             return rc;
         }
     }
