@@ -713,6 +713,7 @@ int upload_items(Solver& S) {
     wst = wst / 4 * 4;  // the tables behind the band rows start on a 16-byte boundary
     S.closure_wst = wst;
     S.closure_smem = closure_smem(S.nR, S.n2, S.n3, max_union, wst, (int)S.tsize);
+    (void)plan_closure((int)S.tsize, S.closure_smem);  // (a launch beyond what the device offers reports it)
     for (int l = 0; l < 3; ++l) {
         const int n_c = rc[2 * l + 1] - rc[2 * l], n_p = rp[2 * l + 1] - rp[2 * l];
         S.range[l].grid_closure = std::max(1, std::min(n_c, S.n_sm * (throughput ? closure_bps : 8)));

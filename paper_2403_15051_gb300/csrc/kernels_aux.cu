@@ -554,8 +554,6 @@ void launch_dens_from_sums(const double* sums, T* dens, long long n, cudaStream_
 template <typename T>
 cudaError_t launch_closure(const ClosureArgs& A, const MomSet& M, int grid, int threads, size_t smem, cudaStream_t s) {
     if (A.wst_elems % 4) return cudaErrorInvalidValue;  // vector loads of the tables behind the band rows
-    const cudaError_t e = allow_dynamic_smem((const void*)closure_kernel<T>, smem);
-    if (e != cudaSuccess) return e;
     return launch_maybe_programmatic(closure_kernel<T>, grid, threads, smem, s, A.programmatic, A, M);
 }
 
@@ -574,9 +572,8 @@ cudaError_t launch_closure_batch(const ClosureArgs& A, const MomSet& M, const Cl
     auto rec = closure_records<T>(B.inline_band);
     const size_t smem = closure_records_smem(M.nR, M.n2, M.n3, B.warps, (int)sizeof(T));
     const size_t band_smem = closure_smem_bytes(M.nR, M.n2, M.n3, 0, 0, (int)sizeof(T));
-    cudaError_t e = allow_dynamic_smem((const void*)rec, smem);
-    if (e == cudaSuccess && !B.inline_band) e = allow_dynamic_smem((const void*)closure_band_kernel<T>, band_smem);
-    if (e == cudaSuccess && !B.inline_band)
+    cudaError_t e = cudaSuccess;
+    if (!B.inline_band)
         e = launch_maybe_programmatic(closure_band_kernel<T>, B.grid_band, kClosureThreads, band_smem, s, A.programmatic, A, M);
     if (e == cudaSuccess) e = launch_maybe_programmatic(rec, B.grid, 32 * B.warps, smem, s, A.programmatic, A, M);
     return e;
@@ -606,6 +603,10 @@ ClosureBatchShape closure_batch_shape(int tsize, int nR, int n2, int n3, int ite
     B.grid_band = clamp((pairs + kClosureWarps - 1) / kClosureWarps,
                         (long long)n_sm * resident(bk, kClosureThreads, closure_smem_bytes(nR, n2, n3, 0, 0, tsize)));
     return B;
+}
+
+cudaError_t plan_closure(int tsize, size_t smem) {
+    return allow_dynamic_smem(tsize == 4 ? (const void*)closure_kernel<float> : (const void*)closure_kernel<double>, smem);
 }
 
 int closure_blocks_per_sm(int tsize, size_t smem) {

@@ -20,8 +20,11 @@ inline __host__ __device__ int rec_off_g3(int nR, int n2) { return kCellScalars 
 // Lets `kern` be launched with `smem` bytes of dynamic shared memory.  A function's limit is the process's,
 // shared by every handle and thread: it is never set to one launch's size (a handle with a smaller momentum
 // set would then make another's next launch fail) but raised, where the launch needs more than it allows, to
-// what the device offers beside the function's static shared memory.
+// what the device offers beside the function's static shared memory.  Called where a launch is planned (a handle's
+// shapes change), not at each launch of a stage: asking the runtime took 0.3 us a launch.  Up to 32 KB the default
+// limit of 48 KB holds for every kernel here, whose static shared memory is less than 16 KB.
 inline cudaError_t allow_dynamic_smem(const void* kern, size_t smem) {
+    if (smem <= 32 * 1024) return cudaSuccess;
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, kern);
     if (e != cudaSuccess || smem <= (size_t)a.maxDynamicSharedSizeBytes) return e;
@@ -156,6 +159,8 @@ cudaError_t launch_closure(const ClosureArgs& A, const MomSet& M, int grid, int 
 size_t closure_smem(int nR, int n2, int n3, int max_union, int wst_elems, int tsize);
 // Blocks of the closure kernel that fit on an SM with `smem` bytes of dynamic shared memory each.
 int closure_blocks_per_sm(int tsize, size_t smem);
+// Lets the closure kernel be launched with `smem` bytes (before launch_closure).
+cudaError_t plan_closure(int tsize, size_t smem);
 // The batch form of the closure: closure_records_kernel, a warp per item of at most kClosureCells
 // cells, after closure_band_kernel unless the bands are short enough for it to sum them itself.
 constexpr int kInlineBandMax = 128;  // columns of the widest band the records kernel sums

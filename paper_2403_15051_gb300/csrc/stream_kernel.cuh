@@ -1110,13 +1110,14 @@ __global__ void __launch_bounds__(stage_max_threads<T, VW, MINB>(), MINB) stream
         march_body<T, GEOM, VW, NV, NR_, N2_, N3_>(A, M);
 }
 
-// Launches, or with `blocks_per_sm` reports how many blocks of the shape reside on an SM.
+// Launches, or with `blocks_per_sm` plans the launch: reports how many blocks of the shape reside on an SM.
 template <typename... Args>
 cudaError_t stage_launch(void (*kern)(Args...), const StageArgs& A, const MomSet& M, int grid, int threads, size_t smem,
                          cudaStream_t s, int* blocks_per_sm) {
-    cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
-    if (e != cudaSuccess) return e;
-    if (blocks_per_sm) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, threads, smem);
+    if (blocks_per_sm) {
+        const cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
+        return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, threads, smem);
+    }
     return launch_maybe_programmatic(kern, grid, threads, smem, s, A.programmatic, A, M);
 }
 template <typename T, int GEOM, int VW, int NV, int NR_, int N2_, int N3_, int MINB = 1>
