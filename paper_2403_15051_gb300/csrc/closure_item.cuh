@@ -232,23 +232,25 @@ __device__ __forceinline__ void clo_fields(const Wide<T> (&sv)[kSums], Wide<T>& 
     using W = Wide<T>;
     n = sv[0];
     const W tr = w_add(w_add(sv[4], sv[5]), sv[6]);
+    T tuu;  // |u|^2, rounded once
     if constexpr (sizeof(T) == 8) {
         // one division for the four quotients by n (a division is nine FP64 operations)
         const T in = T(1) / n.v;
         u[0].v = mul_rn(sv[1].v, in);
         u[1].v = mul_rn(sv[2].v, in);
         u[2].v = mul_rn(sv[3].v, in);
-        const T uu = fma(u[0].v, u[0].v, fma(u[1].v, u[1].v, mul_rn(u[2].v, u[2].v)));
-        Tc.v = mul_rn(mul_rn(fma(-n.v, uu, tr.v), in), T(1.0 / 3.0));
+        tuu = fma(u[0].v, u[0].v, fma(u[1].v, u[1].v, mul_rn(u[2].v, u[2].v)));
+        Tc.v = mul_rn(mul_rn(fma(-n.v, tuu, tr.v), in), T(1.0 / 3.0));
     } else {
         u[0] = w_div(sv[1], n);
         u[1] = w_div(sv[2], n);
         u[2] = w_div(sv[3], n);
         const W uu = w_add(w_add(w_mul(u[0], u[0]), w_mul(u[1], u[1])), w_mul(u[2], u[2]));
         Tc = w_div(w_sub(tr, w_mul(n, uu)), w_scale(n, T(3)));
+        tuu = w_hi(uu);
     }
     const T tn = w_hi(n), t0 = w_hi(u[0]), t1 = w_hi(u[1]), t2 = w_hi(u[2]), ttr = w_hi(tr);
-    const T tuu = fma(t0, t0, fma(t1, t1, mul_rn(t2, t2))), nuu = mul_rn(tn, tuu);
+    const T nuu = mul_rn(tn, tuu);
     const T s4 = w_hi(sv[4]), s5 = w_hi(sv[5]), s6 = w_hi(sv[6]), s7 = w_hi(sv[7]), s8 = w_hi(sv[8]), s9 = w_hi(sv[9]);
     const T m0 = fma(s4, t0, fma(s7, t1, mul_rn(s8, t2)));
     const T m1 = fma(s7, t0, fma(s5, t1, mul_rn(s9, t2)));
