@@ -232,19 +232,14 @@ __device__ __forceinline__ void clo_fields(const Wide<T> (&sv)[kSums], Wide<T>& 
     using W = Wide<T>;
     n = sv[0];
     const W tr = w_add(w_add(sv[4], sv[5]), sv[6]);
+    u[0] = w_div(sv[1], n);
+    u[1] = w_div(sv[2], n);
+    u[2] = w_div(sv[3], n);
     T tuu;  // |u|^2, rounded once
     if constexpr (sizeof(T) == 8) {
-        // one division for the four quotients by n (a division is nine FP64 operations)
-        const T in = T(1) / n.v;
-        u[0].v = mul_rn(sv[1].v, in);
-        u[1].v = mul_rn(sv[2].v, in);
-        u[2].v = mul_rn(sv[3].v, in);
         tuu = fma(u[0].v, u[0].v, fma(u[1].v, u[1].v, mul_rn(u[2].v, u[2].v)));
-        Tc.v = mul_rn(mul_rn(fma(-n.v, tuu, tr.v), in), T(1.0 / 3.0));
+        Tc.v = fma(-n.v, tuu, tr.v) / mul_rn(T(3), n.v);
     } else {
-        u[0] = w_div(sv[1], n);
-        u[1] = w_div(sv[2], n);
-        u[2] = w_div(sv[3], n);
         const W uu = w_add(w_add(w_mul(u[0], u[0]), w_mul(u[1], u[1])), w_mul(u[2], u[2]));
         Tc = w_div(w_sub(tr, w_mul(n, uu)), w_scale(n, T(3)));
         tuu = w_hi(uu);

@@ -38,3 +38,14 @@ def test_heat_flux_takes_the_rounded_wide_kinetic_energy(tmp_path):
     q = f32(nuu * f32(u))
     assert np.mean(y[:3] != f32(u)) < 1e-3
     assert np.mean(y[3:6] != q) < 1e-3
+
+
+def test_fp64_velocities_and_temperature_are_rounded_quotients(tmp_path):
+    # u = (n u) / n and, at rest, T = tr / (3 n), each the correctly rounded quotient
+    x = _sums(20000, 5)
+    y = device_unit.run(tmp_path, "double", FIELDS % ("sv[k].v = x[k]", "u[a].v", "Tc.v"), x, 7)
+    assert np.array_equal(y[:3], x[1:4] / x[0])
+    x[1:4] = 0.0
+    x[4:7] = np.exp(np.random.default_rng(6).uniform(-1, 1, (3, x.shape[1]))) * x[0]
+    y = device_unit.run(tmp_path, "double", FIELDS % ("sv[k].v = x[k]", "u[a].v", "Tc.v"), x, 7)
+    assert np.array_equal(y[6], ((x[4] + x[5]) + x[6]) / (3.0 * x[0]))
