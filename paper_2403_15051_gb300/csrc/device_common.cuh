@@ -190,21 +190,10 @@ __device__ __forceinline__ float2 weno5_pair(float2 w0, float2 w1, float2 w2, fl
 }
 
 // FP64: the FP64 unit takes a warp instruction every 16 cycles, so its operations are what a stage
-// costs, and each of the four quotients above is nine of them.  The weights are taken without a
-// quotient, d_k times the square of the product of the other two indicators, with the indicators'
-// exponents lowered by the smallest one's (an integer operation on the high words, exact) and held
-// below 2^200 (a stencil that much rougher than the smoothest has no weight left either way), so the
-// products stay within the range.  The remaining quotient: the instruction's approximate reciprocal
-// (relative error 2^-20), one cubic step x (1 + e + e^2), e = 1 - d x (2^-60), and the quotient
-// corrected by its residual (correct to an ulp).
-__device__ __forceinline__ double f64_quot(double num, double den) {
-    double x;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(den));
-    const double e = __fma_rn(-den, x, 1.0);
-    x = __fma_rn(x, __fma_rn(e, e, e), x);
-    const double q = __dmul_rn(num, x);
-    return __fma_rn(__fma_rn(-den, q, num), x, q);
-}
+// costs, and a division is a chain of them.  The weights are taken without a quotient, d_k times the square
+// of the product of the other two indicators, with the indicators' exponents lowered by the smallest one's
+// (an integer operation on the high words, exact) and held below 2^200 (a stencil that much rougher than the
+// smoothest has no weight left either way), so the products stay within the range.  One division remains of four.
 __device__ __forceinline__ double f64_lowered(double E, int sh) {
     return __hiloint2double(min(__double2hiint(E) - sh, (1023 + 200) << 20), __double2loint(E));
 }
@@ -229,7 +218,7 @@ __device__ __forceinline__ double weno5_f64(double w0, double w1, double w2, dou
                  aR = __dmul_rn(dR, __dmul_rn(pR, pR));
     const double XL = __fma_rn(s3, tL, D1), XC = __fma_rn(s3, ntC, D2), XR = __fma_rn(-s3, tR, D3);
     const double num = __fma_rn(aR, XR, __fma_rn(aC, XC, __dmul_rn(aL, XL)));
-    return __fma_rn(f64_quot(num, __dadd_rn(__dadd_rn(aL, aC), aR)), 1.0 / 12.0, w2);
+    return __fma_rn(num / __dadd_rn(__dadd_rn(aL, aC), aR), 1.0 / 12.0, w2);
 }
 __device__ __forceinline__ double2 weno5_pair(double2 w0, double2 w1, double2 w2, double2 w3, double2 w4, double2 s3,
                                               double2, double2 dL, double2 dR, double2 e4) {
