@@ -192,10 +192,13 @@ __device__ __forceinline__ float2 weno5_pair(float2 w0, float2 w1, float2 w2, fl
 // FP64: the FP64 unit takes a warp instruction every 16 cycles, so its operations are what a stage
 // costs, and a division is a chain of them.  The weights are taken without a quotient, d_k times the square
 // of the product of the other two indicators, with the indicators' exponents lowered by the smallest one's
-// (an integer operation on the high words, exact) and held below 2^200 (a stencil that much rougher than the
-// smoothest has no weight left either way), so the products stay within the range.  One division remains of four.
-__device__ __forceinline__ double f64_lowered(double E, int sh) {
-    return __hiloint2double(min(__double2hiint(E) - sh, (1023 + 200) << 20), __double2loint(E));
+// (an integer operation on the high words, exact) and held below 2^200, so the products stay within the range.
+// A stencil that much rougher than the smoothest has a weight below 2^-400 and is given none: held at 2^200 it
+// would still count where its candidate differs by more than 2^347.  One division remains of four.
+constexpr int kF64Rough = 200 << 20;
+__device__ __forceinline__ int f64_above(double E, int base) { return __double2hiint(E) - base; }  // (>= 0: base is the least)
+__device__ __forceinline__ double f64_lowered(double E, int above) {
+    return __hiloint2double(min(above, kF64Rough) + (1023 << 20), __double2loint(E));
 }
 __device__ __forceinline__ double weno5_f64(double w0, double w1, double w2, double w3, double w4, double s3, double dL,
                                             double dR, double e4) {
@@ -209,13 +212,15 @@ __device__ __forceinline__ double weno5_f64(double w0, double w1, double w2, dou
     // (positive doubles order like their high words; a window that is not finite keeps the value not
     // finite through the candidates)
     const int hm = min(__double2hiint(EL), min(__double2hiint(EC), __double2hiint(ER)));
-    const int sh = (hm & 0x7ff00000) - (1023 << 20);
-    EL = f64_lowered(EL, sh);
-    EC = f64_lowered(EC, sh);
-    ER = f64_lowered(ER, sh);
+    const int base = hm & 0x7ff00000, xL = f64_above(EL, base), xC = f64_above(EC, base), xR = f64_above(ER, base);
+    EL = f64_lowered(EL, xL);
+    EC = f64_lowered(EC, xC);
+    ER = f64_lowered(ER, xR);
     const double pL = __dmul_rn(EC, ER), pC = __dmul_rn(EL, ER), pR = __dmul_rn(EL, EC);
-    const double aL = __dmul_rn(dL, __dmul_rn(pL, pL)), aC = __dmul_rn(0.6, __dmul_rn(pC, pC)),
-                 aR = __dmul_rn(dR, __dmul_rn(pR, pR));
+    // (a candidate that is not finite gives a product with a weight of zero that is not a number)
+    const double aL = xL > kF64Rough ? 0.0 : __dmul_rn(dL, __dmul_rn(pL, pL));
+    const double aC = xC > kF64Rough ? 0.0 : __dmul_rn(0.6, __dmul_rn(pC, pC));
+    const double aR = xR > kF64Rough ? 0.0 : __dmul_rn(dR, __dmul_rn(pR, pR));
     const double XL = __fma_rn(s3, tL, D1), XC = __fma_rn(s3, ntC, D2), XR = __fma_rn(-s3, tR, D3);
     const double num = __fma_rn(aR, XR, __fma_rn(aC, XC, __dmul_rn(aL, XL)));
     return __fma_rn(num / __dadd_rn(__dadd_rn(aL, aC), aR), 1.0 / 12.0, w2);

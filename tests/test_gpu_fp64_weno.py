@@ -46,3 +46,35 @@ def test_windows_over_many_scales_match_the_direct_form(tmp_path):
         wt = 10.0 ** rng.uniform(-60, 0, n)
         f = g * wt * 10.0 ** rng.uniform(-20, 20, n)
         _compare(tmp_path, f, 4e-6 * wt * wt)
+
+
+def test_indicators_far_apart_match_the_direct_form(tmp_path):
+    # one side of the window 2^50 .. 2^480 times the other: indicators up to 2^960 apart, beyond the ratio from
+    # which a stencil is given no weight, and (the last, by epsilon alone) beyond what a difference of exponents holds
+    rng = np.random.default_rng(10)
+    n = 20000
+    for k in range(6):
+        w = 1.0 + 0.1 * rng.normal(size=(5, n))
+        big = 2.0 ** rng.uniform(50, 480, n)
+        if k < 4:
+            w[k + 1 if k < 2 else 0:5 if k < 2 else k - 1] *= big
+            e4 = np.full(n, 4e-6)
+        elif k == 4:  # (the rough stencils' values around zero, as in a jump back)
+            w[0] *= big
+            w[1] = w[2]
+            e4 = np.full(n, 4e-6)
+        else:  # smooth stencils whose indicator is epsilon alone, 2^-1000
+            w[1:] = 1.0
+            w[0] = 2.0 ** rng.uniform(1, 60, n)
+            e4 = np.full(n, 2.0 ** -1000)
+        _compare(tmp_path, w, e4)
+
+
+def test_windows_that_are_not_finite_stay_so(tmp_path):
+    rng = np.random.default_rng(11)
+    for bad in (np.inf, -np.inf, np.nan):
+        w = 1.0 + 0.1 * rng.normal(size=(5, 500))
+        w[np.arange(500) % 5, np.arange(500)] = bad
+        for sign in (1.0, -1.0):
+            x = np.concatenate([w, np.full((1, 500), 3.0 * sign), np.full((1, 500), 4e-6)])
+            assert not np.any(np.isfinite(device_unit.run(tmp_path, "double", BODY, x, 1)))
