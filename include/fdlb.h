@@ -253,7 +253,11 @@ const char* fdlb_error_string(int code);
 /* Kernel-tuning knobs of the streaming kernel (cells per tile, p_3 values per momentum slice,
  * threads per block); 0 keeps the current value.  A change of the cells per tile alone regroups
  * cells without changing any result; the slice width and the block size change the order of the
- * moment sums (results then agree to rounding).  For the 16 x 8 x 8 FP32 cylinder a block of at
+ * moment sums (results then agree to rounding).  The block has at most the threads asked for where
+ * the momentum set has a kernel of so few (a thread holds at most 8 momenta, so 32 threads per 256
+ * momenta of a slice at the least; the compile-time shapes come in blocks of 256 and 128 threads,
+ * 16 x 8 x 8 in FP32, of 256, 16 x 8 x 8 in FP64, of 288 and 224, 24 x 12 x 12 in FP32, of 448 in
+ * FP64); fdlb_get_tiling reports what came of it.  For the 16 x 8 x 8 FP32 cylinder a block of at
  * most 128 threads selects the row kernel (a whole p_2 row of 8 momenta per thread), the default
  * for handles of more than 64 cells per SM.
  *

@@ -86,7 +86,8 @@ struct Solver {
     MomSet M{};
     // tiling of the stream kernel
     int B = 16, KS = 1, threads = 0;
-    int block_cap = 256;  // threads per block asked for; `threads` follows from it and the shape
+    int block_cap = 256;  // threads per block asked for (or the default); `threads` follows from it and the shape
+    bool block_asked = false;  // by the caller: at most so many then, where the shape has a kernel of so few
     StreamCfg scfg{1, 4, 0};
     size_t smem_stream = 0;
     int march_G = 2, teams = 1;   // cells per group of the stage's march; warps of a block that walk items of their own
@@ -792,22 +793,26 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
         cfg.vw = S.n2 % 4 == 0 ? 4 : (S.n2 % 2 == 0 ? 2 : 1);
     else  // (four FP64 momenta per thread: blocks of up to 256 threads, for their registers)
         cfg.vw = S.n2 % 4 == 0 && Ms <= 1024 ? 4 : (S.n2 % 2 == 0 ? 2 : 1);
+    const int cap = S.block_cap;
+    // whether the caller's block size leaves room for a thread per vector of `vw` momenta
+    auto fits = [&](int vw) { return !S.block_asked || (Ms / vw + 31) / 32 * 32 <= std::max(cap, 32); };
+    const bool spec_cyl = S.geometry == FDLB_CYL && S.nR == 16 && S.n2 == 8 && S.n3 == 8;  // (built for one block size)
+    if (S.tsize == 8 && cfg.vw == 4 && !spec_cyl && !fits(4)) cfg.vw = 2;
     // FP64 over few cells: each of an SM's four partitions takes an FP64 warp instruction every 64 cycles, so a cell
     // whose momenta fit one warp has a quarter of its SM.  Fewer momenta per thread then, as long as cells and warps
     // together do not fill the partitions (one cell's face and update: 41000 cycles by one warp)
     bool spread = false;
     if (S.tsize == 8)
-        while (cfg.vw > 1 && Ms / cfg.vw < 128 && (long long)S.total_cells * ((Ms / cfg.vw + 31) / 32) < 4LL * S.n_sm) {
+        while (cfg.vw > 1 && Ms / cfg.vw < 128 && fits(cfg.vw / 2) && (long long)S.total_cells * ((Ms / cfg.vw + 31) / 32) < 4LL * S.n_sm) {
             cfg.vw /= 2;
             spread = true;
         }
-    const int cap = S.block_cap;
     // rows of eight per thread over many cells, as for the compile-time shape below, and where a block of four
     // momenta per thread would hold two vectors each: the same threads, half the instructions beside the arithmetic
     // (40 x 8 x 8 on 240 cells: 22.2 and 20.5 us)
     const bool rows8 = S.tsize == 4 && S.n2 == 8 && Ms / 8 <= 512 &&
                        ((long long)S.total_cells * S.Np > (long long)S.n_sm * 65536 || Ms / 4 > cap);
-    cfg.spec = ((S.geometry == FDLB_CYL && S.nR == 16 && S.n2 == 8 && S.n3 == 8) ||
+    cfg.spec = (spec_cyl ||
                 (S.geometry == FDLB_SPH && S.nR == 24 && S.n2 == 12 && S.n3 == 12)) &&
                cfg.vw == (S.tsize == 4 || S.geometry == FDLB_CYL ? 4 : 2);
     // the cylinder's FP32 shape in blocks of at most 128 threads: a thread per whole p_2 row (8
@@ -817,7 +822,7 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
     // the sphere's FP32 shape: a thread per row of twelve.  The stage is bound by the shared-memory data unit (four
     // momenta per thread: 86 vector loads per vector, 69% of its rate at 81 us on 2048 cells); a whole row shares
     // the coefficients of K^h and K_3, and K_2's are launch constants.  Not for the mma.sync form, built for four
-    if (cfg.spec && S.tsize == 4 && S.geometry == FDLB_SPH && !S.tensor) cfg.vw = 12;
+    if (cfg.spec && S.tsize == 4 && S.geometry == FDLB_SPH && !S.tensor && fits(12)) cfg.vw = 12;
     const int Vs = Ms / cfg.vw;
     int nt = 0;
     if (cfg.vw == 8 || cfg.vw == 12) {
@@ -833,7 +838,7 @@ int configure_tiling(Solver& S, int B, int KS, int threads) {
         // keep up to 64 of them in one warp
         cfg.nv = cfg.vw == 4 ? (S.tsize == 4 && Vs > 32 ? 2 : 1) : spread ? 1 : 4;
         // (over few cells the second warp is free: 256 momenta on 499 cells 62.2 us per step by one warp, 43.8 by two)
-        if (cfg.nv == 2 && Vs <= 64 && 2LL * S.total_cells <= 16LL * S.n_sm) {
+        if (cfg.nv == 2 && Vs <= 64 && fits(cfg.vw) && 2LL * S.total_cells <= 16LL * S.n_sm) {
             cfg.nv = 1;
             spread = true;
         }
@@ -2273,6 +2278,7 @@ const char* fdlb_error_string(int code) {
 int fdlb_set_tiling(fdlb_handle h, int cells_per_tile, int slice_k, int threads) try {
     Solver* S = SOL(h);
     if (!S || cells_per_tile < 0 || slice_k < 0 || threads < 0) return FDLB_EINVAL;
+    if (threads > 0) S->block_asked = true;
     return fdlb::configure_tiling(*S, cells_per_tile, slice_k, threads);
 } FDLB_HOST_CATCH
 

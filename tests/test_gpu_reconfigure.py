@@ -5,11 +5,12 @@ with one warp per cell, the reduced pair, a block that holds one vector of four 
 import numpy as np
 import pytest
 
+from oracle import solver as osolver
 from paper_2403_15051_gb300 import build as fbuild
 from paper_2403_15051_gb300 import fdlb
 from paper_2403_15051_gb300 import workloads as wl
 
-from .cases import small_case
+from .cases import compare_moments, oracle_problem, perturbed_state, small_case
 
 pytestmark = pytest.mark.gpu
 
@@ -62,3 +63,30 @@ def test_setters_of_other_options_keep_the_kernel(geometry, Q, precision, cells)
                        lambda: S.stage_min_blocks(1), lambda: S.set_tiling(5, 0, 0), lambda: S.set_tiling(0, 0, 0)):
             change()
             assert _kernel(S) == made
+
+
+# (set, precision, cells, threads asked for, the most that may come of it: what the vectors of two FP64 or four FP32
+# momenta, four or two to a thread, took)
+BLOCKS = [(wl.SPH, (12, 12, 12), "fp32", 20, 256, 224), (wl.SPH, (12, 12, 12), "fp32", 20, 288, 288),
+          (wl.CYL, (8, 8, 4), "fp64", 24, 64, 64), (wl.CYL, (8, 8, 4), "fp64", 24, 128, 128), (wl.CYL, (4, 4, 4), "fp64", 24, 32, 32),
+          (wl.CYL, (4, 4, 8), "fp64", 24, 64, 64), (wl.SPH, (4, 4, 4), "fp64", 24, 32, 32), (wl.CYL, (4, 8, 4), "fp32", 24, 32, 32),
+          (wl.CYL, (9, 8, 8), "fp32", 24, 160, 160), (wl.CYL, (8, 8, 8), "fp64", 24, 256, 256)]
+
+
+@pytest.mark.parametrize("geometry,Q,precision,cells,threads,most", BLOCKS)
+def test_the_block_size_asked_for_is_kept(geometry, Q, precision, cells, threads, most):
+    d = small_case(geometry=geometry, precision=precision, n_cells=cells, Q=Q)
+    P = oracle_problem(d)
+    f0 = perturbed_state(P, 8, 0.05)
+    with fdlb.Solver(d) as S:
+        S.set_tiling(0, 0, threads)
+        assert S.tiling()["threads"] <= most
+        S.set_tiling(0, 0, 0)
+        S.set_tensor_contraction(False)
+        assert S.tiling()["threads"] <= most
+        S.set_f(f0)
+        L, L_or = S.eval_rhs(), osolver.rhs(f0, P)
+        assert np.max(np.abs(L - L_or)) <= (1e-10 if precision == "fp64" else 2e-5) * np.max(np.abs(L_or))
+        S.step(2)
+        errs = compare_moments(S.moments(), osolver.moments(osolver.run(f0, P, 2), P), P)
+        assert max(errs.values()) <= (1e-10 if precision == "fp64" else 1e-5), errs
