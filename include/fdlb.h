@@ -252,7 +252,8 @@ const char* fdlb_error_string(int code);
 
 /* Kernel-tuning knobs of the streaming kernel (cells per tile, p_3 values per momentum slice,
  * threads per block); 0 keeps the current value.  A change of the cells per tile alone regroups
- * cells without changing any result; the slice width and the block size change the order of the
+ * cells without changing any result (a lone instance of few cells is cut into smaller tiles unless a
+ * size was asked for, and into a whole number of tiles per SM in any case); the slice width and the block size change the order of the
  * moment sums (results then agree to rounding).  The block has at most the threads asked for where
  * the momentum set has a kernel of so few (a thread holds at most 8 momenta, so 32 threads per 256
  * momenta of a slice at the least; the compile-time shapes come in blocks of 256 and 128 threads,

@@ -85,6 +85,7 @@ struct Solver {
     std::vector<double> tab_h;
     MomSet M{};
     // tiling of the stream kernel
+    bool tile_asked = false;  // B by the caller or the tuner: a lone instance's few cells are not cut smaller then
     int B = 16, KS = 1, threads = 0;
     int block_cap = 256;  // threads per block asked for (or the default); `threads` follows from it and the shape
     bool block_asked = false;  // by the caller: at most so many then, where the shape has a kernel of so few
@@ -588,15 +589,15 @@ int upload_items(Solver& S) {
             const int per_wave = S.n_sm;
             const int r = (nt * slices + per_wave - 1) / per_wave * per_wave / slices;
             if (r >= nt && r * slices % per_wave == 0 && N / r >= 2) nt = r;
-            // not that many: tiles of two cells where they still find an SM each
-            else if (nt * slices < per_wave && N / 2 * slices <= per_wave && N / 2 > nt && !S.fused) nt = N / 2;
+            // not that many (and no tile size asked for): tiles of two cells where they still find an SM each
+            else if (!S.tile_asked && nt * slices < per_wave && N / 2 * slices <= per_wave && N / 2 > nt && !S.fused) nt = N / 2;
             // fewer cells than SMs: one to a tile (each computes both its faces, half as much again, on
             // twice the SMs: the FP64 stage of 64 cells x 128 momenta took 48.8 us in tiles of four)
-            if (!S.fused && !S.tiles && N * slices <= S.n_sm && N * slices <= S.max_sitems) nt = N;
+            if (!S.tile_asked && !S.fused && !S.tiles && N * slices <= S.n_sm && N * slices <= S.max_sitems) nt = N;
             // the march's blocks share an SM: items of two cells up to 16 warps per SM (per step, items of four and
             // two: 256 momenta by two warps on 499 cells 43.8 and 33.6 us, 1000 54.4 and 42.4; 1000 momenta by eight
             // warps on 499 cells 52.5 and 45.4, but on 1000, beyond the line, 59.5 and 72.0)
-            else if (!S.fused && !S.tiles && nt < (N + 1) / 2 && (N + 1LL) / 2 * slices * (S.threads / 32) <= 16LL * S.n_sm)
+            else if (!S.tile_asked && !S.fused && !S.tiles && nt < (N + 1) / 2 && (N + 1LL) / 2 * slices * (S.threads / 32) <= 16LL * S.n_sm)
                 nt = (N + 1) / 2;
         }
         const int base = N / nt, rem = N % nt;
@@ -1305,6 +1306,7 @@ struct TuneKey {
 };
 struct TuneVal {
     int B, closure_cells, minb, batch;
+    bool tile_asked;
 };
 std::map<TuneKey, TuneVal> g_tune_cache;
 std::mutex g_tune_mutex;
@@ -1362,6 +1364,7 @@ int run_autotune(Solver& S, bool use_cache) {
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) {
             S.stage_minb = it->second.minb;
+            S.tile_asked = it->second.tile_asked;
             int rc = configure_tiling(S, it->second.B, 0, 0);
             return rc ? rc : set_closure_grouping(S, it->second.closure_cells, it->second.batch);
         }
@@ -1372,6 +1375,7 @@ int run_autotune(Solver& S, bool use_cache) {
     FDLB_CUDA(cudaEventCreate(&e0));
     FDLB_CUDA(cudaEventCreate(&e1));
     int bestB = S.B, bestC = S.closure_cells, bestM = S.stage_minb, bestBatch = S.closure_batch;
+    bool bestAsked = S.tile_asked;  // (a lone instance's default is a rule, not a tile size)
     float best = time_stages(S, e0, e1);
     if (best < 0.f) best = 1e30f;
     const int Bs[] = {2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
@@ -1385,17 +1389,20 @@ int run_autotune(Solver& S, bool use_cache) {
         if ((mb == 2 || mb == 5) && !rows) continue;
         S.stage_minb = mb;
         for (int B : Bs) {
-            if (B == bestB && mb == bestM) continue;
+            if (B == bestB && mb == bestM && (bestAsked || S.n_inst > 1)) continue;
+            S.tile_asked = true;
             if (configure_tiling(S, B, 0, 0) != FDLB_OK || S.B != B) continue;
             const float ms = time_stages(S, e0, e1);
             if (ms >= 0.f && ms < best) {
                 best = ms;
                 bestB = B;
                 bestM = mb;
+                bestAsked = true;
             }
         }
     }
     S.stage_minb = bestM;
+    S.tile_asked = bestAsked;
     rc = configure_tiling(S, bestB, 0, 0);
     // the closure: the chain form with items of C cells, or the batch form (two launches)
     const int Cs[] = {2, 4, 8, 16};
@@ -1422,7 +1429,7 @@ int run_autotune(Solver& S, bool use_cache) {
     if (!rc) rc = set_closure_grouping(S, bestC, bestBatch);
     if (!rc) {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
-        g_tune_cache[key] = {bestB, bestC, bestM, bestBatch};
+        g_tune_cache[key] = {bestB, bestC, bestM, bestBatch, bestAsked};
     }
     return rc;
 }
@@ -2279,6 +2286,7 @@ int fdlb_set_tiling(fdlb_handle h, int cells_per_tile, int slice_k, int threads)
     Solver* S = SOL(h);
     if (!S || cells_per_tile < 0 || slice_k < 0 || threads < 0) return FDLB_EINVAL;
     if (threads > 0) S->block_asked = true;
+    if (cells_per_tile > 0) S->tile_asked = true;
     return fdlb::configure_tiling(*S, cells_per_tile, slice_k, threads);
 } FDLB_HOST_CATCH
 

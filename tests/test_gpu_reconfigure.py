@@ -90,3 +90,21 @@ def test_the_block_size_asked_for_is_kept(geometry, Q, precision, cells, threads
         S.step(2)
         errs = compare_moments(S.moments(), osolver.moments(osolver.run(f0, P, 2), P), P)
         assert max(errs.values()) <= (1e-10 if precision == "fp64" else 1e-5), errs
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_the_cells_per_tile_asked_for_are_kept_on_a_lone_instance(precision):
+    # 64 cells in one tile are walked by one block, cell after cell: many times the stage's time over the default,
+    # a cell to an item, and the same bits
+    d = small_case(precision=precision, n_cells=64, Q=(4, 4, 4))
+    out = {}
+    for cells in (0, 64):
+        with fdlb.Solver(d) as S:
+            S.set_tiling(cells, 0, 0)
+            S.step(5)
+            out[cells] = S.get_f()
+            S.set_kernel_timing(True)
+            S.step(20)
+            out[cells, "ms"] = S.kernel_times()[0]
+    assert np.array_equal(out[0], out[64])
+    assert out[64, "ms"] > 4.0 * out[0, "ms"]
