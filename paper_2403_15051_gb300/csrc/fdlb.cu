@@ -2331,9 +2331,9 @@ int fdlb_set_tensor_contraction(fdlb_handle h, int enable, int* in_use) try {
     if (!S) return FDLB_EINVAL;
     S->tensor = enable ? 1 : 0;
     if (S->krf) {
-        // radial orders with a contraction kernel: on the tensor cores (FP32); else, where the stage contracts
-        // by default, in the stage, beyond on the CUDA cores
-        const int by_kernel = S->nR >= fdlb::kKrKernelDefaultNodes || (S->tensor && S->krB) ? 1 : 0;
+        // radial orders with a contraction kernel: enabled, by it (in FP32 on the tensor cores); else, where the
+        // stage contracts by default, in the stage, beyond by the kernel on the CUDA cores
+        const int by_kernel = S->nR >= fdlb::kKrKernelDefaultNodes || S->tensor ? 1 : 0;
         S->kr_tc = S->tensor && S->krB ? 1 : 0;
         if (in_use) *in_use = S->kr_tc;
         if (by_kernel != S->krg_on) {
