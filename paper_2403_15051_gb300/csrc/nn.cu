@@ -12,10 +12,10 @@
 // rounding per fused multiply-add).
 //
 // A batch is a few thousand rows of at most a few hundred channels, so a product is microseconds of work
-// and the passes over memory and launches around it are what counts.  A layer is one launch: 64 rows of a
-// sample to a block, which forms the sample's spectral coefficients from the row tiles' partial transforms
-// (left by the launch before), mixes them, adds the inverse transform to the pointwise product, applies
-// bias and GELU and leaves its own rows' partial transform for the next layer.  The head with the loss is
+// and the passes over memory and launches around it are what counts.  A layer is two launches: 64 rows of a
+// sample to a block, which adds the inverse transform of the sample's mixed modes to the pointwise product,
+// applies bias and GELU and leaves its own rows' partial transform, from which a launch between the layers forms
+// the sample's spectral coefficients and mixes them.  The head with the loss is
 // one launch; the backward pass has the same shape, with GELU's derivative in the epilogue that forms its
 // input; the gradients of every weight matrix but the spectral ones are one launch, split over the rows so
 // that they fill the device (as one product after another, each a single block of 64 x 64 outputs over all
@@ -88,24 +88,54 @@ __device__ __forceinline__ void tile_mma(Tile& t, const float* X, const float* Y
         }
     }
 }
+// The same with X by rows, X[row][k] (kKc values of k): per four k's a vector load of each of the thread's rows,
+// as many as above, and the chunk is staged by vectors instead of transposed by scattered stores (forward pass of
+// width 512, 16 modes, 256 points, batch 64: 2693 -> 2169 us, the weights' chunks by vectors too).
+__device__ __forceinline__ void tile_mma_rows(Tile& t, const float* X, const float* Y) {
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll 4
+    for (int k = 0; k < kKc; k += 4) {
+        float xs[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 x = *reinterpret_cast<const float4*>(X + (ty * 4 + i) * kLd + k);
+            xs[i][0] = x.x; xs[i][1] = x.y; xs[i][2] = x.z; xs[i][3] = x.w;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float4 y = *reinterpret_cast<const float4*>(Y + (k + u) * kLd + tx * 4);
+            const float2 y0 = make_float2(y.x, y.y), y1 = make_float2(y.z, y.w);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                t.a[i][0] = __ffma2_rn(p_splat(xs[i][u]), y0, t.a[i][0]);
+                t.a[i][1] = __ffma2_rn(p_splat(xs[i][u]), y1, t.a[i][1]);
+            }
+        }
+    }
+}
 __device__ __forceinline__ float tile_at(const Tile& t, int i, int j) {
     return j == 0 ? t.a[i][0].x : j == 1 ? t.a[i][0].y : j == 2 ? t.a[i][1].x : t.a[i][1].y;
 }
 
+// Four consecutive values, aligned to their size.
+__device__ __forceinline__ float4 ld_four(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 ld_four(const __nv_bfloat16* p) {
+    const uint2 x = *reinterpret_cast<const uint2*>(p);  // (BF16 is the upper half of FP32)
+    return make_float4(__uint_as_float(x.x << 16), __uint_as_float(x.x & 0xFFFF0000u), __uint_as_float(x.y << 16),
+                       __uint_as_float(x.y & 0xFFFF0000u));
+}
 // dst[k][c] = src[(k0 + k) ld + c0 + c], zero outside k0 + k < kn, c0 + c < cn.
 template <typename TS>
 __device__ __forceinline__ void stage_rows(float* dst, const TS* src, long long ld, long long k0, long long kn, int c0, int cn) {
-    if constexpr (sizeof(TS) == 4) {
-        if ((ld & 3) == 0 && (cn & 3) == 0) {  // (rows start on 16-byte boundaries: the buffers do)
+    if ((ld & 3) == 0 && (cn & 3) == 0 && reinterpret_cast<size_t>(src) % (4 * sizeof(TS)) == 0) {
 #pragma unroll
-            for (int e = threadIdx.x; e < kKc * kT / 4; e += kNT) {
-                const int k = e / (kT / 4), c = e % (kT / 4) * 4;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (k0 + k < kn && c0 + c < cn) v = *reinterpret_cast<const float4*>(src + (k0 + k) * ld + c0 + c);
-                *reinterpret_cast<float4*>(dst + k * kLd + c) = v;
-            }
-            return;
+        for (int e = threadIdx.x; e < kKc * kT / 4; e += kNT) {
+            const int k = e / (kT / 4), c = e % (kT / 4) * 4;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (k0 + k < kn && c0 + c < cn) v = ld_four(src + (k0 + k) * ld + c0 + c);
+            *reinterpret_cast<float4*>(dst + k * kLd + c) = v;
         }
+        return;
     }
 #pragma unroll
     for (int e = threadIdx.x; e < kKc * kT; e += kNT) {
@@ -116,6 +146,20 @@ __device__ __forceinline__ void stage_rows(float* dst, const TS* src, long long 
 // dst[k][r] = src[(r0 + r) ld + k0 + k], zero outside r0 + r < rn, k0 + k < kn (a transposed chunk).
 template <typename TS>
 __device__ __forceinline__ void stage_cols(float* dst, const TS* src, long long ld, long long r0, long long rn, int k0, int kn) {
+    if ((ld & 3) == 0 && (kn & 3) == 0 && reinterpret_cast<size_t>(src) % (4 * sizeof(TS)) == 0) {
+        // (a lane per row: the transposed stores of a warp fall on consecutive banks)
+#pragma unroll
+        for (int e = threadIdx.x; e < kKc * kT / 4; e += kNT) {
+            const int r = e % kT, k = e / kT * 4;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (r0 + r < rn && k0 + k < kn) v = ld_four(src + (r0 + r) * ld + k0 + k);
+            dst[k * kLd + r] = v.x;
+            dst[(k + 1) * kLd + r] = v.y;
+            dst[(k + 2) * kLd + r] = v.z;
+            dst[(k + 3) * kLd + r] = v.w;
+        }
+        return;
+    }
 #pragma unroll
     for (int e = threadIdx.x; e < kKc * kT; e += kNT) {
         const int r = e / kKc, k = e % kKc;
@@ -124,12 +168,11 @@ __device__ __forceinline__ void stage_cols(float* dst, const TS* src, long long 
 }
 
 // Shared memory of the tile kernels: two staged chunks, X and Y, the rows of the basis of the partial
-// transform, [kBasis][64], those of the inverse transform's, [2 kModes][kLd], and the spectral coefficients of a
-// chunk of modes, [2 kModes][W].  An output tile takes X's place, [row][kLd].
+// transform, [kBasis][64], and those of the inverse transform's, [2 kModes][kLd].  An output tile takes X's place,
+// [row][kLd].
 __device__ __forceinline__ float* chunk_y(float* sm) { return sm + kKc * kLd; }
 __device__ __forceinline__ float* basis_of(float* sm) { return sm + 2 * kKc * kLd; }
 __device__ __forceinline__ float* inverse_of(float* sm) { return basis_of(sm) + kBasis * kT; }
-__device__ __forceinline__ float* hats_of(float* sm) { return inverse_of(sm) + 2 * kModes * kLd; }
 
 // Rows k0 .. k0 + nk - 1 of a basis at the tile's rows into bs[k][row]: basis(k, row) at basis[k sk + row sr].
 __device__ __forceinline__ void stage_basis(float* bs, const float* basis, long long sk, long long sr, int k0, int nk, int rows) {
@@ -168,120 +211,146 @@ __device__ __forceinline__ void partial_transform(const float* T, const float* b
     }
 }
 
-// The spectral coefficients of `nm` modes from k0 on, summed over the row tiles' partial transforms in
-// order: hats[q][i] = sum_t part[t][mode row][i], rows q < kModes the real, q >= kModes the imaginary parts;
-// kept in `keep` ([2m][W]) where not null.
-__device__ __forceinline__ void sum_hats(float* hats, const float* part, int nt, int m, int W, int k0, int nm, float* keep) {
-#pragma unroll 4
-    for (int e = threadIdx.x; e < 2 * nm * W; e += kNT) {
-        const int q = e / W, i = e % W, im = q >= nm, row = (im ? m : 0) + k0 + (im ? q - nm : q);
-        const float* p = part + (long long)row * W + i;
-        const long long st = 2LL * m * W;
-        float s = 0.f;
-        int t = 0;
-        for (; t + 4 <= nt; t += 4) {
-            const float a = p[t * st], b = p[(t + 1) * st], c = p[(t + 2) * st], d = p[(t + 3) * st];
-            s = (((s + a) + b) + c) + d;
-        }
-        for (; t < nt; ++t) s += p[t * st];
-        hats[((im ? kModes : 0) + (im ? q - nm : q)) * W + i] = s;
-        if (keep) keep[(long long)row * W + i] = s;
+// A value of the row tiles' partial transforms (stride st), added in order.
+__device__ __forceinline__ float sum_parts(const float* p, long long st, int nt) {
+    float s = 0.f;
+    int t = 0;
+    for (; t + 4 <= nt; t += 4) {
+        const float a = p[t * st], b = p[(t + 1) * st], c = p[(t + 2) * st], d = p[(t + 3) * st];
+        s = (((s + a) + b) + c) + d;
     }
+    for (; t < nt; ++t) s += p[t * st];
+    return s;
 }
-
-// The modes' complex mixing into the chunk Y: rows 0 .. nm-1 the real, nm .. 2 nm - 1 the imaginary parts of
-// column n0 + c.  yre = re Rre - im Rim, yim = re Rim + im Rre: a thread per column and quarter of the inputs,
-// the quarters added through `scratch` ([4][2 nm][64], over X and Y; the caller has synchronised).
-__device__ __forceinline__ void mix_forward(float* Y, float* scratch, const float* hats, const __nv_bfloat16* Rre,
-                                            const __nv_bfloat16* Rim, int W, int k0, int nm, int n0) {
-    const int c = threadIdx.x % kT, g = threadIdx.x / kT, col = min(n0 + c, W - 1);
-    // (four quarters of 2 nm rows fit over the chunks for nm <= 17: at most 16 modes at a time)
-#pragma unroll 2
-    for (int q = 0; q < nm; ++q) {
-        const __nv_bfloat16* a = Rre + (long long)(k0 + q) * W * W + col;
-        const __nv_bfloat16* b = Rim + (long long)(k0 + q) * W * W + col;
-        float yr = 0.f, yi = 0.f;
-        for (int i0 = g; i0 < W; i0 += kT) {
-            __nv_bfloat16 ra[kT / 4], rb[kT / 4];
+// The modes' complex mixing of a layer: a mode, 64 columns and kMixB samples to a block, which sums their
+// spectral coefficients from the row tiles' partial transforms (kept in `keep`) and reads the mode's weights
+// once for all of them; forward yre = re Rre - im Rim, yim = re Rim + im Rre, a thread per column and quarter of
+// the inputs; backward dre = dyre Rre^T + dyim Rim^T, dim = dyim Rre^T - dyre Rim^T, eight lanes per row of R.
+// Bound by the latency of its loads on small networks, by FP32 issue on wide ones.  A launch of its own: mixed
+// inside the layer kernels, by every row tile of a sample and every sample again, it was most of a layer on wide
+// networks (us per forward pass, inside and apart, and at the last the tensor-core products that came before:
+// width 64, 6 modes, 256 points, batch 64: 147 and 124; 128, 12, 256, 32: 303 and 214; 512, 4, 64, 16: 659 and 564;
+// 256, 32, 512, 64: 6693, 1598 and 1866; 512, 32, 512, 32: 20979, 2549 and 2762).
+constexpr int kMixB = 8;
+// Shared memory: the coefficients, forward [re, im][i][kMixB], backward [sample][re, im][W]; forward also the
+// quarters' sums [4][2 kMixB][64].  y: [sample][2m][W].
+template <bool kBack>
+__global__ void __launch_bounds__(kNT) mix_kernel(const float* __restrict__ part, int nt, int B, int W, int m,
+                                                  const __nv_bfloat16* __restrict__ Rre, const __nv_bfloat16* __restrict__ Rim,
+                                                  float* __restrict__ keep, float* __restrict__ y) {
+    extern __shared__ __align__(16) float sm[];
+    const int q = blockIdx.x, n0 = blockIdx.y * kT, b0 = blockIdx.z * kMixB, nb = min(kMixB, B - b0);
+    const long long hat = 2LL * m * W;  // of a sample
+    nn_begin();
+    for (int e = threadIdx.x; e < 2 * kMixB * W; e += kNT) {
+        const int i = e % W, im = e / W % 2, s = e / (2 * W);
+        const long long row = (long long)(im ? m + q : q) * W + i;
+        float v = 0.f;
+        if (s < nb) {
+            v = sum_parts(part + (b0 + s) * nt * hat + row, hat, nt);
+            if (blockIdx.y == 0) keep[(b0 + s) * hat + row] = v;
+        }
+        sm[kBack ? (s * 2 + im) * W + i : (im * W + i) * kMixB + s] = v;
+    }
+    __syncthreads();
+    if constexpr (!kBack) {
+        float* scratch = sm + 2 * kMixB * W;
+        const int c = threadIdx.x % kT, g = threadIdx.x / kT, col = min(n0 + c, W - 1);
+        const __nv_bfloat16 *a = Rre + (long long)q * W * W + col, *b = Rim + (long long)q * W * W + col;
+        float yr[kMixB], yi[kMixB];
 #pragma unroll
-            for (int u = 0; u < kT / 4; ++u) {
-                const int i = min(i0 + 4 * u, W - 1);
-                ra[u] = a[(long long)i * W];
-                rb[u] = b[(long long)i * W];
-            }
+        for (int s = 0; s < kMixB; ++s) yr[s] = yi[s] = 0.f;
+#pragma unroll 4
+        for (int i = g; i < W; i += 4) {
+            const float fa = to_f(a[(long long)i * W]), fb = to_f(b[(long long)i * W]);
 #pragma unroll
-            for (int u = 0; u < kT / 4; ++u) {
-                const int i = i0 + 4 * u;
-                if (i < W) {
-                    const float re = hats[q * W + i], im = hats[(kModes + q) * W + i], fa = to_f(ra[u]), fb = to_f(rb[u]);
-                    yr = fmaf(re, fa, fmaf(-im, fb, yr));
-                    yi = fmaf(re, fb, fmaf(im, fa, yi));
+            for (int h = 0; h < kMixB; h += 4) {
+                const float4 r4 = *reinterpret_cast<const float4*>(sm + i * kMixB + h);
+                const float4 i4 = *reinterpret_cast<const float4*>(sm + (W + i) * kMixB + h);
+                const float re[4] = {r4.x, r4.y, r4.z, r4.w}, im[4] = {i4.x, i4.y, i4.z, i4.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    yr[h + u] = fmaf(re[u], fa, fmaf(-im[u], fb, yr[h + u]));
+                    yi[h + u] = fmaf(re[u], fb, fmaf(im[u], fa, yi[h + u]));
                 }
             }
         }
-        scratch[(g * 2 * nm + q) * kT + c] = yr;
-        scratch[(g * 2 * nm + nm + q) * kT + c] = yi;
-    }
-    __syncthreads();
-    float v[2 * kModes * kT / kNT];
 #pragma unroll
-    for (int h = 0; h < 2 * kModes * kT / kNT; ++h) {
-        const int e = threadIdx.x + h * kNT;
-        if (e < 2 * nm * kT) {
-            const int st = 2 * nm * kT;
-            v[h] = (scratch[e] + scratch[st + e]) + (scratch[2 * st + e] + scratch[3 * st + e]);
+        for (int s = 0; s < kMixB; ++s) {
+            scratch[(g * 2 * kMixB + 2 * s) * kT + c] = yr[s];
+            scratch[(g * 2 * kMixB + 2 * s + 1) * kT + c] = yi[s];
         }
-    }
-    __syncthreads();
+        __syncthreads();
+        for (int e = threadIdx.x; e < 2 * nb * kT; e += kNT) {
+            const int st = 2 * kMixB * kT, cc = e % kT, r = e / kT;
+            const float v = (scratch[e] + scratch[st + e]) + (scratch[2 * st + e] + scratch[3 * st + e]);
+            if (n0 + cc < W) y[(b0 + r / 2) * hat + (long long)(r % 2 ? m + q : q) * W + n0 + cc] = v;
+        }
+    } else {
+        const int sub = threadIdx.x & 7;
+        for (int c = threadIdx.x >> 3; c < kT; c += kNT / 8) {
+            float dr[kMixB], di[kMixB];
 #pragma unroll
-    for (int h = 0; h < 2 * kModes * kT / kNT; ++h) {
-        const int e = threadIdx.x + h * kNT;
-        if (e < 2 * nm * kT) Y[e / kT * kLd + e % kT] = n0 + e % kT < W ? v[h] : 0.f;
-    }
-}
-
-// The backward mixing into Y: dre = dyre Rre^T + dyim Rim^T, dim = dyim Rre^T - dyre Rim^T, column n0 + c
-// being row n0 + c of R: eight lanes per row, eight outputs a lane at a time.
-__device__ __forceinline__ void mix_backward(float* Y, const float* hats, const __nv_bfloat16* Rre, const __nv_bfloat16* Rim, int W,
-                                             int k0, int nm, int n0) {
-    const int sub = threadIdx.x & 7;
-    for (int e0 = 0; e0 < nm * kT; e0 += kNT / 8) {
-        const int e = e0 + (threadIdx.x >> 3), q = min(e / kT, nm - 1), c = e % kT;
-        float dr = 0.f, di = 0.f;
-        if (e < nm * kT && n0 + c < W) {
-            const __nv_bfloat16* a = Rre + ((long long)(k0 + q) * W + n0 + c) * W;
-            const __nv_bfloat16* b = Rim + ((long long)(k0 + q) * W + n0 + c) * W;
-            const float *re = hats + q * W, *im = hats + (kModes + q) * W;
-            if (W % 8 == 0) {  // (rows of eight BF16 values start on 16-byte boundaries)
-#pragma unroll 2
-                for (int o = sub * 8; o < W; o += 64) {
-                    const uint4 xa = *reinterpret_cast<const uint4*>(a + o), xb = *reinterpret_cast<const uint4*>(b + o);
-                    const uint32_t ua[4] = {xa.x, xa.y, xa.z, xa.w}, ub[4] = {xb.x, xb.y, xb.z, xb.w};
+            for (int s = 0; s < kMixB; ++s) dr[s] = di[s] = 0.f;
+            if (n0 + c < W) {
+                const __nv_bfloat16 *a = Rre + ((long long)q * W + n0 + c) * W, *b = Rim + ((long long)q * W + n0 + c) * W;
+                if (W % 8 == 0) {  // (rows of eight BF16 values start on 16-byte boundaries)
+                    for (int o = sub * 8; o < W; o += 64) {
+                        const uint4 xa = *reinterpret_cast<const uint4*>(a + o), xb = *reinterpret_cast<const uint4*>(b + o);
+                        const uint32_t ua[4] = {xa.x, xa.y, xa.z, xa.w}, ub[4] = {xb.x, xb.y, xb.z, xb.w};
 #pragma unroll
-                    for (int h = 0; h < 8; ++h) {
-                        const float fa = __uint_as_float(h & 1 ? ua[h / 2] & 0xFFFF0000u : ua[h / 2] << 16);
-                        const float fb = __uint_as_float(h & 1 ? ub[h / 2] & 0xFFFF0000u : ub[h / 2] << 16);
-                        dr = fmaf(re[o + h], fa, fmaf(im[o + h], fb, dr));
-                        di = fmaf(im[o + h], fa, fmaf(-re[o + h], fb, di));
+                        for (int s = 0; s < kMixB; ++s)
+#pragma unroll
+                            for (int h = 0; h < 8; h += 4) {
+                                const float4 r4 = *reinterpret_cast<const float4*>(sm + 2 * s * W + o + h);
+                                const float4 i4 = *reinterpret_cast<const float4*>(sm + (2 * s + 1) * W + o + h);
+                                const float re[4] = {r4.x, r4.y, r4.z, r4.w}, im[4] = {i4.x, i4.y, i4.z, i4.w};
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) {
+                                    const uint32_t wa = ua[(h + u) / 2], wb = ub[(h + u) / 2];
+                                    const float fa = __uint_as_float(u & 1 ? wa & 0xFFFF0000u : wa << 16);
+                                    const float fb = __uint_as_float(u & 1 ? wb & 0xFFFF0000u : wb << 16);
+                                    dr[s] = fmaf(re[u], fa, fmaf(im[u], fb, dr[s]));
+                                    di[s] = fmaf(im[u], fa, fmaf(-re[u], fb, di[s]));
+                                }
+                            }
+                    }
+                } else {
+                    for (int o = sub; o < W; o += 8) {
+                        const float fa = to_f(a[o]), fb = to_f(b[o]);
+#pragma unroll
+                        for (int s = 0; s < kMixB; ++s) {
+                            const float re = sm[2 * s * W + o], im = sm[(2 * s + 1) * W + o];
+                            dr[s] = fmaf(re, fa, fmaf(im, fb, dr[s]));
+                            di[s] = fmaf(im, fa, fmaf(-re, fb, di[s]));
+                        }
                     }
                 }
-            } else {
-                for (int o = sub; o < W; o += 8) {
-                    const float fa = to_f(a[o]), fb = to_f(b[o]);
-                    dr = fmaf(re[o], fa, fmaf(im[o], fb, dr));
-                    di = fmaf(im[o], fa, fmaf(-re[o], fb, di));
+            }
+#pragma unroll
+            for (int s = 0; s < kMixB; ++s) {
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) {
+                    dr[s] += __shfl_xor_sync(0xffffffffu, dr[s], o);
+                    di[s] += __shfl_xor_sync(0xffffffffu, di[s], o);
+                }
+                if (sub == 0 && s < nb && n0 + c < W) {
+                    y[(b0 + s) * hat + (long long)q * W + n0 + c] = dr[s];
+                    y[(b0 + s) * hat + (long long)(m + q) * W + n0 + c] = di[s];
                 }
             }
         }
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) {
-            dr += __shfl_xor_sync(0xffffffffu, dr, o);
-            di += __shfl_xor_sync(0xffffffffu, di, o);
-        }
-        if (sub == 0 && e < nm * kT) {
-            Y[q * kLd + c] = dr;
-            Y[(nm + q) * kLd + c] = di;
-        }
+    }
+}
+size_t mix_smem(int W, bool back) { return ((size_t)2 * kMixB * W + (back ? 0 : 4 * 2 * kMixB * kT)) * sizeof(float); }
+
+// `nm` mixed modes of a sample from k0 on into the chunk Y: rows 0 .. nm-1 the real, nm .. 2 nm - 1 the imaginary
+// parts of column n0 + c.
+__device__ __forceinline__ void stage_mixed(float* Y, const float* yh, int W, int m, int k0, int nm, int n0) {
+#pragma unroll 4
+    for (int e = threadIdx.x; e < 2 * nm * kT; e += kNT) {
+        const int q = e / kT, c = e % kT, row = q < nm ? k0 + q : m + k0 + q - nm;
+        Y[q * kLd + c] = n0 + c < W ? yh[(long long)row * W + n0 + c] : 0.f;
     }
 }
 
@@ -324,16 +393,14 @@ __global__ void __launch_bounds__(kNT) lift_kernel(const float* __restrict__ raw
     partial_transform(sm, F + r0, P, 1, 2 * m, rows, n0, W, basis_of(sm), part + ((long long)b * gridDim.x + blockIdx.x) * 2 * m * W);
 }
 
-// 64 rows of one sample (grid: row tiles, samples, column tiles) through a layer.
-// Forward: u = v W + b + G yh, vout = GELU(u); hat: the layer's spectral coefficients, kept for the
-// gradients; part_out (or null): the partial transform of vout.
-__global__ void __launch_bounds__(kNT) layer_kernel(const float* __restrict__ v, const float* __restrict__ part_in, int P, int W, int m,
+// 64 rows of one sample (grid: row tiles, samples, column tiles) through a layer.  yh: its mixed modes.
+// Forward: u = v W + b + G yh, vout = GELU(u); part_out (or null): the partial transform of vout.
+__global__ void __launch_bounds__(kNT) layer_kernel(const float* __restrict__ v, const float* __restrict__ yh, int P, int W, int m,
                                                     const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
-                                                    const __nv_bfloat16* __restrict__ Rre, const __nv_bfloat16* __restrict__ Rim,
-                                                    const float* __restrict__ F, const float* __restrict__ G, float* __restrict__ hat,
+                                                    const float* __restrict__ F, const float* __restrict__ G,
                                                     float* __restrict__ u, float* __restrict__ vout, float* __restrict__ part_out) {
     extern __shared__ __align__(16) float sm[];
-    float *X = sm, *Y = chunk_y(sm), *Gs = inverse_of(sm), *hats = hats_of(sm);
+    float *X = sm, *Y = chunk_y(sm), *Gs = inverse_of(sm);
     const int nt = gridDim.x, r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT;
     stage_rows(Y, w, W, 0, W, n0, W);
     if (part_out) stage_basis(basis_of(sm), F + r0, P, 1, 0, min(kBasis, 2 * m), min(kT, P - r0));
@@ -348,19 +415,16 @@ __global__ void __launch_bounds__(kNT) layer_kernel(const float* __restrict__ v,
     Tile t;
     tile_zero(t);
     for (int k0 = 0; k0 < W; k0 += kKc) {
-        stage_cols(X, v + (long long)b * P * W, W, r0, P, k0, W);
+        stage_rows(X, v + (long long)b * P * W, W, r0, P, k0, W);
         if (k0 > 0) stage_rows(Y, w, W, k0, W, n0, W);
         __syncthreads();
-        tile_mma(t, X, Y);
+        tile_mma_rows(t, X, Y);
         __syncthreads();
     }
     for (int k0 = 0; k0 < m; k0 += kModes) {
         const int nm = min(kModes, m - k0);
-        sum_hats(hats, part_in + (long long)b * nt * 2 * m * W, nt, m, W, k0, nm,
-                 blockIdx.x == 0 && blockIdx.z == 0 ? hat + (long long)b * 2 * m * W : nullptr);
         if (k0 > 0) inverse_basis(k0, nm);
-        __syncthreads();
-        mix_forward(Y, sm, hats, Rre, Rim, W, k0, nm, n0);
+        stage_mixed(Y, yh + (long long)b * 2 * m * W, W, m, k0, nm, n0);
         __syncthreads();
         tile_mma(t, Gs, Y, 1.f, 2 * nm);
         __syncthreads();
@@ -386,16 +450,14 @@ __global__ void __launch_bounds__(kNT) layer_kernel(const float* __restrict__ v,
                           part_out + ((long long)b * nt + blockIdx.x) * 2 * m * W);
 }
 
-// Backward: dv = du W^T + F^T dvh, and into `out` dv GELU'(u) (in place of u, the layer below's du) with its
+// Backward: dv = du W^T + F^T yh, and into `out` dv GELU'(u) (in place of u, the layer below's du) with its
 // partial transform by G^T, or dv itself where u is null.
-__global__ void __launch_bounds__(kNT) layer_back_kernel(const float* __restrict__ du, const float* __restrict__ part_in, int P, int W,
-                                                         int m, const __nv_bfloat16* __restrict__ w,
-                                                         const __nv_bfloat16* __restrict__ Rre, const __nv_bfloat16* __restrict__ Rim,
-                                                         const float* __restrict__ F, const float* __restrict__ G,
-                                                         float* __restrict__ hat, const float* u, float* out,
+__global__ void __launch_bounds__(kNT) layer_back_kernel(const float* __restrict__ du, const float* __restrict__ yh, int P, int W, int m,
+                                                         const __nv_bfloat16* __restrict__ w, const float* __restrict__ F,
+                                                         const float* __restrict__ G, const float* u, float* out,
                                                          float* __restrict__ part_out) {
     extern __shared__ __align__(16) float sm[];
-    float *X = sm, *Y = chunk_y(sm), *Fs = inverse_of(sm), *hats = hats_of(sm);
+    float *X = sm, *Y = chunk_y(sm), *Fs = inverse_of(sm);
     const int nt = gridDim.x, r0 = blockIdx.x * kT, b = blockIdx.y, n0 = blockIdx.z * kT;
     stage_cols(Y, w, W, n0, W, 0, W);
     if (part_out) stage_basis(basis_of(sm), G + (long long)r0 * 2 * m, 1, 2 * m, 0, min(kBasis, 2 * m), min(kT, P - r0));
@@ -410,19 +472,16 @@ __global__ void __launch_bounds__(kNT) layer_back_kernel(const float* __restrict
     Tile t;
     tile_zero(t);
     for (int k0 = 0; k0 < W; k0 += kKc) {
-        stage_cols(X, du + (long long)b * P * W, W, r0, P, k0, W);
+        stage_rows(X, du + (long long)b * P * W, W, r0, P, k0, W);
         if (k0 > 0) stage_cols(Y, w, W, n0, W, k0, W);
         __syncthreads();
-        tile_mma(t, X, Y);
+        tile_mma_rows(t, X, Y);
         __syncthreads();
     }
     for (int k0 = 0; k0 < m; k0 += kModes) {
         const int nm = min(kModes, m - k0);
-        sum_hats(hats, part_in + (long long)b * nt * 2 * m * W, nt, m, W, k0, nm,
-                 blockIdx.x == 0 && blockIdx.z == 0 ? hat + (long long)b * 2 * m * W : nullptr);
         if (k0 > 0) inverse_basis(k0, nm);
-        __syncthreads();
-        mix_backward(Y, hats, Rre, Rim, W, k0, nm, n0);
+        stage_mixed(Y, yh + (long long)b * 2 * m * W, W, m, k0, nm, n0);
         __syncthreads();
         tile_mma(t, Fs, Y, 1.f, 2 * nm);
         __syncthreads();
@@ -469,10 +528,10 @@ __global__ void __launch_bounds__(kNT) head_kernel(const float* __restrict__ v, 
         Tile t;
         tile_zero(t);
         for (int k0 = 0; k0 < W; k0 += kKc) {
-            if (W > kKc || n0 == 0) stage_cols(X, v, W, r0, rows, k0, W);  // (one chunk: staged once)
+            if (W > kKc || n0 == 0) stage_rows(X, v, W, r0, rows, k0, W);  // (one chunk: staged once)
             if (n0 > 0 || k0 > 0) stage_rows(Y, p1, H, k0, W, n0, H);
             __syncthreads();
-            tile_mma(t, X, Y);
+            tile_mma_rows(t, X, Y);
             __syncthreads();
         }
 #pragma unroll
@@ -559,11 +618,11 @@ __global__ void __launch_bounds__(kNT) head_back_kernel(const float* __restrict_
                 d = s * gelu_grad_f(z);
                 if (blockIdx.z == 0) dz[(base + rr) * H + col] = d;
             }
-            X[k * kLd + rr] = d;
+            X[rr * kLd + k] = d;
         }
         if (k0 > 0) stage_cols(Y, p1, H, n0, W, k0, H);
         __syncthreads();
-        tile_mma(t, X, Y);
+        tile_mma_rows(t, X, Y);
         __syncthreads();
     }
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -741,6 +800,7 @@ struct NNet {
     float *raw = nullptr, *a = nullptr, *vs = nullptr, *us = nullptr, *vh = nullptr;
     float *z1 = nullptr, *dz = nullptr, *h = nullptr, *out = nullptr, *tgt = nullptr, *dout = nullptr;
     float *dv = nullptr, *dyh = nullptr, *loss = nullptr, *part = nullptr;
+    float* yh = nullptr;                      // a layer's mixed modes
     float* hat_part[2] = {nullptr, nullptr};  // the row tiles' partial transforms, of a layer and the next
     double* loss_part = nullptr;
     long long n_rows_params = 0;  // parameters without the spectral weights
@@ -770,7 +830,13 @@ void nn_launch(NNet& n, void (*kern)(KA...), dim3 grid, size_t smem, A... args) 
 unsigned tiles(long long n) { return (unsigned)((n + kT - 1) / kT); }
 constexpr size_t kChunks = 2 * (size_t)kKc * kLd * sizeof(float);  // shared memory of two staged chunks
 constexpr size_t kTileSmem = kChunks + (size_t)kBasis * kT * sizeof(float);
-size_t layer_smem(int W) { return kTileSmem + 2 * (size_t)kModes * (kLd + W) * sizeof(float); }
+constexpr size_t kLayerSmem = kTileSmem + 2 * (size_t)kModes * kLd * sizeof(float);
+// The mixing of layer l: its coefficients into `keep`, the mixed modes into n.yh.
+template <bool kBack>
+void launch_mix(NNet& n, int B, int l, float* keep) {
+    nn_launch(n, mix_kernel<kBack>, dim3(n.m, tiles(n.W), (B + kMixB - 1) / kMixB), mix_smem(n.W, kBack), n.hat_part[l & 1],
+              (int)tiles(n.P), B, n.W, n.m, n.wb + n.o_rre[l], n.wb + n.o_rim[l], keep, n.yh);
+}
 int grad_splits(long long rows) { return (int)std::min<long long>((rows + 127) / 128, kMaxSplits); }
 
 // Forward pass for B samples whose raw parameters are in n.raw; for training (targets in n.tgt) leaves every
@@ -782,8 +848,8 @@ int forward(NNet& n, int B, bool train) {
     nn_launch(n, lift_kernel, grid, kTileSmem, n.raw, P, W, m, n.wb + n.o_lw, n.w + n.o_lb, n.F, n.a, n.vs, n.hat_part[0]);
     for (int l = 0; l < n.L; ++l) {
         float* v = n.vs + (long long)l * rows * W;
-        nn_launch(n, layer_kernel, grid, layer_smem(W), v, n.hat_part[l & 1], P, W, m, n.wb + n.o_w[l], n.w + n.o_b[l],
-                  n.wb + n.o_rre[l], n.wb + n.o_rim[l], n.F, n.G, n.vh + (long long)l * B * 2 * m * W,
+        launch_mix<false>(n, B, l, n.vh + (long long)l * B * 2 * m * W);
+        nn_launch(n, layer_kernel, grid, kLayerSmem, v, n.yh, P, W, m, n.wb + n.o_w[l], n.w + n.o_b[l], n.F, n.G,
                   n.us + (long long)l * rows * W, v + rows * W, l + 1 < n.L ? n.hat_part[(l + 1) & 1] : nullptr);
     }
     nn_launch(n, head_kernel, dim3(tiles(rows)), kChunks, n.vs + (long long)n.L * rows * W, rows, W, H, n.wb + n.o_p1w, n.w + n.o_p1b,
@@ -801,9 +867,9 @@ int backward(NNet& n, int B) {
               n.hat_part[(L - 1) & 1]);
     for (int l = L - 1; l >= 0; --l) {
         float* below = l > 0 ? us(l - 1) : nullptr;
-        nn_launch(n, layer_back_kernel, grid, layer_smem(W), us(l), n.hat_part[l & 1], P, W, m, n.wb + n.o_w[l], n.wb + n.o_rre[l],
-                  n.wb + n.o_rim[l], n.F, n.G, n.dyh + l * hat, below, l > 0 ? below : n.dv,
-                  l > 0 ? n.hat_part[(l - 1) & 1] : nullptr);
+        launch_mix<true>(n, B, l, n.dyh + l * hat);
+        nn_launch(n, layer_back_kernel, grid, kLayerSmem, us(l), n.yh, P, W, m, n.wb + n.o_w[l], n.F, n.G, below,
+                  l > 0 ? below : n.dv, l > 0 ? n.hat_part[(l - 1) & 1] : nullptr);
     }
     GradTasks T{};
     int tile = 0;
@@ -886,6 +952,7 @@ int fdlb_nn_create(int width, int modes, int layers, int hidden, int n_points, i
         {(void**)&n->G, (size_t)2 * modes * n_points * 4}, {(void**)&n->raw, (size_t)max_batch * 5 * 4},
         {(void**)&n->a, rows * fdlb::kCin * 4}, {(void**)&n->vs, (size_t)(layers + 1) * rows * W * 4},
         {(void**)&n->us, (size_t)layers * rows * W * 4}, {(void**)&n->vh, (size_t)layers * max_batch * 2 * modes * W * 4},
+        {(void**)&n->yh, (size_t)max_batch * 2 * modes * W * 4},
         {(void**)&n->hat_part[0], (size_t)max_batch * fdlb::tiles(n_points) * 2 * modes * W * 4},
         {(void**)&n->hat_part[1], (size_t)max_batch * fdlb::tiles(n_points) * 2 * modes * W * 4},
         {(void**)&n->z1, rows * hidden * 4}, {(void**)&n->dz, rows * hidden * 4},
@@ -905,8 +972,8 @@ int fdlb_nn_create(int width, int modes, int layers, int hidden, int n_points, i
         *b.first = n->ws + o;
         o += (b.second + 255) / 256 * 256;
     }
-    // dynamic shared memory beyond the default limit (a function's limit is the process's: the widest network's)
-    const int layer_sm = (int)fdlb::layer_smem(fdlb::kMaxWidth), two = (int)(2 * fdlb::kChunks);
+    // dynamic shared memory beyond the default limit (a function's limit is the process's: one size for all networks)
+    const int layer_sm = (int)fdlb::kLayerSmem, two = (int)(2 * fdlb::kChunks);
     if (cudaFuncSetAttribute(fdlb::layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, layer_sm) != cudaSuccess ||
         cudaFuncSetAttribute(fdlb::layer_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, layer_sm) != cudaSuccess ||
         cudaFuncSetAttribute(fdlb::grad_spectral_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, two) != cudaSuccess) {
