@@ -837,7 +837,14 @@ void launch_mix(NNet& n, int B, int l, float* keep) {
     nn_launch(n, mix_kernel<kBack>, dim3(n.m, tiles(n.W), (B + kMixB - 1) / kMixB), mix_smem(n.W, kBack), n.hat_part[l & 1],
               (int)tiles(n.P), B, n.W, n.m, n.wb + n.o_rre[l], n.wb + n.o_rim[l], keep, n.yh);
 }
-int grad_splits(long long rows) { return (int)std::min<long long>((rows + 127) / 128, kMaxSplits); }
+// Splits of the rows in the weight gradients: enough that the tiles of every matrix make sixteen blocks for each
+// of 152 SMs, whose last wave is then short (four per SM: 3 to 5% more time per training step at widths 256 and
+// 512), and no more: each split is a copy of the parameters in the workspace (64 of them were 1.2 GB for 16 layers
+// of 512 channels).
+int grad_splits(long long rows, int W, int H, int L) {
+    const long long all = tiles(W) + (long long)L * tiles(W) * tiles(W) + tiles(W) * tiles(H) + tiles(H);
+    return (int)std::min<long long>(std::min<long long>((rows + 127) / 128, kMaxSplits), (16 * 152 + all - 1) / all);
+}
 
 // Forward pass for B samples whose raw parameters are in n.raw; for training (targets in n.tgt) leaves every
 // activation the backward pass needs, dout and the loss's parts.
@@ -883,7 +890,7 @@ int backward(NNet& n, int B) {
     for (int l = 0; l < L; ++l) task(n.vs + (long long)l * rows * W, W, us(l), W);
     task(n.vs + (long long)L * rows * W, W, n.dz, H);
     task(n.h, H, n.dout, kCout);
-    const int splits = grad_splits(rows);
+    const int splits = grad_splits(rows, W, H, L);
     nn_launch(n, grad_kernel, dim3(tile, splits), kChunks, T, rows, splits, n.part, n.n_rows_params);
     const long long spectral = 2LL * m * W * W, per_layer = (long long)W * W + W;
     nn_launch(n, grad_spectral_kernel, dim3(L * m, tiles(W), tiles(W)), 2 * kChunks, n.vh, n.dyh, B, W, m, n.g, n.o_rre[0],
@@ -959,7 +966,7 @@ int fdlb_nn_create(int width, int modes, int layers, int hidden, int n_points, i
         {(void**)&n->h, rows * hidden * 4}, {(void**)&n->out, rows * fdlb::kCout * 4},
         {(void**)&n->tgt, rows * fdlb::kCout * 4}, {(void**)&n->dout, rows * fdlb::kCout * 4}, {(void**)&n->dv, rows * W * 4},
         {(void**)&n->dyh, (size_t)layers * max_batch * 2 * modes * W * 4},
-        {(void**)&n->part, (size_t)fdlb::grad_splits(rows) * n->n_rows_params * 4},
+        {(void**)&n->part, (size_t)fdlb::grad_splits(rows, W, hidden, layers) * n->n_rows_params * 4},
         {(void**)&n->loss_part, (size_t)((rows + fdlb::kT - 1) / fdlb::kT) * 8}, {(void**)&n->loss, 256}};
     size_t total = 0;
     for (auto& b : bufs) total += (b.second + 255) / 256 * 256;

@@ -60,3 +60,18 @@ def test_a_wide_network_runs_at_the_arithmetic_rate():
     net.close()
     flops = 2.0 * B * P * (6 * W + L * W * W + W * H + 4 * H) + L * (2 * 2.0 * B * 2 * m * W * P + 8.0 * B * m * W * W)
     assert flops / best > 0.1 * 1e12 * fdlb.fp32_fma_peak()[0]
+
+
+def test_a_wide_networks_workspace_is_its_activations_and_parameters():
+    # the activations of the passes, four parameter vectors and the BF16 copy; the rest (bases, spectral
+    # coefficients, the splits of the weight gradients) a few dozen megabytes
+    torch = pytest.importorskip("torch")
+    W, m, L, H, P, B = 512, 2, 16, 512, 256, 64
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    net = fdlb.WarmStartNet(W, m, L, H, P, max_batch=B)
+    used = free - torch.cuda.mem_get_info()[0]
+    lay, n = onn.layout(W, m, L, H)
+    need = 18 * n + 4 * B * P * ((2 * L + 2) * W + 3 * H + 3 * 4 + 6)
+    net.close()
+    assert used <= need + (128 << 20)
