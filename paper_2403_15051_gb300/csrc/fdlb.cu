@@ -24,10 +24,12 @@ constexpr double kPiH = 3.14159265358979323846;
 constexpr size_t kAlign = 256;
 // Radial node counts from which the K^h contraction can run as its own kernel (the fused stage then
 // reads K^h f), and from which it does by default: below, the stage contracts from a K^h table in shared
-// memory.  At 40 nodes the kernel's launch and its pass over f cost more than the 40 multiply-adds it
-// takes off the stage (step of 240 cells x 2560 momenta 63 us against 81, of 1000 cells 154 against 212, of
-// 96 cells x 640 momenta 36 against 70; FP64 488 either way).  Beyond 48 nodes the table itself and,
-// in FP32, the range of K^h (entries as sqrt(w_i / w_a), the weights below 1e-30) speak for the kernel.
+// memory.  Up to 48 nodes the kernel's launch and its pass over f cost more than the multiply-adds it takes off
+// the stage (us per step, in the stage and by the kernel: FP32 240 cells x 40 x 8 x 8 momenta 56 and 85, 48 x 8 x 8
+// 60 and 90, 1000 cells 147 and 228, 96 cells x 48 x 4 x 4 37 and 68, between spheres 39 and 70; FP64 240 cells x
+// 40 x 8 x 8 821 and 999, 48 x 8 x 8 1007 and 1127, 96 cells x 48 x 4 x 4 191 and 353; FP64 32 x 4 x 4 on 240 cells
+// 312 and 302 the one exception of 46).  Beyond 48 nodes the table itself and, in FP32, the range of K^h (entries
+// as sqrt(w_i / w_a), the weights below 1e-30) speak for the kernel.
 constexpr int kKrKernelMinNodes = 32;
 constexpr int kKrKernelDefaultNodes = 50;
 
@@ -96,7 +98,8 @@ struct Solver {
     int step_B = 0;               // persistent step kernel: cells of its staged tiles
     int use_bulk = 0;
     int closure_cells = 4, closure_threads = 128;  // own cells per closure item (<= kClosureCells)
-    int closure_batch = 0;  // the closure as two launches over all items (items of kClosureCells cells)
+    int closure_batch = 0;  // the closure in its batch form: a warp per item (of up to kClosureCells cells), the bands
+                            // in the same launch or, wider than kInlineBandMax columns, in one before it
     int wall_parts = kWallParts;  // closure work items per wall
     int autotune_mode = 1;  // 0 off; 1 tune on the first step of a batch; 2 also of a single instance
     int stall_checks = 0;   // run_to_steady: checks without halving the best residual before an instance stops
@@ -1404,7 +1407,7 @@ int run_autotune(Solver& S, bool use_cache) {
     S.stage_minb = bestM;
     S.tile_asked = bestAsked;
     rc = configure_tiling(S, bestB, 0, 0);
-    // the closure: the chain form with items of C cells, or the batch form (two launches)
+    // the closure: the chain form with items of C cells, or the batch form
     const int Cs[] = {2, 4, 8, 16};
     for (int C : Cs) {
         if (rc || (C == bestC && !bestBatch)) continue;
